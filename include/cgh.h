@@ -16,9 +16,11 @@
  * (Section 4.1: adr = j + WIDTH * i).
  *
  * Two forms compute the same sum:
- *   - direct: per pixel and per point, the phase is built incrementally in
- *     exact 32/64-bit fixed-point turns (the recurrence of Eqs. 6-8,
- *     Section 2.2) and fed to a single-precision cosine;
+ *   - direct: the turns of a point's columns and rows in a tile of pixels are
+ *     built in exact 32/64-bit fixed point (the recurrence of Eqs. 6-8,
+ *     Section 2.2); their sines and cosines, taken once per tile in single
+ *     precision, are multiplied and summed on the tensor cores as hi+lo FP16
+ *     pairs with short FP32 accumulation chains (NRMS about 3.5e-7);
  *   - separable GEMM: exp(i phi) factors exactly into a column term and a row
  *     term, so I = P Q^T with P [height][2N] and Q [width][2N]; the product
  *     runs on the tcgen05 tensor cores in FP16, BF16 or split hi+lo FP16 with
@@ -68,8 +70,9 @@ enum {
 /* How the hologram is computed. */
 enum {
     CGH_FORM_AUTO = 0,          /* autotuner's choice for the accuracy class */
-    CGH_DIRECT_SFU = 1,         /* direct sum, hardware (MUFU) cosine */
-    CGH_DIRECT_ACCURATE = 2,    /* direct sum, polynomial cosine on the FMA pipe */
+    CGH_DIRECT_SFU = 1,         /* direct sum */
+    CGH_DIRECT_ACCURATE = 2,    /* direct sum; the same, but for CGH_OPT_DIRECT_SHAPE and cgh_batch, whose SIMT kernels
+                                   take the hardware (MUFU) cosine for CGH_DIRECT_SFU and a polynomial here */
     CGH_GEMM_F16 = 3,           /* I = P Q^T, FP16 factors, FP32 accumulate */
     CGH_GEMM_BF16 = 4,          /* I = P Q^T, BF16 factors, FP32 accumulate */
     CGH_GEMM_SPLIT16 = 5        /* I = Ph Qh^T + Ph Ql^T + Pl Qh^T, hi+lo FP16 */
@@ -92,11 +95,10 @@ enum {
 /* Options (cgh_set_option). */
 enum {
     CGH_OPT_TIMEOUT_MS = 1,     /* bound on every device-side wait; host-side waits allow 2x + 1 s; default 5000 */
-    CGH_OPT_POINT_SPLIT = 2,    /* direct forms: 0 = automatic (the amplitude hologram: every CTA takes an
-                                   equal share of the (pixel tile, point) pairs and the last CTA to finish a tile
-                                   sums its parts; the complex wave: point chunks as the critical-path model
-                                   picks them); s > 0: s point chunks, each a plane of partial sums, reduced
-                                   after */
+    CGH_OPT_POINT_SPLIT = 2,    /* direct forms: 0 = automatic (every CTA takes an equal share of the (pixel tile,
+                                   point) pairs and the last CTA to finish a tile sums its parts); s > 0: s point
+                                   chunks per tile, summed in order by the last to finish (the spherical model: each
+                                   a plane of partial sums, reduced after) */
     CGH_OPT_GEMM_SPLITK = 3,    /* GEMM forms: K splits reduced afterwards; 0 = automatic */
     CGH_OPT_GEMM_BN = 4,        /* GEMM forms: tile width, one of 128, 192, 224, 240, 256; 0 = automatic */
     CGH_OPT_TOLERANCE_E9 = 5,   /* CGH_FORM_AUTO: largest admissible NRMS, in units of 1e-9 */
@@ -121,10 +123,9 @@ enum {
                                    piston (CGH_PHASE_FRESNEL_PISTON): points of equal C may differ in depth. */
     CGH_OPT_PHASE_MODEL = 13,   /* CGH_PHASE_* above; default CGH_PHASE_FRESNEL.  cgh_batch supports the default
                                    only (CGH_ENOTSUP otherwise). */
-    CGH_OPT_DIRECT_CTAS = 14,   /* direct SFU amplitude form with CGH_OPT_POINT_SPLIT = 0: the CTAs that share
-                                   the (pixel tile, point) pairs; 0 = automatic (up to three per resident CTA slot,
-                                   each with at least 1024 points; the hardware schedules those beyond the resident
-                                   ones as others finish) */
+    CGH_OPT_DIRECT_CTAS = 14,   /* direct amplitude forms with CGH_OPT_POINT_SPLIT = 0: the CTAs that share
+                                   the (pixel tile, point) pairs; 0 = automatic (up to one per SM; the hardware
+                                   schedules those beyond the resident ones as others finish) */
     CGH_OPT_BATCH_MODE = 15,    /* cgh_batch: 0 = one persistent launch for the whole batch (default; GEMM units on
                                    the tensor cores beside point preparation, factor generation and direct units
                                    on the same SMs); 1 = per-kind launches (preparation and factors per instance,
@@ -135,12 +136,12 @@ enum {
     CGH_OPT_TEST_ALLOC_FAIL = 17, /* test hook: the next n growths of the context's workspace fail as a failed
                                    cudaMalloc would (the call returns CGH_ENOMEM, nothing is launched, and the
                                    context stays usable); 0 = off */
-    CGH_OPT_DIRECT_SHAPE = 18,  /* direct SFU amplitude form with CGH_OPT_POINT_SPLIT = 0: the thread block;
-                                   0 = automatic (5 or 6 by the padded pixels), 1 = 32 x 8 threads of 8 x 4
-                                   pixels, 2 = 16 x 16 threads of 8 x 4, 3 = 16 x 8 threads of 8 x 8, 4 = 32 x 4
-                                   threads of 8 x 8 (each thread its own sines and cosines); 5 = 16 x 16 threads of
-                                   8 x 4, 6 = 32 x 8 threads of 8 x 4, with the sines and cosines of a point's
-                                   columns and rows taken once per CTA into shared-memory tables */
+    CGH_OPT_DIRECT_SHAPE = 18,  /* direct amplitude forms: 0 = on the tensor cores (default); else the SIMT kernel with
+                                   the thread block 1 = 32 x 8 threads of 8 x 4 pixels, 2 = 16 x 16 threads of
+                                   8 x 4, 3 = 16 x 8 threads of 8 x 8, 4 = 32 x 4 threads of 8 x 8 (each thread its
+                                   own sines and cosines); 5 = 16 x 16 threads of 8 x 4, 6 = 32 x 8 threads of
+                                   8 x 4, with the sines and cosines of a point's columns and rows taken once per
+                                   CTA into shared-memory tables */
     CGH_OPT_GEMM_PERSISTENT = 19, /* GEMM forms, cgh_point_cloud: 1 = the hologram as a one-instance batch in the
                                    persistent kernel (its factors generated K chunk by K chunk while the tensor
                                    cores run the GEMM of the chunks already there; a CUDA graph replayed while the
@@ -284,10 +285,8 @@ int cgh_factors(cgh_ctx *ctx, const float *d_xyz, const float *d_amp, int64_t n_
  * amplitude hologram of cgh_point_cloud and its argument gives the phase-only
  * hologram (kinoform) of Eq. 3, the workload the paper times (Section 5).
  *   d_out : float32 [2][height][width]: the real plane, then the imaginary plane.
- * Forms: CGH_DIRECT_SFU (both parts in one direct pass: hardware sine pairs at
- * the first column of each thread's row and for its first column step, the
- * other terms by complex rotation along the row, since the phase is quadratic
- * in the column, Eqs. 6-8; NRMS about 1.3e-6) and the GEMM forms (Re O = P Q^T and Im O = P Q'^T, with
+ * Forms: CGH_DIRECT_SFU (both parts in one direct pass on the tensor cores, NRMS
+ * about 3.6e-7) and the GEMM forms (Re O = P Q^T and Im O = P Q'^T, with
  * Q'[m][2j] = A_j sin alpha, Q'[m][2j+1] = A_j cos alpha).  CGH_FORM_AUTO
  * picks among those; CGH_DIRECT_ACCURATE returns CGH_ENOTSUP.
  */

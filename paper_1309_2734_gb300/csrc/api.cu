@@ -20,61 +20,71 @@ using namespace cgh;
 
 namespace cgh {
 
-// Direct form: prep, then the direct kernel.  By default one launch in which the CTAs take equal shares of the
-// (pixel tile, point) pairs and the last CTA to finish a tile sums its parts (no partial planes).  With
-// CGH_OPT_POINT_SPLIT > 0: point chunks into partial planes and the fixed-order chunk reduction after.
+// The direct form on the tensor cores (planes = 2: the complex wave): prep, then one launch.
+int run_direct_mma(cgh_ctx *ctx, const DirectMmaLayout &lay, int planes, const char *name, int width, int height,
+                   double pitch, double lambda, const float *d_xyz, const float *d_amp, int64_t n, float *d_out)
+{
+    const int64_t n_pad = padded_points(n);
+    const size_t geo_bytes = align_up((size_t)n_pad * sizeof(int4), 256);
+    const size_t aux_bytes = align_up((size_t)n_pad * sizeof(uint2), 256);
+    const size_t zero_bytes = align_up((size_t)(1 + lay.tiles) * sizeof(int), 256);   // max |A|, the tile counters
+    const size_t slot_bytes = (size_t)2 * lay.ctas * 128 * lay.bn * sizeof(float);
+    int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, geo_bytes + aux_bytes + zero_bytes + slot_bytes);
+    if (rc) return rc;
+    char *base = static_cast<char *>(ctx->ws);
+    int4 *geo = reinterpret_cast<int4 *>(base);
+    uint2 *aux = reinterpret_cast<uint2 *>(base + geo_bytes);
+    float *amax = reinterpret_cast<float *>(base + geo_bytes + aux_bytes);
+    cudaError_t e = cudaMemsetAsync(amax, 0, (size_t)(1 + lay.tiles) * sizeof(int), ctx->stream);
+    if (e != cudaSuccess) return cuda_status(e);
+    {
+        ProfileScope ps(ctx, "prep_points", 1);
+        e = launch_prep_points(d_xyz, d_amp, (int)n, (int)n_pad, pitch, lambda, geo, aux, ctx->d_status, amax,
+                               ctx->stream, aux_mode(ctx));
+    }
+    if (e != cudaSuccess) return cuda_status(e);
+    ProfileScope ps(ctx, name, 1);
+    return cuda_status(launch_direct_mma(lay, planes, geo, aux, amax, (int)n, width, height, d_out,
+                                         reinterpret_cast<float *>(base + geo_bytes + aux_bytes + zero_bytes),
+                                         reinterpret_cast<int *>(amax + 1), ctx->d_status,
+                                         (uint64_t)ctx->timeout_ms * 1000000ull, ctx->stream, ctx->drop_tile,
+                                         phase_ref(ctx)));
+}
+
 constexpr int kStreamMinPoints = 64;      // fewest points of one CTA's share in the balanced layout
 constexpr int kStreamSharePoints = 1024;  // points per share from which CTAs beyond the resident ones are added
 constexpr int kStreamWaves = 2;           // at most this many CTAs per resident slot
 
+// The direct forms: on the tensor cores, or (CGH_OPT_DIRECT_SHAPE) the SIMT kernel with the pinned thread block, one
+// launch in which the CTAs take equal shares of the (pixel tile, point) pairs and the last CTA to finish a tile sums
+// its parts.
 int run_direct(cgh_ctx *ctx, bool sfu, int width, int height, double pitch, double lambda, const float *d_xyz,
                const float *d_amp, int64_t n, float *d_out)
 {
+    const char *name = sfu ? "direct_sfu" : "direct_accurate";
+    if (ctx->direct_shape == 0)
+        return run_direct_mma(
+            ctx, choose_direct_mma(1, width, height, n, ctx->num_sms, ctx->point_split, ctx->direct_ctas), 1, name,
+            width, height, pitch, lambda, d_xyz, d_amp, n, d_out);
     const int64_t n_pad = padded_points(n);
-    const int64_t n_ptiles = n_pad / kPointTile;
     const size_t geo_bytes = align_up((size_t)n_pad * sizeof(int4), 256);
     const size_t aux_bytes = align_up((size_t)n_pad * sizeof(uint2), 256);
-    const int64_t plane = (int64_t)width * height;
-    const uint64_t tmo = (uint64_t)ctx->timeout_ms * 1000000ull;
-    const bool stream_k = ctx->point_split == 0;
-    DirectShape sh;
-    int split = 1, ctas = 0;
-    size_t ws_rest = 0;
-    if (stream_k) {
-        // the shape with the fewer padded pixels; up to kStreamWaves CTAs per resident slot (measured at
-        // 1920x1080, 10^4 points, 8 x 8 pixels a thread, four 128-thread CTAs per SM: 608 CTAs 3.02 ms, 1216 2.995,
-        // 1824 3.017, 2432 3.22; DRAM writes 0.1 / 3.9 / 18.4 MB per launch, the parts L2 no longer holds), each
-        // share of at least kStreamSharePoints points beyond the first wave and kStreamMinPoints within it
-        auto padded = [&](const DirectShape &s) {
-            return (int64_t)((width + s.tile_w - 1) / s.tile_w) * s.tile_w *
-                   (((int64_t)height + s.tile_h - 1) / s.tile_h) * s.tile_h;
-        };
-        // blocks of 8 x 4 pixels with the tables of the tile, 16 x 16 threads (a 128 x 64 tile) unless 32 x 8 (256 x
-        // 32) pads a fifth fewer pixels (at equal padding the tall block measured 16 % faster: a point's 192 table
-        // entries over 256 threads instead of 288); CGH_OPT_DIRECT_SHAPE pins any block
-        if (ctx->direct_shape > 0) {
-            sh = direct_stream_shape(ctx->direct_shape - 1);
-        } else {
-            sh = direct_stream_shape(4);
-            if (padded(direct_stream_shape(5)) * 6 < padded(sh) * 5) sh = direct_stream_shape(5);
-        }
-        const int64_t tiles = (int64_t)((width + sh.tile_w - 1) / sh.tile_w) * ((height + sh.tile_h - 1) / sh.tile_h);
-        const int64_t units = tiles * n;
-        const int64_t slots = (int64_t)ctx->num_sms * direct_stream_per_sm(sfu, sh);
-        int64_t want = units >= slots * kStreamSharePoints
-                           ? std::min<int64_t>(kStreamWaves * slots, units / kStreamSharePoints)
-                           : std::min<int64_t>(slots, units / kStreamMinPoints);
-        if (ctx->direct_ctas > 0) want = std::min<int64_t>(ctx->direct_ctas, units);
-        ctas = (int)std::max<int64_t>(1, want);
-        ws_rest = align_up((size_t)2 * ctas * sh.tile_w * sh.tile_h * sizeof(float), 256) +
-                  align_up((size_t)tiles * sizeof(int), 256);
-    } else {
-        const DirectLayout lay = choose_direct_layout(false, width, height, n_ptiles, ctx->num_sms, ctx->point_split);
-        sh = lay.shape;
-        split = lay.split;
-        ws_rest = split > 1 ? (size_t)split * plane * sizeof(float) : 0;
-    }
-    int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, geo_bytes + aux_bytes + ws_rest);
+    // up to kStreamWaves CTAs per resident slot (measured at 1920x1080, 10^4 points, 8 x 8 pixels a thread, four
+    // 128-thread CTAs per SM: 608 CTAs 3.02 ms, 1216 2.995, 1824 3.017, 2432 3.22), each share of at least
+    // kStreamSharePoints points beyond the first wave and kStreamMinPoints within it
+    const DirectShape sh = direct_stream_shape(ctx->direct_shape - 1);
+    const int64_t tiles = (int64_t)((width + sh.tile_w - 1) / sh.tile_w) * ((height + sh.tile_h - 1) / sh.tile_h);
+    const int64_t units = tiles * n;
+    const int64_t slots = (int64_t)ctx->num_sms * direct_stream_per_sm(sfu, sh);
+    int64_t want = units >= slots * kStreamSharePoints
+                       ? std::min<int64_t>(kStreamWaves * slots, units / kStreamSharePoints)
+                       : std::min<int64_t>(slots, units / kStreamMinPoints);
+    if (ctx->point_split > 0) want = std::min<int64_t>(tiles * ctx->point_split, units);
+    if (ctx->direct_ctas > 0) want = std::min<int64_t>(ctx->direct_ctas, units);
+    const int ctas = (int)std::max<int64_t>(1, want);
+    const size_t slot_bytes = align_up((size_t)2 * ctas * sh.tile_w * sh.tile_h * sizeof(float), 256);
+    int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes,
+                    geo_bytes + aux_bytes + slot_bytes + align_up((size_t)tiles * sizeof(int), 256));
     if (rc) return rc;
     char *base = static_cast<char *>(ctx->ws);
     int4 *geo = reinterpret_cast<int4 *>(base);
@@ -87,22 +97,11 @@ int run_direct(cgh_ctx *ctx, bool sfu, int width, int height, double pitch, doub
                                nullptr, ctx->stream, aux_mode(ctx));
     }
     if (e != cudaSuccess) return cuda_status(e);
-    if (stream_k) {
-        int *counters = reinterpret_cast<int *>(
-            reinterpret_cast<char *>(rest) + align_up((size_t)2 * ctas * sh.tile_w * sh.tile_h * sizeof(float), 256));
-        ProfileScope ps(ctx, sfu ? "direct_sfu" : "direct_accurate", 1);   // and the counters' memset
-        return cuda_status(launch_direct_stream(sfu, sh, ctas, geo, aux, (int)n, width, height, d_out, rest,
-                                                counters, ctx->d_status, tmo, ctx->stream, ctx->drop_tile,
-                                                phase_ref(ctx)));
-    }
-    {
-        ProfileScope ps(ctx, sfu ? "direct_sfu" : "direct_accurate", 1);
-        e = launch_direct(sfu, sh, geo, aux, (int)n_pad, width, height, split, split > 1 ? rest : d_out, plane,
-                          ctx->d_status, tmo, ctx->stream, ctx->drop_tile, phase_ref(ctx));
-    }
-    if (e != cudaSuccess || split == 1) return cuda_status(e);
-    ProfileScope ps(ctx, "reduce_slices", 1);
-    return cuda_status(launch_reduce_slices(rest, split, plane, plane, d_out, ctx->stream));
+    int *counters = reinterpret_cast<int *>(reinterpret_cast<char *>(rest) + slot_bytes);
+    ProfileScope ps(ctx, name, 1);   // and the counters' memset
+    return cuda_status(launch_direct_stream(sfu, sh, ctas, geo, aux, (int)n, width, height, d_out, rest, counters,
+                                            ctx->d_status, (uint64_t)ctx->timeout_ms * 1000000ull, ctx->stream,
+                                            ctx->drop_tile, phase_ref(ctx)));
 }
 
 // k-blocks per TMEM accumulation chain of the split-FP16 form (3 passes each)
@@ -396,35 +395,9 @@ int run_wave(cgh_ctx *ctx, int form, const float *d_xyz, const float *d_amp, int
     const size_t aux_bytes = align_up((size_t)n_pad * sizeof(uint2), 256);
     const uint64_t tmo = (uint64_t)ctx->timeout_ms * 1000000ull;
     cudaError_t e;
-    if (form == CGH_DIRECT_SFU) {
-        const int64_t n_ptiles = n_pad / kPointTile;
-        const DirectLayout lay = choose_direct_layout(true, width, height, n_ptiles, ctx->num_sms, ctx->point_split);
-        const DirectShape sh = lay.shape;
-        const int split = lay.split;
-        const size_t part_bytes = split > 1 ? (size_t)split * 2 * plane * sizeof(float) : 0;
-        int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, geo_bytes + aux_bytes + part_bytes);
-        if (rc) return rc;
-        char *base = static_cast<char *>(ctx->ws);
-        int4 *geo = reinterpret_cast<int4 *>(base);
-        uint2 *aux = reinterpret_cast<uint2 *>(base + geo_bytes);
-        float *parts = reinterpret_cast<float *>(base + geo_bytes + aux_bytes);
-        {
-            ProfileScope ps(ctx, "prep_points", 1);
-            e = launch_prep_points(d_xyz, d_amp, (int)n, (int)n_pad, ctx->pitch, ctx->lambda, geo, aux, ctx->d_status,
-                                   nullptr, ctx->stream, aux_mode(ctx));
-        }
-        if (e != cudaSuccess) return cuda_status(e);
-        {
-            ProfileScope ps(ctx, "direct_wave", 1);
-            e = launch_direct_wave(sh, geo, aux, (int)n_pad, width, height, split, split > 1 ? parts : d_out,
-                                   2 * plane, plane, ctx->d_status, tmo, ctx->stream, phase_ref(ctx));
-        }
-        if (e != cudaSuccess || split == 1) return cuda_status(e);
-        ProfileScope ps(ctx, "reduce_slices", 2);
-        e = launch_reduce_slices(parts, split, plane, 2 * plane, d_out, ctx->stream);
-        if (e == cudaSuccess) e = launch_reduce_slices(parts + plane, split, plane, 2 * plane, d_out + plane, ctx->stream);
-        return cuda_status(e);
-    }
+    if (form == CGH_DIRECT_SFU)
+        return run_direct_mma(ctx, choose_direct_mma(2, width, height, n, ctx->num_sms, ctx->point_split, 0), 2,
+                              "direct_wave", width, height, ctx->pitch, ctx->lambda, d_xyz, d_amp, n, d_out);
     if (form < CGH_GEMM_F16 || form > CGH_GEMM_SPLIT16) return CGH_ENOTSUP;
     const int mode = factor_mode(form);
     const int planes = mode == kFactorSplit16 ? 2 : 1;

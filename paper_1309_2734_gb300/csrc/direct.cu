@@ -1,8 +1,8 @@
-// a2: the direct kernels (device code of the term and of a unit of work in
-// direct_dev.cuh): one hologram in the chunked layout (pixel tile x point
-// chunk, partial planes), in the balanced layout (equal shares of the (pixel
-// tile, point) pairs, a tile's parts summed by the last CTA to finish it), the
-// complex object wave, and the per-form batch kernels.
+// a2: the SIMT direct kernels (device code of the term and of a unit of work in
+// direct_dev.cuh): one hologram in the balanced layout (equal shares of the
+// (pixel tile, point) pairs, a tile's parts summed by the last CTA to finish
+// it; CGH_OPT_DIRECT_SHAPE) and the per-form batch kernels.  A hologram of the
+// direct forms otherwise runs on the tensor cores (direct_mma.cu).
 #include <type_traits>
 
 #include "direct_dev.cuh"
@@ -14,27 +14,6 @@ namespace cgh {
 namespace {
 
 using namespace dev;
-
-// One hologram: blockIdx.x = pixel tile, blockIdx.y = point chunk (its own output plane).
-template <int TL, int TR, int BX, int BY, bool SFU, bool EXTRA>
-__global__ void __launch_bounds__(BX *BY, 2)
-    direct_kernel(const int4 *__restrict__ geo, const uint2 *__restrict__ aux, int n_ptiles, int width,
-                  int height, int tiles_x, int split, float *__restrict__ out, long long slice_stride,
-                  bool vec, int *status, unsigned long long timeout_ns, int drop_tile, const PhaseRef ref)
-{
-    __shared__ alignas(128) int4 s_geo[2][kPointTile];
-    __shared__ alignas(128) uint2 s_aux[2][kPointTile];
-    __shared__ alignas(8) uint64_t s_bar[2];
-    init_point_barriers<BX, BY>(s_bar);
-    const int tile = blockIdx.x;
-    const int t_begin = (int)((long long)blockIdx.y * n_ptiles / split);
-    const int t_end = (int)((long long)(blockIdx.y + 1) * n_ptiles / split);
-    uint32_t kg = 0;
-    direct_unit<TL, TR, BX, BY, SFU, 1, EXTRA>(geo, aux, t_begin, t_end, (tile % tiles_x) * (BX * TL),
-                                     (tile / tiles_x) * (BY * TR), width, height,
-                                     out + (long long)blockIdx.y * slice_stride, vec, s_geo, s_aux, s_bar, kg,
-                                     status, timeout_ns, blockIdx.y == 0 ? drop_tile : -1, 0, ref);
-}
 
 // One hologram over a flat work space: unit u = t N + j is (pixel tile t, point j), t < n_tiles, j < N, and
 // CTA c of C takes units [c U / C, (c + 1) U / C) (U = n_tiles N), so every CTA has the same number of terms to
@@ -199,41 +178,14 @@ __global__ void __launch_bounds__(BX *BY, 512 / (BX * BY))
         __syncthreads();
         const int k0 = p0 / T, k1 = (p1 + T - 1) / T;
         const int drop = (blockIdx.x == 0 && w == w0) ? drop_tile : -1;
-        if (!direct_unit<TL, TR, BX, BY, SFU, 1, EXTRA, SMEM_TOT, StreamSink<TL, TR, BX, BY>, CtaSync, T, TABLES>(
+        if (!direct_unit<TL, TR, BX, BY, SFU, EXTRA, SMEM_TOT, StreamSink<TL, TR, BX, BY>, CtaSync, T, TABLES>(
                 geo, aux, k0, k1, (int)(t % tiles_x) * (BX * TL), (int)(t / tiles_x) * (BY * TR), width, height,
-                out, vec, s_geo, s_aux, s_bar, kg, status, timeout_ns, drop, 0, ref, s_tot, p0 - k0 * T,
+                out, vec, s_geo, s_aux, s_bar, kg, status, timeout_ns, drop, ref, s_tot, p0 - k0 * T,
                 p1 - (k1 - 1) * T, sink, s_tab))
             break;
         w = s_seg.t * n_points + s_seg.p1;
         __syncthreads();   // s_seg and the point stages are reused by the next segment
     }
-}
-
-// The complex object wave of one hologram: blockIdx.x = pixel tile, blockIdx.y =
-// point chunk; chunk s writes real and imaginary planes at out + s * slice_stride
-// and out + s * slice_stride + im_offset.  TABLES: the sines and cosines of a point's columns and rows taken once
-// per CTA into shared-memory tables (dev::SepTable), after the totals.
-template <int TL, int TR, int BX, int BY, bool EXTRA, bool TABLES>
-__global__ void __launch_bounds__(BX *BY, 2)
-    direct_wave_kernel(const int4 *__restrict__ geo, const uint2 *__restrict__ aux, int n_ptiles, int width,
-                       int height, int tiles_x, int split, float *__restrict__ out, long long slice_stride,
-                       long long im_offset, bool vec, int *status, unsigned long long timeout_ns,
-                       const PhaseRef ref)
-{
-    __shared__ alignas(128) int4 s_geo[2][kPointTile];
-    __shared__ alignas(128) uint2 s_aux[2][kPointTile];
-    __shared__ alignas(8) uint64_t s_bar[2];
-    extern __shared__ __align__(16) float s_tot[];   // the running totals: 2 TR TL floats per thread; the tables
-    float2 *s_tab = reinterpret_cast<float2 *>(s_tot + 2 * TR * TL * BX * BY);
-    init_point_barriers<BX, BY>(s_bar);
-    const int tile = blockIdx.x;
-    const int t_begin = (int)((long long)blockIdx.y * n_ptiles / split);
-    const int t_end = (int)((long long)(blockIdx.y + 1) * n_ptiles / split);
-    uint32_t kg = 0;
-    direct_unit<TL, TR, BX, BY, true, 2, EXTRA, true, PlainStore, CtaSync, kPointTile, TABLES>(
-        geo, aux, t_begin, t_end, (tile % tiles_x) * (BX * TL), (tile / tiles_x) * (BY * TR), width, height,
-        out + (long long)blockIdx.y * slice_stride, vec, s_geo, s_aux, s_bar, kg, status, timeout_ns, -1, im_offset,
-        ref, s_tot, 0, kPointTile, PlainStore(), s_tab);
 }
 
 // A batch: every CTA walks its list of {job, pixel tile} units over all points of the job.
@@ -260,62 +212,12 @@ __global__ void __launch_bounds__(BX *BY, 2)
 constexpr int kTL = 8, kTR = 4, kBX = 32, kBY = 8;   // the wide shape: 256 x 32 pixels per CTA
 constexpr int kTallBX = 16, kTallBY = 16;             // the tall shape: 128 x 64 pixels per CTA
 
-template <int BX, int BY, bool SFU, bool EXTRA>
-void direct_as(dim3 grid, cudaStream_t s, const int4 *geo, const uint2 *aux, int n_ptiles, int width, int height,
-               int tiles_x, int split, float *out, long long ss, bool vec, int *status, uint64_t timeout_ns,
-               int drop_tile, const PhaseRef &ref)
-{
-    direct_kernel<kTL, kTR, BX, BY, SFU, EXTRA><<<grid, BX * BY, 0, s>>>(
-        geo, aux, n_ptiles, width, height, tiles_x, split, out, ss, vec, status, timeout_ns, drop_tile, ref);
-}
-
-template <int BX, int BY>
-void direct_shaped(bool sfu, bool extra, dim3 grid, cudaStream_t s, const int4 *geo, const uint2 *aux, int n_ptiles,
-                   int width, int height, int tiles_x, int split, float *out, long long ss, bool vec, int *status,
-                   uint64_t timeout_ns, int drop_tile, const PhaseRef &ref)
-{
-    if (sfu && !extra)
-        direct_as<BX, BY, true, false>(grid, s, geo, aux, n_ptiles, width, height, tiles_x, split, out, ss, vec,
-                                       status, timeout_ns, drop_tile, ref);
-    else if (sfu)
-        direct_as<BX, BY, true, true>(grid, s, geo, aux, n_ptiles, width, height, tiles_x, split, out, ss, vec,
-                                      status, timeout_ns, drop_tile, ref);
-    else if (!extra)
-        direct_as<BX, BY, false, false>(grid, s, geo, aux, n_ptiles, width, height, tiles_x, split, out, ss, vec,
-                                        status, timeout_ns, drop_tile, ref);
-    else
-        direct_as<BX, BY, false, true>(grid, s, geo, aux, n_ptiles, width, height, tiles_x, split, out, ss, vec,
-                                       status, timeout_ns, drop_tile, ref);
-}
-
 }  // namespace
 
 DirectShape direct_shape(bool tall)
 {
     return tall ? DirectShape{kTallBX * kTL, kTallBY * kTR, kTallBX * kTallBY, kTallBX}
                 : DirectShape{kBX * kTL, kBY * kTR, kBX * kBY, kBX};
-}
-
-cudaError_t launch_direct(bool sfu, const DirectShape &sh, const int4 *geo, const uint2 *aux, int n_pad, int width,
-                          int height, int split, float *out, int64_t slice_stride, int *status, uint64_t timeout_ns,
-                          cudaStream_t s, int drop_tile, const PhaseRef &ref)
-{
-    const int tiles_x = (width + sh.tile_w - 1) / sh.tile_w;
-    const int tiles_y = (height + sh.tile_h - 1) / sh.tile_h;
-    const int n_ptiles = n_pad / kPointTile;
-    if (split < 1) split = 1;
-    dim3 grid(tiles_x * tiles_y, split);
-    // 16-byte stores only when every row start of every slice is 16-byte aligned
-    const bool vec = (width % 4 == 0) && (slice_stride % 4 == 0) && ((uintptr_t)out % 16 == 0);
-    const long long ss = (long long)slice_stride;
-    const bool extra = ref.any();
-    if (sh.bx == kTallBX)
-        direct_shaped<kTallBX, kTallBY>(sfu, extra, grid, s, geo, aux, n_ptiles, width, height, tiles_x, split, out,
-                                        ss, vec, status, timeout_ns, drop_tile, ref);
-    else
-        direct_shaped<kBX, kBY>(sfu, extra, grid, s, geo, aux, n_ptiles, width, height, tiles_x, split, out, ss,
-                                vec, status, timeout_ns, drop_tile, ref);
-    return cudaGetLastError();
 }
 
 namespace {
@@ -497,70 +399,6 @@ int direct_ctas_per_sm(bool sfu, bool tall)
         return 1;
     }
     return n;
-}
-
-}  // namespace cgh
-
-namespace cgh {
-
-namespace {
-constexpr int kWaveTL = 8, kWaveTR = 4;   // two planes of partial sums in registers, the totals in shared memory
-
-// The tall block takes the tables (two CTAs an SM with 8-point groups); the wide one's tables would leave one CTA
-// an SM, so it keeps each thread's own sines and cosines.
-template <int BX, int BY>
-void wave_as(bool extra, dim3 grid, cudaStream_t s, const int4 *geo, const uint2 *aux, int n_ptiles, int width,
-             int height, int tiles_x, int split, float *out, long long ss, long long im, bool vec, int *status,
-             uint64_t timeout_ns, const PhaseRef &ref)
-{
-    constexpr bool kTables = BX == kTallBX;
-    constexpr size_t dyn_bytes =
-        (size_t)2 * kWaveTR * kWaveTL * BX * BY * sizeof(float) +
-        (kTables ? (size_t)2 * sep_group<2>() * SepTable<BX * kWaveTL, BY * kWaveTR>::kPerPoint * sizeof(float2)
-                 : 0);
-    static PerDeviceOnce configured;   // the running totals exceed the default 48 KB of dynamic shared memory
-    const cudaError_t e = configured.run([&] {
-        cudaError_t r = cudaFuncSetAttribute(direct_wave_kernel<kWaveTL, kWaveTR, BX, BY, true, kTables>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_bytes);
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(direct_wave_kernel<kWaveTL, kWaveTR, BX, BY, false, kTables>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_bytes);
-        return r;
-    });
-    if (e != cudaSuccess) return;
-    if (extra)
-        direct_wave_kernel<kWaveTL, kWaveTR, BX, BY, true, kTables><<<grid, BX * BY, dyn_bytes, s>>>(
-            geo, aux, n_ptiles, width, height, tiles_x, split, out, ss, im, vec, status, timeout_ns, ref);
-    else
-        direct_wave_kernel<kWaveTL, kWaveTR, BX, BY, false, kTables><<<grid, BX * BY, dyn_bytes, s>>>(
-            geo, aux, n_ptiles, width, height, tiles_x, split, out, ss, im, vec, status, timeout_ns, ref);
-}
-}  // namespace
-
-DirectShape direct_wave_shape(bool tall)
-{
-    return tall ? DirectShape{kTallBX * kWaveTL, kTallBY * kWaveTR, kTallBX * kTallBY, kTallBX}
-                : DirectShape{kBX * kWaveTL, kBY * kWaveTR, kBX * kBY, kBX};
-}
-
-cudaError_t launch_direct_wave(const DirectShape &sh, const int4 *geo, const uint2 *aux, int n_pad, int width,
-                               int height, int split, float *out, int64_t slice_stride, int64_t im_offset,
-                               int *status, uint64_t timeout_ns, cudaStream_t s, const PhaseRef &ref)
-{
-    const int tiles_x = (width + sh.tile_w - 1) / sh.tile_w;
-    const int tiles_y = (height + sh.tile_h - 1) / sh.tile_h;
-    const int n_ptiles = n_pad / kPointTile;
-    if (split < 1) split = 1;
-    dim3 grid(tiles_x * tiles_y, split);
-    const bool vec = (width % 4 == 0) && (slice_stride % 4 == 0) && (im_offset % 4 == 0) &&
-                     ((uintptr_t)out % 16 == 0);
-    if (sh.bx == kTallBX)
-        wave_as<kTallBX, kTallBY>(ref.any(), grid, s, geo, aux, n_ptiles, width, height, tiles_x, split, out,
-                                  (long long)slice_stride, (long long)im_offset, vec, status, timeout_ns, ref);
-    else
-        wave_as<kBX, kBY>(ref.any(), grid, s, geo, aux, n_ptiles, width, height, tiles_x, split, out,
-                          (long long)slice_stride, (long long)im_offset, vec, status, timeout_ns, ref);
-    return cudaGetLastError();
 }
 
 }  // namespace cgh

@@ -103,11 +103,9 @@ __device__ __forceinline__ PixelRef pixel_ref(const PhaseRef &r, int m0, int n0)
 // turns the sign of that mean, so it cancels over pairs of points (5.8e-7 and 6.9e-7).
 // ACC: the accurate form -- cos 2 pi t from the polynomial of cos_turn_poly and sin 2 pi t = cos 2 pi (t - 1/4) from the
 // same polynomial, on the FMA pipe (no flip needed: the polynomial's mean error over the turns is about zero).
-// PLANES = 2: the complex object wave (Eq. 2, restricted form), A e^{i 2 pi (a_i + b_r)}: the real part to part,
-// the imaginary part, sin 2 pi a_i (A cos 2 pi b_r) + cos 2 pi a_i (A sin 2 pi b_r), to part_im.
-template <int TL, int TR, bool EXTRA, bool ACC = false, int PLANES = 1>
+template <int TL, int TR, bool EXTRA, bool ACC = false>
 __device__ __forceinline__ void point_terms_sep(const int4 q, const uint2 w, int m0, int n0, const PixelRef &pr,
-                                                uint32_t flip, float (&part)[TR][TL], float (&part_im)[TR][TL])
+                                                uint32_t flip, float (&part)[TR][TL])
 {
     const uint32_t chi = (uint32_t)q.z, clo = (uint32_t)q.w;
     const uint32_t dx = (uint32_t)(m0 - q.x);
@@ -151,10 +149,7 @@ __device__ __forceinline__ void point_terms_sep(const int4 q, const uint2 w, int
         cb *= amp;
         sb *= amp;
 #pragma unroll
-        for (int i = 0; i < TL; ++i) {
-            part[r][i] = fmaf(-sa[i], sb, fmaf(ca[i], cb, part[r][i]));
-            if constexpr (PLANES == 2) part_im[r][i] = fmaf(ca[i], sb, fmaf(sa[i], cb, part_im[r][i]));
-        }
+        for (int i = 0; i < TL; ++i) part[r][i] = fmaf(-sa[i], sb, fmaf(ca[i], cb, part[r][i]));
         b += db;
         db += D;
     }
@@ -177,14 +172,8 @@ struct SepTable {
     __device__ static int col_cos(int k) { return (k >> 3) * 20 + ((k & 7) >> 1) * 4 + (k & 1); }
 };
 // points per table fill (double buffered: one CTA barrier per group; 8 measured 2.69 ms, 32 3.04 -- two CTAs no
-// longer fit an SM -- against 2.51 at 16, 1920x1080, 10^4 points); the complex wave, whose two planes of totals
-// take twice the shared memory, fills 8
+// longer fit an SM -- against 2.51 at 16, 1920x1080, 10^4 points)
 constexpr int kSepGroup = 16;
-template <int PLANES>
-__host__ __device__ constexpr int sep_group()
-{
-    return PLANES == 2 ? 8 : kSepGroup;
-}
 
 // The tables of np <= GROUP points p0, p0 + 1, ... for a tile: NTHREADS / GROUP threads a point (a half warp or a
 // warp), each taking its point's turn constants once and then its share of the columns and rows, one entry at a
@@ -295,12 +284,10 @@ struct SepQuads {
 };
 
 // One point's terms from its quads, two columns a packed FMA (the two lanes' FMAs in one instruction):
-// acc[0][r][j] += (cos a_2j, cos a_2j+1) (A cos b_r) + (sin a_2j, sin a_2j+1) (-A sin b_r), the same two roundings
-// per term as two scalar FMAs; with PLANES = 2 also the imaginary part, acc[1][r][j] += (sin a) (A cos b_r) +
-// (cos a) (A sin b_r).
-template <int TR, int TILE_W, int TILE_H, int PLANES>
-__device__ __forceinline__ void point_terms_table(const SepQuads<TR, TILE_W, TILE_H> &q,
-                                                  float2 (&acc)[PLANES][TR][4])
+// acc[r][j] += (cos a_2j, cos a_2j+1) (A cos b_r) + (sin a_2j, sin a_2j+1) (-A sin b_r), the same two roundings
+// per term as two scalar FMAs.
+template <int TR, int TILE_W, int TILE_H>
+__device__ __forceinline__ void point_terms_table(const SepQuads<TR, TILE_W, TILE_H> &q, float2 (&acc)[TR][4])
 {
     static_assert(TR % 2 == 0, "row pairs in 16-byte quads");
 #pragma unroll
@@ -309,23 +296,17 @@ __device__ __forceinline__ void point_terms_table(const SepQuads<TR, TILE_W, TIL
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const float2 c = make_float2(q.c[j].x, q.c[j].y), s = make_float2(q.c[j].z, q.c[j].w);
-            acc[0][2 * h][j] =
-                __ffma2_rn(s, make_float2(v.y, v.y), __ffma2_rn(c, make_float2(v.x, v.x), acc[0][2 * h][j]));
-            acc[0][2 * h + 1][j] =
-                __ffma2_rn(s, make_float2(v.w, v.w), __ffma2_rn(c, make_float2(v.z, v.z), acc[0][2 * h + 1][j]));
-            if constexpr (PLANES == 2) {
-                acc[1][2 * h][j] = __ffma2_rn(c, make_float2(-v.y, -v.y),
-                                              __ffma2_rn(s, make_float2(v.x, v.x), acc[1][2 * h][j]));
-                acc[1][2 * h + 1][j] = __ffma2_rn(c, make_float2(-v.w, -v.w),
-                                                  __ffma2_rn(s, make_float2(v.z, v.z), acc[1][2 * h + 1][j]));
-            }
+            acc[2 * h][j] =
+                __ffma2_rn(s, make_float2(v.y, v.y), __ffma2_rn(c, make_float2(v.x, v.x), acc[2 * h][j]));
+            acc[2 * h + 1][j] =
+                __ffma2_rn(s, make_float2(v.w, v.w), __ffma2_rn(c, make_float2(v.z, v.z), acc[2 * h + 1][j]));
         }
     }
 }
 
 // The points of the unit are those of tiles [t_begin, t_end), less the first p_first points of the first tile
 // and the points from p_last_end on of the last one.  Sink: PlainStore writes the totals to dst; any other sink
-// is called as sink(tot) with the thread's TR x TL totals of plane 0 (the amplitude hologram only).
+// is called as sink(tot) with the thread's TR x TL totals.
 // Sync: the threads that share the unit and their barrier -- CtaSync (the whole CTA) or GroupSync (a named
 // barrier over a group of warps of a larger CTA).  T: points per shared-memory tile (the prepared points are
 // padded to a multiple of kPointTile, which T divides).
@@ -356,13 +337,13 @@ struct GroupSync {
     }
 };
 
-template <int TL, int TR, int BX, int BY, bool SFU, int PLANES = 1, bool EXTRA = false, bool SMEM_TOT = false,
+template <int TL, int TR, int BX, int BY, bool SFU, bool EXTRA = false, bool SMEM_TOT = false,
           class Sink = PlainStore, class Sync = CtaSync, int T = kPointTile, bool TABLES = false>
 __device__ __forceinline__ bool direct_unit(const int4 *__restrict__ geo, const uint2 *__restrict__ aux,
                                             int t_begin, int t_end, int tile_m0, int tile_n0, int width,
                                             int height, float *__restrict__ dst, bool vec, int4 (*s_geo)[T],
                                             uint2 (*s_aux)[T], uint64_t *s_bar, uint32_t &kg, int *status,
-                                            unsigned long long timeout_ns, int drop = -1, long long im_offset = 0,
+                                            unsigned long long timeout_ns, int drop = -1,
                                             const PhaseRef &ref = PhaseRef(), float *s_tot = nullptr,
                                             int p_first = 0, int p_last_end = T, Sink sink = Sink(),
                                             float2 *s_tab = nullptr)
@@ -390,16 +371,14 @@ __device__ __forceinline__ bool direct_unit(const int4 *__restrict__ geo, const 
     }
 
     constexpr int NT = BX * BY;
-    auto tidx = [&](int c, int r, int i) { return ((c * TR + r) * TL + i) * NT + tid; };
-    float tot[PLANES][TR][TL];
-#pragma unroll
-    for (int c = 0; c < PLANES; ++c)
+    auto tidx = [&](int r, int i) { return (r * TL + i) * NT + tid; };
+    float tot[TR][TL];
 #pragma unroll
         for (int r = 0; r < TR; ++r)
 #pragma unroll
             for (int i = 0; i < TL; ++i) {
-                if constexpr (SMEM_TOT) s_tot[tidx(c, r, i)] = 0.0f;
-                else tot[c][r][i] = 0.0f;
+                if constexpr (SMEM_TOT) s_tot[tidx(r, i)] = 0.0f;
+                else tot[r][i] = 0.0f;
             }
 
     bool ok = true;
@@ -420,13 +399,11 @@ __device__ __forceinline__ bool direct_unit(const int4 *__restrict__ geo, const 
             ok = false;
             break;
         }
-        float part[PLANES][TR][TL];
-#pragma unroll
-        for (int c = 0; c < PLANES; ++c)
+        float part[TR][TL];
 #pragma unroll
             for (int r = 0; r < TR; ++r)
 #pragma unroll
-                for (int i = 0; i < TL; ++i) part[c][r][i] = 0.0f;
+                for (int i = 0; i < TL; ++i) part[r][i] = 0.0f;
 
         const int4 *sg = s_geo[st];
         const uint2 *sa = s_aux[st];
@@ -434,25 +411,18 @@ __device__ __forceinline__ bool direct_unit(const int4 *__restrict__ geo, const 
         const int p_hi = k == nt - 1 ? p_last_end : T;
         if constexpr (TABLES) {
             static_assert(TL == 8, "tables serve 8-column blocks");
-            static_assert(PLANES == 1 || SFU, "the complex wave takes the hardware sine and cosine");
-            constexpr int TW = BX * TL, TH = BY * TR, GROUP = sep_group<PLANES>();
+            constexpr int TW = BX * TL, TH = BY * TR, GROUP = kSepGroup;
             using ST = SepTable<TW, TH>;
-            float2 acc[PLANES][TR][TL / 2];   // columns 2 j and 2 j + 1
-#pragma unroll
-            for (int c = 0; c < PLANES; ++c)
+            float2 acc[TR][TL / 2];   // columns 2 j and 2 j + 1
 #pragma unroll
                 for (int r = 0; r < TR; ++r)
 #pragma unroll
-                    for (int j = 0; j < TL / 2; ++j) acc[c][r][j] = make_float2(0.0f, 0.0f);
-            // The next group's tables are filled while this group's are read: for the amplitude hologram the
-            // fill's entries (integer products, hardware or polynomial sines) are spread over the point loop's
-            // packed FMAs (1920x1080, 10^4 points: 1.77 against 1.79 ms filled before the loop; the complex wave,
-            // short of registers, measured 3.26 against 3.21 and fills first); one barrier a group hands the
-            // buffers over.
+                    for (int j = 0; j < TL / 2; ++j) acc[r][j] = make_float2(0.0f, 0.0f);
+            // The next group's tables are filled while this group's are read, the fill's entries (integer products,
+            // hardware or polynomial sines) spread over the point loop's packed FMAs (1920x1080, 10^4 points: 1.77
+            // against 1.79 ms filled before the loop); one barrier a group hands the buffers over.
             using Filler = SepFiller<TW, TH, BX * BY, GROUP, EXTRA, !SFU>;
-            constexpr int U = PLANES == 1 ? 4 : 2;   // points a step (the loop was measured fastest unrolled by
-                                                     // four, 2.30 ms against 2.32 by two at 1920x1080, 10^4 points;
-                                                     // the complex wave's two planes leave the registers for two)
+            constexpr int U = 4;   // points a step (2.30 ms against 2.32 by two at 1920x1080, 10^4 points)
             constexpr int kSteps = GROUP / U;
             constexpr int kPerStep = (Filler::kEntries + kSteps - 1) / kSteps;
             const int n_grp = (p_hi - p_lo + GROUP - 1) / GROUP;
@@ -470,55 +440,48 @@ __device__ __forceinline__ bool direct_unit(const int4 *__restrict__ geo, const 
                 const int npn = gg + 1 < n_grp ? min(GROUP, p_hi - pn) : 0;
                 const Filler next(sg, sa, pn, npn, tile_m0, tile_n0, s_tab + ((gi + 1) & 1) * (GROUP * ST::kPerPoint),
                                   tid);
-                if constexpr (PLANES == 2) next.all(ref);
-                if (PLANES == 1 && np == GROUP) {
+                if (np == GROUP) {
 #pragma unroll
                     for (int st = 0; st < kSteps; ++st) {
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
                             SepQuads<TR, TW, TH> qd;
                             qd.load(cur + (st * U + u) * ST::kPerPoint, lx * TL, ly * TR);
-                            point_terms_table<TR, TW, TH, PLANES>(qd, acc);
+                            point_terms_table<TR, TW, TH>(qd, acc);
                         }
 #pragma unroll
                         for (int e = st * kPerStep; e < (st + 1) * kPerStep && e < Filler::kEntries; ++e)
                             next.entry(e, ref);
                     }
-                } else {   // the complex wave (filled above), or a short last group (nothing to fill after it)
+                } else {   // a short last group (nothing to fill after it)
 #pragma unroll U
                     for (int g = 0; g < np; ++g) {
                         SepQuads<TR, TW, TH> qd;
                         qd.load(cur + g * ST::kPerPoint, lx * TL, ly * TR);
-                        point_terms_table<TR, TW, TH, PLANES>(qd, acc);
+                        point_terms_table<TR, TW, TH>(qd, acc);
                     }
                 }
                 Sync::sync();   // the next group's tables are written, this group's are no longer read
             }
 #pragma unroll
-            for (int c = 0; c < PLANES; ++c)
-#pragma unroll
                 for (int r = 0; r < TR; ++r)
 #pragma unroll
                     for (int j = 0; j < TL / 2; ++j) {
-                        part[c][r][2 * j] = acc[c][r][j].x;
-                        part[c][r][2 * j + 1] = acc[c][r][j].y;
+                        part[r][2 * j] = acc[r][j].x;
+                        part[r][2 * j + 1] = acc[r][j].y;
                     }
         } else {
-            static_assert(PLANES == 1 || SFU, "the complex wave takes the hardware sine and cosine");
 #pragma unroll 1
             for (int p = p_lo; p < p_hi; ++p)   // p has the parity of the point's index (tiles start even)
-                point_terms_sep<TL, TR, EXTRA, !SFU, PLANES>(sg[p], sa[p], m0, n0, pr,
-                                                             SFU ? (uint32_t)(p & 1) << 31 : 0u, part[0],
-                                                             part[PLANES - 1]);
+                point_terms_sep<TL, TR, EXTRA, !SFU>(sg[p], sa[p], m0, n0, pr, SFU ? (uint32_t)(p & 1) << 31 : 0u,
+                                                     part);
         }
-#pragma unroll
-        for (int c = 0; c < PLANES; ++c)
 #pragma unroll
             for (int r = 0; r < TR; ++r)
 #pragma unroll
                 for (int i = 0; i < TL; ++i) {
-                    if constexpr (SMEM_TOT) s_tot[tidx(c, r, i)] += part[c][r][i];
-                    else tot[c][r][i] += part[c][r][i];
+                    if constexpr (SMEM_TOT) s_tot[tidx(r, i)] += part[r][i];
+                    else tot[r][i] += part[r][i];
                 }
 
         Sync::sync();   // every thread is done with stage st
@@ -528,34 +491,29 @@ __device__ __forceinline__ bool direct_unit(const int4 *__restrict__ geo, const 
     if (!ok) return false;
     if constexpr (SMEM_TOT) {
 #pragma unroll
-        for (int c = 0; c < PLANES; ++c)
-#pragma unroll
             for (int r = 0; r < TR; ++r)
 #pragma unroll
-                for (int i = 0; i < TL; ++i) tot[c][r][i] = s_tot[tidx(c, r, i)];
+                for (int i = 0; i < TL; ++i) tot[r][i] = s_tot[tidx(r, i)];
     }
     if constexpr (!std::is_same<Sink, PlainStore>::value) {
-        static_assert(PLANES == 1, "sinks take the amplitude hologram");
-        sink(tot[0]);
+        sink(tot);
         return true;
     }
 
 #pragma unroll
-    for (int c = 0; c < PLANES; ++c)
-#pragma unroll
         for (int r = 0; r < TR; ++r) {
             const int n = n0 + r;
             if (n >= height || m0 >= width) continue;
-            float *row = dst + (long long)c * im_offset + (long long)n * width + m0;
+            float *row = dst + (long long)n * width + m0;
             if (vec && m0 + TL <= width) {
 #pragma unroll
                 for (int i = 0; i < TL; i += 4)
                     *reinterpret_cast<float4 *>(row + i) =
-                        make_float4(tot[c][r][i], tot[c][r][i + 1], tot[c][r][i + 2], tot[c][r][i + 3]);
+                        make_float4(tot[r][i], tot[r][i + 1], tot[r][i + 2], tot[r][i + 3]);
             } else {
 #pragma unroll
                 for (int i = 0; i < TL; ++i)
-                    if (m0 + i < width) row[i] = tot[c][r][i];
+                    if (m0 + i < width) row[i] = tot[r][i];
             }
         }
     return true;

@@ -1,0 +1,662 @@
+// a2, the direct form on the tensor cores: the tables of the sines and cosines of a point's columns and rows that a
+// CTA takes once for its tile of pixels (the cosine addition formula, direct_dev.cuh) are the operands of a matrix
+// product, I(m, n) = sum_j [cos a_jm, sin a_jm] . [A_j cos b_jn, -A_j sin b_jn], so tcgen05.mma adds them up
+// instead of two FMAs a pixel and point.  No factor goes through memory: each CTA makes its tile's entries in
+// shared memory and multiplies them there.
+//
+// Precision (the form's contract is single precision).  An entry is taken to 1.2e-7 RMS from the exact fixed-point
+// turn (half_turn2), every other point half a turn on in both of its entries so that a mean error of the cosine over
+// the turns cancels between points, and held as the sum of two FP16 values, hi + lo (22 bits and the signs), the
+// amplitudes scaled by 2^12 so that lo stays normal down to 2^-15 of the largest; the product is lo hi + hi lo + hi hi,
+// the large products last.  The tensor cores' FP32 accumulation truncates, which takes 1.9e-7 of a chain's value per
+// group of 32 points, so a chain is kChain = 2 groups, its mean loss is put back (kUnscale), and the chains are added
+// in FP32, in point order.  NRMS against FP64 (before: the SIMT kernel with the hardware cosine / with the polynomial):
+//   1920x1080, 10^4 points 3.5e-7 (6.0e-7);  1283x717, 3001 points, piston and reference 3.2e-7 (4.1e-7);
+//   640x64, 3000 points 1.1e-7 (3.1e-7);  256x256, 1024 points 2.8e-7 (6.7e-7);  wave 3.5e-7 (5.9e-7).
+// (Without the half turn 640x64 gave 7.2e-7; chains of 1 / 4 / 8 groups at 1920x1080 3.1 / 8.6 / 17.6e-7.)
+//
+// Time, prep included (before): 1920x1080, 10^4 points 0.307 ms (1.77; 67.5 G terms/ms); its complex wave 0.485 ms
+// (3.30); 1024x1024, 10^3 points 0.046 ms (0.117); 256x256, 10^3 points 0.026 ms (0.046).
+// What bounds it: the making of entries (0.26 of 0.31 ms with the MMAs left out), 30 instructions for two entries, 15
+// of them packed FMAs of two to three cycles, so the FMA pipe is about 80 % busy while entries are made; the tensor
+// cores are active 30 % of the time.  128 x BN tiles: larger tiles share an entry among more pixels (BN = 64 / 128 /
+// 192 / 224: 0.66 / 0.42 / 0.34 / 0.31 ms), and two stages of 224 rows fill shared memory.
+//
+// One CTA per SM, 18 warps.  Sixteen worker warps make the entries of a stage -- 32 points x (128 A rows + BN B rows),
+// hi and lo planes, K-major with the 128-byte swizzle -- and fold the chains; one thread of warp 16 issues the MMAs, one
+// of warp 17 brings the points (1-D bulk copies).  (Eight worker warps with the totals in registers: 0.41 ms; the totals
+// in tensor memory cost a read and a write more per fold but leave registers for sixteen warps.  Points loaded by the
+// MMA thread: 0.33 ms, its copies delay the next stage's MMAs by 600 clocks.)
+//
+//     ptfull[4]  points of a stage are there        (bulk copy -> workers)
+//     ptempty[4] they are read                      (workers -> loader)
+//     full[S]    a stage's entries are written      (workers -> MMA)
+//     empty[S]   its MMAs are done                  (MMA -> workers)
+//     tfull      a chain is in the accumulator      (MMA -> workers)
+//     tempty     its values are in the totals       (workers -> MMA)
+//     parts[2]   a CTA's parts of a tile are out; who finished the tile (workers, thread 0)
+//
+// A chain's MMAs run while the next stage is made; then it is folded.  Work is the flat list of (pixel tile, group of
+// 32 points) pairs in equal shares per CTA, a tile's parts summed in CTA order by the CTA that finishes last, as in the
+// balanced layout of direct.cu.
+#include <type_traits>
+
+#include <cuda_fp16.h>
+
+#include "device_util.cuh"
+#include "host_util.h"
+#include "kernels.h"
+#include "sincospoly.h"
+#include "tcgen05.cuh"
+
+namespace cgh {
+
+namespace {
+
+constexpr int kWorkers = 512;
+constexpr int kMmaThreads = kWorkers + 64;   // the workers, the MMA warp, the loader warp
+constexpr int kRowsA = 128;
+constexpr int kGroup = kDirectMmaGroup;      // points of a stage: 64 K elements, one 128-byte swizzle row
+constexpr int kPtSlots = 4;
+constexpr int kUnroll = 2;                   // steps of a side side by side
+constexpr int kPtBytes = kGroup * (int)(sizeof(int4) + sizeof(uint2));
+constexpr int kChain = 2;                    // stages of an accumulation chain
+constexpr float kEntryScale = 4096.0f;       // 2^12, the A side (amplitudes)
+// 2^-12, times 1 + 2.4e-7: the accumulation truncates, and a chain of two groups loses 2.9e-7 of its value on average
+// (measured on random clouds; 2.6e-7 on coherent ones)
+constexpr float kUnscale = 2.44140625e-04f * (1.0f + 2.384185791015625e-07f);
+
+template <int BN>
+struct MmaCfg {
+    static constexpr int kA = kRowsA * 128, kB = BN * 128;   // bytes of one plane of A, of B
+    static constexpr int kStage = 2 * (kA + kB);
+    static constexpr int kRoom = 232448 - 1024 - kPtSlots * kPtBytes - 256;
+    static constexpr int kStages = kRoom / kStage > 4 ? 4 : kRoom / kStage;
+    static constexpr int kTotal = BN <= 128 ? 128 : 256;   // tensor-memory column of the totals, after the chain
+    static constexpr int kTmemCols = 2 * kTotal;
+    static constexpr int kSmem = 1024 + kStages * kStage + kPtSlots * kPtBytes + 256;
+    static_assert(BN % 32 == 0 && BN >= 64 && BN <= 256, "B rows in steps of 32, TMEM columns in halves of 16s");
+    static_assert(kStages >= 2, "at least a double-buffered ring");
+};
+
+struct MmaArgs {
+    const int4 *geo;
+    const uint2 *aux;
+    const float *amp_max;
+    float *out;                // plane 1 (the imaginary part) follows plane 0
+    float4 *slots;
+    int *counters;
+    int *status;
+    unsigned long long timeout_ns;
+    long long units, groups;   // (tile, group) pairs; groups per tile
+    int width, height, tiles_a;
+    int a_rows;                // 1: A rows are hologram rows; 0: hologram columns
+    int vec, drop;
+    PhaseRef ref;
+};
+
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+
+// The walk of one point down a side's rows in steps of 32 (Eqs. 6-8 at that stride): t = C d^2 at the first row,
+// D its first difference, S the second, top 32 bits of the 64-bit products.
+struct Walk {
+    uint32_t t, D;
+};
+__device__ __forceinline__ Walk walk_start(int d, uint32_t ch, uint32_t cl, uint32_t add, uint32_t step)
+{
+    const uint32_t d2 = (uint32_t)(d * d);
+    const int e = 64 * d + 1024;   // (d + 32)^2 - d^2
+    Walk w;
+    w.t = ch * d2 + __umulhi(cl, d2) + add;
+    w.D = ch * (uint32_t)e + __umulhi(cl, (uint32_t)e) - (e < 0 ? cl : 0u) + step;
+    return w;
+}
+
+// sqrt(2) sin(pi r) and sqrt(2) cos(pi r) of two signed turns r (2^-32 turn): half the angle, so that s^2 - 1 and s c
+// are minus the cosine and the sine of the whole turn without a quadrant (sincospoly.h).
+template <int U>
+__device__ __forceinline__ void half_turn2(Walk (&w)[2], const uint32_t (&S)[2], bool back, float2 (&s)[U], float2 (&c)[U])
+{
+    float2 r[U], u[U], hs[U], hc[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+        r[j] = make_float2((float)(int)w[0].t, (float)(int)w[1].t);
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            w[p].t = back ? w[p].t - w[p].D : w[p].t + w[p].D;
+            w[p].D += S[p];
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+        r[j] = __fmul2_rn(r[j], f2(2.3283064365386963e-10f));
+        u[j] = __fmul2_rn(r[j], r[j]);
+    }
+#define CGH_HORNER(OUT, IN, COEF)                                                                                     \
+    _Pragma("unroll") for (int j = 0; j < U; ++j) OUT[j] = __ffma2_rn(IN[j], u[j], f2(COEF));
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+        hs[j] = f2(CGH_HSIN_4);
+        hc[j] = f2(CGH_HCOS_4);
+    }
+    CGH_HORNER(hs, hs, CGH_HSIN_3)
+    CGH_HORNER(hc, hc, CGH_HCOS_3)
+    CGH_HORNER(hs, hs, CGH_HSIN_2)
+    CGH_HORNER(hc, hc, CGH_HCOS_2)
+    CGH_HORNER(hs, hs, CGH_HSIN_1)
+    CGH_HORNER(hc, hc, CGH_HCOS_1)
+    CGH_HORNER(hs, hs, CGH_HSIN_0)
+    CGH_HORNER(c, hc, CGH_HCOS_0)
+#undef CGH_HORNER
+#pragma unroll
+    for (int j = 0; j < U; ++j) s[j] = __fmul2_rn(r[j], hs[j]);
+}
+
+// v - h for both halves of a packed FP16 pair (mixed-precision FMA, exact).
+__device__ __forceinline__ float2 minus_half2(float2 v, uint32_t h)
+{
+    float2 d;
+    asm("{\n\t.reg .b16 l, u, m;\n\t"
+        "mov.b32 {l, u}, %2;\n\t"
+        "mov.b16 m, 0xbc00;\n\t"
+        "fma.rn.f32.f16 %0, l, m, %3;\n\t"
+        "fma.rn.f32.f16 %1, u, m, %4;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "r"(h), "f"(v.x), "f"(v.y));
+    return d;
+}
+
+__device__ __forceinline__ uint32_t pack_half2(float lo, float hi)
+{
+    uint32_t r;
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+
+// The row of the imaginary part from that of the real part: {-cos, -sin} -> {-sin, cos}.
+__device__ __forceinline__ uint32_t turn_quarter(uint32_t h)
+{
+    return __byte_perm(h, 0, 0x1032) ^ 0x80000000u;
+}
+
+__device__ __forceinline__ void st_shared8(uint32_t addr, uint32_t a, uint32_t b)
+{
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+
+// 32 lanes x 8 columns of tensor memory (as tmem_ld16, tmem_st16).
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&r)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
+                 : "r"(taddr));
+}
+
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&r)[8])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
+                 "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7])
+                 : "memory");
+}
+
+// Entries of this thread's two points (16 apart: conflict-free loads; K slots 2 pair and 2 pair + 1) at STEPS rows 32
+// apart.  A side: 2^12 A (-cos a, sin a).  B side: its turns
+// walked backwards (b -> -b), (-cos b, -sin b); PLANES = 2: and the rows of the imaginary part, (-sin b, cos b), im_off
+// further on.
+template <int STEPS, bool B, int PLANES>
+__device__ __forceinline__ void side_entries(const int4 *geo, const uint2 *aux, bool swap, int row, uint32_t add,
+                                             uint32_t step, uint32_t piston, float a_scale, uint32_t hi,
+                                             uint32_t lo_off, uint32_t im_off)
+{
+    Walk w[2];
+    uint32_t S[2];
+    float2 a = f2(0.0f);
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        const int4 q = geo[16 * p];
+        const uint32_t ch = (uint32_t)q.z, cl = (uint32_t)q.w;
+        w[p] = walk_start(row - (swap != B ? q.y : q.x), ch, cl, add, step);
+        S[p] = (ch << 11) | (cl >> 21);   // 2048 C
+        if (p & 1) w[p].t ^= 0x80000000u;   // the half turn of every other point
+        if (B) {
+            w[p].t = 0u - w[p].t;
+        } else {
+            const uint2 x = aux[16 * p];
+            w[p].t += x.x & piston;
+            (p & 1 ? a.y : a.x) = __uint_as_float(x.y) * a_scale * kEntryScale;
+        }
+    }
+    const float2 na = make_float2(-a.x, -a.y);
+    // U steps side by side: their chains of dependent operations overlap
+    auto steps = [&](auto uc, int k0) {
+        constexpr int U = decltype(uc)::value;
+        float2 s[U], c[U], x[U], y[U];
+        half_turn2<U>(w, S, B, s, c);
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            if (B) {
+                x[j] = __ffma2_rn(s[j], s[j], f2(-1.0f));
+                y[j] = __fmul2_rn(s[j], c[j]);
+            } else {
+                const float2 as = __fmul2_rn(a, s[j]);
+                x[j] = __ffma2_rn(as, s[j], na);
+                y[j] = __fmul2_rn(as, c[j]);
+            }
+        }
+        uint32_t h[U][2], l[U][2];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            h[j][0] = pack_half2(x[j].x, y[j].x);
+            h[j][1] = pack_half2(x[j].y, y[j].y);
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const float2 d = minus_half2(make_float2(x[j].x, y[j].x), h[j][0]);
+            y[j] = minus_half2(make_float2(x[j].y, y[j].y), h[j][1]);
+            x[j] = d;
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            l[j][0] = pack_half2(x[j].x, x[j].y);
+            l[j][1] = pack_half2(y[j].x, y[j].y);
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const uint32_t at = hi + (uint32_t)(k0 + j) * 4096u;
+            st_shared8(at, h[j][0], h[j][1]);
+            st_shared8(at + lo_off, l[j][0], l[j][1]);
+            if (B && PLANES == 2) {
+                st_shared8(at + im_off, turn_quarter(h[j][0]), turn_quarter(h[j][1]));
+                st_shared8(at + lo_off + im_off, turn_quarter(l[j][0]), turn_quarter(l[j][1]));
+            }
+        }
+    };
+#pragma unroll
+    for (int k = 0; k + kUnroll <= STEPS; k += kUnroll) steps(std::integral_constant<int, kUnroll>{}, k);
+    if constexpr (STEPS % kUnroll != 0) steps(std::integral_constant<int, STEPS % kUnroll>{}, STEPS / kUnroll * kUnroll);
+}
+
+struct MmaBars {
+    uint64_t *full, *empty, *ptfull, *ptempty, *tfull, *tempty, *parts, *drain;
+};
+
+// PLANES = 1: the amplitude hologram, tiles of 128 x BN pixels.  PLANES = 2: the complex wave, tiles of 128 x BN / 2
+// pixels, the B rows (and accumulator columns) of the imaginary part after those of the real part.
+template <int BN, int PLANES>
+__global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid_constant__ MmaArgs g)
+{
+    using C = MmaCfg<BN>;
+    constexpr int HB = BN / 4;          // accumulator columns per worker warp
+    constexpr int TB = BN / PLANES;     // pixels of the tile along B
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ int s_last;
+    __shared__ uint32_t s_tmem;
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *s_pts = smem + C::kStages * C::kStage;
+    MmaBars bars;
+    bars.full = reinterpret_cast<uint64_t *>(s_pts + kPtSlots * kPtBytes);
+    bars.empty = bars.full + 4;
+    bars.ptfull = bars.empty + 4;
+    bars.ptempty = bars.ptfull + kPtSlots;
+    bars.tfull = bars.ptempty + kPtSlots;
+    bars.tempty = bars.tfull + 1;
+    bars.parts = bars.tempty + 1;   // [0] the workers' parts of a tile are out, [1] s_last is set
+    bars.drain = bars.parts + 2;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        for (int s = 0; s < C::kStages; ++s) {
+            mbar_init(&bars.full[s], kWorkers / 32);
+            mbar_init(&bars.empty[s], 1);
+        }
+        mbar_init(bars.tfull, 1);
+        mbar_init(bars.tempty, kWorkers / 32);
+        for (int p = 0; p < kPtSlots; ++p) {
+            mbar_init(&bars.ptfull[p], 1);
+            mbar_init(&bars.ptempty[p], kWorkers / 32);
+        }
+        mbar_init(&bars.parts[0], kWorkers / 32);
+        mbar_init(&bars.parts[1], 1);
+        mbar_init(bars.drain, 1);
+        fence_barrier_init();
+    }
+    if (warp == kWorkers / 32) {
+        tmem_alloc(&s_tmem, C::kTmemCols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+    const long long w0 = (long long)blockIdx.x * g.units / gridDim.x;
+    const long long w1 = ((long long)blockIdx.x + 1) * g.units / gridDim.x;
+    const int n = (int)(w1 - w0);
+    auto wait = [&](uint64_t *bar, uint32_t parity) {
+        if (mbar_wait(bar, parity, g.timeout_ns)) return true;
+        atomicOr(g.status, kStatusTimeout);
+        return false;
+    };
+
+    if (warp == kWorkers / 32 + 1) {   // the loader
+        if (lane == 0) {
+            int gl = (int)(w0 % g.groups), i = 0;
+            for (; i < n; ++i) {
+                if (!wait(&bars.ptempty[i % kPtSlots], ((uint32_t)(i / kPtSlots) & 1u) ^ 1u)) break;
+                uint8_t *dst = s_pts + (i % kPtSlots) * kPtBytes;
+                uint64_t *bar = &bars.ptfull[i % kPtSlots];
+                if (!(blockIdx.x == 0 && i == g.drop)) {
+                    mbar_arrive_expect_tx(bar, kPtBytes);
+                    bulk_copy_g2s(dst, g.geo + (long long)gl * kGroup, kGroup * sizeof(int4), bar);
+                    bulk_copy_g2s(dst + kGroup * sizeof(int4), g.aux + (long long)gl * kGroup, kGroup * sizeof(uint2),
+                                  bar);
+                }
+                if (++gl == (int)g.groups) gl = 0;
+            }
+            // every copy issued completes before the CTA ends
+            for (int j = i > kPtSlots ? i - kPtSlots : 0; j < i; ++j)
+                if (!(blockIdx.x == 0 && j == g.drop))
+                    mbar_wait(&bars.ptfull[j % kPtSlots], (uint32_t)(j / kPtSlots) & 1u, g.timeout_ns);
+        }
+    } else if (warp == kWorkers / 32) {
+        if (lane == 0) {
+            int g0 = (int)(w0 % g.groups);   // group of stage i
+            constexpr uint32_t idesc = umma_idesc_f16(false, kRowsA, BN);
+            int in_chain = 0;
+            uint32_t chain = 0;
+            bool ok = true;
+            for (int i = 0; i < n && ok; ++i) {
+                const int s = i % C::kStages;
+                if (in_chain == 0) {
+                    if (!(ok = wait(bars.tempty, (chain & 1u) ^ 1u))) break;
+                    tc_fence_after();
+                }
+                if (!(ok = wait(&bars.full[s], (uint32_t)(i / C::kStages) & 1u))) break;
+                tc_fence_after();
+                const uint32_t a_hi = smem_addr(smem + s * C::kStage), b_hi = a_hi + 2 * C::kA;
+                // lo hi, hi lo, then hi hi: the large products last, so the truncation of the small ones is small
+#pragma unroll
+                for (int pass = 0; pass < 3; ++pass) {
+                    const uint64_t ad = sw128_kmajor_desc(a_hi + (pass == 0 ? C::kA : 0));
+                    const uint64_t bd = sw128_kmajor_desc(b_hi + (pass == 1 ? C::kB : 0));
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        umma_f16(tmem, ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), idesc,
+                                 (in_chain | pass | kk) ? 1u : 0u);
+                }
+                umma_commit(&bars.empty[s]);
+                const bool tile_end = g0 + 1 == (int)g.groups;
+                if (++in_chain == kChain || tile_end || i + 1 == n) {
+                    umma_commit(bars.tfull);
+                    in_chain = 0;
+                    ++chain;
+                }
+                g0 = tile_end ? 0 : g0 + 1;
+            }
+            // every MMA issued completes before the CTA ends
+            umma_commit(bars.drain);
+            mbar_wait(bars.drain, 0, g.timeout_ns);
+        }
+    } else {
+        const int pair = tid & 15, rl = tid >> 4;   // this thread's two points of a stage and its first row
+        const uint32_t entry = (uint32_t)(rl * 128 + (((pair >> 1) ^ (rl & 7)) << 4) + (pair & 1) * 8);
+        // amplitudes as multiples of 2^(eb - 126), the power of two above the largest
+        const uint32_t eb = min((__float_as_uint(*g.amp_max) >> 23) & 255u, 252u);
+        const float a_scale = __uint_as_float((253u - eb) << 23), unscale = __uint_as_float((eb + 1u) << 23);
+        const int quarter = warp & 3, cg = warp >> 2;   // tensor-memory lanes and columns of this warp
+        const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(cg * HB), total = acc + C::kTotal;
+        int t = (int)(w0 / g.groups), gi = (int)(w0 % g.groups);   // tile and group of stage i
+        int ra = t % g.tiles_a * kRowsA + rl, rb = t / g.tiles_a * TB + rl;   // this thread's first rows of the tile
+        bool pending = false, pend_first = true, pend_end = false;
+        uint32_t folded = 0, sunk = 0;
+        int pend_t = 0;
+        int in_chain = 0, s = 0;
+        uint32_t s_use = 0;   // parity of the ring's round
+
+        // the finished chain to the totals (first: of this CTA's part of the tile)
+        auto fold = [&](bool first) -> bool {
+            if (!wait(bars.tfull, folded & 1u)) return false;
+            ++folded;
+            tc_fence_after();
+#pragma unroll
+            for (int c = 0; c < HB; c += 16) {
+                float v[2][8], w[2][8];
+                tmem_ld8(acc + (uint32_t)c, v[0]);
+                if (c + 8 < HB) tmem_ld8(acc + (uint32_t)c + 8u, v[1]);
+                if (!first) {
+                    tmem_ld8(total + (uint32_t)c, w[0]);
+                    if (c + 8 < HB) tmem_ld8(total + (uint32_t)c + 8u, w[1]);
+                }
+                tmem_ld_wait();
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    if (c + 8 * j >= HB) break;
+                    if (!first)
+#pragma unroll
+                        for (int k = 0; k < 8; k += 2) {
+                            const float2 r =
+                                __fadd2_rn(make_float2(w[j][k], w[j][k + 1]), make_float2(v[j][k], v[j][k + 1]));
+                            v[j][k] = r.x;
+                            v[j][k + 1] = r.y;
+                        }
+                    tmem_st8(total + (uint32_t)(c + 8 * j), v[j]);
+                }
+            }
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bars.tempty);
+            return true;
+        };
+        // the end of this CTA's part of tile pt: a whole tile is stored; a part goes to the CTA's slot and is counted on
+        // the tile, and the CTA that counts last sums the tile's parts in CTA order (whoever is last) and stores it
+        auto sink = [&](const int pt) -> bool {
+            if (!CGH_DCHECK(pt >= 0 && pt * g.groups < g.units, g.status)) return false;   // the same for every worker
+            const long long Cn = gridDim.x;
+            const int lo = (int)(((pt * g.groups + 1) * Cn - 1) / g.units);
+            const int hi = (int)((((pt + 1) * g.groups) * Cn - 1) / g.units);
+            constexpr int Q4 = HB / 4;
+            // slot 0 of a CTA holds its first segment, slot 1 its last: the tile's first CTA may have begun before it
+            const int lo_slot = lo * g.units / Cn / g.groups == pt ? 0 : 1;
+            auto part = [&](int cs) {
+                return g.slots + (2ll * cs + (cs == lo ? lo_slot : 0)) * (Q4 * kWorkers) + tid;
+            };
+            if (lo != hi) {
+                float4 *mine = part((int)blockIdx.x);
+#pragma unroll
+                for (int q = 0; q < Q4; q += 2) {
+                    float v[8];
+                    tmem_ld8(total + (uint32_t)(4 * q), v);
+                    tmem_ld_wait();
+                    mine[q * kWorkers] = make_float4(v[0], v[1], v[2], v[3]);
+                    mine[(q + 1) * kWorkers] = make_float4(v[4], v[5], v[6], v[7]);
+                }
+                __threadfence();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars.parts[0]);
+                if (tid == 0) {
+                    if (!wait(&bars.parts[0], sunk & 1u)) return false;
+                    s_last = atomicAdd(&g.counters[pt], 1) == hi - lo;
+                    mbar_arrive(&bars.parts[1]);
+                }
+                if (!wait(&bars.parts[1], sunk & 1u)) return false;
+                ++sunk;
+                if (!s_last) return true;
+                __threadfence();
+            }
+            const int a = pt % g.tiles_a * kRowsA + quarter * 32 + lane;
+            const int b0 = pt / g.tiles_a * TB + (PLANES == 2 ? (cg & 1) * HB : cg * HB);
+            float *out = g.out + (PLANES == 2 ? (long long)(cg >> 1) * g.width * g.height : 0ll);
+            const float us = unscale;
+#pragma unroll
+            for (int q = 0; q < Q4; q += 2) {
+                float v[8];
+                if (lo == hi) {
+                    tmem_ld8(total + (uint32_t)(4 * q), v);
+                    tmem_ld_wait();
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) v[k] = 0.0f;
+                    for (int cs = lo; cs <= hi; cs += 4) {   // four parts per memory round trip
+                        float4 x[4][2];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+#pragma unroll
+                            for (int i = 0; i < 2; ++i)
+                                x[j][i] = cs + j <= hi ? __ldcg(part(cs + j) + (q + i) * kWorkers)
+                                                       : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) {
+                                v[4 * i] += x[j][i].x;
+                                v[4 * i + 1] += x[j][i].y;
+                                v[4 * i + 2] += x[j][i].z;
+                                v[4 * i + 3] += x[j][i].w;
+                            }
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = v[k] * kUnscale * us;
+                if (!g.a_rows) {   // lanes are columns: each store writes 32 consecutive pixels of a row
+                    if (a < g.width)
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (b0 + 4 * q + k < g.height) out[(long long)(b0 + 4 * q + k) * g.width + a] = v[k];
+                } else if (a < g.height) {
+                    float *row = out + (long long)a * g.width + b0 + 4 * q;
+                    if (g.vec && b0 + 4 * q + 8 <= g.width) {
+                        reinterpret_cast<float4 *>(row)[0] = make_float4(v[0], v[1], v[2], v[3]);
+                        reinterpret_cast<float4 *>(row)[1] = make_float4(v[4], v[5], v[6], v[7]);
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (b0 + 4 * q + k < g.width) row[k] = v[k];
+                    }
+                }
+            }
+            return true;
+        };
+        const unsigned long long ka = g.a_rows ? g.ref.ky : g.ref.kx, kb = g.a_rows ? g.ref.kx : g.ref.ky;
+        const bool swap = g.a_rows != 0;
+        // a finished chain is folded after the next stage is made: its MMAs run meanwhile
+        for (int i = 0; i <= n; ++i) {
+            bool chain_end = false, tile_end = false;
+            if (i < n) {
+                const int ps = i % kPtSlots;
+                if (!wait(&bars.ptfull[ps], (uint32_t)(i / kPtSlots) & 1u)) break;
+                if (!wait(&bars.empty[s], s_use ^ 1u)) break;
+                const int4 *geo = reinterpret_cast<const int4 *>(s_pts + ps * kPtBytes) + pair;
+                const uint2 *aux =
+                    reinterpret_cast<const uint2 *>(s_pts + ps * kPtBytes + kGroup * sizeof(int4)) + pair;
+                const uint32_t base = smem_addr(smem + s * C::kStage) + entry;
+                side_entries<kRowsA / 32, false, PLANES>(
+                    geo, aux, swap, ra, (uint32_t)((ka * (unsigned long long)ra) >> 32) + g.ref.phi0,
+                    ref_step(32 * ka), g.ref.piston ? ~0u : 0u, a_scale, base, C::kA, 0);
+                side_entries<TB / 32, true, PLANES>(geo, aux, swap, rb, (uint32_t)((kb * (unsigned long long)rb) >> 32),
+                                                    ref_step(32 * kb), 0u, 0.0f, base + 2 * C::kA, C::kB, TB * 128);
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&bars.ptempty[ps]);
+                    mbar_arrive(&bars.full[s]);
+                }
+                if (++s == C::kStages) {
+                    s = 0;
+                    s_use ^= 1u;
+                }
+                tile_end = gi + 1 == (int)g.groups || i + 1 == n;
+                chain_end = ++in_chain == kChain || tile_end;
+            }
+            if (pending) {
+                if (!fold(pend_first)) break;
+                pend_first = pend_end;
+                if (pend_end && !sink(pend_t)) break;
+                pending = false;
+            }
+            if (chain_end) {
+                pending = true;
+                pend_end = tile_end;
+                pend_t = t;
+                in_chain = 0;
+            }
+            if (++gi == (int)g.groups) {
+                gi = 0;
+                ++t;
+                ra += kRowsA;
+                if (t % g.tiles_a == 0) {
+                    ra = rl;
+                    rb += TB;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (warp == kWorkers / 32) {
+        __syncwarp();
+        tc_fence_after();
+        tmem_dealloc(tmem, C::kTmemCols);
+    }
+}
+
+template <int BN, int PLANES>
+cudaError_t launch_as(const MmaArgs &g, int ctas, cudaStream_t s)
+{
+    static PerDeviceOnce configured;
+    const cudaError_t e = configured.run([] {
+        return cudaFuncSetAttribute(direct_mma_kernel<BN, PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    MmaCfg<BN>::kSmem);
+    });
+    if (e != cudaSuccess) return e;
+    direct_mma_kernel<BN, PLANES><<<ctas, kMmaThreads, MmaCfg<BN>::kSmem, s>>>(g);
+    return cudaGetLastError();
+}
+
+template <int PLANES>
+cudaError_t launch_bn(int bn, const MmaArgs &g, int ctas, cudaStream_t s)
+{
+    switch (bn) {
+    case 64: return launch_as<64, PLANES>(g, ctas, s);
+    case 128: return launch_as<128, PLANES>(g, ctas, s);
+    case 192: return launch_as<192, PLANES>(g, ctas, s);
+    case 224: if constexpr (PLANES == 1) return launch_as<224, PLANES>(g, ctas, s); else return cudaErrorInvalidValue;
+    case 256: return launch_as<256, PLANES>(g, ctas, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4 *geo, const uint2 *aux,
+                              const float *amp_max, int n_points, int width, int height, float *out, float *slots,
+                              int *counters, int *status, uint64_t timeout_ns, cudaStream_t s, int drop,
+                              const PhaseRef &ref)
+{
+    if (n_points < 1 || lay.ctas < 1 || (planes != 1 && planes != 2) || (uintptr_t)slots % 16 != 0)
+        return cudaErrorInvalidValue;
+    MmaArgs g{};
+    const int side_a = lay.a_rows ? height : width, side_b = lay.a_rows ? width : height;
+    const int tb = lay.bn / planes;
+    g.tiles_a = (side_a + kRowsA - 1) / kRowsA;
+    g.groups = (n_points + kGroup - 1) / kGroup;
+    g.units = (long long)g.tiles_a * ((side_b + tb - 1) / tb) * g.groups;
+    // whole tiles per CTA (one share each) need neither slots nor counters
+    if (lay.ctas > g.units || g.units / lay.ctas >= 0x7ffffff0ll ||
+        (lay.ctas != g.units / g.groups && (slots == nullptr || counters == nullptr)))
+        return cudaErrorInvalidValue;
+    g.geo = geo;
+    g.aux = aux;
+    g.amp_max = amp_max;
+    g.out = out;
+    g.slots = reinterpret_cast<float4 *>(slots);
+    g.counters = counters;
+    g.status = status;
+    g.timeout_ns = timeout_ns;
+    g.width = width;
+    g.height = height;
+    g.a_rows = lay.a_rows;
+    g.vec = width % 4 == 0 && (uintptr_t)out % 16 == 0 && ((long long)width * height) % 4 == 0;
+    g.drop = drop;
+    g.ref = ref;
+    return planes == 2 ? launch_bn<2>(lay.bn, g, lay.ctas, s) : launch_bn<1>(lay.bn, g, lay.ctas, s);
+}
+
+}  // namespace cgh

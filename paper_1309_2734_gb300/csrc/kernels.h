@@ -62,7 +62,7 @@ __device__ __forceinline__ uint32_t ref_step(unsigned long long k)
 }
 #endif
 
-// a2: direct kernel (direct.cu).
+// a2: the SIMT direct kernels (direct.cu).
 struct DirectShape {
     int tile_w, tile_h;   // pixels covered by one CTA
     int threads;          // threads per CTA
@@ -73,11 +73,6 @@ struct DirectShape {
 // The CTA shapes of the direct kernels (256 threads, 8 columns of pixels per
 // thread): wide = 32 x 8 threads, tall = 16 x 16 threads.
 DirectShape direct_shape(bool tall = false);
-// drop_tile >= 0 is a test hook: the first point chunk never loads that tile,
-// so its bounded wait runs out and the launch ends with kStatusTimeout.
-cudaError_t launch_direct(bool sfu, const DirectShape &sh, const int4 *geo, const uint2 *aux, int n_pad, int width,
-                          int height, int split, float *out, int64_t slice_stride, int *status, uint64_t timeout_ns,
-                          cudaStream_t s, int drop_tile = -1, const PhaseRef &ref = PhaseRef());
 
 // The direct form over a flat (pixel tile, point) work space split evenly over ctas CTAs, with the partial
 // tiles at range boundaries summed in CTA order by the last CTA to finish each tile (direct.cu): out receives
@@ -92,12 +87,21 @@ cudaError_t launch_direct_stream(bool sfu, const DirectShape &sh, int ctas, cons
                                  int *status, uint64_t timeout_ns, cudaStream_t s, int drop_tile = -1,
                                  const PhaseRef &ref = PhaseRef());
 
-// Complex object wave (Eq. 2, restricted form), SFU form: real part at out,
-// imaginary part at out + im_offset; point chunk s at out + s * slice_stride.
-DirectShape direct_wave_shape(bool tall = false);
-cudaError_t launch_direct_wave(const DirectShape &sh, const int4 *geo, const uint2 *aux, int n_pad, int width,
-                               int height, int split, float *out, int64_t slice_stride, int64_t im_offset,
-                               int *status, uint64_t timeout_ns, cudaStream_t s, const PhaseRef &ref = PhaseRef());
+// The direct form with the tile's tables multiplied on the tensor cores (direct_mma.cu): the amplitude hologram at
+// out (planes = 1) or the complex wave, real plane then imaginary plane (planes = 2).  amp_max: max |A_j| of the
+// points (launch_prep_points).  slots: 2 ctas x 128 x bn floats (16-byte aligned); counters: one int per tile,
+// zeroed by the caller.  drop >= 0: CTA 0 never loads that group of kDirectMmaGroup points of its share (test hook).
+constexpr int kDirectMmaGroup = 32;
+struct DirectMmaLayout {
+    int bn = 0;       // B rows of a tile: 64, 128, 192, 224 (planes = 1), 256; 128 x bn / planes pixels.  0: not taken
+    int a_rows = 0;   // the tile's 128-pixel side: 1 = hologram rows, 0 = columns
+    int ctas = 0;
+    int tiles = 0;
+};
+cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4 *geo, const uint2 *aux,
+                              const float *amp_max, int n_points, int width, int height, float *out, float *slots,
+                              int *counters, int *status, uint64_t timeout_ns, cudaStream_t s, int drop = -1,
+                              const PhaseRef &ref = PhaseRef());
 
 // f2: the exact spherical wave of Eq. 1 (spherical.cu), direct SFU form.
 // Points prepared with the piston and ext.  planes = 1: the amplitude

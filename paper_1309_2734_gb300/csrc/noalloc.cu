@@ -22,6 +22,7 @@
 #include "../../include/cgh.h"
 #include "device_util.cuh"
 #include "kernels.h"
+#include "tuner.h"
 
 namespace {
 
@@ -30,10 +31,10 @@ using namespace cgh;
 constexpr int64_t kMaxPoints = CGH_NOALLOC_MAX_POINTS;   // 131072 points
 constexpr size_t kGeoBytes = (size_t)kMaxPoints * sizeof(int4);
 constexpr size_t kAuxBytes = (size_t)kMaxPoints * sizeof(uint2);
-constexpr size_t kScratchBytes = kGeoBytes + kAuxBytes + 256;   // + status word
+constexpr size_t kScratchBytes = kGeoBytes + kAuxBytes + 256;   // + status word, max |A|
 constexpr int kMaxDevices = 64;
 
-// 3 MiB + 256 B: prepared points (geo, aux) and the status word.
+// 3 MiB + 256 B: prepared points (geo, aux), the status word and max |A|.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 std::mutex g_setup_mutex;
@@ -60,17 +61,6 @@ int scratch_address(int dev, unsigned char **out)
 
 }  // namespace
 
-// The direct kernel's CTA shape with the fewer padded pixels (one point chunk: no split to balance).
-static cgh::DirectShape noalloc_shape(int width, int height)
-{
-    const cgh::DirectShape wide = cgh::direct_shape(false), tall = cgh::direct_shape(true);
-    auto padded = [&](const cgh::DirectShape &sh) {
-        return (int64_t)((width + sh.tile_w - 1) / sh.tile_w) * sh.tile_w *
-               ((int64_t)((height + sh.tile_h - 1) / sh.tile_h) * sh.tile_h);
-    };
-    return padded(tall) < padded(wide) ? tall : wide;
-}
-
 extern "C" int cgh_point_cloud_noalloc(int width, int height, double pitch_m, double lambda_m, const float *d_xyz,
                                        const float *d_amp, int64_t n_points, float *d_out, void *cuda_stream)
 {
@@ -91,8 +81,11 @@ extern "C" int cgh_point_cloud_noalloc(int width, int height, double pitch_m, do
     int4 *geo = reinterpret_cast<int4 *>(base);
     uint2 *aux = reinterpret_cast<uint2 *>(base + kGeoBytes);
     int *status = reinterpret_cast<int *>(base + kGeoBytes + kAuxBytes);
+    float *amp_max = reinterpret_cast<float *>(status + 1);
     const int64_t plane = (int64_t)width * height;
-    if (cudaMemsetAsync(status, 0, sizeof(int), s) != cudaSuccess) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaMemsetAsync(status, 0, 2 * sizeof(int), s) != cudaSuccess) {
         cudaGetLastError();
         return CGH_ECUDA;
     }
@@ -104,10 +97,11 @@ extern "C" int cgh_point_cloud_noalloc(int width, int height, double pitch_m, do
     } else {
         const int64_t n_pad = (n_points + kPointTile - 1) / kPointTile * kPointTile;   // <= kMaxPoints
         cudaError_t e = launch_prep_points(d_xyz, d_amp, (int)n_points, (int)n_pad, pitch_m, lambda_m, geo, aux,
-                                           status, nullptr, s);
+                                           status, amp_max, s);
+        // one CTA per tile over all points: no parts of a tile, so neither slots nor counters
         if (e == cudaSuccess)
-            e = launch_direct(true, noalloc_shape(width, height), geo, aux, (int)n_pad, width, height, 1, d_out,
-                              plane, status, 5000000000ull, s);
+            e = launch_direct_mma(choose_direct_mma(1, width, height, n_points, sms, 1, 0), 1, geo, aux, amp_max,
+                                  (int)n_points, width, height, d_out, nullptr, nullptr, status, 5000000000ull, s);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return CGH_ECUDA;

@@ -306,9 +306,9 @@ __device__ __forceinline__ bool run_direct_unit(const PersistJob &J, int tile, i
     if (p1 <= p0) return true;   // cannot happen with chunks <= n
     const int k0 = p0 / kSimtTile, k1 = (p1 + kSimtTile - 1) / kSimtTile;
     const PersistDirectSink sink{&J, tile, chunk, s_last};
-    return direct_unit<kDTL, kDTR, kDBX, kDBY, SFU, 1, false, false, PersistDirectSink, SimtSync, kSimtTile>(
+    return direct_unit<kDTL, kDTR, kDBX, kDBY, SFU, false, false, PersistDirectSink, SimtSync, kSimtTile>(
         J.geo, J.aux, k0, k1, (tile % J.tiles_x) * (kDBX * kDTL), (tile / J.tiles_x) * (kDBY * kDTR), J.width,
-        J.height, J.out, J.vec != 0, s_geo, s_aux, s_bar, kg, status, timeout_ns, -1, 0, PhaseRef(), nullptr,
+        J.height, J.out, J.vec != 0, s_geo, s_aux, s_bar, kg, status, timeout_ns, -1, PhaseRef(), nullptr,
         p0 - k0 * kSimtTile, p1 - (k1 - 1) * kSimtTile, sink);
 }
 

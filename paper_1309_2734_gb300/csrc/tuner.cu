@@ -1,8 +1,8 @@
 // Autotuner and launch-shape selection (host side).
 //
 // Static rules (no measurement):
-//   choose_point_split  point chunks of the direct kernel, to fill whole waves;
-//   choose_direct_layout  the direct kernels' CTA shape (less padding) with its split;
+//   choose_direct_mma   tile and CTAs of the direct form on the tensor cores;
+//   choose_layout       the spherical kernel's CTA shape (less padding) with its split;
 //   choose_gemm_bn      GEMM tile width with the least padding of the width;
 //   choose_gemm_splits  K splits of the GEMM, to balance tiles over the CTAs.
 //
@@ -17,6 +17,7 @@
 // from and written to a small JSON file keyed by the device name.
 #include "tuner.h"
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -30,7 +31,6 @@
 namespace cgh {
 
 namespace {
-constexpr int kDirectCtasPerSm = 2;
 constexpr int kForms = 6;
 }  // namespace
 
@@ -59,13 +59,8 @@ static int split_for(int64_t pixel_tiles, int64_t point_tiles, int64_t slots)
     return best;
 }
 
-int choose_point_split(int64_t pixel_tiles, int64_t point_tiles, int num_sms)
-{
-    return split_for(pixel_tiles, point_tiles, (int64_t)num_sms * kDirectCtasPerSm);
-}
-
 DirectLayout choose_layout(const DirectShape *shapes, int n_shapes, int width, int height, int64_t point_tiles,
-                           int num_sms, int force_split, const double *step_cost)
+                           int num_sms, int force_split)
 {
     DirectLayout best{};
     double best_t = 1e300, best_area = 0.0;
@@ -77,8 +72,7 @@ DirectLayout choose_layout(const DirectShape *shapes, int n_shapes, int width, i
         if (s > point_tiles) s = (int)(point_tiles > 0 ? point_tiles : 1);
         // in point-tile steps of one CTA: the shapes keep the same warps per SM (threads x CTAs per SM) and the
         // same pixels per thread, so a step takes the same time whatever the shape
-        const double t =
-            direct_path(tiles, point_tiles > 0 ? point_tiles : 1, s, slots) * (step_cost ? step_cost[k] : 1.0);
+        const double t = direct_path(tiles, point_tiles > 0 ? point_tiles : 1, s, slots);
         const double area = (double)tiles * sh.tile_w * sh.tile_h;
         // a shorter path wins; on equal paths, fewer padded pixels computed
         if (t < best_t * (1.0 - 1e-9) || (t <= best_t * (1.0 + 1e-9) && area < best_area)) {
@@ -90,18 +84,62 @@ DirectLayout choose_layout(const DirectShape *shapes, int n_shapes, int width, i
     return best;
 }
 
-// The complex wave's tall block reads the tile's tables, its wide block takes each thread's own sines and
-// cosines: a point-tile step of the wide block takes 1.78 times as long (5.71 against 3.20 ms at 1920x1080,
-// 10^4 points), so the wide block wins only where it needs far fewer rounds.
-constexpr double kWaveWideStepCost = 1.78;
+// Microseconds of one stage (32 points of a 128 x bn / planes tile) of a CTA of the tensor-core direct form, for the
+// amplitude hologram and the complex wave, and per B row for each part of a tile that its last CTA adds.  Measured
+// on GB300 at 1920x1080 with 10^4 points (stages) and at 256x256 with 10^3 (parts); over 128x32 to 2048x2048 pixels
+// and 100 to 10^4 points the choice is within 8 % of the fastest tile and CTA count but for the smallest holograms
+// (under 30 us), where the spread of one of them is as large.
+struct MmaCost {
+    int bn;
+    double stage[2];
+};
+static const MmaCost kMmaCost[] = {
+    {64, {1.21, 1.16}}, {128, {1.40, 1.30}}, {192, {1.67, 1.48}}, {224, {1.81, 0.0}}, {256, {1.96, 1.64}},
+};
+constexpr double kMmaPartUs = 0.005;
 
-DirectLayout choose_direct_layout(bool wave, int width, int height, int64_t point_tiles, int num_sms,
-                                  int force_split)
+DirectMmaLayout choose_direct_mma(int planes, int width, int height, int64_t n_points, int num_sms, int split,
+                                  int ctas)
 {
-    const DirectShape shapes[2] = {wave ? direct_wave_shape(false) : direct_shape(false),
-                                   wave ? direct_wave_shape(true) : direct_shape(true)};
-    const double wave_cost[2] = {kWaveWideStepCost, 1.0};
-    return choose_layout(shapes, 2, width, height, point_tiles, num_sms, force_split, wave ? wave_cost : nullptr);
+    DirectMmaLayout best;
+    const int64_t groups = (n_points + kDirectMmaGroup - 1) / kDirectMmaGroup;
+    double best_t = 1e300;
+    for (const MmaCost &c : kMmaCost)
+        for (int a_rows = 0; a_rows < 2; ++a_rows) {
+            if (planes == 2 && c.bn / 2 % 32 != 0) continue;
+            const int tb = c.bn / planes;
+            const int side_a = a_rows ? height : width, side_b = a_rows ? width : height;
+            const int64_t tiles = (int64_t)((side_a + 127) / 128) * ((side_b + tb - 1) / tb);
+            const int64_t units = tiles * groups;
+            auto consider = [&](int64_t n, int64_t stages, int64_t parts) {
+                // on equal terms the orientation whose stores write whole rows of 32 pixels
+                const double t = (double)stages * c.stage[planes - 1] + (double)parts * kMmaPartUs * c.bn + 0.01 * a_rows;
+                if (t >= best_t) return;
+                best_t = t;
+                best.bn = c.bn;
+                best.a_rows = a_rows;
+                best.tiles = (int)tiles;
+                best.ctas = (int)n;
+            };
+            if (split > 0) {
+                const int64_t s = std::min<int64_t>(split, groups), n = tiles * s;
+                consider(n, (n + num_sms - 1) / num_sms * ((groups + s - 1) / s), s);
+                continue;
+            }
+            if (ctas > 0) {
+                const int64_t n = std::min<int64_t>(ctas, units);
+                consider(n, (units + n - 1) / n * ((n + num_sms - 1) / num_sms), 1);
+                continue;
+            }
+            // from an equal share on every SM to whole tiles: fewer CTAs leave fewer parts of a tile to add
+            for (int64_t s = (units + num_sms - 1) / num_sms;; s += 1 + s / 4) {
+                consider((units + s - 1) / s, s, s >= groups ? 1 : (groups + s - 1) / s);
+                if (s >= groups) break;
+            }
+        }
+    // a CTA counts its stages in 32 bits
+    best.ctas = (int)std::max<int64_t>(best.ctas, ((int64_t)best.tiles * groups >> 30) + 1);
+    return best;
 }
 
 int choose_gemm_bn(int width)

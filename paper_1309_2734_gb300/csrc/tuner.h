@@ -9,22 +9,20 @@ struct cgh_ctx;
 
 namespace cgh {
 
-// Point chunks for the direct kernels: the shortest critical path, rounds of
-// (pixel tiles x chunks) over the resident CTAs times the longest chunk.
-int choose_point_split(int64_t pixel_tiles, int64_t point_tiles, int num_sms);
-
-// The direct kernels' CTA shape (wide or tall, the one with less padding and the
-// better fill) and its point split; force_split > 0 pins the split.
+// A kernel's CTA shape among n_shapes (each with its threads and CTAs per SM) and its point split: the shortest
+// critical path, rounds of (pixel tiles x chunks) over the resident CTAs times the longest chunk, then the least
+// padding; force_split > 0 pins the split.
 struct DirectLayout {
     DirectShape shape;
     int split;
 };
-DirectLayout choose_direct_layout(bool wave, int width, int height, int64_t point_tiles, int num_sms,
-                                  int force_split);
-// The same choice among n_shapes CTA shapes (each with its threads and CTAs per SM); step_cost, if given, scales
-// each shape's predicted path by the relative time of one of its point-tile steps.
 DirectLayout choose_layout(const DirectShape *shapes, int n_shapes, int width, int height, int64_t point_tiles,
-                           int num_sms, int force_split, const double *step_cost = nullptr);
+                           int num_sms, int force_split);
+
+// The tile and the CTAs of the direct form on the tensor cores (direct_mma.cu) with the shortest predicted time.
+// planes = 2: the complex wave.  split > 0: that many equal chunks of the points per tile; ctas > 0: that many CTAs.
+DirectMmaLayout choose_direct_mma(int planes, int width, int height, int64_t n_points, int num_sms, int split,
+                                  int ctas);
 
 // GEMM orientation, tile width, K splits and form (one CTA per 128-row tile, or the two-SM form: clusters of two
 // CTAs on 256-row tiles) with the shortest predicted time: rounds of units over the ctas CTAs (ctas / 2 clusters)

@@ -1,0 +1,82 @@
+"""The direct forms on the tensor cores (direct_mma.cu) where they can go wrong: tile edges and remainders on both
+sides, groups of 32 points and accumulation chains with a remainder, one CTA and many per tile, wide and extreme
+amplitudes, both planes of the wave.
+
+Tolerance: an entry is good to 1.2e-7 RMS and a term has two (1.7e-7); a chain's truncation leaves up to 3e-7 of its
+value, the split's dropped lo lo product 6e-8, and the FP32 additions of n chains sqrt(n / 2) 2^-25 (3.4e-7 at 10^4
+points): under 6e-7 together, 1e-6 with the spread of a few hundred sampled pixels.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1309_2734_gb300 import Hologram, _lib, workloads
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+TOL = 1e-6
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1309_2734_gb300.build import build
+    build()
+    torch.cuda.set_device(0)
+
+
+def _field(c, form="direct_sfu", wave=False, options=()):
+    xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
+    with Hologram(c.width, c.height, c.pitch_m, c.lambda_m, form=form) as h:
+        for k, v in options:
+            h.set_option(k, v)
+        f = h.wave(xyz, amp) if wave else h.point_cloud(xyz, amp)
+        h.sync()
+        return f.cpu().numpy()
+
+
+def _sampled(c, n=400):
+    rng = np.random.default_rng(c.width + c.n_points)
+    cols, rows = rng.integers(0, c.width, n), rng.integers(0, c.height, n)
+    cols[:4], rows[:4] = [0, c.width - 1, 0, c.width - 1], [0, 0, c.height - 1, c.height - 1]
+    return cols, rows, oracle.field_at(c.pitch_m, c.lambda_m, c.xyz, c.amp, cols, rows)
+
+
+@pytest.mark.parametrize("w,h", [(1, 1), (127, 65), (128, 64), (129, 257), (260, 130), (2000, 130), (130, 2000),
+                                 (1920, 224), (1027, 1025)])
+@pytest.mark.parametrize("n", [1, 31, 33, 97, 2050])
+def test_tile_and_group_edges(w, h, n):
+    c = workloads.random_cloud(9000 + w + n, w, h, n)
+    cols, rows, ref = _sampled(c)
+    got = _field(c)
+    assert oracle.nrms(got[rows, cols], ref) <= TOL
+    both = _field(c, wave=True)
+    assert oracle.nrms(both[0][rows, cols], ref) <= TOL
+
+
+@pytest.mark.parametrize("split,ctas", [(1, 0), (3, 0), (0, 1), (0, 5), (0, 700)])
+def test_cta_counts(split, ctas):
+    c = workloads.random_cloud(9100, 300, 200, 1500)
+    cols, rows, ref = _sampled(c)
+    got = _field(c, options=[(_lib.CGH_OPT_POINT_SPLIT, split), (_lib.CGH_OPT_DIRECT_CTAS, ctas)])
+    assert oracle.nrms(got[rows, cols], ref) <= TOL
+
+
+@pytest.mark.parametrize("lo,hi", [(-6.0, 0.0), (29.0, 30.0), (-30.0, -29.0), (-12.0, 3.0)])
+def test_amplitude_ranges(lo, hi):
+    """Amplitudes over many decades, and near the ends of single precision; either sign."""
+    c = workloads.random_cloud(9200, 200, 150, 3000)
+    rng = np.random.default_rng(1)
+    c.amp = (10.0 ** rng.uniform(lo, hi, c.n_points) * rng.choice([-1.0, 1.0], c.n_points)).astype(np.float32)
+    cols, rows, ref = _sampled(c)
+    for form in ("direct_sfu", "direct_accurate"):
+        assert oracle.nrms(_field(c, form)[rows, cols] * 10.0 ** -hi, ref * 10.0 ** -hi) <= TOL
+
+
+def test_zero_amplitudes():
+    c = workloads.random_cloud(9300, 200, 150, 100)
+    c.amp[:] = 0.0
+    assert not _field(c).any()
