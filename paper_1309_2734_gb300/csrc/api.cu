@@ -489,31 +489,58 @@ int run_spherical(cgh_ctx *ctx, int width, int height, double pitch, double lamb
     const size_t aux_bytes = align_up((size_t)n_pad * sizeof(uint2), 256);
     const size_t ext_bytes = align_up((size_t)n_pad * sizeof(float4), 256);
     const size_t part_bytes = split > 1 ? (size_t)split * planes * plane * sizeof(float) : 0;
-    int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, geo_bytes + aux_bytes + ext_bytes + part_bytes);
+    // The amplitude hologram goes to the tensor cores where the preparation's bound on the cross phase over the points
+    // allows: with the fastest tile, else (a bound up to four times larger) with the narrowest, else to the SIMT kernel.
+    // All are launched; those whose range the bound is not in return at once.
+    const bool mma = planes == 1;
+    DirectMmaLayout ml[2];
+    if (mma) {
+        ml[0] = choose_direct_mma(0, width, height, n, ctx->num_sms, ctx->point_split, 0);
+        if (ml[0].bn > 64) ml[1] = choose_direct_mma(0, width, height, n, ctx->num_sms, ctx->point_split, 0, 64);
+    }
+    const int n_tiles = std::max(ml[0].tiles, ml[1].tiles);
+    const size_t zero_bytes = align_up((size_t)(2 + n_tiles) * sizeof(int), 256);   // max |A|, the bound, tile counters
+    const size_t slot_bytes = (size_t)2 * 128 * std::max((int64_t)ml[0].ctas * ml[0].bn, (int64_t)ml[1].ctas * ml[1].bn) *
+                              sizeof(float);
+    const float bound_min = sph_mma_max_phase(64);
+    int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes,
+                    geo_bytes + aux_bytes + ext_bytes + zero_bytes + std::max(part_bytes, slot_bytes));
     if (rc) return rc;
     char *base = static_cast<char *>(ctx->ws);
     int4 *geo = reinterpret_cast<int4 *>(base);
     uint2 *aux = reinterpret_cast<uint2 *>(base + geo_bytes);
     float4 *ext = reinterpret_cast<float4 *>(base + geo_bytes + aux_bytes);
-    float *parts = reinterpret_cast<float *>(base + geo_bytes + aux_bytes + ext_bytes);
-    cudaError_t e;
+    float *amax = reinterpret_cast<float *>(base + geo_bytes + aux_bytes + ext_bytes);
+    float *parts = reinterpret_cast<float *>(base + geo_bytes + aux_bytes + ext_bytes + zero_bytes);   // or the slots
+    const float *bound = mma ? amax + 1 : nullptr;
+    cudaError_t e = mma ? cudaMemsetAsync(amax, 0, (size_t)(2 + n_tiles) * sizeof(int), ctx->stream) : cudaSuccess;
+    if (e != cudaSuccess) return cuda_status(e);
     {
         ProfileScope ps(ctx, "prep_points", 1);
-        e = launch_prep_points(d_xyz, d_amp, (int)n, (int)n_pad, pitch, lambda, geo, aux, ctx->d_status, nullptr,
-                               ctx->stream, kAuxPiston, ext, width, height, sph_tile_cols(planes),
-                               sph_tile_rows(planes));
+        e = launch_prep_points(d_xyz, d_amp, (int)n, (int)n_pad, pitch, lambda, geo, aux, ctx->d_status,
+                               mma ? amax : nullptr, ctx->stream, kAuxPiston, ext, width, height,
+                               sph_tile_cols(planes), sph_tile_rows(planes), mma ? amax + 1 : nullptr);
     }
     if (e != cudaSuccess) return cuda_status(e);
+    for (int v = 0; v < 2 && ml[v].bn > 0; ++v) {
+        ProfileScope ps(ctx, "spherical_mma", 1);
+        e = launch_direct_mma(ml[v], 1, geo, aux, amax, (int)n, width, height, d_out, parts,
+                              reinterpret_cast<int *>(amax + 2), ctx->d_status,
+                              (uint64_t)ctx->timeout_ms * 1000000ull, ctx->stream, -1, phase_ref(ctx), ext,
+                              v == 0 ? -1.0f : sph_mma_max_phase(ml[0].bn), sph_mma_max_phase(ml[v].bn));
+        if (e != cudaSuccess) return cuda_status(e);
+    }
     {
         ProfileScope ps(ctx, planes == 2 ? "spherical_wave" : "spherical", 1);
         e = launch_spherical(sh, geo, aux, ext, (int)n_pad, width, height, split, planes, split > 1 ? parts : d_out,
-                             (int64_t)planes * plane, plane, phase_ref(ctx), ctx->stream);
+                             (int64_t)planes * plane, plane, phase_ref(ctx), ctx->stream, bound,
+                             bound_min);
     }
     if (e != cudaSuccess || split == 1) return cuda_status(e);
     ProfileScope ps(ctx, "reduce_slices", planes);
     for (int c = 0; c < planes && e == cudaSuccess; ++c)
         e = launch_reduce_slices(parts + c * plane, split, plane, (int64_t)planes * plane, d_out + c * plane,
-                                 ctx->stream);
+                                 ctx->stream, bound, bound_min);
     return cuda_status(e);
 }
 

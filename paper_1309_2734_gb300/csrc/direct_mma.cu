@@ -16,7 +16,8 @@
 // (Without the half turn 640x64 gave 7.2e-7; chains of 1 / 4 / 8 groups at 1920x1080 3.1 / 8.6 / 17.6e-7.)
 //
 // Time, prep included (before): 1920x1080, 10^4 points 0.307 ms (1.77; 67.5 G terms/ms); its complex wave 0.485 ms
-// (3.30); 1024x1024, 10^3 points 0.046 ms (0.117); 256x256, 10^3 points 0.026 ms (0.046).
+// (3.30); 1024x1024, 10^3 points 0.046 ms (0.117); 256x256, 10^3 points 0.026 ms (0.046); the spherical hologram,
+// 1920x1080, 10^4 points at 0.3-1 m 0.66 ms (7.36; with the narrowest tile, for points at 0.2 m, 1.53).
 // What bounds it: the making of entries (0.26 of 0.31 ms with the MMAs left out), 30 instructions for two entries, 15
 // of them packed FMAs of two to three cycles, so the FMA pipe is about 80 % busy while entries are made; the tensor
 // cores are active 30 % of the time.  128 x BN tiles: larger tiles share an entry among more pixels (BN = 64 / 128 /
@@ -47,6 +48,7 @@
 #include "host_util.h"
 #include "kernels.h"
 #include "sincospoly.h"
+#include "spherical_dev.cuh"
 #include "tcgen05.cuh"
 
 namespace cgh {
@@ -61,10 +63,12 @@ constexpr int kPtSlots = 4;
 constexpr int kUnroll = 2;                   // steps of a side side by side
 constexpr int kPtBytes = kGroup * (int)(sizeof(int4) + sizeof(uint2));
 constexpr int kChain = 2;                    // stages of an accumulation chain
+constexpr int kSphChain = 4;                 // spherical: stages of half as many points
 constexpr float kEntryScale = 4096.0f;       // 2^12, the A side (amplitudes)
 // 2^-12, times 1 + 2.4e-7: the accumulation truncates, and a chain of two groups loses 2.9e-7 of its value on average
-// (measured on random clouds; 2.6e-7 on coherent ones)
+// (measured on random clouds; 2.6e-7 on coherent ones); a spherical chain, with twice the MMAs, 4.6e-7
 constexpr float kUnscale = 2.44140625e-04f * (1.0f + 2.384185791015625e-07f);
+constexpr float kSphUnscale = 2.44140625e-04f * (1.0f + 4.76837158203125e-07f);
 
 template <int BN>
 struct MmaCfg {
@@ -82,7 +86,8 @@ struct MmaCfg {
 struct MmaArgs {
     const int4 *geo;
     const uint2 *aux;
-    const float *amp_max;
+    const float4 *ext;         // the spherical form's constants
+    const float *amp_max;      // [0] max |A|, [1] the spherical form's bound (prep)
     float *out;                // plane 1 (the imaginary part) follows plane 0
     float4 *slots;
     int *counters;
@@ -92,6 +97,7 @@ struct MmaArgs {
     int width, height, tiles_a;
     int a_rows;                // 1: A rows are hologram rows; 0: hologram columns
     int vec, drop;
+    float phase_lo, phase_hi;  // the spherical form: the bounds this launch takes
     PhaseRef ref;
 };
 
@@ -115,30 +121,18 @@ __device__ __forceinline__ Walk walk_start(int d, uint32_t ch, uint32_t cl, uint
 // sqrt(2) sin(pi r) and sqrt(2) cos(pi r) of two signed turns r (2^-32 turn): half the angle, so that s^2 - 1 and s c
 // are minus the cosine and the sine of the whole turn without a quadrant (sincospoly.h).
 template <int U>
-__device__ __forceinline__ void half_turn2(Walk (&w)[2], const uint32_t (&S)[2], bool back, float2 (&s)[U], float2 (&c)[U])
+__device__ __forceinline__ void half_turn2(const float2 (&turn)[U], float2 (&s)[U], float2 (&c)[U])
 {
     float2 r[U], u[U], hs[U], hc[U];
 #pragma unroll
     for (int j = 0; j < U; ++j) {
-        r[j] = make_float2((float)(int)w[0].t, (float)(int)w[1].t);
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            w[p].t = back ? w[p].t - w[p].D : w[p].t + w[p].D;
-            w[p].D += S[p];
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-        r[j] = __fmul2_rn(r[j], f2(2.3283064365386963e-10f));
+        r[j] = __fmul2_rn(turn[j], f2(2.3283064365386963e-10f));
         u[j] = __fmul2_rn(r[j], r[j]);
-    }
-#define CGH_HORNER(OUT, IN, COEF)                                                                                     \
-    _Pragma("unroll") for (int j = 0; j < U; ++j) OUT[j] = __ffma2_rn(IN[j], u[j], f2(COEF));
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
         hs[j] = f2(CGH_HSIN_4);
         hc[j] = f2(CGH_HCOS_4);
     }
+#define CGH_HORNER(OUT, IN, COEF)                                                                                     \
+    _Pragma("unroll") for (int j = 0; j < U; ++j) OUT[j] = __ffma2_rn(IN[j], u[j], f2(COEF));
     CGH_HORNER(hs, hs, CGH_HSIN_3)
     CGH_HORNER(hc, hc, CGH_HCOS_3)
     CGH_HORNER(hs, hs, CGH_HSIN_2)
@@ -182,6 +176,11 @@ __device__ __forceinline__ uint32_t turn_quarter(uint32_t h)
 __device__ __forceinline__ void st_shared8(uint32_t addr, uint32_t a, uint32_t b)
 {
     asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+
+__device__ __forceinline__ void st_shared4(uint32_t addr, uint32_t a)
+{
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(a) : "memory");
 }
 
 // 32 lanes x 8 columns of tensor memory (as tmem_ld16, tmem_st16).
@@ -231,7 +230,16 @@ __device__ __forceinline__ void side_entries(const int4 *geo, const uint2 *aux, 
     auto steps = [&](auto uc, int k0) {
         constexpr int U = decltype(uc)::value;
         float2 s[U], c[U], x[U], y[U];
-        half_turn2<U>(w, S, B, s, c);
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            x[j] = make_float2((float)(int)w[0].t, (float)(int)w[1].t);
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                w[p].t = B ? w[p].t - w[p].D : w[p].t + w[p].D;
+                w[p].D += S[p];
+            }
+        }
+        half_turn2<U>(x, s, c);
 #pragma unroll
         for (int j = 0; j < U; ++j) {
             if (B) {
@@ -276,16 +284,121 @@ __device__ __forceinline__ void side_entries(const int4 *geo, const uint2 *aux, 
     if constexpr (STEPS % kUnroll != 0) steps(std::integral_constant<int, STEPS % kUnroll>{}, STEPS / kUnroll * kUnroll);
 }
 
+// The spherical form.  About the centre of a tile (offsets cx, cy from the point, U0 = (cx^2 + cy^2) q, q = (p / z)^2)
+// a pixel with vx = dx^2 - cx^2 and vy = dy^2 - cy^2 has the turn
+//   Z + C dx^2 + C dy^2 + d0 + P(vx) + P(vy) + X,   P(v) = d1 w + d2 w^2 + d3 w^3, w = q v, Z h(U0 + w) - d0 = P(v)
+// (the Fresnel turn with its piston and the remainder: d0 = Z h(U0), and d1 = Z h1, d2 = Z h2 / 2, d3 = Z h3 / 6 from
+// h's derivatives at U0), where all but the cross term X = 2 d2 F(vx) F(vy), F(v) = w (1 + h3 / (2 h2) w), is a column
+// turn plus a row turn.  With 2 pi X = g(column) f(row) the term's factor exp(i g f) is taken to second order,
+// 1 + i g f - g^2 f^2 / 2: three products of a column's and a row's entry, the first as hi + lo pairs, the other two
+// (at most a few percent) as FP16.  The point preparation bounds |g f| (sph_mma_max_phase) and |P| (kSphRangeTurns)
+// for every point and pixel of a cloud that comes here: at the largest |g f| the third order left out is 4e-7 of a
+// point's term (RMS over the pixels) and the rounding of the second product 5e-7.
+struct SphPoint {
+    float d0, e1, e2, e3;   // turns: d0's fraction, P's coefficients in v (2^-32 turn)
+    float cq, ka, sb;       // F(v) = q v (1 + cq v); g = ka v (1 + cq v), f = sb v (1 + cq v)
+};
+
+// Offsets of the centre along A and B; hb: half the tile's B side.
+__device__ __forceinline__ SphPoint sph_point(const float4 x, int ca, int cb, float hb)
+{
+    const float q = fabsf(x.x), zh = fabsf(x.y);
+    const float fa = (float)ca, fb = (float)cb;
+    SphPoint P;
+    float v0, s0, rs0;
+    P.d0 = dev::sph_d0_frac(fa, fb, x, v0, s0, rs0);
+    const float r2 = rs0 * rs0, r3 = r2 * rs0;
+    const float d2 = -0.25f * zh * r3, q1 = q * 4294967296.0f;
+    P.e1 = -zh * v0 * rs0 * q1;
+    P.e2 = d2 * q * q1;
+    P.e3 = 0.125f * zh * r3 * r2 * q * q * q1;
+    P.cq = -0.75f * r2 * q;
+    const float span = fmaf(2.0f * hb, fabsf(fb), hb * hb);   // max |vy|
+    P.sb = __frcp_rn(span);
+    P.ka = 12.56637061435917295f * d2 * q * q * span;         // 4 pi d2 q^2 / sb
+    return P;
+}
+
+// Entries of this thread's point at STEPS rows 32 apart, two rows a packed operation, in plane 0 the first product's
+// hi and the second product, in plane 1 its lo and the third.  d: the first row's offset from the point, off: from the
+// tile's centre.
+template <int STEPS, bool B>
+__device__ __forceinline__ void sph_entries(const SphPoint &P, const int4 q, int d, int off, bool flip, uint32_t add,
+                                            uint32_t step, float amp, uint32_t at0, uint32_t lo_off)
+{
+    static_assert(STEPS % 2 == 0, "pairs of rows");
+    const uint32_t ch = (uint32_t)q.z, cl = (uint32_t)q.w;
+    Walk w = walk_start(d, ch, cl, add, step);
+    const uint32_t S = (ch << 11) | (cl >> 21);   // 2048 C
+    if (flip) w.t ^= 0x80000000u;                 // the half turn of every other point
+    if (B) w.t = 0u - w.t;
+    float2 a2 = make_float2((float)off, (float)(off + 32));
+    const float2 c2 = f2((float)(2 * (d - off)));
+    const float2 A = f2(amp), nA = f2(-amp);
+#pragma unroll
+    for (int k = 0; k < STEPS; k += 2) {
+        const float2 v = __fmul2_rn(a2, __fadd2_rn(a2, c2));
+        const float2 p = __fmul2_rn(v, __ffma2_rn(v, __ffma2_rn(v, f2(P.e3), f2(P.e2)), f2(P.e1)));
+        const float2 F = __fmul2_rn(v, __ffma2_rn(v, f2(P.cq), f2(1.0f)));
+        const uint32_t t0 = w.t;
+        w.t = B ? w.t - w.D : w.t + w.D;
+        w.D += S;
+        const uint32_t t1 = w.t;
+        w.t = B ? w.t - w.D : w.t + w.D;
+        w.D += S;
+        const uint32_t p0 = (uint32_t)__float2int_rn(p.x), p1 = (uint32_t)__float2int_rn(p.y);
+        float2 turn[1], s[1], c[1], x, y;
+        turn[0] = make_float2((float)(int)(B ? t0 - p0 : t0 + p0), (float)(int)(B ? t1 - p1 : t1 + p1));
+        half_turn2<1>(turn, s, c);
+        float2 x1, y1, x2, y2;
+        if (B) {
+            x = __ffma2_rn(s[0], s[0], f2(-1.0f));
+            y = __fmul2_rn(s[0], c[0]);
+            const float2 f = __fmul2_rn(F, f2(P.sb)), nf = __fmul2_rn(F, f2(-P.sb));
+            x1 = __fmul2_rn(y, nf);   // i times: (-y, x)
+            y1 = __fmul2_rn(x, f);
+            x2 = __fmul2_rn(y1, f);
+            y2 = __fmul2_rn(x1, nf);
+        } else {
+            const float2 as = __fmul2_rn(A, s[0]);
+            x = __ffma2_rn(as, s[0], nA);
+            y = __fmul2_rn(as, c[0]);
+            const float2 gk = __fmul2_rn(F, f2(P.ka)), h = __fmul2_rn(F, f2(-0.5f * P.ka));
+            x1 = __fmul2_rn(x, gk);
+            y1 = __fmul2_rn(y, gk);
+            x2 = __fmul2_rn(x1, h);
+            y2 = __fmul2_rn(y1, h);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float xj = j ? x.y : x.x, yj = j ? y.y : y.x;
+            const uint32_t h = pack_half2(xj, yj);
+            const float2 l = minus_half2(make_float2(xj, yj), h);
+            const uint32_t at = at0 + (uint32_t)(k + j) * 4096u;
+            st_shared4(at, h);
+            st_shared4(at + lo_off, pack_half2(l.x, l.y));
+            st_shared4(at ^ 64u, j ? pack_half2(x1.y, y1.y) : pack_half2(x1.x, y1.x));
+            st_shared4((at ^ 64u) + lo_off, j ? pack_half2(x2.y, y2.y) : pack_half2(x2.x, y2.x));
+        }
+        a2 = __fadd2_rn(a2, f2(64.0f));
+    }
+}
+
 struct MmaBars {
     uint64_t *full, *empty, *ptfull, *ptempty, *tfull, *tempty, *parts, *drain;
 };
 
 // PLANES = 1: the amplitude hologram, tiles of 128 x BN pixels.  PLANES = 2: the complex wave, tiles of 128 x BN / 2
 // pixels, the B rows (and accumulator columns) of the imaginary part after those of the real part.
-template <int BN, int PLANES>
+// SPH: the amplitude hologram of the spherical model, 16 points a stage (three products each).
+template <int BN, int PLANES, bool SPH>
 __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid_constant__ MmaArgs g)
 {
     using C = MmaCfg<BN>;
+    constexpr int GROUP = SPH ? kSphMmaGroup : kGroup;
+    constexpr int CHAIN = SPH ? kSphChain : kChain;
+    static_assert(!SPH || (PLANES == 1 && BN % 64 == 0), "row pairs of the amplitude hologram");
+    if (SPH && !(g.amp_max[1] > g.phase_lo && g.amp_max[1] <= g.phase_hi)) return;   // another kernel's cloud
     constexpr int HB = BN / 4;          // accumulator columns per worker warp
     constexpr int TB = BN / PLANES;     // pixels of the tile along B
     extern __shared__ uint8_t smem_raw[];
@@ -344,10 +457,11 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
                 uint8_t *dst = s_pts + (i % kPtSlots) * kPtBytes;
                 uint64_t *bar = &bars.ptfull[i % kPtSlots];
                 if (!(blockIdx.x == 0 && i == g.drop)) {
-                    mbar_arrive_expect_tx(bar, kPtBytes);
-                    bulk_copy_g2s(dst, g.geo + (long long)gl * kGroup, kGroup * sizeof(int4), bar);
-                    bulk_copy_g2s(dst + kGroup * sizeof(int4), g.aux + (long long)gl * kGroup, kGroup * sizeof(uint2),
-                                  bar);
+                    constexpr uint32_t GB = GROUP * sizeof(int4), AB = GROUP * sizeof(uint2);
+                    mbar_arrive_expect_tx(bar, GB + AB + (SPH ? GB : 0));
+                    bulk_copy_g2s(dst, g.geo + (long long)gl * GROUP, GB, bar);
+                    bulk_copy_g2s(dst + GB, g.aux + (long long)gl * GROUP, AB, bar);
+                    if (SPH) bulk_copy_g2s(dst + GB + AB, g.ext + (long long)gl * GROUP, GB, bar);
                 }
                 if (++gl == (int)g.groups) gl = 0;
             }
@@ -372,19 +486,30 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
                 if (!(ok = wait(&bars.full[s], (uint32_t)(i / C::kStages) & 1u))) break;
                 tc_fence_after();
                 const uint32_t a_hi = smem_addr(smem + s * C::kStage), b_hi = a_hi + 2 * C::kA;
-                // lo hi, hi lo, then hi hi: the large products last, so the truncation of the small ones is small
+                // products of planes (A, B: 0 = hi, 1 = lo), the large ones last, so the truncation of the small ones
+                // is small: lo hi, hi lo, hi hi over the whole row; the spherical form's first product is in the
+                // first half of the row (K steps 0 and 1), its third in the second half of the lo planes, its second
+                // in that of the hi planes
+                bool acc = in_chain != 0;
+                auto product = [&](int pa, int pb, int k0, int k1) {
+                    const uint64_t ad = sw128_kmajor_desc(a_hi + pa * C::kA), bd = sw128_kmajor_desc(b_hi + pb * C::kB);
 #pragma unroll
-                for (int pass = 0; pass < 3; ++pass) {
-                    const uint64_t ad = sw128_kmajor_desc(a_hi + (pass == 0 ? C::kA : 0));
-                    const uint64_t bd = sw128_kmajor_desc(b_hi + (pass == 1 ? C::kB : 0));
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        umma_f16(tmem, ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), idesc,
-                                 (in_chain | pass | kk) ? 1u : 0u);
+                    for (int kk = k0; kk < k1; ++kk) {
+                        umma_f16(tmem, ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), idesc, acc ? 1u : 0u);
+                        acc = true;
+                    }
+                };
+                constexpr int KH = SPH ? 2 : 4;
+                product(1, 0, 0, KH);
+                product(0, 1, 0, KH);
+                if (SPH) {
+                    product(1, 1, 2, 4);
+                    product(0, 0, 2, 4);
                 }
+                product(0, 0, 0, KH);
                 umma_commit(&bars.empty[s]);
                 const bool tile_end = g0 + 1 == (int)g.groups;
-                if (++in_chain == kChain || tile_end || i + 1 == n) {
+                if (++in_chain == CHAIN || tile_end || i + 1 == n) {
                     umma_commit(bars.tfull);
                     in_chain = 0;
                     ++chain;
@@ -396,8 +521,11 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
             mbar_wait(bars.drain, 0, g.timeout_ns);
         }
     } else {
-        const int pair = tid & 15, rl = tid >> 4;   // this thread's two points of a stage and its first row
-        const uint32_t entry = (uint32_t)(rl * 128 + (((pair >> 1) ^ (rl & 7)) << 4) + (pair & 1) * 8);
+        // this thread's two points of a stage (spherical: its point) and its first row; a warp's two rows are 4 apart
+        // in the spherical form, whose halves of a row then fall on different banks
+        const int pair = tid & 15, rl = SPH ? (warp >> 2) * 8 + (warp & 3) + ((tid >> 4) & 1) * 4 : tid >> 4;
+        const uint32_t entry = SPH ? (uint32_t)(rl * 128 + (((pair >> 2) ^ (rl & 7)) << 4) + (pair & 3) * 4)
+                                   : (uint32_t)(rl * 128 + (((pair >> 1) ^ (rl & 7)) << 4) + (pair & 1) * 8);
         // amplitudes as multiples of 2^(eb - 126), the power of two above the largest
         const uint32_t eb = min((__float_as_uint(*g.amp_max) >> 23) & 255u, 252u);
         const float a_scale = __uint_as_float((253u - eb) << 23), unscale = __uint_as_float((eb + 1u) << 23);
@@ -515,7 +643,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
                     }
                 }
 #pragma unroll
-                for (int k = 0; k < 8; ++k) v[k] = v[k] * kUnscale * us;
+                for (int k = 0; k < 8; ++k) v[k] = v[k] * (SPH ? kSphUnscale : kUnscale) * us;
                 if (!g.a_rows) {   // lanes are columns: each store writes 32 consecutive pixels of a row
                     if (a < g.width)
 #pragma unroll
@@ -544,15 +672,31 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
                 const int ps = i % kPtSlots;
                 if (!wait(&bars.ptfull[ps], (uint32_t)(i / kPtSlots) & 1u)) break;
                 if (!wait(&bars.empty[s], s_use ^ 1u)) break;
-                const int4 *geo = reinterpret_cast<const int4 *>(s_pts + ps * kPtBytes) + pair;
-                const uint2 *aux =
-                    reinterpret_cast<const uint2 *>(s_pts + ps * kPtBytes + kGroup * sizeof(int4)) + pair;
+                const uint8_t *pts = s_pts + ps * kPtBytes;
+                const int4 *geo = reinterpret_cast<const int4 *>(pts) + pair;
+                const uint2 *aux = reinterpret_cast<const uint2 *>(pts + GROUP * sizeof(int4)) + pair;
                 const uint32_t base = smem_addr(smem + s * C::kStage) + entry;
-                side_entries<kRowsA / 32, false, PLANES>(
-                    geo, aux, swap, ra, (uint32_t)((ka * (unsigned long long)ra) >> 32) + g.ref.phi0,
-                    ref_step(32 * ka), g.ref.piston ? ~0u : 0u, a_scale, base, C::kA, 0);
-                side_entries<TB / 32, true, PLANES>(geo, aux, swap, rb, (uint32_t)((kb * (unsigned long long)rb) >> 32),
-                                                    ref_step(32 * kb), 0u, 0.0f, base + 2 * C::kA, C::kB, TB * 128);
+                const uint32_t add_a = (uint32_t)((ka * (unsigned long long)ra) >> 32) + g.ref.phi0;
+                const uint32_t add_b = (uint32_t)((kb * (unsigned long long)rb) >> 32);
+                if constexpr (SPH) {
+                    const int4 q = *geo;
+                    const uint2 x = *aux;
+                    const float4 e = *(reinterpret_cast<const float4 *>(pts + GROUP * (sizeof(int4) + sizeof(uint2))) +
+                                       pair);
+                    const int da = ra - (swap ? q.y : q.x), db = rb - (swap ? q.x : q.y);
+                    const int oa = rl - kRowsA / 2, ob = rl - TB / 2;
+                    const SphPoint P = sph_point(e, da - oa, db - ob, 0.5f * TB);
+                    const uint32_t d0 = (uint32_t)__float2int_rn(P.d0 * 2147483648.0f) << 1;
+                    sph_entries<kRowsA / 32, false>(P, q, da, oa, pair & 1, add_a + x.x + d0, ref_step(32 * ka),
+                                                    __uint_as_float(x.y) * a_scale * kEntryScale, base, C::kA);
+                    sph_entries<TB / 32, true>(P, q, db, ob, pair & 1, add_b, ref_step(32 * kb), 0.0f,
+                                               base + 2 * C::kA, C::kB);
+                } else {
+                    side_entries<kRowsA / 32, false, PLANES>(geo, aux, swap, ra, add_a, ref_step(32 * ka),
+                                                             g.ref.piston ? ~0u : 0u, a_scale, base, C::kA, 0);
+                    side_entries<TB / 32, true, PLANES>(geo, aux, swap, rb, add_b, ref_step(32 * kb), 0u, 0.0f,
+                                                        base + 2 * C::kA, C::kB, TB * 128);
+                }
                 fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) {
@@ -564,7 +708,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
                     s_use ^= 1u;
                 }
                 tile_end = gi + 1 == (int)g.groups || i + 1 == n;
-                chain_end = ++in_chain == kChain || tile_end;
+                chain_end = ++in_chain == CHAIN || tile_end;
             }
             if (pending) {
                 if (!fold(pend_first)) break;
@@ -597,28 +741,30 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
     }
 }
 
-template <int BN, int PLANES>
+template <int BN, int PLANES, bool SPH>
 cudaError_t launch_as(const MmaArgs &g, int ctas, cudaStream_t s)
 {
     static PerDeviceOnce configured;
     const cudaError_t e = configured.run([] {
-        return cudaFuncSetAttribute(direct_mma_kernel<BN, PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        return cudaFuncSetAttribute(direct_mma_kernel<BN, PLANES, SPH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     MmaCfg<BN>::kSmem);
     });
     if (e != cudaSuccess) return e;
-    direct_mma_kernel<BN, PLANES><<<ctas, kMmaThreads, MmaCfg<BN>::kSmem, s>>>(g);
+    direct_mma_kernel<BN, PLANES, SPH><<<ctas, kMmaThreads, MmaCfg<BN>::kSmem, s>>>(g);
     return cudaGetLastError();
 }
 
-template <int PLANES>
+template <int PLANES, bool SPH>
 cudaError_t launch_bn(int bn, const MmaArgs &g, int ctas, cudaStream_t s)
 {
     switch (bn) {
-    case 64: return launch_as<64, PLANES>(g, ctas, s);
-    case 128: return launch_as<128, PLANES>(g, ctas, s);
-    case 192: return launch_as<192, PLANES>(g, ctas, s);
-    case 224: if constexpr (PLANES == 1) return launch_as<224, PLANES>(g, ctas, s); else return cudaErrorInvalidValue;
-    case 256: return launch_as<256, PLANES>(g, ctas, s);
+    case 64: return launch_as<64, PLANES, SPH>(g, ctas, s);
+    case 128: return launch_as<128, PLANES, SPH>(g, ctas, s);
+    case 192: return launch_as<192, PLANES, SPH>(g, ctas, s);
+    case 224:
+        if constexpr (PLANES == 1 && !SPH) return launch_as<224, PLANES, SPH>(g, ctas, s);
+        else return cudaErrorInvalidValue;
+    case 256: return launch_as<256, PLANES, SPH>(g, ctas, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -628,15 +774,16 @@ cudaError_t launch_bn(int bn, const MmaArgs &g, int ctas, cudaStream_t s)
 cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4 *geo, const uint2 *aux,
                               const float *amp_max, int n_points, int width, int height, float *out, float *slots,
                               int *counters, int *status, uint64_t timeout_ns, cudaStream_t s, int drop,
-                              const PhaseRef &ref)
+                              const PhaseRef &ref, const float4 *ext, float phase_lo, float phase_hi)
 {
+    const int group = ext != nullptr ? kSphMmaGroup : kGroup;
     if (n_points < 1 || lay.ctas < 1 || (planes != 1 && planes != 2) || (uintptr_t)slots % 16 != 0)
         return cudaErrorInvalidValue;
     MmaArgs g{};
     const int side_a = lay.a_rows ? height : width, side_b = lay.a_rows ? width : height;
     const int tb = lay.bn / planes;
     g.tiles_a = (side_a + kRowsA - 1) / kRowsA;
-    g.groups = (n_points + kGroup - 1) / kGroup;
+    g.groups = (n_points + group - 1) / group;
     g.units = (long long)g.tiles_a * ((side_b + tb - 1) / tb) * g.groups;
     // whole tiles per CTA (one share each) need neither slots nor counters
     if (lay.ctas > g.units || g.units / lay.ctas >= 0x7ffffff0ll ||
@@ -644,6 +791,9 @@ cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4
         return cudaErrorInvalidValue;
     g.geo = geo;
     g.aux = aux;
+    g.ext = ext;
+    g.phase_lo = phase_lo;
+    g.phase_hi = phase_hi;
     g.amp_max = amp_max;
     g.out = out;
     g.slots = reinterpret_cast<float4 *>(slots);
@@ -656,7 +806,8 @@ cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4
     g.vec = width % 4 == 0 && (uintptr_t)out % 16 == 0 && ((long long)width * height) % 4 == 0;
     g.drop = drop;
     g.ref = ref;
-    return planes == 2 ? launch_bn<2>(lay.bn, g, lay.ctas, s) : launch_bn<1>(lay.bn, g, lay.ctas, s);
+    if (ext != nullptr) return planes == 1 ? launch_bn<1, true>(lay.bn, g, lay.ctas, s) : cudaErrorInvalidValue;
+    return planes == 2 ? launch_bn<2, false>(lay.bn, g, lay.ctas, s) : launch_bn<1, false>(lay.bn, g, lay.ctas, s);
 }
 
 }  // namespace cgh

@@ -32,10 +32,13 @@ __host__ __device__ constexpr int sph_tile_cols(int planes) { return planes == 1
 constexpr double kSphFitTurns = 2.98023223876953125e-8;   // 2^-25 turn
 constexpr double kSphRangeTurns = 0.45;
 constexpr double kSeriesU = 0.05;
+// Largest cross phase (rad) the tensor-core spherical form takes with tiles of 128 x bn pixels, as the point
+// preparation bounds it for 128 x 256: it shrinks with the tile.
+__host__ __device__ constexpr float sph_mma_max_phase(int bn) { return 0.05f * 256.0f / (float)bn; }
 cudaError_t launch_prep_points(const float *d_xyz, const float *d_amp, int n, int n_pad, double pitch,
                                double lambda, int4 *geo, uint2 *aux, int *status, float *amp_max,
                                cudaStream_t s, int aux_x = kAuxSecondDiff, float4 *ext = nullptr, int width = 0,
-                               int height = 0, int tile_cols = 4, int tile_rows = 4);
+                               int height = 0, int tile_cols = 4, int tile_rows = 4, float *sph_max = nullptr);
 
 // The plane-wave reference phase of Eq. 5, phi_r(m, n) = kx m + ky n + phi0,
 // common to every point of a launch: kx, ky in 2^-64 turn per pixel, phi0 in
@@ -91,7 +94,9 @@ cudaError_t launch_direct_stream(bool sfu, const DirectShape &sh, int ctas, cons
 // out (planes = 1) or the complex wave, real plane then imaginary plane (planes = 2).  amp_max: max |A_j| of the
 // points (launch_prep_points).  slots: 2 ctas x 128 x bn floats (16-byte aligned); counters: one int per tile,
 // zeroed by the caller.  drop >= 0: CTA 0 never loads that group of kDirectMmaGroup points of its share (test hook).
-constexpr int kDirectMmaGroup = 32;
+// ext != nullptr: the amplitude hologram of the spherical model (points prepared with the piston, ext and its bound
+// amp_max[1]; groups of kSphMmaGroup points); the kernel returns at once unless phase_lo < amp_max[1] <= phase_hi.
+constexpr int kDirectMmaGroup = 32, kSphMmaGroup = 16;
 struct DirectMmaLayout {
     int bn = 0;       // B rows of a tile: 64, 128, 192, 224 (planes = 1), 256; 128 x bn / planes pixels.  0: not taken
     int a_rows = 0;   // the tile's 128-pixel side: 1 = hologram rows, 0 = columns
@@ -101,17 +106,20 @@ struct DirectMmaLayout {
 cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4 *geo, const uint2 *aux,
                               const float *amp_max, int n_points, int width, int height, float *out, float *slots,
                               int *counters, int *status, uint64_t timeout_ns, cudaStream_t s, int drop = -1,
-                              const PhaseRef &ref = PhaseRef());
+                              const PhaseRef &ref = PhaseRef(), const float4 *ext = nullptr, float phase_lo = 0.0f,
+                              float phase_hi = 0.0f);
 
 // f2: the exact spherical wave of Eq. 1 (spherical.cu), direct SFU form.
 // Points prepared with the piston and ext.  planes = 1: the amplitude
-// hologram (Eq. 5, middle line) at out; planes = 2: the complex wave, real part
+// hologram (Eq. 5, middle line) at out (bound: only if *bound > bound_min, else the tensor-core kernel
+// took it; the same in launch_reduce_slices); planes = 2: the complex wave, real part
 // at out and imaginary part at out + im_offset.  Point chunk s at out + s * slice_stride.
 // variant 0: 32 x 8 threads (wide), 1: 16 x 16 (tall), 2: 16 x 8 (short, four CTAs per SM).
 DirectShape spherical_shape(int planes, int variant = 0);
 cudaError_t launch_spherical(const DirectShape &sh, const int4 *geo, const uint2 *aux, const float4 *ext, int n_pad,
                              int width, int height, int split, int planes, float *out, int64_t slice_stride,
-                             int64_t im_offset, const PhaseRef &ref, cudaStream_t s);
+                             int64_t im_offset, const PhaseRef &ref, cudaStream_t s, const float *bound = nullptr,
+                             float bound_min = 0.0f);
 
 // a7: one job (hologram) of a batched direct launch; units are {job, pixel tile}.
 struct DirectJob {
@@ -291,7 +299,7 @@ cudaError_t launch_persist(const PersistParams &p, int ctas, int bn_max, int *st
 
 // a5: fixed-order sum of `slices` planes of n floats (reduce.cu).
 cudaError_t launch_reduce_slices(const float *parts, int slices, int64_t n, int64_t slice_stride, float *out,
-                                 cudaStream_t s);
+                                 cudaStream_t s, const float *bound = nullptr, float bound_min = 0.0f);
 
 // a6: 8-bit min/max quantiser (quantize.cu). scratch holds 2 uint32.
 cudaError_t launch_quantize8(const float *field, int64_t n, uint8_t *out, uint32_t *scratch, cudaStream_t s);

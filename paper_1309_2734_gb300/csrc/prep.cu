@@ -17,23 +17,23 @@ namespace cgh {
 __global__ void prep_points_kernel(const float *__restrict__ xyz, const float *__restrict__ amp, int n,
                                    int n_pad, double pitch, double lambda, int4 *__restrict__ geo,
                                    uint2 *__restrict__ aux, int *status, float *amp_max, int aux_x,
-                                   float4 *__restrict__ ext, int width, int height, int tile_cols, int tile_rows)
+                                   float4 *__restrict__ ext, int width, int height, int tile_cols, int tile_rows, float *sph_max)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n_pad) return;
     dev::prep_point(j, xyz, amp, n, pitch, lambda, geo, aux, status, amp_max, aux_x, ext, width, height, tile_cols,
-                    tile_rows);
+                    tile_rows, sph_max);
 }
 
 cudaError_t launch_prep_points(const float *d_xyz, const float *d_amp, int n, int n_pad, double pitch,
                                double lambda, int4 *geo, uint2 *aux, int *status, float *amp_max,
-                               cudaStream_t s, int aux_x, float4 *ext, int width, int height, int tile_cols, int tile_rows)
+                               cudaStream_t s, int aux_x, float4 *ext, int width, int height, int tile_cols, int tile_rows, float *sph_max)
 {
     if (n_pad <= 0) return cudaSuccess;
     const int threads = 256;
     const int blocks = (n_pad + threads - 1) / threads;
     prep_points_kernel<<<blocks, threads, 0, s>>>(d_xyz, d_amp, n, n_pad, pitch, lambda, geo, aux, status,
-                                                         amp_max, aux_x, ext, width, height, tile_cols, tile_rows);
+                                                         amp_max, aux_x, ext, width, height, tile_cols, tile_rows, sph_max);
     return cudaGetLastError();
 }
 

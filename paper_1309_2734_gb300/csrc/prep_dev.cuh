@@ -24,7 +24,7 @@ __device__ __forceinline__ void prep_point(int j, const float *__restrict__ xyz,
                                            double pitch, double lambda, int4 *__restrict__ geo,
                                            uint2 *__restrict__ aux, int *status, float *amp_max, int aux_x,
                                            float4 *__restrict__ ext, int width, int height, int tile_cols,
-                                           int tile_rows)
+                                           int tile_rows, float *sph_max = nullptr)
 {
     if (ext != nullptr) ext[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (j >= n) {  // padding: zero amplitude, zero phase
@@ -71,6 +71,20 @@ __device__ __forceinline__ void prep_point(int j, const float *__restrict__ xyz,
                           zh * (0.5 * umax) * wmax + 0.25 * zh * wmax * wmax <= kSphRangeTurns;
         const float q = (float)qz, h = (float)zh;   // and the pair's low parts, for the double-float d0
         ext[j] = make_float4(quad ? q : -q, umax < kSeriesU ? h : -h, (float)(qz - (double)q), (float)(zh - (double)h));
+    }
+    if (sph_max != nullptr) {
+        // the tensor-core form's bound: the largest cross phase 4 pi |d2| F F <= (pi Z / 2) wa wb over its tiles (128
+        // pixels of one axis, up to 256 of the other, either way round), and the range of the remainder's variation
+        // along either side, |P| <= (Z / 4) (umax + w) w
+        const double qz = (pitch / (double)fz) * (pitch / (double)fz), Z = (double)fz / lambda;
+        const double cx = fmax(fabs((double)fx), fabs((double)(width - 1) - (double)fx)) + 128.0;
+        const double cy = fmax(fabs((double)fy), fabs((double)(height - 1) - (double)fy)) + 128.0;
+        const double x64 = qz * (128.0 * cx + 4096.0), x128 = qz * (256.0 * cx + 16384.0);
+        const double y64 = qz * (128.0 * cy + 4096.0), y128 = qz * (256.0 * cy + 16384.0);
+        const double phase = 1.5707963267948966 * Z * fmax(x64 * y128, x128 * y64);
+        const double w = fmax(x128, y128), umax = (cx * cx + cy * cy) * qz;
+        const bool ok_range = 0.25 * Z * (umax + w) * w <= kSphRangeTurns;
+        atomicMax(reinterpret_cast<unsigned *>(sph_max), __float_as_uint(ok_range ? (float)phase : 1e30f));
     }
     if (amp_max != nullptr) atomicMax(reinterpret_cast<unsigned *>(amp_max), __float_as_uint(fabsf(a)));
 }

@@ -9,8 +9,9 @@ namespace cgh {
 namespace {
 
 __global__ void reduce_slices_vec4(const float4 *__restrict__ parts, int slices, long long n4, long long stride4,
-                                   float4 *__restrict__ out)
+                                   float4 *__restrict__ out, const float *bound, float bound_min)
 {
+    if (bound != nullptr && !(*bound > bound_min)) return;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n4;
          i += (long long)gridDim.x * blockDim.x) {
         float4 acc = parts[i];
@@ -26,8 +27,9 @@ __global__ void reduce_slices_vec4(const float4 *__restrict__ parts, int slices,
 }
 
 __global__ void reduce_slices_scalar(const float *__restrict__ parts, int slices, long long n, long long stride,
-                                     float *__restrict__ out)
+                                     float *__restrict__ out, const float *bound, float bound_min)
 {
+    if (bound != nullptr && !(*bound > bound_min)) return;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         float acc = parts[i];
@@ -49,7 +51,7 @@ int grid_for(long long work, int threads)
 }  // namespace
 
 cudaError_t launch_reduce_slices(const float *parts, int slices, int64_t n, int64_t slice_stride, float *out,
-                                 cudaStream_t s)
+                                 cudaStream_t s, const float *bound, float bound_min)
 {
     if (n <= 0) return cudaSuccess;
     const int threads = 256;
@@ -57,9 +59,11 @@ cudaError_t launch_reduce_slices(const float *parts, int slices, int64_t n, int6
                      ((uintptr_t)out % 16 == 0);
     if (vec) {
         reduce_slices_vec4<<<grid_for(n / 4, threads), threads, 0, s>>>(
-            reinterpret_cast<const float4 *>(parts), slices, n / 4, slice_stride / 4, reinterpret_cast<float4 *>(out));
+            reinterpret_cast<const float4 *>(parts), slices, n / 4, slice_stride / 4, reinterpret_cast<float4 *>(out),
+            bound, bound_min);
     } else {
-        reduce_slices_scalar<<<grid_for(n, threads), threads, 0, s>>>(parts, slices, n, slice_stride, out);
+        reduce_slices_scalar<<<grid_for(n, threads), threads, 0, s>>>(parts, slices, n, slice_stride, out,
+                                                                        bound, bound_min);
     }
     return cudaGetLastError();
 }

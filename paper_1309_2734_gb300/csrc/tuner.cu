@@ -84,36 +84,41 @@ DirectLayout choose_layout(const DirectShape *shapes, int n_shapes, int width, i
     return best;
 }
 
-// Microseconds of one stage (32 points of a 128 x bn / planes tile) of a CTA of the tensor-core direct form, for the
-// amplitude hologram and the complex wave, and per B row for each part of a tile that its last CTA adds.  Measured
-// on GB300 at 1920x1080 with 10^4 points (stages) and at 256x256 with 10^3 (parts); over 128x32 to 2048x2048 pixels
+// Microseconds of one stage (32 points of a 128 x bn / planes tile; spherical: 16) of a CTA of the tensor-core direct
+// form, for the amplitude hologram, the complex wave and the spherical hologram, and per B row for each part of a tile
+// that its last CTA adds.  Measured on GB300 at 1920x1080 with 10^4 points (stages) and at 256x256 with 10^3 (parts); over 128x32 to 2048x2048 pixels
 // and 100 to 10^4 points the choice is within 8 % of the fastest tile and CTA count but for the smallest holograms
 // (under 30 us), where the spread of one of them is as large.
 struct MmaCost {
     int bn;
-    double stage[2];
+    double stage[3];
 };
 static const MmaCost kMmaCost[] = {
-    {64, {1.21, 1.16}}, {128, {1.40, 1.30}}, {192, {1.67, 1.48}}, {224, {1.81, 0.0}}, {256, {1.96, 1.64}},
+    {64, {1.21, 1.16, 1.43}},  {128, {1.40, 1.30, 1.69}}, {192, {1.67, 1.48, 1.90}},
+    {224, {1.81, 0.0, 0.0}}, {256, {1.96, 1.64, 2.07}},
 };
 constexpr double kMmaPartUs = 0.005;
 
 DirectMmaLayout choose_direct_mma(int planes, int width, int height, int64_t n_points, int num_sms, int split,
-                                  int ctas)
+                                  int ctas, int bn)
 {
     DirectMmaLayout best;
-    const int64_t groups = (n_points + kDirectMmaGroup - 1) / kDirectMmaGroup;
+    const bool sph = planes == 0;   // the spherical amplitude hologram
+    if (sph) planes = 1;
+    const int group = sph ? kSphMmaGroup : kDirectMmaGroup;
+    const int64_t groups = (n_points + group - 1) / group;
     double best_t = 1e300;
     for (const MmaCost &c : kMmaCost)
         for (int a_rows = 0; a_rows < 2; ++a_rows) {
-            if (planes == 2 && c.bn / 2 % 32 != 0) continue;
+            if (bn > 0 && c.bn != bn) continue;
+            if (sph ? c.bn % 64 != 0 : c.bn / planes % 32 != 0) continue;
             const int tb = c.bn / planes;
             const int side_a = a_rows ? height : width, side_b = a_rows ? width : height;
             const int64_t tiles = (int64_t)((side_a + 127) / 128) * ((side_b + tb - 1) / tb);
             const int64_t units = tiles * groups;
             auto consider = [&](int64_t n, int64_t stages, int64_t parts) {
                 // on equal terms the orientation whose stores write whole rows of 32 pixels
-                const double t = (double)stages * c.stage[planes - 1] + (double)parts * kMmaPartUs * c.bn + 0.01 * a_rows;
+                const double t = (double)stages * c.stage[sph ? 2 : planes - 1] + (double)parts * kMmaPartUs * c.bn + 0.01 * a_rows;
                 if (t >= best_t) return;
                 best_t = t;
                 best.bn = c.bn;

@@ -20,9 +20,10 @@ DirectLayout choose_layout(const DirectShape *shapes, int n_shapes, int width, i
                            int num_sms, int force_split);
 
 // The tile and the CTAs of the direct form on the tensor cores (direct_mma.cu) with the shortest predicted time.
-// planes = 2: the complex wave.  split > 0: that many equal chunks of the points per tile; ctas > 0: that many CTAs.
+// planes = 2: the complex wave, 0: the amplitude hologram of the spherical model.  split > 0: that many equal chunks of the points per tile; ctas > 0: that many CTAs; bn > 0:
+// that tile.
 DirectMmaLayout choose_direct_mma(int planes, int width, int height, int64_t n_points, int num_sms, int split,
-                                  int ctas);
+                                  int ctas, int bn = 0);
 
 // GEMM orientation, tile width, K splits and form (one CTA per 128-row tile, or the two-SM form: clusters of two
 // CTAs on 256-row tiles) with the shortest predicted time: rounds of units over the ctas CTAs (ctas / 2 clusters)

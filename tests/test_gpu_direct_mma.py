@@ -80,3 +80,33 @@ def test_zero_amplitudes():
     c = workloads.random_cloud(9300, 200, 150, 100)
     c.amp[:] = 0.0
     assert not _field(c).any()
+
+
+MMA, SIMT = 1.5e-6, 1e-5   # the SIMT kernel's tolerance is that of its own tests
+
+
+@pytest.mark.parametrize("w,h,n,z,tol", [
+    (129, 257, 15, (0.3, 0.5), MMA), (300, 200, 17, (0.2, 0.3), MMA), (1920, 224, 130, (0.4, 1.0), MMA), (130, 2000, 33, (0.5, 0.9), MMA),
+    (1920, 1080, 65, (0.3, 1.0), MMA),      # the widest tile
+    (1920, 1080, 65, (0.2, 0.25), MMA),     # the narrowest tile
+    (1920, 1080, 65, (0.05, 0.1), SIMT),     # beyond its bound: the SIMT kernel
+    (1920, 1080, 65, (0.005, 1.0), SIMT),    # a close point among far ones: the SIMT kernel
+    (1000, 600, 2050, (0.25, 0.6), MMA),
+])
+@pytest.mark.parametrize("ref", [(0.0, 0.0, 0.0), (0.01, -0.02, 0.4)])
+def test_spherical(w, h, n, z, tol, ref):
+    """The spherical model on either side of the bounds that pick its kernel.  The tensor-core form adds to the errors
+    above at most 4e-7 of a term for the third order and 5e-7 for the FP16 products at the largest cross phase."""
+    c = workloads.random_cloud(9400 + w + n, w, h, n, z)
+    rng = np.random.default_rng(3)
+    cols, rows = rng.integers(0, w, 300), rng.integers(0, h, 300)
+    cols[:4], rows[:4] = [0, w - 1, 0, w - 1], [0, 0, h - 1, h - 1]
+    want = oracle.model_wave_at(2, c.pitch_m, c.lambda_m, c.xyz, c.amp, cols, rows, reference=ref).real
+    xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
+    with Hologram(w, h, c.pitch_m, c.lambda_m, form="direct_sfu") as hg:
+        hg.set_phase_model("spherical")
+        hg.set_reference(*ref)
+        f = hg.point_cloud(xyz, amp)
+        hg.sync()
+        got = f.cpu().numpy()
+    assert oracle.nrms(got[rows, cols], want) <= tol
