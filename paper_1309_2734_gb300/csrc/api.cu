@@ -104,8 +104,11 @@ int run_direct(cgh_ctx *ctx, bool sfu, int width, int height, double pitch, doub
                                             ctx->drop_tile, phase_ref(ctx)));
 }
 
-// k-blocks per TMEM accumulation chain of the split-FP16 form (3 passes each)
-constexpr int kSplit16ChunkKb = 8;
+// k-blocks per TMEM accumulation chain of the split-FP16 form (3 passes each).  Between chains the MMAs wait for the
+// fold, so longer chains are faster, and the truncation of the accumulation grows with them: with the small products
+// first (gemm_mma) 8 / 16 / 24 / 32 k-blocks give 0.90 / 1.42 / 1.99 / 2.54e-6 NRMS and 248 / 237 / 232 / 233 us at
+// 1024x1024, 20,011 points (8 with the large products first: 2.8e-6, 245 us)
+constexpr int kSplit16ChunkKb = 24;
 // smallest point chunk worth a pipeline stage of its own
 constexpr int64_t kPipelineMinPoints = 8192;
 // CGH_OPT_GEMM_GROUP = 0 tries the grouped form from this many points

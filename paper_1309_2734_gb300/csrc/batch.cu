@@ -107,7 +107,7 @@ struct Layout {
     }
 };
 
-constexpr int kSplit16ChunkKbBatch = 8;
+constexpr int kSplit16ChunkKbBatch = 16;   // divides a factor group's 32 k-blocks (see kSplit16ChunkKb, api.cu)
 
 // Form (and, for the GEMM forms, tile width) of every instance: the context's form, or the autotuner's choice.
 // forced > 0: that form for every instance.

@@ -119,8 +119,9 @@ __device__ __forceinline__ void gemm_producer(const Units &src, uint8_t *smem, c
         for (int c0 = x.kb0; c0 < x.kb1 && ok; c0 += x.kc) {
             const int c1 = min(x.kb1, c0 + x.kc);
             for (int pass = 0; pass < x.passes && ok; ++pass) {
-                const CUtensorMap *ma = (pass == 2) ? x.mpl : x.mp;
-                const CUtensorMap *mb = (pass == 1) ? x.mql : x.mq;
+                // split FP16: lo hi, hi lo, then hi hi (the small products first, gemm_mma)
+                const CUtensorMap *ma = (pass + 3 == x.passes) ? x.mpl : x.mp;
+                const CUtensorMap *mb = (pass + 2 == x.passes) ? x.mql : x.mq;
                 for (int kb = c0; kb < c1; ++kb, ++it) {
                     const int s = (int)(it % C::kStages);
                     const uint32_t ph = (it / C::kStages) & 1u;
@@ -155,6 +156,9 @@ template <class C, class Units>
 __device__ __forceinline__ void gemm_mma(const Units &src, uint8_t *smem, const GemmBars &bars, uint32_t tmem_base,
                                          int *status, unsigned long long timeout_ns)
 {
+    // Passes in the producer's order, split FP16: lo hi, hi lo, hi hi over a chunk.  The accumulation truncates each
+    // sum, which costs the small products little while the accumulator holds only those; with hi hi first every MMA
+    // truncated at the full magnitude (three times the error at equal chunk length).
     uint64_t *full = bars.full, *empty = bars.empty, *tfull = bars.tfull, *tempty = bars.tempty,
              *drain = bars.drain;
     uint32_t it = 0;
@@ -232,8 +236,9 @@ __device__ __forceinline__ void gemm_producer_pair(const Units &src, uint8_t *sm
         for (int c0 = x.kb0; c0 < x.kb1 && ok; c0 += x.kc) {
             const int c1 = min(x.kb1, c0 + x.kc);
             for (int pass = 0; pass < x.passes && ok; ++pass) {
-                const CUtensorMap *ma = (pass == 2) ? x.mpl : x.mp;
-                const CUtensorMap *mb = (pass == 1) ? x.mql : x.mq;
+                // split FP16: lo hi, hi lo, then hi hi (the small products first, gemm_mma)
+                const CUtensorMap *ma = (pass + 3 == x.passes) ? x.mpl : x.mp;
+                const CUtensorMap *mb = (pass + 2 == x.passes) ? x.mql : x.mq;
                 for (int kb = c0; kb < c1; ++kb, ++it) {
                     const int s = (int)(it % C::kStages);
                     const uint32_t ph = (it / C::kStages) & 1u;
