@@ -648,8 +648,8 @@ int fresnel_run(cgh_ctx *ctx, double z, const float *in, float *d_out)
     return cuda_status(launch_crop(ctx->fft_pad, H, W, d_out, ctx->stream));
 }
 
-// Largest band-list workspace of the WRP record (points x bands x 4 bytes).
-constexpr size_t kMaxBandListBytes = (size_t)1 << 30;
+// Largest band-list workspace of the WRP record (points x bands x 8 bytes).
+constexpr size_t kMaxBandListBytes = (size_t)2 << 30;
 
 // WRP step 1 into the padded work plane (pad, zeroed first) or into planes.
 int wrp_record(cgh_ctx *ctx, const float *d_xyz, const float *d_amp, int64_t n, double z_wrp, float2 *pad,
@@ -658,26 +658,25 @@ int wrp_record(cgh_ctx *ctx, const float *d_xyz, const float *d_amp, int64_t n, 
     const int64_t n_pad = padded_points(n);
     const size_t geo_bytes = align_up((size_t)n_pad * sizeof(int4), 256);
     const size_t win_bytes = align_up((size_t)n_pad * sizeof(uint4), 256);
+    const size_t row_bytes = align_up((size_t)n_pad * sizeof(int2), 256);
     // band lists hold at most every point in every band; beyond kMaxBandListBytes the tiles walk all points
-    const int bands = (ctx->height + 31) / 32;
-    const int cells = wrp_band_cells(ctx->height, (int)n_pad);
-    const size_t list_bytes = (size_t)n_pad * bands * sizeof(int);
+    const size_t list_bytes = wrp_list_bytes(ctx->height, (int)n_pad);
     const bool binned = list_bytes <= kMaxBandListBytes;
-    const size_t band_bytes = binned ? align_up((size_t)(2 * cells + 1) * sizeof(int), 256) + list_bytes : 0;
-    int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, geo_bytes + win_bytes + band_bytes);
+    const size_t count_bytes = binned ? align_up((size_t)wrp_band_cells(ctx->height, (int)n_pad) * sizeof(int), 256) : 0;
+    int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes,
+                    geo_bytes + win_bytes + row_bytes + count_bytes + (binned ? list_bytes : 0));
     if (rc) return rc;
-    int4 *geo = reinterpret_cast<int4 *>(ctx->ws);
-    uint4 *win = reinterpret_cast<uint4 *>(static_cast<char *>(ctx->ws) + geo_bytes);
-    int *count = reinterpret_cast<int *>(static_cast<char *>(ctx->ws) + geo_bytes + win_bytes);
-    int *offset = count + cells;
-    int *list = binned ? reinterpret_cast<int *>(reinterpret_cast<char *>(count) +
-                                                 align_up((size_t)(2 * cells + 1) * sizeof(int), 256))
-                       : nullptr;
+    char *base = static_cast<char *>(ctx->ws);
+    int4 *geo = reinterpret_cast<int4 *>(base);
+    uint4 *win = reinterpret_cast<uint4 *>(base + geo_bytes);
+    int2 *rows = reinterpret_cast<int2 *>(base + geo_bytes + win_bytes);
+    int *count = reinterpret_cast<int *>(base + geo_bytes + win_bytes + row_bytes);
+    int2 *list = binned ? reinterpret_cast<int2 *>(base + geo_bytes + win_bytes + row_bytes + count_bytes) : nullptr;
     cudaError_t e;
     {
         ProfileScope ps(ctx, "wrp_prep", 1);
         e = launch_wrp_prep(d_xyz, d_amp, (int)n, (int)n_pad, ctx->pitch, ctx->lambda, z_wrp, piston_on(ctx), geo, win,
-                            ctx->d_status, ctx->stream);
+                            rows, ctx->d_status, ctx->stream);
     }
     if (e != cudaSuccess) return cuda_status(e);
     // the own FFT reads only the rows < H, columns < W of the work plane; the cuFFT path reads all of it
@@ -688,12 +687,12 @@ int wrp_record(cgh_ctx *ctx, const float *d_xyz, const float *d_amp, int64_t n, 
     }
     const int64_t pad_ld = own ? ctx->fft_g.Lx : 2 * ctx->width;
     if (binned) {
-        ProfileScope ps(ctx, "wrp_bands", 3);
-        e = launch_wrp_bands(geo, win, (int)n_pad, ctx->height, count, offset, list, ctx->stream);
+        ProfileScope ps(ctx, "wrp_bands", 1);
+        e = launch_wrp_bands(geo, win, rows, (int)n_pad, ctx->height, count, list, ctx->stream);
         if (e != cudaSuccess) return cuda_status(e);
     }
     ProfileScope ps(ctx, "wrp_record", 1);
-    return cuda_status(launch_wrp_record(geo, win, (int)n_pad, ctx->height, ctx->width, offset, list, pad, pad_ld,
+    return cuda_status(launch_wrp_record(geo, win, (int)n_pad, ctx->height, ctx->width, count, list, pad, pad_ld,
                                          planes, ctx->stream));
 }
 

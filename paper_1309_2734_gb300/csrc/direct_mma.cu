@@ -45,15 +45,18 @@
 #include <cuda_fp16.h>
 
 #include "device_util.cuh"
+#include "half_turn.cuh"
 #include "host_util.h"
 #include "kernels.h"
-#include "sincospoly.h"
 #include "spherical_dev.cuh"
 #include "tcgen05.cuh"
 
 namespace cgh {
 
 namespace {
+
+using dev::f2;
+using dev::half_turn2;
 
 constexpr int kWorkers = 512;
 constexpr int kMmaThreads = kWorkers + 64;   // the workers, the MMA warp, the loader warp
@@ -101,8 +104,6 @@ struct MmaArgs {
     PhaseRef ref;
 };
 
-__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
-
 // The walk of one point down a side's rows in steps of 32 (Eqs. 6-8 at that stride): t = C d^2 at the first row,
 // D its first difference, S the second, top 32 bits of the 64-bit products.
 struct Walk {
@@ -116,34 +117,6 @@ __device__ __forceinline__ Walk walk_start(int d, uint32_t ch, uint32_t cl, uint
     w.t = ch * d2 + __umulhi(cl, d2) + add;
     w.D = ch * (uint32_t)e + __umulhi(cl, (uint32_t)e) - (e < 0 ? cl : 0u) + step;
     return w;
-}
-
-// sqrt(2) sin(pi r) and sqrt(2) cos(pi r) of two signed turns r (2^-32 turn): half the angle, so that s^2 - 1 and s c
-// are minus the cosine and the sine of the whole turn without a quadrant (sincospoly.h).
-template <int U>
-__device__ __forceinline__ void half_turn2(const float2 (&turn)[U], float2 (&s)[U], float2 (&c)[U])
-{
-    float2 r[U], u[U], hs[U], hc[U];
-#pragma unroll
-    for (int j = 0; j < U; ++j) {
-        r[j] = __fmul2_rn(turn[j], f2(2.3283064365386963e-10f));
-        u[j] = __fmul2_rn(r[j], r[j]);
-        hs[j] = f2(CGH_HSIN_4);
-        hc[j] = f2(CGH_HCOS_4);
-    }
-#define CGH_HORNER(OUT, IN, COEF)                                                                                     \
-    _Pragma("unroll") for (int j = 0; j < U; ++j) OUT[j] = __ffma2_rn(IN[j], u[j], f2(COEF));
-    CGH_HORNER(hs, hs, CGH_HSIN_3)
-    CGH_HORNER(hc, hc, CGH_HCOS_3)
-    CGH_HORNER(hs, hs, CGH_HSIN_2)
-    CGH_HORNER(hc, hc, CGH_HCOS_2)
-    CGH_HORNER(hs, hs, CGH_HSIN_1)
-    CGH_HORNER(hc, hc, CGH_HCOS_1)
-    CGH_HORNER(hs, hs, CGH_HSIN_0)
-    CGH_HORNER(c, hc, CGH_HCOS_0)
-#undef CGH_HORNER
-#pragma unroll
-    for (int j = 0; j < U; ++j) s[j] = __fmul2_rn(r[j], hs[j]);
 }
 
 // v - h for both halves of a packed FP16 pair (mixed-precision FMA, exact).

@@ -194,18 +194,19 @@ cudaError_t launch_fft_chirp_spectrum(const FftGrid &g, float2 *spec, unsigned l
 cudaError_t launch_fft_convolve(const FftGrid &g, const float *in, int H, int W, float2 *pad, const float2 *spec,
                                 const float2 *twx, const float2 *twy, float *out, cudaStream_t s);
 
-// win[j] = {piston (or 0), A, floor(w_j^2), floor(w_j)}; geo as in the point preparation, at d_j = z_j - z_wrp
+// win[j] = {piston (or 0), A, floor(w_j^2), floor(w_j)}, rows[j] = {y - floor(w_j), y + floor(w_j)}; geo as in the point
+// preparation, at d_j = z_j - z_wrp
 cudaError_t launch_wrp_prep(const float *d_xyz, const float *d_amp, int n, int n_pad, double pitch, double lambda,
-                            double z_wrp, bool piston, int4 *geo, uint4 *win, int *status, cudaStream_t s);
-// Band lists (32 rows each, built per segment of 4096 points): count[cells], offset[cells + 1],
-// list[sum of counts] (at most n_pad * bands), cells = bands x segments.
-int wrp_band_cells(int H, int n_pad);
-cudaError_t launch_wrp_bands(const int4 *geo, const uint4 *win, int n_pad, int H, int *count, int *offset, int *list,
-                             cudaStream_t s);
-// into pad (row stride pad_ld) when pad is not null, else into planes [2][H][W]; list == nullptr: every tile
-// walks all points (the same sums)
-cudaError_t launch_wrp_record(const int4 *geo, const uint4 *win, int n_pad, int H, int W, const int *offset,
-                              const int *list, float2 *pad, int64_t pad_ld, float *planes, cudaStream_t s);
+                            double z_wrp, bool piston, int4 *geo, uint4 *win, int2 *rows, int *status, cudaStream_t s);
+// The points that reach each band of 64 rows: wrp_band_cells(H, n_pad) counts and wrp_list_bytes(H, n_pad) of lists.
+int64_t wrp_band_cells(int H, int n_pad);
+size_t wrp_list_bytes(int H, int n_pad);
+cudaError_t launch_wrp_bands(const int4 *geo, const uint4 *win, const int2 *rows, int n_pad, int H, int *count,
+                             int2 *list, cudaStream_t s);
+// Into the padded work plane (pad, leading dimension pad_ld) or into planes [2][H][W]; list == nullptr: no lists, every
+// tile walks all points.
+cudaError_t launch_wrp_record(const int4 *geo, const uint4 *win, int n_pad, int H, int W, const int *count,
+                              const int2 *list, float2 *pad, int64_t pad_ld, float *planes, cudaStream_t s);
 
 // Hardware-sine throughput (results per second) of the whole GPU, measured; -1 on failure (probe.cu).
 double measure_mufu_rate(int num_sms, cudaStream_t s);

@@ -245,3 +245,49 @@ def test_numerical_reconstruction_focuses_on_the_point():
     r, c = np.unravel_index(np.argmax(inten), inten.shape)
     assert (r, c) == (310, 200)
     assert inten[305:316, 195:206].sum() > 0.5 * inten.sum()
+
+
+@pytest.mark.parametrize("w,h,n", [(33, 65, 9), (31, 63, 8193), (65, 130, 20000), (200, 40, 513)])
+def test_record_tile_and_list_edges(w, h, n):
+    """Tiles of 32 x 64 pixels with remainders, lists of several segments of points, batches with a remainder.  An
+    entry is good to 1.2e-7 RMS and a term has two (1.7e-7; 6e-7 with the spread over few points); a pixel adds up to
+    n terms one after the other in single precision, each sum rounded to 2^-25 of its size, which grows as the square
+    root of its terms: sqrt(n) 2^-25 at most (2.7e-6 at 8193 points)."""
+    c = workloads.wrp_cloud(77 + n, w, h, n)
+    ref = oracle.wrp_record(0, c.pitch_m, c.lambda_m, 0.5, c.xyz, c.amp, w, h)
+    xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
+    with Hologram(w, h, c.pitch_m, c.lambda_m) as hg:
+        got = hg.wrp_record(xyz, amp, 0.5)
+        hg.sync()
+    got = got.cpu().numpy()
+    tol = 6e-7 + math.sqrt(n) * 2.0 ** -25
+    assert oracle.nrms(got[0], ref.real) <= tol and oracle.nrms(got[1], ref.imag) <= tol
+
+
+def test_record_without_lists():
+    """Lists too large for their workspace (points x bands): every tile walks all points.  The sum over the cloud is
+    that over its two halves, whose lists fit."""
+    w, h, n = 4, 16384, 1_100_000
+    c = workloads.wrp_cloud(79, w, h, n)
+    xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
+    with Hologram(w, h, c.pitch_m, c.lambda_m) as hg:
+        whole = hg.wrp_record(xyz, amp, 0.5).clone()
+        k = n // 2
+        halves = hg.wrp_record(xyz[:k].contiguous(), amp[:k].contiguous(), 0.5).clone()
+        halves += hg.wrp_record(xyz[k:].contiguous(), amp[k:].contiguous(), 0.5)
+        hg.sync()
+    # a pixel adds about 2000 terms in another order: sqrt(2000) roundings of 2^-24
+    assert ((whole - halves).norm() / whole.norm()).item() <= 3e-6
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 1001, 4096])
+def test_kinoform_remainders(n):
+    """Four pixels a thread or one by one: the same codes whatever the count and the planes' alignment."""
+    rng = np.random.default_rng(n)
+    re, im = rng.standard_normal((2, 4099)).astype(np.float32)
+    with Hologram(8, 8, 8e-6, 532e-9) as hg:
+        want = hg.kinoform8(torch.from_numpy(np.stack([re[:4096], im[:4096]])).cuda()).flatten()
+        wave = torch.from_numpy(np.stack([re[:n], im[:n]])).cuda()
+        got = hg.kinoform8(wave).flatten()
+        hg.sync()
+    assert torch.equal(got, want[:n])
