@@ -549,7 +549,8 @@ int run_spherical(cgh_ctx *ctx, int width, int height, double pitch, double lamb
 
 // Fresnel diffraction state of the context, made on first use: the own FFT's
 // grid (Ly x Lx, powers of two), its twiddle tables, the padded work plane and
-// the chirp's spectrum; for grids beyond its lengths, a cuFFT plan of 2H x 2W.
+// the chirp's spectrum (a row and a column factor); for grids beyond its
+// lengths, a cuFFT plan of 2H x 2W and the spectrum on the whole grid.
 int ensure_fft(cgh_ctx *ctx)
 {
     if (ctx->fft_ready) return CGH_OK;
@@ -565,7 +566,7 @@ int ensure_fft(cgh_ctx *ctx)
         return rc;
     };
     if (cudaMalloc(&ctx->fft_pad, words * sizeof(float2)) != cudaSuccess ||
-        cudaMalloc(&ctx->fft_spec, words * sizeof(float2)) != cudaSuccess)
+        cudaMalloc(&ctx->fft_spec, (g.ok ? (size_t)g.Ly + g.Lx : words) * sizeof(float2)) != cudaSuccess)
         return fail(CGH_ENOMEM);
     if (g.ok) {
         // e^{-2 pi i k / L} in double, rounded once
@@ -608,7 +609,7 @@ int fresnel_run(cgh_ctx *ctx, double z, const float *in, float *d_out)
         const double s = ctx->pitch * ctx->pitch / (ctx->lambda * z) / cells;
         const unsigned long long C = turns_fixed64(ctx->pitch * ctx->pitch / (2.0 * ctx->lambda * z));
         if (g.ok) {
-            ProfileScope ps(ctx, "fresnel_spectrum", 5);
+            ProfileScope ps(ctx, "fresnel_spectrum", 3);
             e = launch_fft_chirp_spectrum(g, ctx->fft_spec, C, s * std::sin(a0), -s * std::cos(a0), ctx->fft_twx,
                                           ctx->fft_twy, ctx->stream);
         } else {

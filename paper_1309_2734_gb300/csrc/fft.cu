@@ -5,18 +5,19 @@
 // Forward 2-D transform of the H x W input, product with the chirp's
 // spectrum, inverse transform, crop:
 //   rows     Lx-point FFT of the H nonzero rows only, the input planes read
-//            straight into shared memory (the zero padding is never stored);
+//            straight into shared memory (the zero padding is never stored),
+//            times the chirp's row spectrum (the chirp is separable);
 //   columns  Ly = L1 L2 four-step: pass A, L1-point FFTs over the rows
 //            L2 a + b (rows >= H are zero: not loaded); pass B, L2-point FFTs
 //            over the contiguous rows L2 c + b, which leaves the spectrum in
 //            the scrambled order ky = c + L1 d at row L2 c + d.  Any fixed
-//            order serves a convolution, so the chirp's spectrum is kept in
-//            that order, and forward pass B, the product and inverse pass B
-//            are ONE pass (the middle kernel), twiddles e^{-2 pi i c b / Ly}
-//            included; inverse pass A writes only the rows < H.  Columns of
+//            order serves a convolution, so forward pass B, the product with
+//            the chirp's column spectrum and inverse pass B are ONE pass (the
+//            middle kernel), twiddles e^{-2 pi i c b / Ly} included; inverse
+//            pass A writes only the rows < H.  Columns of
 //            256 .. 2048 points instead take ONE pass over strips of 8 to 32
 //            whole columns in shared memory (forward transform of the rows
-//            < H, product with the spectrum in natural order, inverse, rows
+//            < H, product with the column spectrum, inverse, rows
 //            < H stored), so the plane crosses HBM once each way; longer
 //            columns do not fit at that strip width (64-byte row segments),
 //            and narrower strips measured slower than the four-step passes;
@@ -486,6 +487,7 @@ struct RowIO {
     float *out;
     long long plane;
     int y0, rows, W, Lx;
+    const float2 *sx;   // the chirp's row spectrum, a factor of the forward rows
     __device__ __forceinline__ float2 load(int q, int x) const
     {
         const int y = y0 + q;
@@ -503,7 +505,7 @@ struct RowIO {
                 out[plane + (long long)y * W + x] = v.y;
             }
         } else {
-            pad[(long long)y * Lx + x] = v;
+            pad[(long long)y * Lx + x] = MODE == kRowInPlace ? v : cmul(v, sx[x]);
         }
     }
 };
@@ -523,19 +525,20 @@ __device__ __forceinline__ bool rows_fft_direct(float2 *s, int Lx, int nseq, con
 }
 
 // Row transforms: nseq rows of length Lx per CTA.
-//   kRowExpand:  rows y < H from the input planes [2][H][W] (zeros beyond W), forward, into pad;
-//   kRowPadRows: rows y < H of pad, columns < W (zeros beyond), forward, in place;
-//   kRowInPlace: rows of pad, forward, in place (the chirp, all Ly rows);
+//   kRowExpand:  rows y < H from the input planes [2][H][W] (zeros beyond W), forward, times sx, into pad;
+//   kRowPadRows: rows y < H of pad, columns < W (zeros beyond), forward, times sx, in place;
+//   kRowInPlace: rows of pad, forward, in place (a line of the chirp);
 //   kRowCrop:    rows y < H of pad, inverse, columns < W into the output planes.
 template <int MODE>
 __global__ void __launch_bounds__(1024) fft_rows_kernel(const float *__restrict__ in, float2 *__restrict__ pad, float *__restrict__ out,
-                                int H, int W, int Lx, int rows, int nseq, const float2 *__restrict__ twx)
+                                int H, int W, int Lx, int rows, int nseq, const float2 *__restrict__ twx,
+                                const float2 *__restrict__ sx)
 {
     extern __shared__ float2 sm[];
     const int y0 = blockIdx.x * nseq;
     const int T = blockDim.x;
     const long long plane = (long long)H * W;
-    if (rows_fft_direct<MODE>(sm, Lx, nseq, twx, RowIO<MODE>{in, pad, out, plane, y0, rows, W, Lx})) return;
+    if (rows_fft_direct<MODE>(sm, Lx, nseq, twx, RowIO<MODE>{in, pad, out, plane, y0, rows, W, Lx, sx})) return;
     for (int q = 0; q < nseq; ++q) {
         const int y = y0 + q;
         for (int x = threadIdx.x; x < Lx; x += T) {
@@ -564,7 +567,10 @@ __global__ void __launch_bounds__(1024) fft_rows_kernel(const float *__restrict_
                 out[plane + (long long)y * W + x] = v.y;
             }
         } else {
-            for (int x = threadIdx.x; x < Lx; x += T) pad[(long long)y * Lx + x] = sm[saddr<kLayoutRows>(x, q, Lx, 0)];
+            for (int x = threadIdx.x; x < Lx; x += T) {
+                const float2 v = sm[saddr<kLayoutRows>(x, q, Lx, 0)];
+                pad[(long long)y * Lx + x] = MODE == kRowInPlace ? v : cmul(v, sx[x]);
+            }
         }
     }
 }
@@ -599,11 +605,11 @@ struct ColsAIO {
     }
 };
 
-// Column pass B, forward: in, rows L2 c + b times the four-step twiddle; out, the product with the spectrum into
-// shared memory (natural order) -- or, building the spectrum itself (spec == nullptr), straight to pad.
+// Column pass B, forward: in, rows L2 c + b times the four-step twiddle; out, the product with the chirp's column
+// spectrum (sy[d]: this c's) into shared memory (natural order).
 struct ColsBFwdIO {
     float2 *pad;
-    const float2 *spec;
+    const float2 *sy;
     float2 *s;
     const float2 *t4;
     int Lx, L2, c, x0, stride;
@@ -611,12 +617,7 @@ struct ColsBFwdIO {
     {
         return cmul(pad[(long long)(L2 * c + b) * Lx + x0 + q], t4[b]);
     }
-    __device__ __forceinline__ void store(int q, int d, float2 v) const
-    {
-        const long long g = (long long)(L2 * c + d) * Lx + x0 + q;
-        if (spec != nullptr) s[d * stride + q] = cmul(v, spec[g]);
-        else pad[g] = v;
-    }
+    __device__ __forceinline__ void store(int q, int d, float2 v) const { s[d * stride + q] = cmul(v, sy[d]); }
 };
 
 // Column pass B, inverse: out, rows L2 c + b times the conjugate four-step twiddle.
@@ -672,11 +673,10 @@ __global__ void __launch_bounds__(256, 4) fft_cols_a_kernel(float2 *__restrict__
 }
 
 // Column pass B over the rows L2 c + b (b < L2) of each strip, with the
-// four-step twiddle e^{-2 pi i c b / Ly}.  spec == nullptr: forward only, the
-// result (the spectrum in scrambled order) stored.  Otherwise: forward,
-// product with spec (same order, its tile loaded together with the data),
-// inverse, conjugate twiddle: the middle of the convolution in one pass.
-__global__ void __launch_bounds__(256, 4) fft_cols_b_kernel(float2 *__restrict__ pad, const float2 *__restrict__ spec, int Lx, int L1, int L2,
+// four-step twiddle e^{-2 pi i c b / Ly}: forward, product with the chirp's
+// column spectrum (spec_y, whose entry of output d is c + L1 d), inverse,
+// conjugate twiddle: the middle of the convolution in one pass.
+__global__ void __launch_bounds__(256, 4) fft_cols_b_kernel(float2 *__restrict__ pad, const float2 *__restrict__ spec_y, int Lx, int L1, int L2,
                                   int sw, const float2 *__restrict__ twy)
 {
     extern __shared__ float2 sm[];
@@ -685,31 +685,24 @@ __global__ void __launch_bounds__(256, 4) fft_cols_b_kernel(float2 *__restrict__
     const int c = blockIdx.x >> lstrips, x0 = (blockIdx.x & ((1 << lstrips) - 1)) << lsw;
     const int stride = sw + 1;
     const int n = L2 << lsw;
-    if (cols_ct(L2, sw) && blockDim.x == 256) {   // first and last stages on global memory: one tile, no spectrum tile
-        float2 *tw = sm + L2 * stride, *t4 = tw + L2;
-        for (int k = threadIdx.x; k < L2; k += blockDim.x) {
-            tw[k] = twy[k * L1];
-            t4[k] = twy[c * k];
-        }
+    // in shared memory: e^{-2 pi i k / L2} = twy[k L1], the four-step twiddles e^{-2 pi i c b / Ly} = twy[c b] and the
+    // spectrum's entries
+    float2 *tw = sm + L2 * stride, *t4 = tw + L2, *sy = t4 + L2;
+    for (int k = threadIdx.x; k < L2; k += blockDim.x) {
+        tw[k] = twy[k * L1];
+        t4[k] = twy[c * k];
+        sy[k] = spec_y[c + L1 * k];
+    }
+    if (cols_ct(L2, sw) && blockDim.x == 256) {   // first and last stages on global memory
         __syncthreads();
-        cols_fft_direct<false, true, true>(sm, L2, sw, tw, ColsBFwdIO{pad, spec, sm, t4, Lx, L2, c, x0, stride});
-        if (spec == nullptr) return;
+        cols_fft_direct<false, true, true>(sm, L2, sw, tw, ColsBFwdIO{pad, sy, sm, t4, Lx, L2, c, x0, stride});
         __syncthreads();   // the products are in shared memory
         cols_fft_direct<true, false, true>(sm, L2, sw, tw, ColsBInvIO{pad, t4, Lx, L2, c, x0});
         return;
     }
-    float2 *sp = sm + L2 * stride;   // the spectrum's tile
-    // in shared memory: e^{-2 pi i k / L2} = twy[k L1] and the four-step twiddles e^{-2 pi i c b / Ly} = twy[c b]
-    float2 *tw = sm + (spec != nullptr ? 2 : 1) * L2 * stride, *t4 = tw + L2;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const int b = i >> lsw, q = i & (sw - 1);
-        const long long g = (long long)(L2 * c + b) * Lx + x0 + q;
-        cp_async8(&sm[b * stride + q], pad + g);
-        if (spec != nullptr) cp_async8(&sp[b * stride + q], spec + g);
-    }
-    for (int k = threadIdx.x; k < L2; k += blockDim.x) {
-        tw[k] = twy[k * L1];
-        t4[k] = twy[c * k];
+        cp_async8(&sm[b * stride + q], pad + (long long)(L2 * c + b) * Lx + x0 + q);
     }
     cp_async_wait_all();
     __syncthreads();
@@ -719,17 +712,9 @@ __global__ void __launch_bounds__(256, 4) fft_cols_b_kernel(float2 *__restrict__
     }
     __syncthreads();
     cols_fft<false>(sm, L2, sw, stride, tw);
-    if (spec == nullptr) {
-#pragma unroll 4
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const int d = i >> lsw, q = i & (sw - 1);
-            pad[(long long)(L2 * c + d) * Lx + x0 + q] = sm[d * stride + q];
-        }
-        return;
-    }
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const int d = i >> lsw, q = i & (sw - 1);
-        sm[d * stride + q] = cmul(sm[d * stride + q], sp[d * stride + q]);
+        sm[d * stride + q] = cmul(sm[d * stride + q], sy[d]);
     }
     __syncthreads();
     cols_fft<true>(sm, L2, sw, stride, tw);
@@ -742,13 +727,10 @@ __global__ void __launch_bounds__(256, 4) fft_cols_b_kernel(float2 *__restrict__
 }
 
 // The fused column pass's global side: sequence q is column x0 + q, element e is row e (natural order).  Loads
-// read the rows below nz_rows (the rest are zero).  Stores: with spec, the product with the spectrum into shared
-// memory (the input of the inverse transform); without, the rows below keep_rows into pad.
+// read the rows below nz_rows (the rest are zero), stores write the rows below keep_rows.
 template <int LQ>
 struct StripIO {
     float2 *pad;
-    const float2 *spec;
-    float2 *s;
     int Lx, x0, nz_rows, keep_rows;
     __device__ __forceinline__ float2 load(int q, int e) const
     {
@@ -756,48 +738,41 @@ struct StripIO {
     }
     __device__ __forceinline__ void store(int q, int e, float2 v) const
     {
-        const int g = e * Lx + x0 + q;
-        if (spec != nullptr) s[strip_addr<LQ>(e, q)] = cmul(v, spec[g]);
-        else if (e < keep_rows) pad[g] = v;
+        if (e < keep_rows) pad[e * Lx + x0 + q] = v;
     }
 };
 
 // The columns in one pass, where a whole column fits in shared memory: per strip of 2^LQ columns, the forward
-// Ly-point transform (Ly = 2^LM) of the rows below nz_rows, the product with the spectrum (natural order) as the
-// last forward stage stores, the inverse transform, and the rows below keep_rows stored -- the plane crosses
-// HBM once each way instead of three times.  spec == nullptr: the forward transform alone, every row below
-// keep_rows stored (the chirp's spectrum).  2^(LM + LQ - 4) threads, each holding 16 values per stage.
+// Ly-point transform (Ly = 2^LM) of the rows below nz_rows, the product with the chirp's column spectrum, the inverse
+// transform, and the rows below keep_rows stored -- the plane crosses HBM once each way instead of three times.
+// 2^(LM + LQ - 4) threads, each holding 16 values per stage.
 template <int LM, int LQ>
 __global__ void __launch_bounds__(1 << (LM + LQ - 4), 1024 >> (LM + LQ - 4))
-    fft_cols_full_kernel(float2 *__restrict__ pad, const float2 *__restrict__ spec, int Lx, int nz_rows,
+    fft_cols_full_kernel(float2 *__restrict__ pad, const float2 *__restrict__ spec_y, int Lx, int nz_rows,
                          int keep_rows, const float2 *__restrict__ twy)
 {
     extern __shared__ float2 sm[];
     constexpr int T = 1 << (LM + LQ - 4);
     const int x0 = blockIdx.x << LQ;
-    const StripIO<LQ> io{pad, nullptr, sm, Lx, x0, nz_rows, keep_rows};
-    if (spec == nullptr) {
-        fft_io<false, kLayoutStrip, LM, LQ, true, true, 0>(sm, twy, io);
-        return;
-    }
+    const StripIO<LQ> io{pad, Lx, x0, nz_rows, keep_rows};
     fft_io<false, kLayoutStrip, LM, LQ, true, false, 0>(sm, twy, io);   // natural order in shared memory
 #pragma unroll 4
     for (int i = threadIdx.x; i < (1 << (LM + LQ)); i += T) {
         const int q = i & ((1 << LQ) - 1), e = i >> LQ;
         float2 &v = sm[strip_addr<LQ>(e, q)];
-        v = cmul(v, spec[e * Lx + x0 + q]);
+        v = cmul(v, spec_y[e]);
     }
     __syncthreads();
     fft_io<true, kLayoutStrip, LM, LQ, false, true, 0>(sm, twy, io);
 }
 
-// The chirp on the Ly x Lx grid, h(k, l) = pre exp(i 2 pi C (k'^2 + l'^2) / 2^64) (k' = k or k - Ly, the signed
-// offset; likewise l'), as the product of its separable factors: a(l) = exp(i 2 pi C l'^2 / 2^64) for the thread's
-// kChirpCols columns, computed once, and pre a(k) for each of the block's kChirpRows rows -- a complex product per
-// entry in place of a sine and cosine (the turns of the two factors add to the joint turn within 2^-31; each factor
-// is an accurate single-precision sine and cosine, the product adds about two units of rounding).
-constexpr int kChirpCols = 8, kChirpRows = 64;
-
+// The chirp h(k, l) = pre exp(i 2 pi C (k'^2 + l'^2) / 2^64) on the Ly x Lx grid (k' = k or k - Ly, the signed offset;
+// likewise l') is the product of a line over l, which carries pre, and one over k, so its spectrum is the product of the
+// lines' transforms: the forward rows take the one, the column pass the other, and no two-dimensional spectrum is
+// built or read (2048x2048: the middle column pass, 134 of 400 MB less, 73 -> 59 us; the call 206 -> 188 us).  What bounds
+// the column passes now is latency and issue: in blocks of columns that stay in L2 they were slower (198 us in two
+// blocks, 227 in four).
+// Entry l < Lx of h: the line over l; entry Lx + k: the line over k.
 __device__ __forceinline__ float2 chirp_factor(unsigned long long C, int k, int L)
 {
     const long long kk = k <= L / 2 ? k : k - L;
@@ -807,25 +782,12 @@ __device__ __forceinline__ float2 chirp_factor(unsigned long long C, int k, int 
     return make_float2(c, s);
 }
 
-__global__ void chirp_grid_kernel(float2 *__restrict__ h, int Ly, int Lx, unsigned long long C, float pre_re,
-                                  float pre_im)
+__global__ void chirp_lines_kernel(float2 *__restrict__ h, int Ly, int Lx, unsigned long long C, float pre_re,
+                                   float pre_im)
 {
-    const int l0 = blockIdx.x * blockDim.x * kChirpCols + threadIdx.x;
-    float2 a[kChirpCols];
-#pragma unroll
-    for (int j = 0; j < kChirpCols; ++j) {
-        const int l = l0 + j * (int)blockDim.x;
-        a[j] = l < Lx ? chirp_factor(C, l, Lx) : make_float2(0.0f, 0.0f);
-    }
-    const int k1 = min(Ly, (int)(blockIdx.y + 1) * kChirpRows);
-    for (int k = blockIdx.y * kChirpRows; k < k1; ++k) {
-        const float2 b = cmul(chirp_factor(C, k, Ly), make_float2(pre_re, pre_im));
-#pragma unroll
-        for (int j = 0; j < kChirpCols; ++j) {
-            const int l = l0 + j * (int)blockDim.x;
-            if (l < Lx) h[(long long)k * Lx + l] = cmul(b, a[j]);
-        }
-    }
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < Lx) h[i] = cmul(chirp_factor(C, i, Lx), make_float2(pre_re, pre_im));
+    else if (i < Lx + Ly) h[i] = chirp_factor(C, i - Lx, Ly);
 }
 
 int threads_for(int work)
@@ -893,23 +855,22 @@ static size_t cols_a_smem(const FftGrid &g, int swa)
     return ((size_t)g.L1 * (swa + 1) + g.L1) * sizeof(float2);
 }
 
-static size_t cols_b_smem(const FftGrid &g, int swb, bool product)
+static size_t cols_b_smem(const FftGrid &g, int swb)
 {
-    const int tiles = product && !cols_ct(g.L2, swb) ? 2 : 1;   // the compile-time form reads the spectrum directly
-    return ((size_t)tiles * g.L2 * (swb + 1) + 2 * g.L2) * sizeof(float2);
+    return ((size_t)g.L2 * (swb + 1) + 3 * g.L2) * sizeof(float2);
 }
 
 static cudaError_t configure_cols(const FftGrid &g)
 {
     static size_t done_a = 0, done_b = 0;
-    const size_t a = cols_a_smem(g, strip_width(g.Lx, g.L1)), b = cols_b_smem(g, strip_width(g.Lx, g.L2), true);
+    const size_t a = cols_a_smem(g, strip_width(g.Lx, g.L1)), b = cols_b_smem(g, strip_width(g.Lx, g.L2));
     cudaError_t e = cudaSuccess;
     if (a > 48 * 1024 && a > done_a) {
         for (auto fn : {(const void *)fft_cols_a_kernel<false>, (const void *)fft_cols_a_kernel<true>})
             if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a);
         if (e == cudaSuccess) done_a = a;
     }
-    if (e == cudaSuccess && b > 48 * 1024 && b > done_b) {   // the product pass holds two tiles
+    if (e == cudaSuccess && b > 48 * 1024 && b > done_b) {
         e = cudaFuncSetAttribute(fft_cols_b_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b);
         if (e == cudaSuccess) done_b = b;
     }
@@ -932,7 +893,7 @@ static int cols_full_lq(const FftGrid &g)
 }
 
 template <int LM, int LQ>
-static cudaError_t launch_cols_full_as(const FftGrid &g, float2 *pad, const float2 *spec, int nz_rows, int keep_rows,
+static cudaError_t launch_cols_full_as(const FftGrid &g, float2 *pad, const float2 *spec_y, int nz_rows, int keep_rows,
                                        const float2 *twy, cudaStream_t s)
 {
     constexpr int M = 1 << LM;
@@ -943,16 +904,16 @@ static cudaError_t launch_cols_full_as(const FftGrid &g, float2 *pad, const floa
                                     (int)bytes);
     });
     if (e != cudaSuccess) return e;
-    fft_cols_full_kernel<LM, LQ><<<g.Lx >> LQ, 1 << (LM + LQ - 4), bytes, s>>>(pad, spec, g.Lx, nz_rows, keep_rows, twy);
+    fft_cols_full_kernel<LM, LQ><<<g.Lx >> LQ, 1 << (LM + LQ - 4), bytes, s>>>(pad, spec_y, g.Lx, nz_rows, keep_rows, twy);
     return cudaGetLastError();
 }
 
-static cudaError_t launch_cols_full(const FftGrid &g, float2 *pad, const float2 *spec, int nz_rows, int keep_rows,
+static cudaError_t launch_cols_full(const FftGrid &g, float2 *pad, const float2 *spec_y, int nz_rows, int keep_rows,
                                     const float2 *twy, cudaStream_t s)
 {
     const int lq = cols_full_lq(g);
 #define CGH_COLS_FULL(LMV, LQV) \
-    if (g.Ly == (1 << LMV) && lq == LQV) return launch_cols_full_as<LMV, LQV>(g, pad, spec, nz_rows, keep_rows, twy, s);
+    if (g.Ly == (1 << LMV) && lq == LQV) return launch_cols_full_as<LMV, LQV>(g, pad, spec_y, nz_rows, keep_rows, twy, s);
     CGH_COLS_FULL(11, 3)
     CGH_COLS_FULL(10, 3)
     CGH_COLS_FULL(9, 4)
@@ -964,22 +925,15 @@ static cudaError_t launch_cols_full(const FftGrid &g, float2 *pad, const float2 
 cudaError_t launch_fft_chirp_spectrum(const FftGrid &g, float2 *spec, unsigned long long C, double pre_re,
                                       double pre_im, const float2 *twx, const float2 *twy, cudaStream_t s)
 {
-    chirp_grid_kernel<<<dim3((g.Lx + 256 * kChirpCols - 1) / (256 * kChirpCols), (g.Ly + kChirpRows - 1) / kChirpRows),
-                        256, 0, s>>>(spec, g.Ly, g.Lx, C, (float)pre_re, (float)pre_im);
-    const int nseq = rows_per_cta(g.Lx);
-    const size_t rs = rows_smem(g.Lx, nseq);
-    cudaError_t e = configure_rows(rs);
-    if (e != cudaSuccess) return e;
-    fft_rows_kernel<kRowInPlace><<<(g.Ly + nseq - 1) / nseq, threads_for(nseq * g.Lx), rs, s>>>(
-        nullptr, spec, nullptr, 0, 0, g.Lx, g.Ly, nseq, twx);
-    if (cols_full_lq(g) >= 0) return launch_cols_full(g, spec, nullptr, g.Ly, g.Ly, twy, s);
-    const int swa = strip_width(g.Lx, g.L1), swb = strip_width(g.Lx, g.L2);
-    e = configure_cols(g);
-    if (e != cudaSuccess) return e;
-    fft_cols_a_kernel<false><<<g.L2 * (g.Lx / swa), threads_for(g.L1 * swa), cols_a_smem(g, swa), s>>>(
-        spec, g.Lx, g.L1, g.L2, swa, g.Ly, g.Ly, twy);
-    fft_cols_b_kernel<<<g.L1 * (g.Lx / swb), threads_for(g.L2 * swb), cols_b_smem(g, swb, false), s>>>(
-        spec, nullptr, g.Lx, g.L1, g.L2, swb, twy);
+    chirp_lines_kernel<<<(g.Lx + g.Ly + 255) / 256, 256, 0, s>>>(spec, g.Ly, g.Lx, C, (float)pre_re, (float)pre_im);
+    for (int line = 0; line < 2; ++line) {
+        const int L = line == 0 ? g.Lx : g.Ly, nseq = rows_per_cta(L);
+        const size_t rs = rows_smem(L, nseq);
+        const cudaError_t e = configure_rows(rs);
+        if (e != cudaSuccess) return e;
+        fft_rows_kernel<kRowInPlace><<<1, threads_for(nseq * L), rs, s>>>(nullptr, line == 0 ? spec : spec + g.Lx, nullptr,
+                                                                        0, 0, L, 1, nseq, line == 0 ? twx : twy, nullptr);
+    }
     return cudaGetLastError();
 }
 
@@ -992,28 +946,29 @@ cudaError_t launch_fft_convolve(const FftGrid &g, const float *in, int H, int W,
     if (e != cudaSuccess) return e;
     if (in != nullptr)
         fft_rows_kernel<kRowExpand><<<(H + nseq - 1) / nseq, threads_for(nseq * g.Lx), rs, s>>>(in, pad, nullptr, H, W,
-                                                                                             g.Lx, H, nseq, twx);
+                                                                                             g.Lx, H, nseq, twx, spec);
     else
         fft_rows_kernel<kRowPadRows><<<(H + nseq - 1) / nseq, threads_for(nseq * g.Lx), rs, s>>>(nullptr, pad, nullptr,
-                                                                                              H, W, g.Lx, H, nseq, twx);
+                                                                                              H, W, g.Lx, H, nseq, twx, spec);
     if (cols_full_lq(g) >= 0) {
-        e = launch_cols_full(g, pad, spec, H, H, twy, s);
+        e = launch_cols_full(g, pad, spec + g.Lx, H, H, twy, s);
         if (e != cudaSuccess) return e;
         fft_rows_kernel<kRowCrop><<<(H + nseq - 1) / nseq, threads_for(nseq * g.Lx), rs, s>>>(nullptr, pad, out, H, W,
-                                                                                           g.Lx, H, nseq, twx);
+                                                                                           g.Lx, H, nseq, twx, spec);
         return cudaGetLastError();
     }
     const int swa = strip_width(g.Lx, g.L1), swb = strip_width(g.Lx, g.L2);
-    const size_t sa = cols_a_smem(g, swa), sb = cols_b_smem(g, swb, true);
+    const size_t sa = cols_a_smem(g, swa), sb = cols_b_smem(g, swb);
     e = configure_cols(g);
     if (e != cudaSuccess) return e;
     fft_cols_a_kernel<false><<<g.L2 * (g.Lx / swa), threads_for(g.L1 * swa), sa, s>>>(pad, g.Lx, g.L1, g.L2, swa, H,
                                                                                      g.Ly, twy);
-    fft_cols_b_kernel<<<g.L1 * (g.Lx / swb), threads_for(g.L2 * swb), sb, s>>>(pad, spec, g.Lx, g.L1, g.L2, swb, twy);
+    fft_cols_b_kernel<<<g.L1 * (g.Lx / swb), threads_for(g.L2 * swb), sb, s>>>(pad, spec + g.Lx, g.Lx, g.L1, g.L2, swb,
+                                                                             twy);
     fft_cols_a_kernel<true><<<g.L2 * (g.Lx / swa), threads_for(g.L1 * swa), sa, s>>>(pad, g.Lx, g.L1, g.L2, swa, g.Ly,
                                                                                     H, twy);
     fft_rows_kernel<kRowCrop><<<(H + nseq - 1) / nseq, threads_for(nseq * g.Lx), rs, s>>>(nullptr, pad, out, H, W,
-                                                                                       g.Lx, H, nseq, twx);
+                                                                                       g.Lx, H, nseq, twx, spec);
     return cudaGetLastError();
 }
 

@@ -185,8 +185,8 @@ struct FftGrid {
     bool ok = false;
 };
 FftGrid fft_grid(int H, int W);
-// The chirp pre * exp(i 2 pi C (k^2 + l^2) / 2^64) on the grid, transformed: its spectrum in the
-// scrambled column order the convolution uses.
+// The spectrum of the chirp pre * exp(i 2 pi C (k^2 + l^2) / 2^64) on the grid as its factors: spec[0 .. Lx) over the
+// columns (with pre), spec[Lx .. Lx + Ly) over the rows.
 cudaError_t launch_fft_chirp_spectrum(const FftGrid &g, float2 *spec, unsigned long long C, double pre_re,
                                       double pre_im, const float2 *twx, const float2 *twy, cudaStream_t s);
 // out ([2][H][W]) = crop(IFFT(FFT(input) * spec)); input = the planes in, or (in == nullptr) the rows
