@@ -126,9 +126,12 @@ enum {
     CGH_OPT_DIRECT_CTAS = 14,   /* direct amplitude forms with CGH_OPT_POINT_SPLIT = 0: the CTAs that share
                                    the (pixel tile, point) pairs; 0 = automatic (up to one per SM; the hardware
                                    schedules those beyond the resident ones as others finish) */
-    CGH_OPT_BATCH_MODE = 15,    /* cgh_batch: 0 = one persistent launch for the whole batch (default; GEMM units on
-                                   the tensor cores beside point preparation, factor generation and direct units
-                                   on the same SMs); 1 = per-kind launches (preparation and factors per instance,
+    CGH_OPT_BATCH_MODE = 15,    /* cgh_batch: 0 = default: a batch of 10^11 terms (width x height x points) or more
+                                   hologram by hologram on two streams of the context's own (not under stream
+                                   capture, nor with another batch option, GEMM_BN or GEMM_CHUNK set); else one
+                                   persistent launch for the whole batch (GEMM units on the tensor cores beside
+                                   point preparation, factor generation and direct units on the same SMs); 1 =
+                                   per-kind launches (preparation and factors per instance,
                                    then one GEMM launch and one direct launch per direct form) */
     CGH_OPT_BATCH_OVERLAP = 16, /* cgh_batch, persistent launch: 1 = a GEMM unit starts as soon as its own
                                    hologram's factors are written (default); 0 = once every hologram's factors
@@ -303,13 +306,15 @@ typedef struct {
 } cgh_instance;
 
 /*
- * Many holograms (for example the frames of a holographic video) in one
- * persistent launch.  inst is a host array of n_inst instances (the context's
- * own width/height/pitch/lambda are not used).  The form of each instance is
- * the autotuner's choice under the context's tolerance (CGH_FORM_AUTO) or the
- * context's form.  The first call with a given set of shapes builds the work
- * list and captures the launch in a CUDA graph; later calls with the same
- * shapes and buffers replay it.
+ * Many holograms (for example the frames of a holographic video) in one call.
+ * inst is a host array of n_inst instances (the context's own
+ * width/height/pitch/lambda are not used).  The form of each instance is the
+ * autotuner's choice under the context's tolerance (CGH_FORM_AUTO) or the
+ * context's form.  A large batch (CGH_OPT_BATCH_MODE) runs hologram by hologram
+ * on two streams that the context's stream waits for, with a workspace for the
+ * largest hologram on each.  A smaller one is one persistent launch: the first
+ * call with a given set of shapes builds the work list and captures the launch
+ * in a CUDA graph; later calls with the same shapes and buffers replay it.
  */
 int cgh_batch(cgh_ctx *ctx, const cgh_instance *inst, int n_inst);
 

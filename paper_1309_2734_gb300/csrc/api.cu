@@ -793,6 +793,7 @@ int cgh_destroy(cgh_ctx *ctx)
     if (!ctx) return CGH_OK;
     DeviceGuard g(ctx->device);
     int rc = cgh_sync(ctx);
+    destroy_batch_lanes(ctx->lanes);
     if (ctx->ws) cudaFree(ctx->ws);
     if (ctx->pws) cudaFree(ctx->pws);
     for (float2 *p : {ctx->fft_pad, ctx->fft_spec, ctx->fft_twx, ctx->fft_twy})
@@ -1177,6 +1178,7 @@ int cgh_sync(cgh_ctx *ctx)
         if (ms.count() > 2 * ctx->timeout_ms + 1000) return CGH_ETIMEOUT;
         std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
+    if (!ctx->d_status) return CGH_OK;   // a batch's lane: its status is the batch's
     int bits = 0;
     if (cudaMemcpy(&bits, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
         return cuda_status(cudaGetLastError());

@@ -16,6 +16,7 @@
 // per-CTA unit lists and one persistent direct launch per direct form.
 #include <algorithm>
 #include <cstring>
+#include <new>
 #include <vector>
 
 #include "context.h"
@@ -717,10 +718,117 @@ int batch_forms(const cgh_ctx *ctx, int *forms, int max_entries)
     return n;
 }
 
+// Contexts with streams and workspaces of their own that share the batch's status word.
+struct BatchLanes {
+    static constexpr int kCount = 2;
+    cgh_ctx *lane[kCount] = {};
+    cudaEvent_t start = nullptr, done[kCount] = {};
+};
+
+static BatchLanes *make_lanes(cgh_ctx *ctx)
+{
+    BatchLanes *L = new (std::nothrow) BatchLanes();
+    if (!L) return nullptr;
+    bool ok = cudaEventCreateWithFlags(&L->start, cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 0; i < BatchLanes::kCount && ok; ++i) {
+        L->lane[i] = new (std::nothrow) cgh_ctx();
+        ok = L->lane[i] != nullptr;
+        if (!ok) break;
+        L->lane[i]->device = ctx->device;
+        L->lane[i]->num_sms = ctx->num_sms;
+        L->lane[i]->d_status = ctx->d_status;
+        ok = cudaStreamCreateWithFlags(&L->lane[i]->stream, cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&L->done[i], cudaEventDisableTiming) == cudaSuccess;
+    }
+    if (ok) return L;
+    cudaGetLastError();
+    destroy_batch_lanes(L);
+    return nullptr;
+}
+
+void destroy_batch_lanes(BatchLanes *L)
+{
+    if (!L) return;
+    for (int i = 0; i < BatchLanes::kCount; ++i) {
+        if (L->done[i]) cudaEventDestroy(L->done[i]);
+        cgh_ctx *c = L->lane[i];
+        if (!c) continue;
+        cudaStream_t s = c->stream;
+        c->d_status = nullptr;   // the batch's context owns it
+        cgh_destroy(c);
+        if (s) cudaStreamDestroy(s);
+    }
+    if (L->start) cudaEventDestroy(L->start);
+    delete L;
+}
+
+// Whether the batch's holograms go one by one through the single-hologram forms on two streams: their GEMMs take the
+// two-SM tiles and layouts of the time model, run at 0.8 of the tensor peak against the persistent launch's 0.6, and
+// one hologram's preparation and factors fill the other's tails.  From kLanesEvals terms in all; below it the
+// launches of many small holograms cost more than that gains.  12 frames of 10^3 to 10^5 points, split FP16: 9.9 ms
+// against 10.7 (FP16 3.5 against 3.8; one stream 9.7 but 3.65, three 9.9); 6 frames of 3 10^3 to 3 10^4 points (1.7
+// 10^11 terms) 1.48 against 1.68 (FP16 0.56 against 0.64); 4 small ones (4 10^10 terms) 0.41 against 0.44 (FP16 0.181
+// against 0.171).  Not under capture (the forms grow their workspaces), nor with options of the other modes.
+constexpr double kLanesEvals = 1e11;
+
+static bool lanes_serve(const cgh_ctx *ctx, const cgh_instance *inst, int n)
+{
+    if (ctx->batch_mode != 0 || ctx->batch_overlap != 1 || ctx->batch_chunk_mb != 0 || ctx->batch_premade_pct >= 0 ||
+        ctx->drop_tile >= 0 || ctx->test_alloc_fail > 0 || ctx->gemm_bn != 0 || ctx->gemm_chunk != 0)
+        return false;
+    double evals = 0.0;
+    for (int i = 0; i < n; ++i) evals += (double)inst[i].width * inst[i].height * (double)inst[i].n_points;
+    if (evals < kLanesEvals) return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cs == cudaStreamCaptureStatusNone;
+}
+
+// The largest first, alternately on the lanes.
+static int run_batch_lanes(cgh_ctx *ctx, const cgh_instance *inst, int n, const std::vector<int> &forms)
+{
+    if (!ctx->lanes && !(ctx->lanes = make_lanes(ctx))) return CGH_ENOMEM;
+    BatchLanes &L = *ctx->lanes;
+    constexpr int count = BatchLanes::kCount;
+    std::vector<int> order(n);
+    for (int i = 0; i < n; ++i) order[i] = i;
+    auto work = [&](int i) { return (double)inst[i].width * inst[i].height * (double)inst[i].n_points; };
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work(a) > work(b); });
+    cudaError_t e = cudaEventRecord(L.start, ctx->stream);
+    for (int k = 0; k < count && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(L.lane[k]->stream, L.start, 0);
+    if (e != cudaSuccess) return cuda_status(e);
+    int rc = CGH_OK;
+    for (int j = 0; j < n && rc == CGH_OK; ++j) {
+        const cgh_instance &I = inst[order[j]];
+        cgh_ctx *c = L.lane[j % count];
+        c->timeout_ms = ctx->timeout_ms;
+        c->factor_budget_mb = ctx->factor_budget_mb;
+        c->form = forms[order[j]];
+        c->gemm_group = 1;   // as in the other modes
+        rc = compute_hologram(c, I.width, I.height, I.pitch_m, I.lambda_m, I.d_xyz, I.d_amp, I.n_points, I.d_out);
+    }
+    // the context's stream goes on after every lane, also after a failure
+    for (int k = 0; k < count; ++k) {
+        if (e == cudaSuccess) e = cudaEventRecord(L.done[k], L.lane[k]->stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, L.done[k], 0);
+    }
+    return rc != CGH_OK ? rc : cuda_status(e);
+}
+
 int run_batch(cgh_ctx *ctx, const cgh_instance *inst, int n)
 {
     if (!ctx->batch) ctx->batch = new BatchPlan();
     BatchPlan *plan = ctx->batch;
+    if (lanes_serve(ctx, inst, n)) {
+        std::vector<int> bn;
+        choose_forms(ctx, inst, n, plan, bn);
+        plan->key.clear();   // the forms are this batch's now
+        ProfileScope ps(ctx, "batch_lanes", 1);
+        return run_batch_lanes(ctx, inst, n, plan->forms);
+    }
     const std::vector<uint64_t> key = plan_key(ctx, inst, n);
     if (!(plan->exec && plan->key == key)) {
         // the previous graph may still be running on the context's stream

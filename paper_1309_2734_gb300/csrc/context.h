@@ -19,8 +19,10 @@
 namespace cgh {
 constexpr int64_t kDefaultFactorBudgetMb = 2048;   // factor workspace of one chunk of points, MiB
 struct BatchPlan;
+struct BatchLanes;
 struct TuneState;
 void destroy_batch_plan(BatchPlan *plan);
+void destroy_batch_lanes(BatchLanes *lanes);
 void destroy_tune_state(TuneState *t);
 }  // namespace cgh
 
@@ -87,6 +89,7 @@ struct cgh_ctx {
     std::vector<cudaEvent_t> event_pool;
     std::vector<Total> totals;
     cgh::BatchPlan *batch = nullptr;   // cgh_batch: cached plan and CUDA graph
+    cgh::BatchLanes *lanes = nullptr;  // cgh_batch on streams: contexts with workspaces of their own
     cgh::BatchPlan *single = nullptr;  // CGH_OPT_GEMM_PERSISTENT: one hologram's persistent plan and graph
     cgh::TuneState *tune = nullptr;    // autotuner measurements
 };

@@ -232,3 +232,44 @@ def test_video_batch_64_frames_sampled(tol_e9):
         ref = oracle.field_at(c.pitch_m, c.lambda_m, c.xyz, c.amp, cols, rows)
         got = o[torch.from_numpy(rows).cuda(), torch.from_numpy(cols).cuda()].cpu().numpy()
         assert oracle.nrms(got, ref) <= tol_e9 * 1e-9, c.name
+
+
+@pytest.mark.parametrize("form", ["gemm_split16", "gemm_f16", "direct_sfu"])
+def test_large_batch_on_streams(form):
+    """A batch of 10^11 terms or more runs on two streams of its own: ragged frames and an empty one, the same bits on a
+    second call and as each hologram alone, work queued before and after on the caller's stream, new data in the same
+    buffers, and a bad point reported."""
+    clouds = [workloads.random_cloud(900 + i, w, h, n) for i, (w, h, n) in
+              enumerate([(1920, 1080, 20000), (1283, 717, 30001), (64, 64, 0), (1920, 1080, 18001), (130, 257, 9000)])]
+    dev = _dev(clouds)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        src = [(x.clone(), a.clone()) for x, a, *_ in dev]
+        outs = [torch.full((c.height, c.width), 5.0, device="cuda") for c in clouds]
+        with Hologram(8, 8, 8e-6, 532e-9, form=form) as h:
+            for (x, a, *_), (sx, sa) in zip(dev, src):
+                x.copy_(sx)
+                a.copy_(sa)
+            batch(h, dev, outs)
+            first = [o.clone() for o in outs]   # on the same stream, without waiting
+            batch(h, dev, outs)
+            h.sync()
+            assert len(_lib.cgh_batch_forms(h.ctx)) == len(clouds)
+            for c, a, b, (x, amp, *_) in zip(clouds, first, outs, dev):
+                assert torch.equal(a, b)
+                with Hologram(c.width, c.height, c.pitch_m, c.lambda_m, form=form) as one:
+                    alone = one.point_cloud(x, amp)
+                    one.sync()
+                assert torch.equal(a, alone)
+            small = clouds[4]
+            ref = oracle.field(small.pitch_m, small.lambda_m, small.xyz, small.amp, small.width, small.height)
+            assert oracle.nrms(first[4].cpu().numpy(), ref) <= NRMS[form]
+            dev[1][1].mul_(2.0)
+            batch(h, dev, outs)
+            h.sync()
+            assert ((outs[1] - 2.0 * first[1]).norm() / first[1].norm()).item() < 1e-3
+            dev[0][0][17, 2] = -1.0
+            batch(h, dev, outs)
+            with pytest.raises(CghError) as ei:
+                h.sync()
+            assert ei.value.code == _lib.CGH_EINPUT
