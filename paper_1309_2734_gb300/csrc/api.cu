@@ -27,26 +27,28 @@ int run_direct_mma(cgh_ctx *ctx, const DirectMmaLayout &lay, int planes, const c
     const int64_t n_pad = padded_points(n);
     const size_t geo_bytes = align_up((size_t)n_pad * sizeof(int4), 256);
     const size_t aux_bytes = align_up((size_t)n_pad * sizeof(uint2), 256);
-    const size_t zero_bytes = align_up((size_t)(1 + lay.tiles) * sizeof(int), 256);   // max |A|, the tile counters
+    const int amp_parts = (int)((n_pad + kPrepBlock - 1) / kPrepBlock);
+    const size_t amp_bytes = align_up((size_t)amp_parts * sizeof(float), 256);
+    const size_t cnt_bytes = align_up((size_t)lay.tiles * sizeof(int), 256);
     const size_t slot_bytes = (size_t)2 * lay.ctas * 128 * lay.bn * sizeof(float);
-    int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, geo_bytes + aux_bytes + zero_bytes + slot_bytes);
+    int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, geo_bytes + aux_bytes + amp_bytes + cnt_bytes + slot_bytes);
     if (rc) return rc;
     char *base = static_cast<char *>(ctx->ws);
     int4 *geo = reinterpret_cast<int4 *>(base);
     uint2 *aux = reinterpret_cast<uint2 *>(base + geo_bytes);
     float *amax = reinterpret_cast<float *>(base + geo_bytes + aux_bytes);
-    cudaError_t e = cudaMemsetAsync(amax, 0, (size_t)(1 + lay.tiles) * sizeof(int), ctx->stream);
-    if (e != cudaSuccess) return cuda_status(e);
+    int *counters = reinterpret_cast<int *>(base + geo_bytes + aux_bytes + amp_bytes);
+    cudaError_t e = cudaSuccess;
     {
         ProfileScope ps(ctx, "prep_points", 1);
         e = launch_prep_points(d_xyz, d_amp, (int)n, (int)n_pad, pitch, lambda, geo, aux, ctx->d_status, amax,
-                               ctx->stream, aux_mode(ctx));
+                               ctx->stream, aux_mode(ctx), nullptr, 0, 0, 4, 4, nullptr, counters, lay.tiles);
     }
     if (e != cudaSuccess) return cuda_status(e);
     ProfileScope ps(ctx, name, 1);
-    return cuda_status(launch_direct_mma(lay, planes, geo, aux, amax, (int)n, width, height, d_out,
-                                         reinterpret_cast<float *>(base + geo_bytes + aux_bytes + zero_bytes),
-                                         reinterpret_cast<int *>(amax + 1), ctx->d_status,
+    return cuda_status(launch_direct_mma(lay, planes, geo, aux, amax, amp_parts, (int)n, width, height, d_out,
+                                         reinterpret_cast<float *>(reinterpret_cast<char *>(counters) + cnt_bytes), counters,
+                                         ctx->d_status,
                                          (uint64_t)ctx->timeout_ms * 1000000ull, ctx->stream, ctx->drop_tile,
                                          phase_ref(ctx)));
 }
@@ -527,7 +529,7 @@ int run_spherical(cgh_ctx *ctx, int width, int height, double pitch, double lamb
     if (e != cudaSuccess) return cuda_status(e);
     for (int v = 0; v < 2 && ml[v].bn > 0; ++v) {
         ProfileScope ps(ctx, "spherical_mma", 1);
-        e = launch_direct_mma(ml[v], 1, geo, aux, amax, (int)n, width, height, d_out, parts,
+        e = launch_direct_mma(ml[v], 1, geo, aux, amax, 1, (int)n, width, height, d_out, parts,
                               reinterpret_cast<int *>(amax + 2), ctx->d_status,
                               (uint64_t)ctx->timeout_ms * 1000000ull, ctx->stream, -1, phase_ref(ctx), ext,
                               v == 0 ? -1.0f : sph_mma_max_phase(ml[0].bn), sph_mma_max_phase(ml[v].bn));
@@ -777,8 +779,8 @@ int cgh_create(int width, int height, double pitch_m, double lambda_m, cgh_ctx *
     ctx->lambda = lambda_m;
     ctx->device = dev;
     ctx->num_sms = sms;
-    if (cudaMalloc(&ctx->d_status, 4 * sizeof(int)) != cudaSuccess ||
-        cudaMemset(ctx->d_status, 0, 4 * sizeof(int)) != cudaSuccess) {
+    if (cudaMalloc(&ctx->d_status, kStatusWords * sizeof(int)) != cudaSuccess ||
+        cudaMemset(ctx->d_status, 0, kStatusWords * sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         if (ctx->d_status) cudaFree(ctx->d_status);
         delete ctx;
@@ -1111,9 +1113,9 @@ int cgh_quantize8(cgh_ctx *ctx, const float *d_field, int64_t n, int mode, uint8
         ProfileScope ps(ctx, "kinoform8", 1);
         return cuda_status(launch_kinoform8(d_field, d_field + n, n, d_out, ctx->stream));
     }
-    ProfileScope ps(ctx, "quantize8", 3);
+    ProfileScope ps(ctx, "quantize8", 2);
     return cuda_status(
-        launch_quantize8(d_field, n, d_out, reinterpret_cast<uint32_t *>(ctx->d_status + 1), ctx->stream));
+        launch_quantize8(d_field, n, d_out, reinterpret_cast<uint32_t *>(ctx->d_status + 2), ctx->stream));
 }
 
 int cgh_profile_read(cgh_ctx *ctx, cgh_kernel_time *out, int max_entries, int *n_entries, int reset)

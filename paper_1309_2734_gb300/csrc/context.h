@@ -17,6 +17,7 @@
 #include "kernels.h"
 
 namespace cgh {
+constexpr int kStatusWords = 2 + 2 * kQuantParts;
 constexpr int64_t kDefaultFactorBudgetMb = 2048;   // factor workspace of one chunk of points, MiB
 struct BatchPlan;
 struct BatchLanes;
@@ -50,7 +51,7 @@ struct cgh_ctx {
     cudaStream_t side_stream = nullptr;   // factor generation of the next point chunk
     cudaEvent_t ev_ready = nullptr, ev_fact[2] = {nullptr, nullptr}, ev_gemm[2] = {nullptr, nullptr};
     int64_t tol_e9 = 10000;   // 1e-5
-    int *d_status = nullptr;  // [0] status bits, [1..2] quantiser scratch, [3] spare
+    int *d_status = nullptr;  // [0] status bits, [2 ..] quantiser scratch (kStatusWords)
     void *ws = nullptr;       // grow-only workspace
     size_t ws_bytes = 0;
     void *pws = nullptr;      // GEMM forms: prepared points and their groups (grow-only)

@@ -123,6 +123,19 @@ __device__ __forceinline__ bool wait_count(const int *count, int need, unsigned 
     }
 }
 
+// Programmatic dependent launch: lets the next kernel of the stream start, up to its own grid_wait, while this one still
+// runs (launch_dependent, host_util.h); grid_wait returns when the kernels before have completed and their writes are
+// visible.  Either does nothing in a plain launch.
+__device__ __forceinline__ void grid_launch_dependents()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+__device__ __forceinline__ void grid_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // 1-D bulk copy (TMA, non-tensor) global -> shared; completes tx bytes on bar.
 // dst, src and bytes must be multiples of 16.
 __device__ __forceinline__ void bulk_copy_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)

@@ -15,6 +15,10 @@
 //   640x64, 3000 points 1.1e-7 (3.1e-7);  256x256, 1024 points 2.8e-7 (6.7e-7);  wave 3.5e-7 (5.9e-7).
 // (Without the half turn 640x64 gave 7.2e-7; chains of 1 / 4 / 8 groups at 1920x1080 3.1 / 8.6 / 17.6e-7.)
 //
+// The kernel starts while the points are being prepared (dependent launch) and reduces max |A| itself, so nothing is
+// cleared before: 256x256, 10^3 points with the quantiser 25.7 us (35.4 with plain launches, clears and prep blocks of
+// 256 points).
+//
 // Time, prep included (before): 1920x1080, 10^4 points 0.307 ms (1.77; 67.5 G terms/ms); its complex wave 0.485 ms
 // (3.30); 1024x1024, 10^3 points 0.046 ms (0.117); 256x256, 10^3 points 0.026 ms (0.046); the spherical hologram,
 // 1920x1080, 10^4 points at 0.3-1 m 0.66 ms (7.36; with the narrowest tile, for points at 0.2 m, 1.53).
@@ -90,7 +94,8 @@ struct MmaArgs {
     const int4 *geo;
     const uint2 *aux;
     const float4 *ext;         // the spherical form's constants
-    const float *amp_max;      // [0] max |A|, [1] the spherical form's bound (prep)
+    const float *amp_max;      // max |A| in amp_parts values; spherical: [0] max |A|, [1] the bound (prep)
+    int amp_parts;
     float *out;                // plane 1 (the imaginary part) follows plane 0
     float4 *slots;
     int *counters;
@@ -371,12 +376,14 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
     constexpr int GROUP = SPH ? kSphMmaGroup : kGroup;
     constexpr int CHAIN = SPH ? kSphChain : kChain;
     static_assert(!SPH || (PLANES == 1 && BN % 64 == 0), "row pairs of the amplitude hologram");
+    if (SPH) grid_wait();
     if (SPH && !(g.amp_max[1] > g.phase_lo && g.amp_max[1] <= g.phase_hi)) return;   // another kernel's cloud
     constexpr int HB = BN / 4;          // accumulator columns per worker warp
     constexpr int TB = BN / PLANES;     // pixels of the tile along B
     extern __shared__ uint8_t smem_raw[];
     __shared__ int s_last;
     __shared__ uint32_t s_tmem;
+    __shared__ uint32_t s_amp[kMmaThreads / 32];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *s_pts = smem + C::kStages * C::kStage;
     MmaBars bars;
@@ -409,6 +416,11 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
         tmem_alloc(&s_tmem, C::kTmemCols);
         tmem_relinquish();
     }
+    grid_wait();   // the barriers and tensor memory above are set up while the points are still being prepared
+    uint32_t amp = 0;
+    for (int i = tid; i < g.amp_parts; i += kMmaThreads) amp = max(amp, __float_as_uint(__ldcg(g.amp_max + i)));
+    amp = __reduce_max_sync(0xffffffffu, amp);
+    if (lane == 0) s_amp[warp] = amp;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -500,7 +512,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
         const uint32_t entry = SPH ? (uint32_t)(rl * 128 + (((pair >> 2) ^ (rl & 7)) << 4) + (pair & 3) * 4)
                                    : (uint32_t)(rl * 128 + (((pair >> 1) ^ (rl & 7)) << 4) + (pair & 1) * 8);
         // amplitudes as multiples of 2^(eb - 126), the power of two above the largest
-        const uint32_t eb = min((__float_as_uint(*g.amp_max) >> 23) & 255u, 252u);
+        const uint32_t amax = __reduce_max_sync(0xffffffffu, s_amp[lane < kMmaThreads / 32 ? lane : 0]);
+        const uint32_t eb = min((amax >> 23) & 255u, 252u);
         const float a_scale = __uint_as_float((253u - eb) << 23), unscale = __uint_as_float((eb + 1u) << 23);
         const int quarter = warp & 3, cg = warp >> 2;   // tensor-memory lanes and columns of this warp
         const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(cg * HB), total = acc + C::kTotal;
@@ -723,8 +736,7 @@ cudaError_t launch_as(const MmaArgs &g, int ctas, cudaStream_t s)
                                     MmaCfg<BN>::kSmem);
     });
     if (e != cudaSuccess) return e;
-    direct_mma_kernel<BN, PLANES, SPH><<<ctas, kMmaThreads, MmaCfg<BN>::kSmem, s>>>(g);
-    return cudaGetLastError();
+    return launch_dependent(direct_mma_kernel<BN, PLANES, SPH>, dim3(ctas), dim3(kMmaThreads), MmaCfg<BN>::kSmem, s, g);
 }
 
 template <int PLANES, bool SPH>
@@ -745,8 +757,8 @@ cudaError_t launch_bn(int bn, const MmaArgs &g, int ctas, cudaStream_t s)
 }  // namespace
 
 cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4 *geo, const uint2 *aux,
-                              const float *amp_max, int n_points, int width, int height, float *out, float *slots,
-                              int *counters, int *status, uint64_t timeout_ns, cudaStream_t s, int drop,
+                              const float *amp_max, int amp_parts, int n_points, int width, int height, float *out,
+                              float *slots, int *counters, int *status, uint64_t timeout_ns, cudaStream_t s, int drop,
                               const PhaseRef &ref, const float4 *ext, float phase_lo, float phase_hi)
 {
     const int group = ext != nullptr ? kSphMmaGroup : kGroup;
@@ -768,6 +780,7 @@ cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4
     g.phase_lo = phase_lo;
     g.phase_hi = phase_hi;
     g.amp_max = amp_max;
+    g.amp_parts = amp_parts;
     g.out = out;
     g.slots = reinterpret_cast<float4 *>(slots);
     g.counters = counters;

@@ -12,7 +12,9 @@ namespace cgh {
 constexpr int kPointTile = 256;
 
 // a1: per-point constants and validation (prep.cu).  amp_max (optional, zeroed
-// by the caller) receives max_j |A_j|.  geo[j] = {x, y, C_hi, C_lo},
+// by the caller) receives max_j |A_j|; with `zero` given it receives one value
+// per kPrepBlock points instead (not zeroed before) and the kernel clears the
+// n_zero words at `zero`.  geo[j] = {x, y, C_hi, C_lo},
 // aux[j] = {w, A} with w per aux_x: kAuxSecondDiff: the second difference
 // 2 C_j (top 32 bits) of the recurrence; kAuxPiston: the piston
 // frac(z_j / lambda) in 2^-32 turn (the phase of Eq. 2 with its first term);
@@ -38,7 +40,10 @@ __host__ __device__ constexpr float sph_mma_max_phase(int bn) { return 0.05f * 2
 cudaError_t launch_prep_points(const float *d_xyz, const float *d_amp, int n, int n_pad, double pitch,
                                double lambda, int4 *geo, uint2 *aux, int *status, float *amp_max,
                                cudaStream_t s, int aux_x = kAuxSecondDiff, float4 *ext = nullptr, int width = 0,
-                               int height = 0, int tile_cols = 4, int tile_rows = 4, float *sph_max = nullptr);
+                               int height = 0, int tile_cols = 4, int tile_rows = 4, float *sph_max = nullptr,
+                               int *zero = nullptr, int n_zero = 0);
+// points per block: the FP64 pipe bounds a block, so small ones spread a small cloud over all SMs
+constexpr int kPrepBlock = 64;
 
 // The plane-wave reference phase of Eq. 5, phi_r(m, n) = kx m + ky n + phi0,
 // common to every point of a launch: kx, ky in 2^-64 turn per pixel, phi0 in
@@ -92,7 +97,7 @@ cudaError_t launch_direct_stream(bool sfu, const DirectShape &sh, int ctas, cons
 
 // The direct form with the tile's tables multiplied on the tensor cores (direct_mma.cu): the amplitude hologram at
 // out (planes = 1) or the complex wave, real plane then imaginary plane (planes = 2).  amp_max: max |A_j| of the
-// points (launch_prep_points).  slots: 2 ctas x 128 x bn floats (16-byte aligned); counters: one int per tile,
+// points, as amp_parts values (launch_prep_points).  slots: 2 ctas x 128 x bn floats (16-byte aligned); counters: one int per tile,
 // zeroed by the caller.  drop >= 0: CTA 0 never loads that group of kDirectMmaGroup points of its share (test hook).
 // ext != nullptr: the amplitude hologram of the spherical model (points prepared with the piston, ext and its bound
 // amp_max[1]; groups of kSphMmaGroup points); the kernel returns at once unless phase_lo < amp_max[1] <= phase_hi.
@@ -104,8 +109,8 @@ struct DirectMmaLayout {
     int tiles = 0;
 };
 cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4 *geo, const uint2 *aux,
-                              const float *amp_max, int n_points, int width, int height, float *out, float *slots,
-                              int *counters, int *status, uint64_t timeout_ns, cudaStream_t s, int drop = -1,
+                              const float *amp_max, int amp_parts, int n_points, int width, int height, float *out,
+                              float *slots, int *counters, int *status, uint64_t timeout_ns, cudaStream_t s, int drop = -1,
                               const PhaseRef &ref = PhaseRef(), const float4 *ext = nullptr, float phase_lo = 0.0f,
                               float phase_hi = 0.0f);
 
@@ -302,7 +307,8 @@ cudaError_t launch_persist(const PersistParams &p, int ctas, int bn_max, int *st
 cudaError_t launch_reduce_slices(const float *parts, int slices, int64_t n, int64_t slice_stride, float *out,
                                  cudaStream_t s, const float *bound = nullptr, float bound_min = 0.0f);
 
-// a6: 8-bit min/max quantiser (quantize.cu). scratch holds 2 uint32.
+// a6: 8-bit min/max quantiser (quantize.cu). scratch holds 2 kQuantParts uint32 (8-byte aligned).
+constexpr int kQuantParts = 2048;
 cudaError_t launch_quantize8(const float *field, int64_t n, uint8_t *out, uint32_t *scratch, cudaStream_t s);
 // Kinoform (phase-only hologram, Eq. 3) quantiser: 255/(2 pi) per radian of
 // atan2(im, re) taken in [0, 2 pi).

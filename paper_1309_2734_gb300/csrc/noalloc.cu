@@ -100,7 +100,7 @@ extern "C" int cgh_point_cloud_noalloc(int width, int height, double pitch_m, do
                                            status, amp_max, s);
         // one CTA per tile over all points: no parts of a tile, so neither slots nor counters
         if (e == cudaSuccess)
-            e = launch_direct_mma(choose_direct_mma(1, width, height, n_points, sms, 1, 0), 1, geo, aux, amp_max,
+            e = launch_direct_mma(choose_direct_mma(1, width, height, n_points, sms, 1, 0), 1, geo, aux, amp_max, 1,
                                   (int)n_points, width, height, d_out, nullptr, nullptr, status, 5000000000ull, s);
         if (e != cudaSuccess) {
             cudaGetLastError();

@@ -232,6 +232,19 @@ def test_quantize_bit_exact_on_same_field(n, offset):
     assert np.array_equal(_q_gpu(f, offset), want)
 
 
+@pytest.mark.parametrize("n", [15, 16, 4095, 4096, 4097, 8191, 65552, 304 * 4096 + 13, 1216 * 4096 + 4097])
+@pytest.mark.parametrize("offset", [0, 1, 4])
+def test_quantize_block_edges(n, offset):
+    # the smallest and the largest value where one block's share (16 values a thread) ends and the next begins
+    rng = np.random.default_rng(n)
+    f = rng.uniform(-1, 1, n).astype(np.float32)
+    for at in (0, n - 1, min(n, 4096) - 1, min(n - 1, 4096), n // 16 * 16 - 1):
+        for v in (3.0, -5.0):
+            g = f.copy()
+            g[at] = v
+            assert np.array_equal(_q_gpu(g, offset), oracle.quantize8(g)[0]), (at, v)
+
+
 def test_quantize_special_fields():
     f = np.full(100, 3.25, np.float32)
     assert np.all(_q_gpu(f) == 0)

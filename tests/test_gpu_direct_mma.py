@@ -110,3 +110,20 @@ def test_spherical(w, h, n, z, tol, ref):
         hg.sync()
         got = f.cpu().numpy()
     assert oracle.nrms(got[rows, cols], want) <= tol
+
+
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 256, 257, 1500])
+def test_largest_amplitude_in_any_block(n):
+    # max |A| comes from one value per 64 points: wherever the largest stands, the scaled entries stay in FP16's range
+    c = workloads.random_cloud(77 + n, 200, 150, n)
+    cols, rows, _ = _sampled(c)
+    for at in sorted({0, n // 2, min(n, 64) - 1, n - 1}):
+        amp = c.amp.copy()
+        amp[at] = -3e8
+        ref = oracle.field_at(c.pitch_m, c.lambda_m, c.xyz, amp, cols, rows)
+        for wave in (False, True):
+            with Hologram(200, 150, c.pitch_m, c.lambda_m, form="direct_sfu") as h:
+                x, a = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(amp).cuda()
+                f = h.wave(x, a)[0] if wave else h.point_cloud(x, a)
+                h.sync()
+                assert oracle.nrms(f.cpu().numpy()[rows, cols], ref) <= TOL
