@@ -289,8 +289,10 @@ int cgh_factors(cgh_ctx *ctx, const float *d_xyz, const float *d_amp, int64_t n_
  * hologram (kinoform) of Eq. 3, the workload the paper times (Section 5).
  *   d_out : float32 [2][height][width]: the real plane, then the imaginary plane.
  * Forms: CGH_DIRECT_SFU (both parts in one direct pass on the tensor cores, NRMS
- * about 3.6e-7) and the GEMM forms (Re O = P Q^T and Im O = P Q'^T, with
- * Q'[m][2j] = A_j sin alpha, Q'[m][2j+1] = A_j cos alpha).  CGH_FORM_AUTO
+ * about 3.6e-7) and the GEMM forms (Re O = P Q^T and, with the factor of the
+ * shorter side turned by a quarter, Im O = P' Q^T, P'[n][2j] = sin beta,
+ * P'[n][2j+1] = -cos beta, or Im O = P Q'^T, Q'[m][2j] = A_j sin alpha,
+ * Q'[m][2j+1] = A_j cos alpha).  CGH_FORM_AUTO
  * picks among those; CGH_DIRECT_ACCURATE returns CGH_ENOTSUP.
  */
 int cgh_wave(cgh_ctx *ctx, const float *d_xyz, const float *d_amp, int64_t n_points, float *d_out);

@@ -383,14 +383,14 @@ int run_gemm(cgh_ctx *ctx, int form, int width, int height, double pitch, double
         }
     }
     const FactorLaunch pf = [&](int64_t u0, int64_t nu, void *P, void *Q, int64_t ld, cudaStream_t s) {
-        return launch_factors(mode, geo + u0, aux + u0, (int)nu, height, width, P, Q, ld, amax, s, false, ref);
+        return launch_factors(mode, geo + u0, aux + u0, (int)nu, height, width, P, Q, ld, amax, s, ref);
     };
     return gemm_units(ctx, mode, width, height, n, "factors", pf, amax, d_out);
 }
 
 // The complex object wave: real plane at d_out, imaginary plane at d_out + W H.
 // Direct form: one pass accumulating both parts.  GEMM forms: per chunk of
-// points, Re = P Q^T and Im = P Q'^T (the same P), later chunks adding.
+// points, Re = P Q^T and Im = X Q^T or P X^T (launch_factors), later chunks adding.
 int run_wave(cgh_ctx *ctx, int form, const float *d_xyz, const float *d_amp, int64_t n, float *d_out)
 {
     const int width = ctx->width, height = ctx->height;
@@ -406,10 +406,13 @@ int run_wave(cgh_ctx *ctx, int form, const float *d_xyz, const float *d_amp, int
     if (form < CGH_GEMM_F16 || form > CGH_GEMM_SPLIT16) return CGH_ENOTSUP;
     const int mode = factor_mode(form);
     const int planes = mode == kFactorSplit16 ? 2 : 1;
-    const int64_t bytes_per_point = (int64_t)planes * (width + height) * 2 * 2;
-    int64_t chunk = (ctx->factor_budget_mb << 20) / bytes_per_point / 32 * 32;
-    if (chunk < 32) chunk = 32;
-    if (chunk >= n) chunk = n;
+    // P, Q and the imaginary part's factor beside the shorter of them within the budget, in even chunks.  One stream:
+    // with the next chunk's factors on a second one the GEMMs lost more than the factors' time (1920x1080, 10^5 points,
+    // split FP16: 3.75 ms in two chunks, 3.88 in four, against 3.48 in one).
+    const int64_t bytes_per_point = (int64_t)planes * (width + height + std::min(width, height)) * 2 * 2;
+    const int64_t most = std::max<int64_t>(32, (ctx->factor_budget_mb << 20) / bytes_per_point / 32 * 32);
+    const int64_t n_chunks = (n + most - 1) / most;
+    const int64_t chunk = std::min(n, ((n + n_chunks - 1) / n_chunks + 31) / 32 * 32);
     const int64_t ld_max = (2 * chunk + 63) / 64 * 64;
     GemmPlan plan;
     plan.mode = mode;
@@ -428,16 +431,18 @@ int run_wave(cgh_ctx *ctx, int form, const float *d_xyz, const float *d_amp, int
     const size_t amax_bytes = 256;
     const size_t p_bytes = align_up((size_t)planes * height * ld_max * 2, 256);
     const size_t q_bytes = align_up((size_t)planes * width * ld_max * 2, 256);
+    const bool beside_p = imag_beside_p(height, width);
+    const size_t x_bytes = beside_p ? p_bytes : q_bytes;
     const size_t part_bytes = plan.splits > 1 ? (size_t)plan.splits * 2 * plane * sizeof(float) : 0;
-    int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, geo_bytes + aux_bytes + amax_bytes + p_bytes + q_bytes + part_bytes);
+    int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, geo_bytes + aux_bytes + amax_bytes + p_bytes + q_bytes + x_bytes +
+                                                     part_bytes);
     if (rc) return rc;
     char *base = static_cast<char *>(ctx->ws);
     int4 *geo = reinterpret_cast<int4 *>(base);
     uint2 *aux = reinterpret_cast<uint2 *>(base + geo_bytes);
     float *amax = reinterpret_cast<float *>(base + geo_bytes + aux_bytes);
-    void *P = base + geo_bytes + aux_bytes + amax_bytes;
-    void *Q = base + geo_bytes + aux_bytes + amax_bytes + p_bytes;
-    float *parts = reinterpret_cast<float *>(base + geo_bytes + aux_bytes + amax_bytes + p_bytes + q_bytes);
+    char *P = base + geo_bytes + aux_bytes + amax_bytes, *Q = P + p_bytes, *X = Q + q_bytes;
+    float *parts = reinterpret_cast<float *>(X + x_bytes);
     e = cudaMemsetAsync(amax, 0, sizeof(float), ctx->stream);
     if (e != cudaSuccess) return cuda_status(e);
     {
@@ -452,22 +457,19 @@ int run_wave(cgh_ctx *ctx, int form, const float *d_xyz, const float *d_amp, int
     for (int64_t c0 = 0; c0 < n; c0 += chunk) {
         const int64_t nc = n - c0 < chunk ? n - c0 : chunk;
         const int64_t ld = (2 * nc + 63) / 64 * 64;
+        {
+            ProfileScope ps(ctx, "factors", 1);
+            e = launch_factors(mode, geo + c0, aux + c0, (int)nc, height, width, P, Q, ld, amax, ctx->stream, ref, X);
+        }
+        if (e != cudaSuccess) return cuda_status(e);
         GemmPlan pc = plan;
         pc.accumulate = c0 > 0;
-        for (int part = 0; part < 2; ++part) {
-            {
-                ProfileScope ps(ctx, "factors", 1);
-                e = launch_factors(mode, geo + c0, aux + c0, (int)nc, height, width, P, Q, ld, amax, ctx->stream,
-                                   part == 1, ref);
-            }
-            if (e != cudaSuccess) return cuda_status(e);
-            {
-                ProfileScope ps(ctx, "gemm_tcgen05", 1);
-                e = launch_gemm(pc, P, Q, height, width, ld, part == 0 ? re_out : im_out, plane, amax, ctx->d_status,
-                                tmo, ctx->stream);
-            }
-            if (e != cudaSuccess) return cuda_status(e);
-        }
+        ProfileScope ps(ctx, "gemm_tcgen05", 2);
+        e = launch_gemm(pc, P, Q, height, width, ld, re_out, plane, amax, ctx->d_status, tmo, ctx->stream);
+        if (e == cudaSuccess)
+            e = launch_gemm(pc, beside_p ? X : P, beside_p ? Q : X, height, width, ld, im_out, plane, amax, ctx->d_status,
+                            tmo, ctx->stream);
+        if (e != cudaSuccess) return cuda_status(e);
     }
     if (plan.splits == 1) return CGH_OK;
     ProfileScope ps(ctx, "reduce_slices", 2);
@@ -1014,7 +1016,7 @@ int cgh_factors(cgh_ctx *ctx, const float *d_xyz, const float *d_amp, int64_t n_
     if (e != cudaSuccess) return cuda_status(e);
     ProfileScope ps(ctx, "factors", 1);
     return cuda_status(launch_factors(factor_mode(dtype_form), geo, aux, (int)n_points, ctx->height, ctx->width,
-                                      d_p, d_q, ld, nullptr, ctx->stream, false, phase_ref(ctx)));
+                                      d_p, d_q, ld, nullptr, ctx->stream, phase_ref(ctx)));
 }
 
 int cgh_batch(cgh_ctx *ctx, const cgh_instance *inst, int n_inst)

@@ -37,18 +37,21 @@ __device__ __forceinline__ uint32_t pack(float lo_col, float hi_col, int mode, b
 constexpr float kTurnK1 = 6.28318595886230469f;   // 0x40c90fdc
 constexpr float kTurnK0 = 9.42477893829345703f;   // 1.5 * kTurnK1, exact
 
-// One point's entry of a row: P (cos b, sin b); Q, the amplitude times (cos a, -sin a), or with IMAG
-// (sin a, cos a) -- the imaginary part's factor.
-template <bool IS_P, bool IMAG>
-__device__ __forceinline__ void factor_entry(float s, float c, float a, float &re, float &im)
+// The imaginary part's factor beside P or beside Q (none: the real part alone).
+enum { kDualNone = 0, kDualP = 1, kDualQ = 2 };
+
+// The imaginary part's entries from the real part's: P (cos b, sin b) -> (sin b, -cos b), Q (A cos a, -A sin a) ->
+// (A sin a, A cos a), a swap and a sign of the packed pair (hi and lo alike: rounding is symmetric).
+template <bool IS_P>
+__device__ __forceinline__ uint32_t imag_entry(uint32_t pair)
 {
-    if (IS_P) {
-        re = c;
-        im = s;
-    } else {
-        re = IMAG ? a * s : a * c;
-        im = IMAG ? a * c : -a * s;
-    }
+    return __byte_perm(pair, 0, 0x1032) ^ (IS_P ? 0x80000000u : 0x8000u);
+}
+
+template <bool IS_P>
+__device__ __forceinline__ uint4 imag_entries(uint4 v)
+{
+    return make_uint4(imag_entry<IS_P>(v.x), imag_entry<IS_P>(v.y), imag_entry<IS_P>(v.z), imag_entry<IS_P>(v.w));
 }
 
 // FP16 / BF16 factors of rows [line0, line1) of P (IS_P) or Q for the thread's four points: the turn walked down the
@@ -56,11 +59,11 @@ __device__ __forceinline__ void factor_entry(float s, float c, float a, float &r
 // line0 (drift below 32^2 / 2 units of 2^-32 turn over a block's 32 rows, far below the factors' 2^-11), converted
 // by its top 23 bits as a float mantissa with a half turn added (so (f - 1.5) K1 is the angle itself in [-pi, pi)):
 // no 64-bit product and no conversion instruction per entry.
-template <int MODE, bool IS_P, bool IMAG>
+template <int MODE, bool IS_P, bool DUAL>
 __device__ __forceinline__ void factor_rows_walk(int line0, int line1, const int (&coord)[4], const uint32_t (&chi)[4],
                                                  const uint32_t (&clo)[4], const uint32_t (&pist)[4],
                                                  const float (&a)[4], const bool (&live)[4], uint16_t *base,
-                                                 long long ld, int j0, const PhaseRef &ref)
+                                                 uint16_t *X, long long ld, int j0, const PhaseRef &ref)
 {
     if (line0 >= line1) return;
     uint32_t g[4], e[4], D[4];
@@ -82,27 +85,28 @@ __device__ __forceinline__ void factor_rows_walk(int line0, int line1, const int
             const float f = __uint_as_float(__funnelshift_r(g[q] + radd, 0x7fu, 9));
             float s, c;
             __sincosf(fmaf(f, kTurnK1, -kTurnK0), &s, &c);
-            float re, im;
-            factor_entry<IS_P, IMAG>(s, c, a[q], re, im);
-            v[2 * q] = live[q] ? re : 0.0f;
-            v[2 * q + 1] = live[q] ? im : 0.0f;
+            v[2 * q] = live[q] ? (IS_P ? c : a[q] * c) : 0.0f;
+            v[2 * q + 1] = live[q] ? (IS_P ? s : -a[q] * s) : 0.0f;
             g[q] += e[q];
             e[q] += D[q];
         }
-        uint16_t *dst = base + (long long)line * ld + 2 * j0;
-        *reinterpret_cast<uint4 *>(dst) = make_uint4(pack(v[0], v[1], MODE, false), pack(v[2], v[3], MODE, false),
-                                                     pack(v[4], v[5], MODE, false), pack(v[6], v[7], MODE, false));
+        const long long at = (long long)line * ld + 2 * j0;
+        const uint4 w = make_uint4(pack(v[0], v[1], MODE, false), pack(v[2], v[3], MODE, false),
+                                   pack(v[4], v[5], MODE, false), pack(v[6], v[7], MODE, false));
+        *reinterpret_cast<uint4 *>(base + at) = w;
+        if (DUAL) *reinterpret_cast<uint4 *>(X + at) = imag_entries<IS_P>(w);
     }
 }
 
 // The factors of one thread's four points j0 .. j0 + 3 (those below n_points; the rest of the slots are zero
 // columns) on rows [r_begin, r_end) of the stacked rows (P's rows below height, then Q's rows), Q scaled by
-// scale (1 / max|A|).
-template <int MODE, bool IMAG>
+// scale (1 / max|A|).  DUAL: and the imaginary part's factor beside one of them, to X in that one's layout.
+template <int MODE, int DUAL>
 __device__ __forceinline__ void factor_thread(int j0, int r_begin, int r_end, const int4 *__restrict__ geo,
                                               const uint2 *__restrict__ aux, int n_points, int height, int width,
-                                              uint16_t *__restrict__ P, uint16_t *__restrict__ Q, long long ld,
-                                              long long plane_p, long long plane_q, float scale, const PhaseRef &ref)
+                                              uint16_t *__restrict__ P, uint16_t *__restrict__ Q,
+                                              uint16_t *__restrict__ X, long long ld, long long plane_p,
+                                              long long plane_q, float scale, const PhaseRef &ref)
 {
     int px[4], py[4];
     uint32_t chi[4], clo[4], pist[4];
@@ -129,9 +133,10 @@ __device__ __forceinline__ void factor_thread(int j0, int r_begin, int r_end, co
     }
     if constexpr (MODE != kFactorSplit16) {
         // P rows below height, Q rows (columns) above
-        factor_rows_walk<MODE, true, IMAG>(r_begin, min(r_end, height), py, chi, clo, pist, a, live, P, ld, j0, ref);
-        factor_rows_walk<MODE, false, IMAG>(max(r_begin, height) - height, r_end - height, px, chi, clo, pist, a, live,
-                                            Q, ld, j0, ref);
+        factor_rows_walk<MODE, true, DUAL == kDualP>(r_begin, min(r_end, height), py, chi, clo, pist, a, live, P, X, ld,
+                                                     j0, ref);
+        factor_rows_walk<MODE, false, DUAL == kDualQ>(max(r_begin, height) - height, r_end - height, px, chi, clo, pist,
+                                                      a, live, Q, X, ld, j0, ref);
         return;
     }
     // split FP16: the exact turn of every entry (its hi + lo pair carries 2^-22 of it)
@@ -151,21 +156,25 @@ __device__ __forceinline__ void factor_thread(int j0, int r_begin, int r_end, co
                 const float t = (float)(int)g * 2.3283064365386963e-10f;     // [-1/2, 1/2)
                 sincos_turn(t, s, c);
                 if (!is_p) {
-                    const float cc = c;
-                    c = IMAG ? a[q] * s : a[q] * c;
-                    s = IMAG ? a[q] * cc : -a[q] * s;
+                    c = a[q] * c;
+                    s = -a[q] * s;
                 }
             }
             v[2 * q] = c;
             v[2 * q + 1] = s;
         }
-        uint16_t *dst = (is_p ? P + (long long)line * ld : Q + (long long)line * ld) + 2 * j0;
+        const long long at = (long long)line * ld + 2 * j0, lo_at = at + (is_p ? plane_p : plane_q);
+        uint16_t *base = is_p ? P : Q;
         const uint4 hi = make_uint4(pack(v[0], v[1], MODE, false), pack(v[2], v[3], MODE, false),
                                     pack(v[4], v[5], MODE, false), pack(v[6], v[7], MODE, false));
-        *reinterpret_cast<uint4 *>(dst) = hi;
+        *reinterpret_cast<uint4 *>(base + at) = hi;
         const uint4 lo = make_uint4(pack(v[0], v[1], MODE, true), pack(v[2], v[3], MODE, true),
                                     pack(v[4], v[5], MODE, true), pack(v[6], v[7], MODE, true));
-        *reinterpret_cast<uint4 *>(dst + (is_p ? plane_p : plane_q)) = lo;
+        *reinterpret_cast<uint4 *>(base + lo_at) = lo;
+        if (DUAL != kDualNone && is_p == (DUAL == kDualP)) {
+            *reinterpret_cast<uint4 *>(X + at) = imag_entries<DUAL == kDualP>(hi);
+            *reinterpret_cast<uint4 *>(X + lo_at) = imag_entries<DUAL == kDualP>(lo);
+        }
     }
 }
 

@@ -143,12 +143,14 @@ int direct_ctas_per_sm(bool sfu, bool tall);
 // kFactorSplit16 the lo planes follow the hi planes (offset rows * ld).
 // amp_max (optional) scales Q by 1 / max|A|.
 enum { kFactorF16 = 0, kFactorBF16 = 1, kFactorSplit16 = 2 };
-// imag_q_only: write only Q' (the factor of the imaginary part) into Q.
+// X != nullptr: and the factor of the imaginary part, beside P (Im = X Q^T) when
+// imag_beside_p, else beside Q (Im = P X^T), in that one's layout.
 // The reference phase goes to both factors (ky n into P, kx m + phi0 into Q),
 // the piston (aux.x) into Q.
 cudaError_t launch_factors(int mode, const int4 *geo, const uint2 *aux, int n_points, int height, int width,
                            void *P, void *Q, int64_t ld, const float *amp_max, cudaStream_t s,
-                           bool imag_q_only = false, const PhaseRef &ref = PhaseRef());
+                           const PhaseRef &ref = PhaseRef(), void *X = nullptr);
+inline bool imag_beside_p(int height, int width) { return height <= width; }
 
 // Grouped GEMM form (groups.cu, factors.cu).  Groups: points with the same
 // plane constant C and the same column x.  meta (device, 4 ints): [0] planes

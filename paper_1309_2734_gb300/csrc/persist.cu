@@ -322,7 +322,7 @@ __device__ __forceinline__ void run_factor_unit(const PersistJob &J, int band, i
     const int r0 = band * kFactorRows;
     const int r1 = min(J.height + J.width, r0 + kFactorRows);
     if (j0 < J.point_slots)
-        factor_thread<MODE, false>(j0, r0, r1, J.geo, J.aux, J.n, J.height, J.width, J.P, J.Q, J.ld, J.plane_p,
+        factor_thread<MODE, kDualNone>(j0, r0, r1, J.geo, J.aux, J.n, J.height, J.width, J.P, J.Q, nullptr, J.ld, J.plane_p,
                                    J.plane_q, scale, PhaseRef());
 }
 

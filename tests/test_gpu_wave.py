@@ -142,3 +142,25 @@ def test_wave_gemm_orientations(trans):
     ref = oracle.wave(c.pitch_m, c.lambda_m, c.xyz, c.amp, 300, 140)
     got, _ = _wave(c, "gemm_split16", {_lib.CGH_OPT_GEMM_TRANSPOSE: trans})
     _check_wave(got, ref, 1e-5)
+
+
+@pytest.mark.parametrize("form", ["gemm_f16", "gemm_bf16", "gemm_split16"])
+@pytest.mark.parametrize("w,h", [(1, 5), (5, 1), (64, 64), (300, 33), (33, 300), (130, 257)])
+@pytest.mark.parametrize("n,budget", [(1, 0), (35, 0), (1029, 0), (1029, 1)])
+def test_imaginary_factor_beside_either_side(form, w, h, n, budget):
+    # the imaginary part's factor is written beside the side with fewer rows; rows in blocks of 32, four points a
+    # thread, chunks of points with a remainder
+    c = workloads.random_cloud(4400 + w + n, w, h, n)
+    ref = oracle.wave(c.pitch_m, c.lambda_m, c.xyz, c.amp, w, h)
+    with Hologram(w, h, c.pitch_m, c.lambda_m, form=form) as hh:
+        if budget:
+            hh.set_option(_lib.CGH_OPT_FACTOR_BUDGET_MB, budget)
+        got = hh.wave(torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()).cpu().numpy()
+    # an entry is off by up to 2^-11, 2^-9, 2^-22 of itself and a term has two; split FP16 adds the hardware sine's
+    # 4e-7 of each and the accumulation's 3e-6.  Where the terms add in phase (64x64: the chirps barely turn) both are
+    # proportional to the sum: the accumulation truncates in proportion to it, and equal angles err alike.
+    rel = {"gemm_f16": 1.2e-3, "gemm_bf16": 9e-3, "gemm_split16": 6e-6}[form]
+    scale = max(np.sqrt((c.amp.astype(np.float64) ** 2).sum()), np.sqrt((np.abs(ref) ** 2).mean()))
+    for plane, want in zip(got, (ref.real, ref.imag)):
+        d = plane.astype(np.float64) - want
+        assert np.sqrt((d * d).mean()) <= rel * scale
