@@ -7,8 +7,10 @@ Workload (default): a 1920x1080 hologram of 10,000 seeded synthetic points
 (z ~ U[0.3, 1.0] m, A ~ U[0.5, 1.0], lambda = 532 nm, p = 8 um), the
 display-size case of the paper's direct-calculation experiments.  One step is
 one pass of the hot path over that cloud: point preparation, the direct
-kernel (SFU cosine; the CTAs take equal shares of the (pixel tile, point)
-pairs and sum each tile's parts in the kernel), and the 8-bit quantiser.
+kernel (each CTA makes the sines and cosines of its tile's columns and rows
+as split FP16 and multiplies them on the tensor cores; the CTAs take equal
+shares of the (pixel tile, point) pairs and sum each tile's parts in the
+kernel), and the 8-bit quantiser.
 Inputs and outputs are far below L2, so a 256 MiB buffer is written between
 timed steps to flush L2; the flush is not timed.
 
@@ -35,12 +37,13 @@ if ROOT not in sys.path:
 
 METRIC = "G point-pixel evals/s and holograms/s, direct FP32 vs tensor GEMM, at stated NRMS error"
 UNIT = "Gevals/s"
-MUFU_PER_SM_PER_CLK = 16        # MUFU (hardware sine / cosine) operations per SM per clock
 FMA_PER_SM_PER_CLK = 128        # FP32 FMA-pipe operations per SM per clock
+DIRECT_FLOPS = 12               # direct forms, per evaluation: K = 2 (cosine, sine), three products of split FP16
 
 
 def direct_ops(form, width, height, n_points):
-    """The direct kernel's work per launch in FMA-pipe operations, as the kernel does it: a CTA covers a 128 x 64
+    """The SIMT direct kernel's work per launch in FMA-pipe operations (the direct forms with a pinned thread block,
+    CGH_OPT_DIRECT_SHAPE; by default they run on the tensor cores, DIRECT_FLOPS), as the kernel does it: a CTA covers a 128 x 64
     tile (256 x 32 where that pads a fifth fewer pixels); per point it takes the sine and cosine of the tile's
     columns and rows once (the SFU form: one FFMA and the sine's range multiply per entry, and the amplitude's two
     multiplies per row entry; the accurate form: two polynomials of 8 FMA-pipe operations per entry), then every
@@ -431,13 +434,11 @@ def run_ours(args):
             # the whole hologram (prep, factors, GEMM, reduction) against the same tensor peak
             rec["e2e_tensor_frac"] = 4.0 * wc.evals * passes / (ms * 1e-3) / 1e12 / peak_tc
         elif extra in kp:
-            ops, pipe, per_clk, per_eval = direct_ops(extra, wc.width, wc.height, wc.n_points)
-            pk = per_clk * torch.cuda.get_device_properties(local).multi_processor_count * \
-                (_peaks().get("sm_max_mhz") or 2070.0) * 1e6
+            peak_tc = _peaks().get("bf16_tflops") or 1939.7
             dms = kp[extra][1] / max(kp[extra][0], 1)
-            rec["roofline"] = {"kernel": extra, "bound": "alu", "achieved": ops / (dms * 1e-3) / 1e9,
-                               "peak": pk / 1e9, "unit": f"G {pipe} op/s", "ops_per_eval": round(per_eval, 4),
-                               "frac": ops / (dms * 1e-3) / pk,
+            tflops = DIRECT_FLOPS * wc.evals / (dms * 1e-3) / 1e12
+            rec["roofline"] = {"kernel": extra, "bound": "tensor", "achieved": tflops, "peak": peak_tc,
+                               "unit": "TFLOP/s", "frac": tflops / peak_tc, "flops_per_eval": DIRECT_FLOPS,
                                "traffic": ncu_traffic(extra, extra, wc.name)}
         key = f"{extra}@{wc.name}"
         forms[key] = rec
@@ -644,7 +645,7 @@ def run_ours(args):
                 "gevals_per_s": evals_all / (ms * 1e-3) / 1e9, "_samples": picked,
                 "forms": {v: sum(1 for f in forms_b if f == k) for k, v in names.items()
                           if any(f == k for f in forms_b)},
-                # one persistent launch per batch (and the memset of its counters), timed with CUDA events
+                # the batch's two streams, or its one persistent launch, timed with CUDA events
                 "kernel_ms": {k: v[1] / reps for k, v in kp.items()},
                 "gemm_tflops": flops / (ms * 1e-3) / 1e12,
                 "tensor_frac": flops / (ms * 1e-3) / 1e12 / peak_tc}
@@ -677,16 +678,12 @@ def run_ours(args):
 
     evals_all = cloud.evals * args.steps * world
     value = evals_all / (total_ms * 1e-3) / 1e9
-    props = torch.cuda.get_device_properties(local)
-    peaks = _peaks()
-    sm_max = peaks.get("sm_max_mhz") or clocks.get("sm_max_mhz") or 2070.0
+    peak = _peaks().get("bf16_tflops") or 1939.7
     if args.form.startswith("gemm"):
         # tensor-bound: 4 flop per evaluation per product (3 products for split FP16)
         dom = "gemm_tcgen05"
-        src = "gemm.cu"
         dom_launches, dom_ms = prof.get(dom, (0, 0.0))
         passes = 3 if args.form == "gemm_split16" else 1
-        peak = peaks.get("bf16_tflops") or 1939.7
         # the GEMM's K: 2 per point, or 2 per (plane, column) group when the grouped form ran; the flops of all
         # timed steps over the kernel's total time = flops per launch over the average launch (chunks included)
         grouped = "group_factors" in prof
@@ -695,24 +692,13 @@ def run_ours(args):
         roof = {"bound": "tensor", "unit": "TFLOP/s", "gemm_k": 2 * k_units,
                 "peak_basis": "measured dense bf16 burst (fp16 nominal rate is the same)"}
     else:
-        # the FMA pipe of the implemented evaluation, see direct_ops
+        # the tensor cores' part; what bounds the kernel is the making of the operands on the FMA pipe
         dom = args.form
-        src = "direct.cu"
         dom_launches, dom_ms = prof.get(dom, (0, 0.0))
-        ops, pipe, per_clk, per_eval = direct_ops(args.form, W, H, N)
-        peak = per_clk * props.multi_processor_count * sm_max * 1e6 / 1e9
-        achieved = ops / (dom_ms / max(dom_launches, 1) * 1e-3) / 1e9 if dom_ms > 0 else None
-        roof = {"bound": "alu", "unit": f"G {pipe} op/s",
-                "peak_basis": f"{per_clk} {pipe} op/clk/SM x {props.multi_processor_count} SMs x {sm_max:.0f} MHz "
-                              f"(sm_max_mhz of measured peaks); {per_eval:.4f} {pipe} op per evaluation "
-                              "(two FMAs a pixel and point, and per point the sines and cosines of the CTA's "
-                              "tile columns and rows)"}
-        if pipe == "MUFU":
-            # the same pipe measured in this run: independent hardware sines on every SM (cgh_measure_mufu)
-            from paper_1309_2734_gb300 import _lib
-            probe = _lib.cgh_measure_mufu(h.ctx) / 1e9
-            roof["peak_probe"] = probe
-            roof["frac_of_probe"] = achieved / probe if achieved else None
+        achieved = (DIRECT_FLOPS * W * H * N / (dom_ms / max(dom_launches, 1) * 1e-3) / 1e12) if dom_ms > 0 else None
+        roof = {"bound": "tensor", "unit": "TFLOP/s",
+                "peak_basis": f"measured dense bf16 burst (fp16 nominal rate is the same); {DIRECT_FLOPS} flop per "
+                              "evaluation (K = 2, three products of split FP16)"}
     traffic = ncu_traffic(dom, args.form, cloud.name)
 
     cpu, nrms = (None, None)
@@ -737,9 +723,8 @@ def run_ours(args):
         "config": {"workload": cloud.name, "width": W, "height": H, "n_points": N, "form": args.form,
                    "step": ("prep + factors + tcgen05 GEMM (+ split reduction) + quantize8"
                             if args.form.startswith("gemm") else
-                            "prep + direct kernel (equal shares of the (tile, point) pairs, each tile's parts "
-                            "summed in the kernel) + quantize8" if args.form == "direct_sfu" else
-                            "prep + direct kernel (+ chunk reduction) + quantize8"),
+                            "prep + direct kernel on the tensor cores (equal shares of the (tile, point) pairs, each "
+                            "tile's parts summed in the kernel) + quantize8"),
                    "l2": "flushed between timed steps (256 MiB write, untimed)",
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
         "holograms_per_s": args.steps * world / (total_ms * 1e-3),
@@ -749,9 +734,7 @@ def run_ours(args):
         "kernel_ms": {k: v[1] / max(v[0], 1) for k, v in prof.items()},
         "roofline": {"kernel": dom, "bound": roof["bound"], "achieved": achieved, "peak": peak,
                      "unit": roof["unit"], "frac": (achieved / peak) if achieved else None,
-                     "traffic": traffic, "peak_basis": roof["peak_basis"],
-                     **({"peak_probe": roof["peak_probe"], "frac_of_probe": roof["frac_of_probe"]}
-                        if "peak_probe" in roof else {})},
+                     "traffic": traffic, "peak_basis": roof["peak_basis"]},
         "clocks": clocks,
         "e2e": {"value": cloud.evals * args.steps * world / e2e_total / 1e9, "unit": UNIT,
                 "h2d_bytes_per_step": int(cloud.xyz.nbytes + cloud.amp.nbytes),

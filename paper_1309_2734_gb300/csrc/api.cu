@@ -29,7 +29,9 @@ int run_direct_mma(cgh_ctx *ctx, const DirectMmaLayout &lay, int planes, const c
     const size_t aux_bytes = align_up((size_t)n_pad * sizeof(uint2), 256);
     const int amp_parts = (int)((n_pad + kPrepBlock - 1) / kPrepBlock);
     const size_t amp_bytes = align_up((size_t)amp_parts * sizeof(float), 256);
-    const size_t cnt_bytes = align_up((size_t)lay.tiles * sizeof(int), 256);
+    const int launches = direct_mma_launches(lay, kDirectMmaGroup, n);
+    const int64_t n_counters = (int64_t)lay.tiles * launches;
+    const size_t cnt_bytes = align_up((size_t)n_counters * sizeof(int), 256);
     const size_t slot_bytes = (size_t)2 * lay.ctas * 128 * lay.bn * sizeof(float);
     int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, geo_bytes + aux_bytes + amp_bytes + cnt_bytes + slot_bytes);
     if (rc) return rc;
@@ -42,14 +44,13 @@ int run_direct_mma(cgh_ctx *ctx, const DirectMmaLayout &lay, int planes, const c
     {
         ProfileScope ps(ctx, "prep_points", 1);
         e = launch_prep_points(d_xyz, d_amp, (int)n, (int)n_pad, pitch, lambda, geo, aux, ctx->d_status, amax,
-                               ctx->stream, aux_mode(ctx), nullptr, 0, 0, 4, 4, nullptr, counters, lay.tiles);
+                               ctx->stream, aux_mode(ctx), nullptr, 0, 0, 4, 4, nullptr, counters, n_counters);
     }
     if (e != cudaSuccess) return cuda_status(e);
-    ProfileScope ps(ctx, name, 1);
-    return cuda_status(launch_direct_mma(lay, planes, geo, aux, amax, amp_parts, (int)n, width, height, d_out,
-                                         reinterpret_cast<float *>(reinterpret_cast<char *>(counters) + cnt_bytes), counters,
-                                         ctx->d_status,
-                                         (uint64_t)ctx->timeout_ms * 1000000ull, ctx->stream, ctx->drop_tile,
+    ProfileScope ps(ctx, name, launches);
+    float *slots = reinterpret_cast<float *>(reinterpret_cast<char *>(counters) + cnt_bytes);
+    return cuda_status(launch_direct_mma(lay, planes, geo, aux, amax, amp_parts, (int)n, width, height, d_out, slots,
+                                         counters, ctx->d_status, (uint64_t)ctx->timeout_ms * 1000000ull, ctx->stream, ctx->drop_tile,
                                          phase_ref(ctx)));
 }
 
@@ -505,7 +506,9 @@ int run_spherical(cgh_ctx *ctx, int width, int height, double pitch, double lamb
         ml[0] = choose_direct_mma(0, width, height, n, ctx->num_sms, ctx->point_split, 0);
         if (ml[0].bn > 64) ml[1] = choose_direct_mma(0, width, height, n, ctx->num_sms, ctx->point_split, 0, 64);
     }
-    const int n_tiles = std::max(ml[0].tiles, ml[1].tiles);
+    int64_t n_tiles = 0;   // counters: of every tile and launch
+    for (int v = 0; v < 2 && ml[v].bn > 0; ++v)
+        n_tiles = std::max(n_tiles, (int64_t)ml[v].tiles * direct_mma_launches(ml[v], kSphMmaGroup, n));
     const size_t zero_bytes = align_up((size_t)(2 + n_tiles) * sizeof(int), 256);   // max |A|, the bound, tile counters
     const size_t slot_bytes = (size_t)2 * 128 * std::max((int64_t)ml[0].ctas * ml[0].bn, (int64_t)ml[1].ctas * ml[1].bn) *
                               sizeof(float);
@@ -530,7 +533,7 @@ int run_spherical(cgh_ctx *ctx, int width, int height, double pitch, double lamb
     }
     if (e != cudaSuccess) return cuda_status(e);
     for (int v = 0; v < 2 && ml[v].bn > 0; ++v) {
-        ProfileScope ps(ctx, "spherical_mma", 1);
+        ProfileScope ps(ctx, "spherical_mma", direct_mma_launches(ml[v], kSphMmaGroup, n));
         e = launch_direct_mma(ml[v], 1, geo, aux, amax, 1, (int)n, width, height, d_out, parts,
                               reinterpret_cast<int *>(amax + 2), ctx->d_status,
                               (uint64_t)ctx->timeout_ms * 1000000ull, ctx->stream, -1, phase_ref(ctx), ext,

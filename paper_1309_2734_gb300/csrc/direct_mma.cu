@@ -44,6 +44,7 @@
 // A chain's MMAs run while the next stage is made; then it is folded.  Work is the flat list of (pixel tile, group of
 // 32 points) pairs in equal shares per CTA, a tile's parts summed in CTA order by the CTA that finishes last, as in the
 // balanced layout of direct.cu.
+#include <algorithm>
 #include <type_traits>
 
 #include <cuda_fp16.h>
@@ -105,6 +106,7 @@ struct MmaArgs {
     int width, height, tiles_a;
     int a_rows;                // 1: A rows are hologram rows; 0: hologram columns
     int vec, drop;
+    int add;                   // add to out: a later launch over the points
     float phase_lo, phase_hi;  // the spherical form: the bounds this launch takes
     PhaseRef ref;
 };
@@ -634,16 +636,24 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
                     if (a < g.width)
 #pragma unroll
                         for (int k = 0; k < 8; ++k)
-                            if (b0 + 4 * q + k < g.height) out[(long long)(b0 + 4 * q + k) * g.width + a] = v[k];
+                            if (b0 + 4 * q + k < g.height) {
+                                float *o = out + (long long)(b0 + 4 * q + k) * g.width + a;
+                                *o = g.add ? *o + v[k] : v[k];
+                            }
                 } else if (a < g.height) {
                     float *row = out + (long long)a * g.width + b0 + 4 * q;
                     if (g.vec && b0 + 4 * q + 8 <= g.width) {
-                        reinterpret_cast<float4 *>(row)[0] = make_float4(v[0], v[1], v[2], v[3]);
-                        reinterpret_cast<float4 *>(row)[1] = make_float4(v[4], v[5], v[6], v[7]);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            float4 *o = reinterpret_cast<float4 *>(row) + h;
+                            const float4 old = g.add ? *o : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                            *o = make_float4(old.x + v[4 * h], old.y + v[4 * h + 1], old.z + v[4 * h + 2],
+                                             old.w + v[4 * h + 3]);
+                        }
                     } else {
 #pragma unroll
                         for (int k = 0; k < 8; ++k)
-                            if (b0 + 4 * q + k < g.width) row[k] = v[k];
+                            if (b0 + 4 * q + k < g.width) row[k] = g.add ? row[k] + v[k] : v[k];
                     }
                 }
             }
@@ -756,6 +766,16 @@ cudaError_t launch_bn(int bn, const MmaArgs &g, int ctas, cudaStream_t s)
 
 }  // namespace
 
+// The totals take one FP32 addition per chain of 64 points, whose rounding grows with the square root of their number:
+// a launch adds at most kMmaLaunchPoints points of a tile in one CTA, and the next launch adds to its output
+// (2048x2048, 5 10^5 points: NRMS 4.3e-7; the SIMT kernel's 8.9e-7, one launch about 1.6e-6).
+int direct_mma_launches(const DirectMmaLayout &lay, int group, int64_t n_points)
+{
+    const int64_t groups = (n_points + group - 1) / group;
+    const int64_t share = (lay.tiles * groups + lay.ctas - 1) / lay.ctas;   // of a CTA; of a tile at most all groups
+    return (int)(((share < groups ? share : groups) * group + kMmaLaunchPoints - 1) / kMmaLaunchPoints);
+}
+
 cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4 *geo, const uint2 *aux,
                               const float *amp_max, int amp_parts, int n_points, int width, int height, float *out,
                               float *slots, int *counters, int *status, uint64_t timeout_ns, cudaStream_t s, int drop,
@@ -765,35 +785,45 @@ cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4
     if (n_points < 1 || lay.ctas < 1 || (planes != 1 && planes != 2) || (uintptr_t)slots % 16 != 0)
         return cudaErrorInvalidValue;
     MmaArgs g{};
+    const int launches = direct_mma_launches(lay, group, n_points);
+    const long long all_groups = (n_points + group - 1) / group, per = (all_groups + launches - 1) / launches;
     const int side_a = lay.a_rows ? height : width, side_b = lay.a_rows ? width : height;
     const int tb = lay.bn / planes;
     g.tiles_a = (side_a + kRowsA - 1) / kRowsA;
-    g.groups = (n_points + group - 1) / group;
-    g.units = (long long)g.tiles_a * ((side_b + tb - 1) / tb) * g.groups;
+    const long long tiles = (long long)g.tiles_a * ((side_b + tb - 1) / tb);
     // whole tiles per CTA (one share each) need neither slots nor counters
-    if (lay.ctas > g.units || g.units / lay.ctas >= 0x7ffffff0ll ||
-        (lay.ctas != g.units / g.groups && (slots == nullptr || counters == nullptr)))
+    if (tiles != lay.tiles || (lay.ctas != tiles && (slots == nullptr || counters == nullptr)))
         return cudaErrorInvalidValue;
-    g.geo = geo;
-    g.aux = aux;
-    g.ext = ext;
     g.phase_lo = phase_lo;
     g.phase_hi = phase_hi;
     g.amp_max = amp_max;
     g.amp_parts = amp_parts;
     g.out = out;
     g.slots = reinterpret_cast<float4 *>(slots);
-    g.counters = counters;
     g.status = status;
     g.timeout_ns = timeout_ns;
     g.width = width;
     g.height = height;
     g.a_rows = lay.a_rows;
     g.vec = width % 4 == 0 && (uintptr_t)out % 16 == 0 && ((long long)width * height) % 4 == 0;
-    g.drop = drop;
     g.ref = ref;
-    if (ext != nullptr) return planes == 1 ? launch_bn<1, true>(lay.bn, g, lay.ctas, s) : cudaErrorInvalidValue;
-    return planes == 2 ? launch_bn<2, false>(lay.bn, g, lay.ctas, s) : launch_bn<1, false>(lay.bn, g, lay.ctas, s);
+    if (ext != nullptr && planes != 1) return cudaErrorInvalidValue;
+    for (long long first = 0, k = 0; first < all_groups; first += per, ++k) {
+        g.groups = std::min(per, all_groups - first);
+        g.units = tiles * g.groups;
+        if (lay.ctas > g.units || g.units / lay.ctas >= 0x7ffffff0ll) return cudaErrorInvalidValue;
+        g.geo = geo + first * group;
+        g.aux = aux + first * group;
+        g.ext = ext != nullptr ? ext + first * group : nullptr;
+        g.counters = counters != nullptr ? counters + k * tiles : nullptr;
+        g.drop = k == 0 ? drop : -1;
+        g.add = k > 0;
+        const cudaError_t e = ext != nullptr ? launch_bn<1, true>(lay.bn, g, lay.ctas, s)
+                              : planes == 2  ? launch_bn<2, false>(lay.bn, g, lay.ctas, s)
+                                             : launch_bn<1, false>(lay.bn, g, lay.ctas, s);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace cgh

@@ -41,7 +41,7 @@ cudaError_t launch_prep_points(const float *d_xyz, const float *d_amp, int n, in
                                double lambda, int4 *geo, uint2 *aux, int *status, float *amp_max,
                                cudaStream_t s, int aux_x = kAuxSecondDiff, float4 *ext = nullptr, int width = 0,
                                int height = 0, int tile_cols = 4, int tile_rows = 4, float *sph_max = nullptr,
-                               int *zero = nullptr, int n_zero = 0);
+                               int *zero = nullptr, int64_t n_zero = 0);
 // points per block: the FP64 pipe bounds a block, so small ones spread a small cloud over all SMs
 constexpr int kPrepBlock = 64;
 
@@ -97,17 +97,19 @@ cudaError_t launch_direct_stream(bool sfu, const DirectShape &sh, int ctas, cons
 
 // The direct form with the tile's tables multiplied on the tensor cores (direct_mma.cu): the amplitude hologram at
 // out (planes = 1) or the complex wave, real plane then imaginary plane (planes = 2).  amp_max: max |A_j| of the
-// points, as amp_parts values (launch_prep_points).  slots: 2 ctas x 128 x bn floats (16-byte aligned); counters: one int per tile,
-// zeroed by the caller.  drop >= 0: CTA 0 never loads that group of kDirectMmaGroup points of its share (test hook).
+// points, as amp_parts values (launch_prep_points).  slots: 2 ctas x 128 x bn floats (16-byte aligned); counters: one int per tile
+// and launch (direct_mma_launches), zeroed by the caller.  drop >= 0: CTA 0 never loads that group of kDirectMmaGroup points of its share (test hook).
 // ext != nullptr: the amplitude hologram of the spherical model (points prepared with the piston, ext and its bound
 // amp_max[1]; groups of kSphMmaGroup points); the kernel returns at once unless phase_lo < amp_max[1] <= phase_hi.
 constexpr int kDirectMmaGroup = 32, kSphMmaGroup = 16;
+constexpr int64_t kMmaLaunchPoints = 20480;
 struct DirectMmaLayout {
     int bn = 0;       // B rows of a tile: 64, 128, 192, 224 (planes = 1), 256; 128 x bn / planes pixels.  0: not taken
     int a_rows = 0;   // the tile's 128-pixel side: 1 = hologram rows, 0 = columns
     int ctas = 0;
     int tiles = 0;
 };
+int direct_mma_launches(const DirectMmaLayout &lay, int group, int64_t n_points);
 cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4 *geo, const uint2 *aux,
                               const float *amp_max, int amp_parts, int n_points, int width, int height, float *out,
                               float *slots, int *counters, int *status, uint64_t timeout_ns, cudaStream_t s, int drop = -1,

@@ -19,13 +19,13 @@ __global__ void __launch_bounds__(kPrepBlock) prep_points_kernel(const float *__
                                    int n_pad, double pitch, double lambda, int4 *__restrict__ geo,
                                    uint2 *__restrict__ aux, int *status, float *amp_max, int aux_x,
                                    float4 *__restrict__ ext, int width, int height, int tile_cols, int tile_rows, float *sph_max,
-                                   int *zero, int n_zero)
+                                   int *zero, int64_t n_zero)
 {
     __shared__ float s_max;
     grid_launch_dependents();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (zero != nullptr) {   // a part of max |A| per block: no clearing pass before this kernel
-        for (int i = j; i < n_zero; i += gridDim.x * blockDim.x) zero[i] = 0;
+        for (int64_t i = j; i < n_zero; i += gridDim.x * blockDim.x) zero[i] = 0;
         if (threadIdx.x == 0) s_max = 0.0f;
         __syncthreads();
         if (j < n_pad)
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(kPrepBlock) prep_points_kernel(const float *__
 cudaError_t launch_prep_points(const float *d_xyz, const float *d_amp, int n, int n_pad, double pitch,
                                double lambda, int4 *geo, uint2 *aux, int *status, float *amp_max,
                                cudaStream_t s, int aux_x, float4 *ext, int width, int height, int tile_cols, int tile_rows, float *sph_max,
-                               int *zero, int n_zero)
+                               int *zero, int64_t n_zero)
 {
     if (n_pad <= 0) return cudaSuccess;
     const int blocks = (n_pad + kPrepBlock - 1) / kPrepBlock;

@@ -127,3 +127,14 @@ def test_largest_amplitude_in_any_block(n):
                 f = h.wave(x, a)[0] if wave else h.point_cloud(x, a)
                 h.sync()
                 assert oracle.nrms(f.cpu().numpy()[rows, cols], ref) <= TOL
+
+
+@pytest.mark.parametrize("w,h", [(130, 67), (67, 132)])
+@pytest.mark.parametrize("n", [20480, 20481, 41000])
+def test_points_beyond_one_launch(w, h, n):
+    # one CTA takes every point of a tile: beyond 20480 points a second launch adds to the first one's output
+    c = workloads.random_cloud(500 + n + w, w, h, n)
+    cols, rows, ref = _sampled(c)
+    for wave in (False, True):
+        f = _field(c, wave=wave, options=((_lib.CGH_OPT_POINT_SPLIT, 1),))
+        assert oracle.nrms((f[0] if wave else f)[rows, cols], ref) <= TOL
