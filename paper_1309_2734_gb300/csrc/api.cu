@@ -573,7 +573,7 @@ int ensure_fft(cgh_ctx *ctx)
         return rc;
     };
     if (cudaMalloc(&ctx->fft_pad, words * sizeof(float2)) != cudaSuccess ||
-        cudaMalloc(&ctx->fft_spec, (g.ok ? (size_t)g.Ly + g.Lx : words) * sizeof(float2)) != cudaSuccess)
+        cudaMalloc(&ctx->fft_spec, (g.ok ? fft_spec_words(g) : words) * sizeof(float2)) != cudaSuccess)
         return fail(CGH_ENOMEM);
     if (g.ok) {
         // e^{-2 pi i k / L} in double, rounded once
@@ -617,8 +617,7 @@ int fresnel_run(cgh_ctx *ctx, double z, const float *in, float *d_out)
         const unsigned long long C = turns_fixed64(ctx->pitch * ctx->pitch / (2.0 * ctx->lambda * z));
         if (g.ok) {
             ProfileScope ps(ctx, "fresnel_spectrum", 3);
-            e = launch_fft_chirp_spectrum(g, ctx->fft_spec, C, s * std::sin(a0), -s * std::cos(a0), ctx->fft_twx,
-                                          ctx->fft_twy, ctx->stream);
+            e = launch_fft_chirp_spectrum(g, ctx->fft_spec, C, s * std::sin(a0), -s * std::cos(a0), ctx->stream);
         } else {
             {
                 ProfileScope ps(ctx, "fresnel_chirp", 1);

@@ -364,7 +364,7 @@ __device__ __forceinline__ void cols_fft(float2 *s, int M, int nseq, int stride,
     else smem_fft<INV, kLayoutCols>(s, M, nseq, stride, tw, 1);
 }
 
-enum { kRowExpand = 0, kRowInPlace = 1, kRowCrop = 2, kRowPadRows = 3 };
+enum { kRowExpand = 0, kRowCrop = 1, kRowPadRows = 2 };
 
 // Transforms of compile-time length whose first stage reads its values from,
 // and whose last stage writes them to, an IO object instead of shared memory
@@ -505,7 +505,7 @@ struct RowIO {
                 out[plane + (long long)y * W + x] = v.y;
             }
         } else {
-            pad[(long long)y * Lx + x] = MODE == kRowInPlace ? v : cmul(v, sx[x]);
+            pad[(long long)y * Lx + x] = cmul(v, sx[x]);
         }
     }
 };
@@ -527,7 +527,6 @@ __device__ __forceinline__ bool rows_fft_direct(float2 *s, int Lx, int nseq, con
 // Row transforms: nseq rows of length Lx per CTA.
 //   kRowExpand:  rows y < H from the input planes [2][H][W] (zeros beyond W), forward, times sx, into pad;
 //   kRowPadRows: rows y < H of pad, columns < W (zeros beyond), forward, times sx, in place;
-//   kRowInPlace: rows of pad, forward, in place (a line of the chirp);
 //   kRowCrop:    rows y < H of pad, inverse, columns < W into the output planes.
 template <int MODE>
 __global__ void __launch_bounds__(1024) fft_rows_kernel(const float *__restrict__ in, float2 *__restrict__ pad, float *__restrict__ out,
@@ -543,7 +542,7 @@ __global__ void __launch_bounds__(1024) fft_rows_kernel(const float *__restrict_
         const int y = y0 + q;
         for (int x = threadIdx.x; x < Lx; x += T) {
             float2 *d = &sm[saddr<kLayoutRows>(x, q, Lx, 0)];
-            const bool live = y < rows && (MODE == kRowInPlace || MODE == kRowCrop || x < W);
+            const bool live = y < rows && (MODE == kRowCrop || x < W);
             if (!live) {
                 *d = make_float2(0.0f, 0.0f);
             } else if (MODE == kRowExpand) {
@@ -569,7 +568,7 @@ __global__ void __launch_bounds__(1024) fft_rows_kernel(const float *__restrict_
         } else {
             for (int x = threadIdx.x; x < Lx; x += T) {
                 const float2 v = sm[saddr<kLayoutRows>(x, q, Lx, 0)];
-                pad[(long long)y * Lx + x] = MODE == kRowInPlace ? v : cmul(v, sx[x]);
+                pad[(long long)y * Lx + x] = cmul(v, sx[x]);
             }
         }
     }
@@ -772,22 +771,77 @@ __global__ void __launch_bounds__(1 << (LM + LQ - 4), 1024 >> (LM + LQ - 4))
 // built or read (2048x2048: the middle column pass, 134 of 400 MB less, 73 -> 59 us; the call 206 -> 188 us).  What bounds
 // the column passes now is latency and issue: in blocks of columns that stay in L2 they were slower (198 us in two
 // blocks, 227 in four).
-// Entry l < Lx of h: the line over l; entry Lx + k: the line over k.
-__device__ __forceinline__ float2 chirp_factor(unsigned long long C, int k, int L)
+// Both lines' transforms are taken in FP64 and rounded once when z changes: in FP32 they left the result with 5.0e-7 of
+// error at 2048x2048 (the two-dimensional spectrum before: 4.8e-7), now 3.6e-7.  FP64 runs at two FMAs a clock and SM,
+// so each line is a four-step transform of plain sums over all SMs: 54 us at 2048x2048, 74 at 4096x4096 (the
+// two-dimensional FP32 spectrum 159 and 664; a radix-2 transform of one block a line about 160 at 2048x2048).
+// L = L1 L2, n = L2 n1 + n2, k = k1 + L1 k2:
+// X[k] = sum_n2 W_L2^(n2 k2) W_L^(n2 k1) sum_n1 W_L1^(n1 k1) x[n].
+constexpr int kChirpThreads = 64;
+struct ChirpLine {
+    double2 *x, *w, *y;   // the line, W_L^m, the inner sums
+    int L, L1, L2, i;     // this thread's element
+};
+
+// The line of this thread (the one over l, then the one over k) in the scratch.
+__device__ __forceinline__ bool chirp_line(double2 *work, int Lx, int Ly, ChirpLine &c)
 {
-    const long long kk = k <= L / 2 ? k : k - L;
-    const uint32_t t = (uint32_t)((C * (unsigned long long)(kk * kk)) >> 32);
-    float s, c;
-    sincospif((float)(int)t * (1.0f / 2147483648.0f), &s, &c);
-    return make_float2(c, s);
+    const int i = blockIdx.x * kChirpThreads + threadIdx.x;
+    if (i >= Lx + Ly) return false;
+    const bool first = i < Lx;
+    c.L = first ? Lx : Ly;
+    c.i = first ? i : i - Lx;
+    c.x = work + (first ? 0 : 3ll * Lx);
+    c.w = c.x + c.L;
+    c.y = c.w + c.L;
+    const int lg = 31 - __clz(c.L);
+    c.L1 = 1 << ((lg + 1) / 2);
+    c.L2 = c.L / c.L1;
+    return true;
 }
 
-__global__ void chirp_lines_kernel(float2 *__restrict__ h, int Ly, int Lx, unsigned long long C, float pre_re,
-                                   float pre_im)
+__global__ void __launch_bounds__(kChirpThreads) chirp_lines_kernel(double2 *work, int Lx, int Ly, unsigned long long C)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < Lx) h[i] = cmul(chirp_factor(C, i, Lx), make_float2(pre_re, pre_im));
-    else if (i < Lx + Ly) h[i] = chirp_factor(C, i - Lx, Ly);
+    ChirpLine c;
+    if (!chirp_line(work, Lx, Ly, c)) return;
+    const long long k = c.i <= c.L / 2 ? c.i : c.i - c.L;
+    double sn, cs;
+    sincospi((double)(long long)(C * (unsigned long long)(k * k)) * 1.0842021724855044e-19, &sn, &cs);   // 2^-63
+    c.x[c.i] = make_double2(cs, sn);
+    sincospi(-2.0 * (double)c.i / (double)c.L, &sn, &cs);
+    c.w[c.i] = make_double2(cs, sn);
+}
+
+__device__ __forceinline__ double2 dft_sum(const double2 *x, int stride, int n, const double2 *w, int step, int mask)
+{
+    double2 s = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+        const double2 a = x[(long long)j * stride], t = w[(j * step) & mask];
+        s.x += a.x * t.x - a.y * t.y;
+        s.y += a.x * t.y + a.y * t.x;
+    }
+    return s;
+}
+
+__global__ void __launch_bounds__(kChirpThreads) chirp_inner_kernel(double2 *work, int Lx, int Ly)
+{
+    ChirpLine c;
+    if (!chirp_line(work, Lx, Ly, c)) return;
+    const int n2 = c.i & (c.L2 - 1), k1 = c.i / c.L2;
+    const double2 s = dft_sum(c.x + n2, c.L2, c.L1, c.w, c.L2 * k1, c.L - 1), t = c.w[n2 * k1];
+    c.y[c.i] = make_double2(s.x * t.x - s.y * t.y, s.x * t.y + s.y * t.x);   // [k1][n2]
+}
+
+__global__ void __launch_bounds__(kChirpThreads) chirp_outer_kernel(float2 *spec, double2 *work, int Lx, int Ly,
+                                                                    double pre_re, double pre_im)
+{
+    ChirpLine c;
+    if (!chirp_line(work, Lx, Ly, c)) return;
+    const int k1 = c.i & (c.L1 - 1), k2 = c.i / c.L1;
+    const double2 s = dft_sum(c.y + k1 * c.L2, 1, c.L2, c.w, c.L1 * k2, c.L - 1);
+    if (c.x == work) spec[c.i] = make_float2((float)(s.x * pre_re - s.y * pre_im), (float)(s.x * pre_im + s.y * pre_re));
+    else spec[Lx + c.i] = make_float2((float)s.x, (float)s.y);
 }
 
 int threads_for(int work)
@@ -842,8 +896,8 @@ static cudaError_t configure_rows(size_t bytes)
     static size_t done = 0;
     if (bytes <= 48 * 1024 || bytes <= done) return cudaSuccess;
     cudaError_t e = cudaSuccess;
-    for (auto fn : {(const void *)fft_rows_kernel<kRowExpand>, (const void *)fft_rows_kernel<kRowInPlace>,
-                    (const void *)fft_rows_kernel<kRowCrop>, (const void *)fft_rows_kernel<kRowPadRows>})
+    for (auto fn : {(const void *)fft_rows_kernel<kRowExpand>, (const void *)fft_rows_kernel<kRowCrop>,
+                    (const void *)fft_rows_kernel<kRowPadRows>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess) done = bytes;
     return e;
@@ -923,17 +977,13 @@ static cudaError_t launch_cols_full(const FftGrid &g, float2 *pad, const float2 
 }
 
 cudaError_t launch_fft_chirp_spectrum(const FftGrid &g, float2 *spec, unsigned long long C, double pre_re,
-                                      double pre_im, const float2 *twx, const float2 *twy, cudaStream_t s)
+                                      double pre_im, cudaStream_t s)
 {
-    chirp_lines_kernel<<<(g.Lx + g.Ly + 255) / 256, 256, 0, s>>>(spec, g.Ly, g.Lx, C, (float)pre_re, (float)pre_im);
-    for (int line = 0; line < 2; ++line) {
-        const int L = line == 0 ? g.Lx : g.Ly, nseq = rows_per_cta(L);
-        const size_t rs = rows_smem(L, nseq);
-        const cudaError_t e = configure_rows(rs);
-        if (e != cudaSuccess) return e;
-        fft_rows_kernel<kRowInPlace><<<1, threads_for(nseq * L), rs, s>>>(nullptr, line == 0 ? spec : spec + g.Lx, nullptr,
-                                                                        0, 0, L, 1, nseq, line == 0 ? twx : twy, nullptr);
-    }
+    double2 *work = reinterpret_cast<double2 *>(spec + (g.Lx + g.Ly + 1) / 2 * 2);
+    const int blocks = (g.Lx + g.Ly + kChirpThreads - 1) / kChirpThreads;
+    chirp_lines_kernel<<<blocks, kChirpThreads, 0, s>>>(work, g.Lx, g.Ly, C);
+    chirp_inner_kernel<<<blocks, kChirpThreads, 0, s>>>(work, g.Lx, g.Ly);
+    chirp_outer_kernel<<<blocks, kChirpThreads, 0, s>>>(spec, work, g.Lx, g.Ly, pre_re, pre_im);
     return cudaGetLastError();
 }
 

@@ -195,9 +195,10 @@ struct FftGrid {
 };
 FftGrid fft_grid(int H, int W);
 // The spectrum of the chirp pre * exp(i 2 pi C (k^2 + l^2) / 2^64) on the grid as its factors: spec[0 .. Lx) over the
-// columns (with pre), spec[Lx .. Lx + Ly) over the rows.
+// columns (with pre), spec[Lx .. Lx + Ly) over the rows, then the scratch: fft_spec_words in all.
+inline size_t fft_spec_words(const FftGrid &g) { return 7 * ((size_t)g.Lx + g.Ly) + 1; }
 cudaError_t launch_fft_chirp_spectrum(const FftGrid &g, float2 *spec, unsigned long long C, double pre_re,
-                                      double pre_im, const float2 *twx, const float2 *twy, cudaStream_t s);
+                                      double pre_im, cudaStream_t s);
 // out ([2][H][W]) = crop(IFFT(FFT(input) * spec)); input = the planes in, or (in == nullptr) the rows
 // y < H, columns x < W of pad.
 cudaError_t launch_fft_convolve(const FftGrid &g, const float *in, int H, int W, float2 *pad, const float2 *spec,

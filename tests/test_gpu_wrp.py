@@ -291,3 +291,15 @@ def test_kinoform_remainders(n):
         got = hg.kinoform8(wave).flatten()
         hg.sync()
     assert torch.equal(got, want[:n])
+
+
+@pytest.mark.parametrize("w,h", [(1, 1), (1, 2), (2, 1), (3, 2), (1, 9), (5, 65), (129, 3), (257, 64)])
+def test_fresnel_spectrum_line_lengths(w, h):
+    # the chirp's lines by four-step sums: lengths 1 to 1024, odd and even powers of two, a new z per call.  Two
+    # transforms of at most 2^10 x 2^8 in FP32 leave about 20 roundings of 2^-25 (RMS) each on a path: under 5e-7
+    rng = np.random.default_rng(w * 1000 + h)
+    u = rng.standard_normal((2, h, w)).astype(np.float32)
+    with Hologram(w, h, 8e-6, 532e-9) as hol:
+        for z in (0.02, 0.3):
+            got = _cplx(hol.fresnel(torch.from_numpy(u).cuda(), z))
+            assert _nrms_c(got, oracle.fresnel(u[0].astype(np.float64) + 1j * u[1], 8e-6, 532e-9, z)) <= 1e-6
