@@ -63,14 +63,14 @@ def direct_ops(form, width, height, n_points):
 # dram__bytes_write.sum), keyed by the SHA-1 of the kernel's sources they were
 # taken on; a changed source reports null until it is profiled again.
 NCU_TRAFFIC = [
-    # profiles/direct_sfu-1920x1080-n10000.md (api.cu holds the launch's CTA count)
+    # profiles/direct_mma-1920x1080-n10000.md: 0.341 MB read + 0.008 MB written (tuner.cu picks the tile and CTAs)
     {"kernel": "direct_sfu", "form": "direct_sfu", "workload": "direct-1920x1080-n10000",
-     "src": ["direct.cu", "direct_dev.cuh", "device_util.cuh", "api.cu"],
-     "sha1": "9b424be116a5758083538cced11cb2c3dd771817", "bytes_per_launch": 365056},
-    # profiles/gemm_f16-1920x1080-n50000.md: 600.731 MB read + 3.053 MB written per launch
+     "src": ["direct_mma.cu", "half_turn.cuh", "sincospoly.h", "device_util.cuh", "tcgen05.cuh", "tuner.cu"],
+     "sha1": "ed26b1de3845b336541b4128f56a9381a2366171", "bytes_per_launch": 349184},
+    # profiles/gemm_f16-1920x1080-n50000.md: 600.757 MB read + 3.468 MB written per launch
     {"kernel": "gemm_tcgen05", "form": "gemm_f16", "workload": "gemm-1920x1080-n50000",
      "src": ["gemm.cu", "gemm_dev.cuh", "tcgen05.cuh", "device_util.cuh"],
-     "sha1": "1b3da24ffb355250d6467758d091b4a7b91d7b3a", "bytes_per_launch": 603784192},
+     "sha1": "8274f926cfd50de78410d514bc0c38633b9c90c0", "bytes_per_launch": 604224768},
 ]
 
 
@@ -435,7 +435,7 @@ def run_ours(args):
             rec["e2e_tensor_frac"] = 4.0 * wc.evals * passes / (ms * 1e-3) / 1e12 / peak_tc
         elif extra in kp:
             peak_tc = _peaks().get("bf16_tflops") or 1939.7
-            dms = kp[extra][1] / max(kp[extra][0], 1)
+            dms = kp[extra][1] / reps   # one launch per 20480 points of a tile: time per hologram
             tflops = DIRECT_FLOPS * wc.evals / (dms * 1e-3) / 1e12
             rec["roofline"] = {"kernel": extra, "bound": "tensor", "achieved": tflops, "peak": peak_tc,
                                "unit": "TFLOP/s", "frac": tflops / peak_tc, "flops_per_eval": DIRECT_FLOPS,
@@ -695,7 +695,7 @@ def run_ours(args):
         # the tensor cores' part; what bounds the kernel is the making of the operands on the FMA pipe
         dom = args.form
         dom_launches, dom_ms = prof.get(dom, (0, 0.0))
-        achieved = (DIRECT_FLOPS * W * H * N / (dom_ms / max(dom_launches, 1) * 1e-3) / 1e12) if dom_ms > 0 else None
+        achieved = (DIRECT_FLOPS * W * H * N * args.steps / (dom_ms * 1e-3) / 1e12) if dom_ms > 0 else None
         roof = {"bound": "tensor", "unit": "TFLOP/s",
                 "peak_basis": f"measured dense bf16 burst (fp16 nominal rate is the same); {DIRECT_FLOPS} flop per "
                               "evaluation (K = 2, three products of split FP16)"}

@@ -1,4 +1,4 @@
-// Device-side code of the direct form, shared by its kernels (direct.cu) and by the persistent batch kernel
+// Device-side code of the SIMT direct form, shared by its kernels (direct.cu) and by the persistent batch kernel
 // (persist.cu): the terms of one point in a thread's block of pixels and the unit of work that sums the points of a
 // range into a tile of pixels.
 //

@@ -19,13 +19,18 @@
 // cleared before: 256x256, 10^3 points with the quantiser 25.7 us (35.4 with plain launches, clears and prep blocks of
 // 256 points).
 //
-// Time, prep included (before): 1920x1080, 10^4 points 0.307 ms (1.77; 67.5 G terms/ms); its complex wave 0.485 ms
-// (3.30); 1024x1024, 10^3 points 0.046 ms (0.117); 256x256, 10^3 points 0.026 ms (0.046); the spherical hologram,
-// 1920x1080, 10^4 points at 0.3-1 m 0.66 ms (7.36; with the narrowest tile, for points at 0.2 m, 1.53).
+// Time, prep included (before): 1920x1080, 10^4 points 0.305 ms (1.77; 68 G terms/ms); its complex wave 0.480 ms
+// (3.30); 1024x1024, 10^3 points 0.042 ms (0.117); 256x256, 10^3 points 0.021 ms (0.046); the spherical hologram,
+// 1920x1080, 10^4 points at 0.3-1 m 0.643 ms (7.36; with the narrowest tile, for points at 0.2 m, 1.53).
 // What bounds it: the making of entries (0.26 of 0.31 ms with the MMAs left out), 30 instructions for two entries, 15
-// of them packed FMAs of two to three cycles, so the FMA pipe is about 80 % busy while entries are made; the tensor
-// cores are active 30 % of the time.  128 x BN tiles: larger tiles share an entry among more pixels (BN = 64 / 128 /
+// of them packed FMAs of two to three cycles, so the FMA pipe is about 80 % busy while entries are made (52 % over the
+// kernel); the tensor cores are active 36 % of the time.  128 x BN tiles: larger tiles share an entry among more pixels (BN = 64 / 128 /
 // 192 / 224: 0.66 / 0.42 / 0.34 / 0.31 ms), and two stages of 224 rows fill shared memory.
+//
+// Measured and not used: a pair of CTAs (cta_group::2) on tiles of 256 rows, half of B's entries each, 0.322 ms and the
+// wave 0.557 -- two fifths fewer entries, but then the loop of MMAs, fold and next chain (tensor memory holds one
+// accumulator beside the totals) and the cluster's round trips are as long; four warps of their own for the folds 0.306
+// and 0.563 ms (80 registers a thread, and the folds take longer than the next stage's entries).
 //
 // One CTA per SM, 18 warps.  Sixteen worker warps make the entries of a stage -- 32 points x (128 A rows + BN B rows),
 // hi and lo planes, K-major with the 128-byte swizzle -- and fold the chains; one thread of warp 16 issues the MMAs, one

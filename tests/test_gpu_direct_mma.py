@@ -138,3 +138,43 @@ def test_points_beyond_one_launch(w, h, n):
     for wave in (False, True):
         f = _field(c, wave=wave, options=((_lib.CGH_OPT_POINT_SPLIT, 1),))
         assert oracle.nrms((f[0] if wave else f)[rows, cols], ref) <= TOL
+
+
+@pytest.mark.parametrize("what", ["cloud", "accurate", "wave", "spherical", "gemm_wave", "launches"])
+def test_captured_and_replayed(what):
+    # dependent launches and the kernels' own clears inside a CUDA graph: a replay on new amplitudes gives the bits of
+    # a plain call
+    c = workloads.random_cloud(811, 300, 200, 21000 if what == "launches" else 900)
+    xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
+    form = {"accurate": "direct_accurate", "gemm_wave": "gemm_split16"}.get(what, "direct_sfu")
+    s = torch.cuda.Stream()
+    with Hologram(300, 200, c.pitch_m, c.lambda_m, form=form, stream=s) as h:
+        if what == "spherical":
+            h.set_phase_model("spherical")
+        if what == "launches":
+            h.set_option(_lib.CGH_OPT_POINT_SPLIT, 1)
+
+        def call():
+            if "wave" in what:
+                w = h.wave(xyz, amp)
+                return w, h.kinoform8(w)
+            f = h.point_cloud(xyz, amp)
+            return f, h.quantize8(f)
+        s.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(s):
+            call()
+        h.sync()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            f, q = call()
+        amp.mul_(-3.0)
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        got = f.clone(), q.clone()
+        with torch.cuda.stream(s):
+            want = call()
+        h.sync()
+        torch.cuda.synchronize()
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
