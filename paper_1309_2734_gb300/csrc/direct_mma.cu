@@ -23,7 +23,7 @@
 // (3.30); 1024x1024, 10^3 points 0.042 ms (0.117); 256x256, 10^3 points 0.021 ms (0.046); the spherical hologram,
 // 1920x1080, 10^4 points at 0.3-1 m 0.643 ms (7.36; with the narrowest tile, for points at 0.2 m, 1.53).
 // What bounds it: the making of entries (0.26 of 0.31 ms with the MMAs left out), 30 instructions for two entries, 15
-// of them packed FMAs of two to three cycles, so the FMA pipe is about 80 % busy while entries are made (52 % over the
+// of them packed FMAs of two to three cycles, so the FMA pipe is about 80 % busy while entries are made (53 % over the
 // kernel); the tensor cores are active 36 % of the time.  128 x BN tiles: larger tiles share an entry among more pixels (BN = 64 / 128 /
 // 192 / 224: 0.66 / 0.42 / 0.34 / 0.31 ms), and two stages of 224 rows fill shared memory.
 //
@@ -73,7 +73,6 @@ constexpr int kMmaThreads = kWorkers + 64;   // the workers, the MMA warp, the l
 constexpr int kRowsA = 128;
 constexpr int kGroup = kDirectMmaGroup;      // points of a stage: 64 K elements, one 128-byte swizzle row
 constexpr int kPtSlots = 4;
-constexpr int kUnroll = 2;                   // steps of a side side by side
 constexpr int kPtBytes = kGroup * (int)(sizeof(int4) + sizeof(uint2));
 constexpr int kChain = 2;                    // stages of an accumulation chain
 constexpr int kSphChain = 4;                 // spherical: stages of half as many points
@@ -211,7 +210,8 @@ __device__ __forceinline__ void side_entries(const int4 *geo, const uint2 *aux, 
         }
     }
     const float2 na = make_float2(-a.x, -a.y);
-    // U steps side by side: their chains of dependent operations overlap
+    // U steps side by side: their chains of dependent operations overlap (one plane: 1.5 % over two; two planes: as two)
+    constexpr int kUnroll = PLANES == 1 ? 4 : 2;
     auto steps = [&](auto uc, int k0) {
         constexpr int U = decltype(uc)::value;
         float2 s[U], c[U], x[U], y[U];
