@@ -66,11 +66,11 @@ NCU_TRAFFIC = [
     # profiles/direct_mma-1920x1080-n10000.md: 0.340 MB read + 0.007 MB written (tuner.cu picks the tile and CTAs)
     {"kernel": "direct_sfu", "form": "direct_sfu", "workload": "direct-1920x1080-n10000",
      "src": ["direct_mma.cu", "half_turn.cuh", "sincospoly.h", "device_util.cuh", "tcgen05.cuh", "tuner.cu"],
-     "sha1": "77c3559fbae764d01ff25a7ac70fc2eedd11afb6", "bytes_per_launch": 347392},
+     "sha1": "3dcbd9d362a6953c3166959594f5a5d04ab321bc", "bytes_per_launch": 347392},
     # profiles/gemm_f16-1920x1080-n50000.md: 600.757 MB read + 3.468 MB written per launch
     {"kernel": "gemm_tcgen05", "form": "gemm_f16", "workload": "gemm-1920x1080-n50000",
      "src": ["gemm.cu", "gemm_dev.cuh", "tcgen05.cuh", "device_util.cuh"],
-     "sha1": "8274f926cfd50de78410d514bc0c38633b9c90c0", "bytes_per_launch": 604224768},
+     "sha1": "ff92f49acbffe6a904d2ffea048dc0fce8339410", "bytes_per_launch": 604224768},
 ]
 
 

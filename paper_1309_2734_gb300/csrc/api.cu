@@ -137,6 +137,9 @@ using FactorLaunch = std::function<cudaError_t(int64_t u0, int64_t nu, void *P, 
 // 5x10^4 points: 0.428 ms without, 0.428-0.46 ms with 2-4 stages, so it is
 // off by default.)  The epilogue multiplies by *scale, the factor of Q (or
 // P) that keeps the FP16 operands within range.
+// Largest W x H x points that prep, factors, GEMM and reduction are dependent launches for (about 0.2 ms; 1920x1080,
+// 5 10^4 points, FP16: 2 % slower with them, 377 -> 383 us).
+constexpr int64_t kDependentTerms = 30000000000ll;
 // Points (K units) per factor chunk when one chunk's P and Q may take budget bytes.
 static int64_t gemm_chunk_units(int mode, int width, int height, int64_t budget)
 {
@@ -166,6 +169,8 @@ int gemm_units(cgh_ctx *ctx, int mode, int width, int height, int64_t n, const c
     plan.ctas = gemm_max_ctas(ctx->num_sms);
     const GemmLayout lay = choose_gemm_layout(width, height, nkb_max, plan.ctas, mode == kFactorSplit16,
                                               ctx->gemm_bn, ctx->gemm_splitk, ctx->gemm_trans, ctx->gemm_pair);
+    const bool dependent = (int64_t)width * height * n <= kDependentTerms;
+    plan.dependent = dependent;
     plan.pair = lay.pair;
     plan.bn = lay.bn;
     plan.splits = lay.splits;
@@ -234,7 +239,8 @@ int gemm_units(cgh_ctx *ctx, int mode, int width, int height, int64_t n, const c
     }
     if (plan.splits == 1) return CGH_OK;
     ProfileScope ps(ctx, "reduce_slices", 1);
-    return cuda_status(launch_reduce_slices(parts, plan.splits, plane, plane, d_out, ctx->stream));
+    return cuda_status(
+        launch_reduce_slices(parts, plan.splits, plane, plane, d_out, ctx->stream, nullptr, 0.0f, dependent));
 }
 
 }  // namespace cgh
@@ -384,7 +390,8 @@ int run_gemm(cgh_ctx *ctx, int form, int width, int height, double pitch, double
         }
     }
     const FactorLaunch pf = [&](int64_t u0, int64_t nu, void *P, void *Q, int64_t ld, cudaStream_t s) {
-        return launch_factors(mode, geo + u0, aux + u0, (int)nu, height, width, P, Q, ld, amax, s, ref);
+        return launch_factors(mode, geo + u0, aux + u0, (int)nu, height, width, P, Q, ld, amax, s, ref, nullptr,
+                              (int64_t)width * height * n <= kDependentTerms);
     };
     return gemm_units(ctx, mode, width, height, n, "factors", pf, amax, d_out);
 }
@@ -427,6 +434,8 @@ int run_wave(cgh_ctx *ctx, int form, const float *d_xyz, const float *d_amp, int
     if (!gemm_bn_supported(plan.bn)) return CGH_ENOTSUP;
     plan.chunk_kb = ctx->gemm_chunk > 0 ? ctx->gemm_chunk : (mode == kFactorSplit16 ? kSplit16ChunkKb : 0);
     plan.accumulate = false;
+    const bool dependent = plane * n <= kDependentTerms;
+    plan.dependent = dependent;
     const int64_t last = n - (n - 1) / chunk * chunk;
     if (plan.splits > (2 * last + 63) / 64) plan.splits = (int)((2 * last + 63) / 64);
     const size_t amax_bytes = 256;
@@ -460,7 +469,8 @@ int run_wave(cgh_ctx *ctx, int form, const float *d_xyz, const float *d_amp, int
         const int64_t ld = (2 * nc + 63) / 64 * 64;
         {
             ProfileScope ps(ctx, "factors", 1);
-            e = launch_factors(mode, geo + c0, aux + c0, (int)nc, height, width, P, Q, ld, amax, ctx->stream, ref, X);
+            e = launch_factors(mode, geo + c0, aux + c0, (int)nc, height, width, P, Q, ld, amax, ctx->stream, ref, X,
+                               dependent);
         }
         if (e != cudaSuccess) return cuda_status(e);
         GemmPlan pc = plan;
@@ -474,8 +484,9 @@ int run_wave(cgh_ctx *ctx, int form, const float *d_xyz, const float *d_amp, int
     }
     if (plan.splits == 1) return CGH_OK;
     ProfileScope ps(ctx, "reduce_slices", 2);
-    e = launch_reduce_slices(re_out, plan.splits, plane, plane, d_out, ctx->stream);
-    if (e == cudaSuccess) e = launch_reduce_slices(im_out, plan.splits, plane, plane, d_out + plane, ctx->stream);
+    e = launch_reduce_slices(re_out, plan.splits, plane, plane, d_out, ctx->stream, nullptr, 0.0f, dependent);
+    if (e == cudaSuccess)
+        e = launch_reduce_slices(im_out, plan.splits, plane, plane, d_out + plane, ctx->stream, nullptr, 0.0f, dependent);
     return cuda_status(e);
 }
 

@@ -751,7 +751,7 @@ cudaError_t launch_as(const MmaArgs &g, int ctas, cudaStream_t s)
                                     MmaCfg<BN>::kSmem);
     });
     if (e != cudaSuccess) return e;
-    return launch_dependent(direct_mma_kernel<BN, PLANES, SPH>, dim3(ctas), dim3(kMmaThreads), MmaCfg<BN>::kSmem, s, g);
+    return launch_dependent(direct_mma_kernel<BN, PLANES, SPH>, dim3(ctas), dim3(kMmaThreads), MmaCfg<BN>::kSmem, s, true, g);
 }
 
 template <int PLANES, bool SPH>

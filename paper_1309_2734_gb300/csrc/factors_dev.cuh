@@ -102,8 +102,8 @@ __device__ __forceinline__ void factor_rows_walk(int line0, int line1, const int
 // columns) on rows [r_begin, r_end) of the stacked rows (P's rows below height, then Q's rows), Q scaled by
 // scale (1 / max|A|).  DUAL: and the imaginary part's factor beside one of them, to X in that one's layout.
 template <int MODE, int DUAL>
-__device__ __forceinline__ void factor_thread(int j0, int r_begin, int r_end, const int4 *__restrict__ geo,
-                                              const uint2 *__restrict__ aux, int n_points, int height, int width,
+__device__ __forceinline__ void factor_thread(int j0, int r_begin, int r_end, const int4 *geo,
+                                              const uint2 *aux, int n_points, int height, int width,
                                               uint16_t *__restrict__ P, uint16_t *__restrict__ Q,
                                               uint16_t *__restrict__ X, long long ld, long long plane_p,
                                               long long plane_q, float scale, const PhaseRef &ref)

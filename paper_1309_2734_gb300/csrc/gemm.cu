@@ -173,6 +173,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         tmem_alloc(tmem_slot, C::kTmemCols);
         tmem_relinquish();
     }
+    grid_wait();
+    grid_launch_dependents();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -292,6 +294,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         tmem_alloc_pair(tmem_slot, C::kTmemCols);
         tmem_relinquish_pair();
     }
+    grid_wait();
+    grid_launch_dependents();
     tc_fence_before();
     cluster_sync();   // both CTAs' barriers initialised and tensor memory allocated
     tc_fence_after();
@@ -316,7 +320,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 }
 
 template <int BN>
-cudaError_t launch_pair(const PairUnits &u, int clusters, int *status, uint64_t timeout_ns, cudaStream_t s)
+cudaError_t launch_pair(const PairUnits &u, int clusters, int *status, uint64_t timeout_ns, cudaStream_t s, bool dependent)
 {
     using C = GemmPairCfg<BN>;
     static PerDeviceOnce configured;
@@ -329,13 +333,15 @@ cudaError_t launch_pair(const PairUnits &u, int clusters, int *status, uint64_t 
     cfg.blockDim = dim3(kGemmThreads, 1, 1);
     cfg.dynamicSmemBytes = C::kSmemBytes;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, gemm_pair_kernel<BN>, u, status, (unsigned long long)timeout_ns);
 }
 
@@ -366,12 +372,12 @@ cudaError_t configure()
 }
 
 template <int BN>
-cudaError_t launch_single(const SingleUnits &u, int ctas, int *status, uint64_t timeout_ns, cudaStream_t s)
+cudaError_t launch_single(const SingleUnits &u, int ctas, int *status, uint64_t timeout_ns, cudaStream_t s, bool dependent)
 {
     cudaError_t e = configure<BN, SingleUnits>();
     if (e != cudaSuccess) return e;
-    gemm_kernel<BN, SingleUnits><<<ctas, kGemmThreads, GemmCfg<BN>::kSmemBytes, s>>>(u, status, timeout_ns);
-    return cudaGetLastError();
+    return launch_dependent(gemm_kernel<BN, SingleUnits>, dim3(ctas), dim3(kGemmThreads), GemmCfg<BN>::kSmemBytes, s, dependent, u, status,
+                            (unsigned long long)timeout_ns);
 }
 
 }  // namespace
@@ -475,20 +481,20 @@ cudaError_t launch_gemm(const GemmPlan &plan, const void *P, const void *Q, int 
         const int pair_units = v.tiles_m * v.tiles_n * v.splits;
         const int clusters = std::min(plan.ctas / 2, pair_units);
         switch (bn) {
-        case 128: return launch_pair<128>(v, clusters, status, timeout_ns, s);
-        case 192: return launch_pair<192>(v, clusters, status, timeout_ns, s);
-        case 224: return launch_pair<224>(v, clusters, status, timeout_ns, s);
-        default: return launch_pair<256>(v, clusters, status, timeout_ns, s);
+        case 128: return launch_pair<128>(v, clusters, status, timeout_ns, s, plan.dependent);
+        case 192: return launch_pair<192>(v, clusters, status, timeout_ns, s, plan.dependent);
+        case 224: return launch_pair<224>(v, clusters, status, timeout_ns, s, plan.dependent);
+        default: return launch_pair<256>(v, clusters, status, timeout_ns, s, plan.dependent);
         }
     }
     const int units = u.tiles_m * u.tiles_n * u.splits;
     const int ctas = plan.ctas < units ? plan.ctas : units;
     switch (bn) {
-    case 128: return launch_single<128>(u, ctas, status, timeout_ns, s);
-    case 192: return launch_single<192>(u, ctas, status, timeout_ns, s);
-    case 224: return launch_single<224>(u, ctas, status, timeout_ns, s);
-    case 240: return launch_single<240>(u, ctas, status, timeout_ns, s);
-    default: return launch_single<256>(u, ctas, status, timeout_ns, s);
+    case 128: return launch_single<128>(u, ctas, status, timeout_ns, s, plan.dependent);
+    case 192: return launch_single<192>(u, ctas, status, timeout_ns, s, plan.dependent);
+    case 224: return launch_single<224>(u, ctas, status, timeout_ns, s, plan.dependent);
+    case 240: return launch_single<240>(u, ctas, status, timeout_ns, s, plan.dependent);
+    default: return launch_single<256>(u, ctas, status, timeout_ns, s, plan.dependent);
     }
 }
 

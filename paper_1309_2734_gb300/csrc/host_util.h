@@ -31,9 +31,9 @@ class PerDeviceOnce {
 };
 
 // Launches a kernel that calls grid_wait() before it touches memory, so that its launch and its first steps overlap the
-// kernel before it in the stream.
+// kernel before it in the stream; allow false: a plain launch.
 template <class... Params, class... Args>
-cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args)
+cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool allow, Args... args)
 {
     cudaLaunchConfig_t c = {};
     c.gridDim = grid;
@@ -42,7 +42,7 @@ cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, s
     c.stream = s;
     cudaLaunchAttribute a[1];
     a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    a[0].val.programmaticStreamSerializationAllowed = 1;
+    a[0].val.programmaticStreamSerializationAllowed = allow ? 1 : 0;
     c.attrs = a;
     c.numAttrs = 1;
     return cudaLaunchKernelEx(&c, kernel, static_cast<Params>(args)...);

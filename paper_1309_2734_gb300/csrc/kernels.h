@@ -151,7 +151,7 @@ enum { kFactorF16 = 0, kFactorBF16 = 1, kFactorSplit16 = 2 };
 // the piston (aux.x) into Q.
 cudaError_t launch_factors(int mode, const int4 *geo, const uint2 *aux, int n_points, int height, int width,
                            void *P, void *Q, int64_t ld, const float *amp_max, cudaStream_t s,
-                           const PhaseRef &ref = PhaseRef(), void *X = nullptr);
+                           const PhaseRef &ref = PhaseRef(), void *X = nullptr, bool dependent = false);
 inline bool imag_beside_p(int height, int width) { return height <= width; }
 
 // Grouped GEMM form (groups.cu, factors.cu).  Groups: points with the same
@@ -230,6 +230,7 @@ struct GemmPlan {
     int chunk_kb;      // k-blocks (of 64) per TMEM accumulation chain; 0 = whole split
     bool accumulate;   // add to the output (or partial planes) instead of overwriting
     bool trans;        // A = Q (128-row tiles of hologram columns), B = P; writes out transposed back
+    bool dependent = false;   // a dependent launch (after the factors)
     bool pair = false; // the two-SM form (clusters of two CTAs, 256-row tiles, half of B in each CTA); bn != 240
 };
 int gemm_max_ctas(int num_sms);
@@ -310,7 +311,7 @@ cudaError_t launch_persist(const PersistParams &p, int ctas, int bn_max, int *st
 
 // a5: fixed-order sum of `slices` planes of n floats (reduce.cu).
 cudaError_t launch_reduce_slices(const float *parts, int slices, int64_t n, int64_t slice_stride, float *out,
-                                 cudaStream_t s, const float *bound = nullptr, float bound_min = 0.0f);
+                                 cudaStream_t s, const float *bound = nullptr, float bound_min = 0.0f, bool dependent = false);
 
 // a6: 8-bit min/max quantiser (quantize.cu). scratch holds 2 kQuantParts uint32 (8-byte aligned).
 constexpr int kQuantParts = 2048;

@@ -181,10 +181,10 @@ cudaError_t launch_quantize8(const float *field, int64_t n, uint8_t *out, uint32
     const bool vec = ((uintptr_t)field % 16 == 0) && ((uintptr_t)out % 16 == 0);
     // 16 values a thread, so that a small field leaves few parts to the mapping blocks
     const int blocks = std::min(quant_grid(n / 16), kQuantParts);
-    cudaError_t e = launch_dependent(minmax_kernel, dim3(blocks), dim3(256), 0, s, field, (long long)n, part,
+    cudaError_t e = launch_dependent(minmax_kernel, dim3(blocks), dim3(256), 0, s, true, field, (long long)n, part,
                                      (uintptr_t)field % 16 == 0);
     if (e != cudaSuccess) return e;
-    return launch_dependent(map_kernel, dim3(quant_grid(vec ? n / 8 : n)), dim3(256), 0, s, field, (long long)n, part,
+    return launch_dependent(map_kernel, dim3(quant_grid(vec ? n / 8 : n)), dim3(256), 0, s, true, field, (long long)n, part,
                             blocks, out, vec);
 }
 

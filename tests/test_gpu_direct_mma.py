@@ -140,17 +140,23 @@ def test_points_beyond_one_launch(w, h, n):
         assert oracle.nrms((f[0] if wave else f)[rows, cols], ref) <= TOL
 
 
-@pytest.mark.parametrize("what", ["cloud", "accurate", "wave", "spherical", "gemm_wave", "launches"])
+@pytest.mark.parametrize("what", ["cloud", "accurate", "wave", "spherical", "gemm_wave", "launches", "gemm", "gemm_pair",
+                                  "gemm_chunks"])
 def test_captured_and_replayed(what):
     # dependent launches and the kernels' own clears inside a CUDA graph: a replay on new amplitudes gives the bits of
     # a plain call
     c = workloads.random_cloud(811, 300, 200, 21000 if what == "launches" else 900)
     xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
-    form = {"accurate": "direct_accurate", "gemm_wave": "gemm_split16"}.get(what, "direct_sfu")
+    form = {"accurate": "direct_accurate", "gemm_wave": "gemm_split16", "gemm": "gemm_f16", "gemm_pair": "gemm_split16",
+            "gemm_chunks": "gemm_bf16"}.get(what, "direct_sfu")
     s = torch.cuda.Stream()
     with Hologram(300, 200, c.pitch_m, c.lambda_m, form=form, stream=s) as h:
         if what == "spherical":
             h.set_phase_model("spherical")
+        if what == "gemm_pair":
+            h.set_option(_lib.CGH_OPT_GEMM_PAIR, 1)
+        if what == "gemm_chunks":
+            h.set_option(_lib.CGH_OPT_FACTOR_BUDGET_MB, 1)
         if what == "launches":
             h.set_option(_lib.CGH_OPT_POINT_SPLIT, 1)
 
