@@ -70,7 +70,7 @@ NCU_TRAFFIC = [
     # profiles/gemm_f16-1920x1080-n50000.md: 600.757 MB read + 3.468 MB written per launch
     {"kernel": "gemm_tcgen05", "form": "gemm_f16", "workload": "gemm-1920x1080-n50000",
      "src": ["gemm.cu", "gemm_dev.cuh", "tcgen05.cuh", "device_util.cuh"],
-     "sha1": "ff92f49acbffe6a904d2ffea048dc0fce8339410", "bytes_per_launch": 604224768},
+     "sha1": "43ea28564d17d32a63c9bd0dc4d6cbbcad3f1cca", "bytes_per_launch": 604224768},
 ]
 
 

@@ -335,13 +335,13 @@ cudaError_t launch_pair(const PairUnits &u, int clusters, int *status, uint64_t 
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = dependent ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, gemm_pair_kernel<BN>, u, status, (unsigned long long)timeout_ns);
 }
 

@@ -42,9 +42,9 @@ cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, s
     c.stream = s;
     cudaLaunchAttribute a[1];
     a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    a[0].val.programmaticStreamSerializationAllowed = allow ? 1 : 0;
+    a[0].val.programmaticStreamSerializationAllowed = 1;
     c.attrs = a;
-    c.numAttrs = 1;
+    c.numAttrs = allow ? 1 : 0;
     return cudaLaunchKernelEx(&c, kernel, static_cast<Params>(args)...);
 }
 
