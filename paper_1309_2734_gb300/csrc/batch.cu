@@ -111,9 +111,9 @@ struct Layout {
 constexpr int kSplit16ChunkKbBatch = 16;   // divides a factor group's 32 k-blocks (see kSplit16ChunkKb, api.cu)
 
 // Form (and, for the GEMM forms, tile width) of every instance: the context's form, or the autotuner's choice.
-// forced > 0: that form for every instance.
+// forced > 0: that form for every instance; single: for the single-hologram forms of the lanes.
 void choose_forms(cgh_ctx *ctx, const cgh_instance *inst, int n, BatchPlan *plan, std::vector<int> &bn,
-                  int forced = 0)
+                  int forced = 0, bool single = false)
 {
     const double tol = (double)ctx->tol_e9 * 1e-9;
     plan->forms.assign(n, CGH_DIRECT_SFU);
@@ -123,7 +123,7 @@ void choose_forms(cgh_ctx *ctx, const cgh_instance *inst, int n, BatchPlan *plan
         const int f = forced > 0 ? forced
                       : ctx->form != CGH_FORM_AUTO
                           ? ctx->form
-                          : tune_choose_form(ctx, inst[i].width, inst[i].height, inst[i].n_points, tol);
+                          : tune_choose_form(ctx, inst[i].width, inst[i].height, inst[i].n_points, tol, !single);
         plan->forms[i] = f;
         if (f >= CGH_GEMM_F16)
             bn[i] = ctx->gemm_bn > 0 ? ctx->gemm_bn
@@ -824,7 +824,7 @@ int run_batch(cgh_ctx *ctx, const cgh_instance *inst, int n)
     BatchPlan *plan = ctx->batch;
     if (lanes_serve(ctx, inst, n)) {
         std::vector<int> bn;
-        choose_forms(ctx, inst, n, plan, bn);
+        choose_forms(ctx, inst, n, plan, bn, 0, true);
         plan->key.clear();   // the forms are this batch's now
         ProfileScope ps(ctx, "batch_lanes", 1);
         return run_batch_lanes(ctx, inst, n, plan->forms);

@@ -536,7 +536,11 @@ double tune_predict(cgh_ctx *ctx, int form, int width, int height, int64_t n)
     return c[0] + c[1] * (double)width * height * (double)n + c[2] * (double)(width + height) * (double)n;
 }
 
-int tune_choose_form(cgh_ctx *ctx, int width, int height, int64_t n, double tol)
+// The persistent launch and the per-kind launches run direct units on the SIMT kernel, which the single hologram's times
+// say nothing about: there a GEMM form is taken wherever one is admissible.  Persistent launch, direct / split FP16:
+// 64 x 512x512, 2000 points 7386 / 539 us; 8 x 1920x1080, 100 points 424 / 90; 16 x 64x64, 100 points 42 / 33; the
+// direct form was ahead by 3 % at most (256 x 64x64, 100 points 287 / 295).
+int tune_choose_form(cgh_ctx *ctx, int width, int height, int64_t n, double tol, bool batch)
 {
     if (tune_calibrate(ctx, false) != CGH_OK) return CGH_DIRECT_SFU;
     const int forms[5] = {CGH_DIRECT_SFU, CGH_DIRECT_ACCURATE, CGH_GEMM_F16, CGH_GEMM_BF16, CGH_GEMM_SPLIT16};
@@ -544,6 +548,7 @@ int tune_choose_form(cgh_ctx *ctx, int width, int height, int64_t n, double tol)
     double best_t = 1e300;
     for (int f : forms) {
         if (form_nrms_bound(f) > tol) continue;
+        if (batch && f < CGH_GEMM_F16 && tol >= form_nrms_bound(CGH_GEMM_SPLIT16)) continue;
         const double tp = tune_predict(ctx, f, width, height, n);
         if (tp < best_t) {
             best_t = tp;

@@ -204,6 +204,25 @@ def test_autotuned_batch_meets_tolerance(tol_e9, allowed):
     _check_all(clouds, outs, tol_e9 * 1e-9)
 
 
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("tol_e9,allowed", [(10000, {_lib.CGH_GEMM_SPLIT16}), (2_000_000, {_lib.CGH_GEMM_SPLIT16, _lib.CGH_GEMM_F16}),
+                                            (3000, {_lib.CGH_DIRECT_ACCURATE})])
+def test_auto_in_a_small_batch_takes_the_gemm_forms(tol_e9, allowed, mode):
+    # below 10^11 terms direct units run on the SIMT kernel, up to twenty times slower than the GEMM: they serve only
+    # where no GEMM form is accurate enough
+    clouds = [workloads.random_cloud(720 + i, w, h, n) for i, (w, h, n) in
+              enumerate([(512, 512, 2000), (256, 256, 1024), (64, 64, 100), (1920, 1080, 100)])]
+    dev = _dev(clouds)
+    outs = [torch.zeros((c.height, c.width), device="cuda") for c in clouds]
+    with Hologram(8, 8, 8e-6, 532e-9, form="auto") as h:
+        h.set_option(_lib.CGH_OPT_TOLERANCE_E9, tol_e9)
+        h.set_option(_lib.CGH_OPT_BATCH_MODE, mode)
+        batch(h, dev, outs)
+        h.sync()
+        assert set(_lib.cgh_batch_forms(h.ctx)) <= allowed
+    _check_all(clouds, outs, tol_e9 * 1e-9)
+
+
 def test_auto_single_hologram_meets_tolerance():
     c = workloads.random_cloud(710, 640, 360, 6000)
     xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
