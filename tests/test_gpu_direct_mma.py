@@ -140,6 +140,15 @@ def test_points_beyond_one_launch(w, h, n):
         assert oracle.nrms((f[0] if wave else f)[rows, cols], ref) <= TOL
 
 
+def test_launches_share_the_points_evenly():
+    # 12 tiles of 480,943 groups on 13 CTAs: 694 launches, none with fewer groups than the CTAs need.  To the tolerance
+    # above come the launches' additions to the output, sqrt(694 / 2) 2^-25 = 5.6e-7
+    c = workloads.random_cloud(611, 384, 896, 15390145)
+    cols, rows, ref = _sampled(c, 24)
+    got = _field(c, options=[(_lib.CGH_OPT_DIRECT_CTAS, 13)])
+    assert oracle.nrms(got[rows, cols], ref) <= TOL + 6e-7
+
+
 @pytest.mark.parametrize("what", ["cloud", "accurate", "wave", "spherical", "gemm_wave", "launches", "gemm", "gemm_pair",
                                   "gemm_chunks"])
 def test_captured_and_replayed(what):
