@@ -128,7 +128,8 @@ enum {
                                    schedules those beyond the resident ones as others finish) */
     CGH_OPT_BATCH_MODE = 15,    /* cgh_batch: 0 = default: a batch of 10^11 terms (width x height x points) or more
                                    hologram by hologram on two streams of the context's own (not under stream
-                                   capture, nor with another batch option, GEMM_BN or GEMM_CHUNK set); else one
+                                   capture, nor with another batch option, GEMM_BN, GEMM_CHUNK or
+                                   GEMM_TRANSPOSE set); else one
                                    persistent launch for the whole batch (GEMM units on the tensor cores beside
                                    point preparation, factor generation and direct units on the same SMs); 1 =
                                    per-kind launches (preparation and factors per instance,

@@ -768,13 +768,15 @@ void destroy_batch_lanes(BatchLanes *L)
 // launches of many small holograms cost more than that gains.  12 frames of 10^3 to 10^5 points, split FP16: 9.9 ms
 // against 10.7 (FP16 3.5 against 3.8; one stream 9.7 but 3.65, three 9.9); 6 frames of 3 10^3 to 3 10^4 points (1.7
 // 10^11 terms) 1.48 against 1.68 (FP16 0.56 against 0.64); 4 small ones (4 10^10 terms) 0.41 against 0.44 (FP16 0.181
-// against 0.171).  Not under capture (the forms grow their workspaces), nor with options of the other modes.
+// against 0.171).  Not under capture (the forms grow their workspaces), nor with options of the other
+// modes, a pinned tile width, chain or orientation among them.
 constexpr double kLanesEvals = 1e11;
 
 static bool lanes_serve(const cgh_ctx *ctx, const cgh_instance *inst, int n)
 {
     if (ctx->batch_mode != 0 || ctx->batch_overlap != 1 || ctx->batch_chunk_mb != 0 || ctx->batch_premade_pct >= 0 ||
-        ctx->drop_tile >= 0 || ctx->test_alloc_fail > 0 || ctx->gemm_bn != 0 || ctx->gemm_chunk != 0)
+        ctx->drop_tile >= 0 || ctx->test_alloc_fail > 0 || ctx->gemm_bn != 0 || ctx->gemm_chunk != 0 ||
+        ctx->gemm_trans != 0)
         return false;
     double evals = 0.0;
     for (int i = 0; i < n; ++i) evals += (double)inst[i].width * inst[i].height * (double)inst[i].n_points;

@@ -292,3 +292,24 @@ def test_large_batch_on_streams(form):
             with pytest.raises(CghError) as ei:
                 h.sync()
             assert ei.value.code == _lib.CGH_EINPUT
+
+
+@pytest.mark.parametrize("option,value", [(None, 0), (_lib.CGH_OPT_GEMM_TRANSPOSE, 1), (_lib.CGH_OPT_GEMM_TRANSPOSE, 2),
+                                          (_lib.CGH_OPT_GEMM_BN, 192), (_lib.CGH_OPT_GEMM_CHUNK, 8)])
+def test_large_batch_honours_pinned_tiles(option, value):
+    # a pinned orientation, tile width or chain is the persistent launch's; without one 10^11 terms run on the streams
+    clouds = [workloads.random_cloud(940 + i, 1283, 717, 60001) for i in range(2)]
+    dev = _dev(clouds)
+    outs = [torch.empty((c.height, c.width), device="cuda") for c in clouds]
+    with Hologram(8, 8, 8e-6, 532e-9, form="gemm_f16") as h:
+        if option is not None:
+            h.set_option(option, value)
+        h.profile()
+        batch(h, dev, outs)
+        h.sync()
+        assert set(h.profile_read()) == ({"batch_lanes"} if option is None else {"batch_persist"})
+    rng = np.random.default_rng(94)
+    for c, o in zip(clouds, outs):
+        cols, rows = rng.integers(0, c.width, 64), rng.integers(0, c.height, 64)
+        ref = oracle.field_at(c.pitch_m, c.lambda_m, c.xyz, c.amp, cols, rows)
+        assert oracle.nrms(o.cpu().numpy()[rows, cols], ref) <= NRMS["gemm_f16"]
