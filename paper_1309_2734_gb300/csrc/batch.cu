@@ -125,7 +125,7 @@ void choose_forms(cgh_ctx *ctx, const cgh_instance *inst, int n, BatchPlan *plan
                           ? ctx->form
                           : tune_choose_form(ctx, inst[i].width, inst[i].height, inst[i].n_points, tol, !single);
         plan->forms[i] = f;
-        if (f >= CGH_GEMM_F16)
+        if (f >= CGH_GEMM_F16 && !single)   // the single-hologram forms choose their own tiles
             bn[i] = ctx->gemm_bn > 0 ? ctx->gemm_bn
                                      : (ctx->form == CGH_FORM_AUTO ? tune_choose_bn(ctx, inst[i].width, inst[i].height, f)
                                                                    : choose_gemm_bn(inst[i].width));

@@ -313,3 +313,18 @@ def test_large_batch_honours_pinned_tiles(option, value):
         cols, rows = rng.integers(0, c.width, 64), rng.integers(0, c.height, 64)
         ref = oracle.field_at(c.pitch_m, c.lambda_m, c.xyz, c.amp, cols, rows)
         assert oracle.nrms(o.cpu().numpy()[rows, cols], ref) <= NRMS["gemm_f16"]
+
+
+def test_large_auto_batch_measures_no_tile_widths(tmp_path, monkeypatch):
+    # the streams' forms choose their tiles by the time model: no shape's five widths are timed (with a wait
+    # each) for a batch that does not use them
+    cache = tmp_path / "tune.json"
+    monkeypatch.setenv("CGH_TUNE_CACHE", str(cache))
+    clouds = [workloads.random_cloud(950 + i, 1280, 720, 60000) for i in range(2)]
+    dev = _dev(clouds)
+    outs = [torch.empty((c.height, c.width), device="cuda") for c in clouds]
+    with Hologram(8, 8, 8e-6, 532e-9, form="auto") as h:
+        batch(h, dev, outs)
+        h.sync()
+        assert set(_lib.cgh_batch_forms(h.ctx)) <= {_lib.CGH_GEMM_SPLIT16, _lib.CGH_DIRECT_SFU, _lib.CGH_DIRECT_ACCURATE}
+    assert '"bn": {}' in cache.read_text()
