@@ -34,7 +34,7 @@ int run_direct_mma(cgh_ctx *ctx, const DirectMmaLayout &lay, int planes, const c
     const size_t cnt_bytes = align_up((size_t)n_counters * sizeof(int), 256);
     const size_t slot_bytes = (size_t)2 * lay.ctas * 128 * lay.bn * sizeof(float);
     int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, geo_bytes + aux_bytes + amp_bytes + cnt_bytes + slot_bytes);
-    if (rc) return rc;
+    if (rc || ctx->reserve_only) return rc;
     char *base = static_cast<char *>(ctx->ws);
     int4 *geo = reinterpret_cast<int4 *>(base);
     uint2 *aux = reinterpret_cast<uint2 *>(base + geo_bytes);
@@ -188,7 +188,7 @@ int gemm_units(cgh_ctx *ctx, int mode, int width, int height, int64_t n, const c
     const size_t q_bytes = align_up((size_t)planes * width * ld_max * 2, 256);
     const size_t part_bytes = plan.splits > 1 ? (size_t)plan.splits * plane * sizeof(float) : 0;
     int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, nbuf * (p_bytes + q_bytes) + part_bytes);
-    if (rc) return rc;
+    if (rc || ctx->reserve_only) return rc;
     char *fac = static_cast<char *>(ctx->ws);
     float *parts = reinterpret_cast<float *>(fac + nbuf * (p_bytes + q_bytes));
     cudaError_t e;
@@ -346,6 +346,11 @@ int run_gemm(cgh_ctx *ctx, int form, int width, int height, double pitch, double
     char *gscratch = base + geo_bytes + aux_bytes + meta_bytes;
     int4 *groups = reinterpret_cast<int4 *>(gscratch + gscratch_bytes);
     int2 *members = reinterpret_cast<int2 *>(gscratch + gscratch_bytes + groups_bytes);
+    const FactorLaunch pf = [&](int64_t u0, int64_t nu, void *P, void *Q, int64_t ld, cudaStream_t s) {
+        return launch_factors(mode, geo + u0, aux + u0, (int)nu, height, width, P, Q, ld, amax, s, ref, nullptr,
+                              (int64_t)width * height * n <= kDependentTerms);
+    };
+    if (ctx->reserve_only) return gemm_units(ctx, mode, width, height, n, "factors", pf, amax, d_out);
     cudaError_t e = cudaMemsetAsync(amax, 0, sizeof(float), ctx->stream);
     if (e != cudaSuccess) return cuda_status(e);
     {
@@ -389,10 +394,6 @@ int run_gemm(cgh_ctx *ctx, int form, int width, int height, double pitch, double
             }
         }
     }
-    const FactorLaunch pf = [&](int64_t u0, int64_t nu, void *P, void *Q, int64_t ld, cudaStream_t s) {
-        return launch_factors(mode, geo + u0, aux + u0, (int)nu, height, width, P, Q, ld, amax, s, ref, nullptr,
-                              (int64_t)width * height * n <= kDependentTerms);
-    };
     return gemm_units(ctx, mode, width, height, n, "factors", pf, amax, d_out);
 }
 

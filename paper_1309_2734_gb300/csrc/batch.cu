@@ -775,8 +775,7 @@ constexpr double kLanesEvals = 1e11;
 static bool lanes_serve(const cgh_ctx *ctx, const cgh_instance *inst, int n)
 {
     if (ctx->batch_mode != 0 || ctx->batch_overlap != 1 || ctx->batch_chunk_mb != 0 || ctx->batch_premade_pct >= 0 ||
-        ctx->drop_tile >= 0 || ctx->test_alloc_fail > 0 || ctx->gemm_bn != 0 || ctx->gemm_chunk != 0 ||
-        ctx->gemm_trans != 0)
+        ctx->drop_tile >= 0 || ctx->gemm_bn != 0 || ctx->gemm_chunk != 0 || ctx->gemm_trans != 0)
         return false;
     double evals = 0.0;
     for (int i = 0; i < n; ++i) evals += (double)inst[i].width * inst[i].height * (double)inst[i].n_points;
@@ -799,19 +798,31 @@ static int run_batch_lanes(cgh_ctx *ctx, const cgh_instance *inst, int n, const 
     for (int i = 0; i < n; ++i) order[i] = i;
     auto work = [&](int i) { return (double)inst[i].width * inst[i].height * (double)inst[i].n_points; };
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work(a) > work(b); });
-    cudaError_t e = cudaEventRecord(L.start, ctx->stream);
-    for (int k = 0; k < count && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(L.lane[k]->stream, L.start, 0);
-    if (e != cudaSuccess) return cuda_status(e);
-    int rc = CGH_OK;
-    for (int j = 0; j < n && rc == CGH_OK; ++j) {
+    auto run = [&](int j) {
         const cgh_instance &I = inst[order[j]];
         cgh_ctx *c = L.lane[j % count];
         c->timeout_ms = ctx->timeout_ms;
         c->factor_budget_mb = ctx->factor_budget_mb;
         c->form = forms[order[j]];
         c->gemm_group = 1;   // as in the other modes
-        rc = compute_hologram(c, I.width, I.height, I.pitch_m, I.lambda_m, I.d_xyz, I.d_amp, I.n_points, I.d_out);
+        return compute_hologram(c, I.width, I.height, I.pitch_m, I.lambda_m, I.d_xyz, I.d_amp, I.n_points, I.d_out);
+    };
+    // every workspace before the first launch: a growth that fails leaves all outputs as they were
+    for (int j = 0; j < n && inst[order[j]].n_points > 0; ++j) {
+        cgh_ctx *c = L.lane[j % count];
+        c->test_alloc_fail = ctx->test_alloc_fail;
+        c->reserve_only = true;
+        const int rc = run(j);
+        c->reserve_only = false;
+        ctx->test_alloc_fail = c->test_alloc_fail;
+        c->test_alloc_fail = 0;
+        if (rc != CGH_OK) return rc;
     }
+    cudaError_t e = cudaEventRecord(L.start, ctx->stream);
+    for (int k = 0; k < count && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(L.lane[k]->stream, L.start, 0);
+    if (e != cudaSuccess) return cuda_status(e);
+    int rc = CGH_OK;
+    for (int j = 0; j < n && rc == CGH_OK; ++j) rc = run(j);
     // the context's stream goes on after every lane, also after a failure
     for (int k = 0; k < count; ++k) {
         if (e == cudaSuccess) e = cudaEventRecord(L.done[k], L.lane[k]->stream);

@@ -39,6 +39,7 @@ struct cgh_ctx {
     int direct_ctas = 0;      // CGH_OPT_DIRECT_CTAS
     int direct_shape = 0;     // CGH_OPT_DIRECT_SHAPE
     int test_alloc_fail = 0;  // CGH_OPT_TEST_ALLOC_FAIL: workspace growths still to refuse
+    bool reserve_only = false;   // a batch's lane: the forms grow their workspaces and return before any launch
     int batch_mode = 0;       // CGH_OPT_BATCH_MODE
     int batch_overlap = 1;    // CGH_OPT_BATCH_OVERLAP
     int gemm_splitk = 0;

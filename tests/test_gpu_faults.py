@@ -122,3 +122,34 @@ def test_refused_batch_arena_then_recovery():
     for c, o in zip(clouds, outs):
         ref = oracle.field(c.pitch_m, c.lambda_m, c.xyz, c.amp, c.width, c.height)
         assert oracle.nrms(o.cpu().numpy(), ref) <= 1e-5
+
+
+@pytest.mark.parametrize("form", ["direct_sfu", "gemm_split16"])
+def test_refused_growth_of_a_large_batch_leaves_every_output(form):
+    """A large batch (two streams) whose second hologram needs more workspace than the batch before: the growth is refused,
+    CGH_ENOMEM, and no output is written, that of the hologram with enough workspace neither."""
+    def make(second):
+        clouds = [workloads.random_cloud(914, 1920, 1080, 60000), workloads.random_cloud(915, 200, 150, second)]
+        dev = [(torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda(), c.width, c.height, c.pitch_m,
+                c.lambda_m) for c in clouds]
+        return clouds, dev, [torch.full((c.height, c.width), 7.0, device="cuda") for c in clouds]
+    with Hologram(8, 8, 8e-6, 532e-9, form=form) as h:
+        _, dev, outs = make(1000)
+        batch(h, dev, outs)
+        h.sync()
+        clouds, dev, outs = make(3000000 if form == "direct_sfu" else 300000)
+        h.set_option(_lib.CGH_OPT_TEST_ALLOC_FAIL, 1)
+        with pytest.raises(CghError) as ei:
+            batch(h, dev, outs)
+        assert ei.value.code == _lib.CGH_ENOMEM
+        h.sync()
+        torch.cuda.synchronize()
+        for o in outs:
+            assert bool((o == 7.0).all())
+        batch(h, dev, outs)
+        h.sync()
+    rng = np.random.default_rng(9)
+    for c, o in zip(clouds, outs):
+        cols, rows = rng.integers(0, c.width, 32), rng.integers(0, c.height, 32)
+        ref = oracle.field_at(c.pitch_m, c.lambda_m, c.xyz, c.amp, cols, rows)
+        assert oracle.nrms(o.cpu().numpy()[rows, cols], ref) <= 1e-5
