@@ -262,7 +262,7 @@ struct TuneState {
     bool calibrated = false;
     double coef[kForms][3] = {};   // seconds: c0, per W*H*N, per (W+H)*N
     std::map<std::string, int> bn;
-    std::string device;
+    std::string device;   // tune_key
 };
 
 void destroy_tune_state(TuneState *t)
@@ -272,14 +272,21 @@ void destroy_tune_state(TuneState *t)
 
 namespace {
 
-std::string device_name(int dev)
+// Revision of what the cached coefficients describe, part of the key a cache is accepted by: counted up with the kernels
+// that a form runs (2: the direct forms on the tensor cores, six times faster than what files without a revision
+// describe).
+constexpr int kTuneRevision = 2;
+
+// The device and the revision, as the cache names them.
+std::string tune_key(int dev)
 {
+    const std::string rev = ":r" + std::to_string(kTuneRevision);
     cudaDeviceProp p;
     if (cudaGetDeviceProperties(&p, dev) != cudaSuccess) {
         cudaGetLastError();
-        return "unknown";
+        return "unknown" + rev;
     }
-    return std::string(p.name) + ":" + std::to_string(p.multiProcessorCount);
+    return std::string(p.name) + ":" + std::to_string(p.multiProcessorCount) + rev;
 }
 
 const char *cache_path()
@@ -307,7 +314,7 @@ void save_cache(const TuneState &t)
     std::fclose(f);
 }
 
-// Parses a cache written by save_cache: accepted only when it names this device and ABI and every one of the
+// Parses a cache written by save_cache: accepted only when it names this device (with the revision of its kernels, tune_key) and ABI and every one of the
 // kForms x 3 coefficients is finite and not negative (they are seconds, and seconds per evaluation); anything
 // else -- a truncated or edited file, another device, another ABI -- is refused as a whole and the tuner
 // calibrates instead.  Tile widths that the GEMM does not support are skipped.
@@ -495,7 +502,7 @@ TuneState *state(cgh_ctx *ctx)
 {
     if (!ctx->tune) {
         ctx->tune = new TuneState();
-        ctx->tune->device = device_name(ctx->device);
+        ctx->tune->device = tune_key(ctx->device);
         load_cache(*ctx->tune);
     }
     return ctx->tune;

@@ -88,6 +88,22 @@ def test_damaged_cache_is_recalibrated(cache, damage):
     _auto_hologram_ok()
 
 
+@pytest.mark.parametrize("revision", ["", ":r1", ":r999"])
+def test_cache_of_other_kernels_is_recalibrated(cache, revision):
+    """Coefficients measured on other kernels (a file without the revision, or with another one) are refused."""
+    with Hologram(8, 8, 8e-6, 532e-9, form="auto") as h:
+        _lib.check(_lib.cgh_autotune(h.ctx, 1), "cgh_autotune")
+    device = _device_of(cache)
+    name, sms = device.split(":")[:2]
+    rows = ", ".join("[1.0e-06, 8.6e-14, 0.0e+00]" for _ in range(6))
+    old = '{\n "abi": 1,\n "device": "%s:%s%s",\n "coef": [%s],\n "bn": {}\n}\n' % (name, sms, revision, rows)
+    cache.write_text(old)
+    with Hologram(8, 8, 8e-6, 532e-9, form="auto") as h:
+        _lib.check(_lib.cgh_autotune(h.ctx, 0), "cgh_autotune")
+    assert cache.read_text() != old
+    assert _lib.cgh_tune_cache_check(str(cache), device)
+
+
 @pytest.mark.parametrize("form", ["direct_sfu", "gemm_split16"])
 def test_refused_allocation_then_recovery(form):
     """The first workspace growth is refused (as a failed cudaMalloc): CGH_ENOMEM, nothing launched; the same
