@@ -140,8 +140,7 @@ using FactorLaunch = std::function<cudaError_t(int64_t u0, int64_t nu, void *P, 
 // Largest W x H x points that prep, factors, GEMM and reduction are dependent launches for (about 0.2 ms; 1920x1080,
 // 5 10^4 points, FP16: 2 % slower with them, 377 -> 383 us).
 constexpr int64_t kDependentTerms = 30000000000ll;
-// Points (K units) per factor chunk when one chunk's P and Q may take budget bytes.
-static int64_t gemm_chunk_units(int mode, int width, int height, int64_t budget)
+int64_t gemm_chunk_units(int mode, int width, int height, int64_t budget)
 {
     const int planes = mode == kFactorSplit16 ? 2 : 1;
     const int64_t bytes_per_unit = (int64_t)planes * (width + height) * 2 * 2;

@@ -108,6 +108,7 @@ struct DirectMmaLayout {
     int a_rows = 0;   // the tile's 128-pixel side: 1 = hologram rows, 0 = columns
     int ctas = 0;
     int tiles = 0;
+    double us = 0.0;  // predicted time of the launches
 };
 int direct_mma_launches(const DirectMmaLayout &lay, int group, int64_t n_points);
 cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4 *geo, const uint2 *aux,

@@ -7,8 +7,9 @@
 //   choose_gemm_splits  K splits of the GEMM, to balance tiles over the CTAs.
 //
 // Measured rules (a context, outside any stream capture):
-//   tune_calibrate      times every form on three synthetic clouds on this
-//                       device and fits, per form, t = c0 + c1 W H N + c2 (W + H) N;
+//   tune_calibrate      times every form on seven synthetic clouds on this
+//                       device and fits, per form, the scale of its kernel's
+//                       time model and what that leaves out (form_terms);
 //   tune_choose_form    the fastest form whose stated NRMS bound is within the
 //                       requested tolerance, by that model;
 //   tune_choose_bn      the fastest GEMM tile width for a hologram shape and
@@ -18,6 +19,7 @@
 #include "tuner.h"
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -125,6 +127,7 @@ DirectMmaLayout choose_direct_mma(int planes, int width, int height, int64_t n_p
                 best.a_rows = a_rows;
                 best.tiles = (int)tiles;
                 best.ctas = (int)n;
+                best.us = t;
             };
             if (split > 0) {
                 const int64_t s = std::min<int64_t>(split, groups), n = tiles * s;
@@ -184,7 +187,7 @@ constexpr double kReduceBytesPerUs = 3.0e6;
 GemmLayout choose_gemm_layout(int width, int height, int64_t k_blocks, int ctas, bool split_form, int force_bn,
                               int force_splits, int force_trans, int force_pair)
 {
-    GemmLayout best{false, 256, 1, false};
+    GemmLayout best{false, 256, 1, false, 0.0};
     double best_t = 1e300;
     for (int pair = 0; pair < 2; ++pair) {
         if ((force_pair == 1 && !pair) || (force_pair == 2 && pair)) continue;   // 1: always, 2: never
@@ -214,7 +217,7 @@ GemmLayout choose_gemm_layout(int width, int height, int64_t k_blocks, int ctas,
                     if (tr) t *= 0.995;
                     if (t < best_t * (1.0 - 1e-9)) {
                         best_t = t;
-                        best = GemmLayout{tr != 0, bn, (int)s, pair != 0};
+                        best = GemmLayout{tr != 0, bn, (int)s, pair != 0, t};
                     }
                 }
             }
@@ -260,7 +263,20 @@ double form_nrms_bound(int form)
 
 struct TuneState {
     bool calibrated = false;
-    double coef[kForms][3] = {};   // seconds: c0, per W*H*N, per (W+H)*N
+    double coef[kForms][3] = {};   // seconds: c0, then the factors of form_terms
+    struct Choice {
+        int width = 0, height = 0;
+        int64_t n = 0;
+        double tol = 0.0;
+        int64_t budget_mb = 0;
+        bool batch = false;
+        int form = 0;
+        bool same(const Choice &o) const
+        {
+            return width == o.width && height == o.height && n == o.n && tol == o.tol && budget_mb == o.budget_mb &&
+                   batch == o.batch;
+        }
+    } last;   // the choice of the call before: a program's holograms are mostly of one size
     std::map<std::string, int> bn;
     std::string device;   // tune_key
 };
@@ -274,8 +290,8 @@ namespace {
 
 // Revision of what the cached coefficients describe, part of the key a cache is accepted by: counted up with the kernels
 // that a form runs (2: the direct forms on the tensor cores, six times faster than what files without a revision
-// describe).
-constexpr int kTuneRevision = 2;
+// describe; 3: coefficients of the kernels' time models).
+constexpr int kTuneRevision = 3;
 
 // The device and the revision, as the cache names them.
 std::string tune_key(int dev)
@@ -401,30 +417,38 @@ void synth_points(int width, int height, int64_t n, std::vector<float> &xyz, std
     }
 }
 
-struct Scratch {
+// A synthetic cloud and its hologram on the device.
+struct Synth {
+    int width, height;
+    int64_t n;
     float *xyz = nullptr, *amp = nullptr, *out = nullptr;
-    ~Scratch()
+    bool ok = false;
+    Synth(int width, int height, int64_t n) : width(width), height(height), n(n)
+    {
+        std::vector<float> hx, ha;
+        synth_points(width, height, n, hx, ha);
+        ok = cudaMalloc(&xyz, hx.size() * sizeof(float)) == cudaSuccess &&
+             cudaMalloc(&amp, ha.size() * sizeof(float)) == cudaSuccess &&
+             cudaMalloc(&out, (size_t)width * height * sizeof(float)) == cudaSuccess &&
+             cudaMemcpy(xyz, hx.data(), hx.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
+             cudaMemcpy(amp, ha.data(), ha.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
+        if (!ok) cudaGetLastError();
+    }
+    ~Synth()
     {
         if (xyz) cudaFree(xyz);
         if (amp) cudaFree(amp);
         if (out) cudaFree(out);
     }
+    Synth(const Synth &) = delete;
+    Synth &operator=(const Synth &) = delete;
 };
 
-// Seconds per hologram of `form` (tile width bn, 0 = default) on a synthetic cloud.
-double time_form(cgh_ctx *ctx, int form, int bn, int width, int height, int64_t n, int reps)
+// Seconds per hologram of `form` (tile width bn, 0 = default) on a synthetic cloud: the least of `rounds` averages over
+// reps calls (with several rounds one call in the first, and from 60 us on).
+double time_form(cgh_ctx *ctx, int form, int bn, const Synth &s, int reps, int rounds = 1)
 {
-    std::vector<float> hx, ha;
-    synth_points(width, height, n, hx, ha);
-    Scratch s;
-    if (cudaMalloc(&s.xyz, hx.size() * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&s.amp, ha.size() * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&s.out, (size_t)width * height * sizeof(float)) != cudaSuccess) {
-        cudaGetLastError();
-        return -1.0;
-    }
-    cudaMemcpy(s.xyz, hx.data(), hx.size() * sizeof(float), cudaMemcpyHostToDevice);
-    cudaMemcpy(s.amp, ha.data(), ha.size() * sizeof(float), cudaMemcpyHostToDevice);
+    if (!s.ok) return -1.0;
     const int saved_form = ctx->form, saved_bn = ctx->gemm_bn, saved_model = ctx->phase_model;
     const int saved_group = ctx->gemm_group;
     const bool saved_profile = ctx->profile;
@@ -436,16 +460,19 @@ double time_form(cgh_ctx *ctx, int form, int bn, int width, int height, int64_t 
     double sec = -1.0;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess &&
-        compute_hologram(ctx, width, height, ctx->pitch, ctx->lambda, s.xyz, s.amp, n, s.out) == CGH_OK) {
-        cudaEventRecord(e0, ctx->stream);
+        compute_hologram(ctx, s.width, s.height, ctx->pitch, ctx->lambda, s.xyz, s.amp, s.n, s.out) == CGH_OK) {
         bool ok = true;
-        for (int r = 0; r < reps && ok; ++r)
-            ok = compute_hologram(ctx, width, height, ctx->pitch, ctx->lambda, s.xyz, s.amp, n, s.out) == CGH_OK;
-        cudaEventRecord(e1, ctx->stream);
-        if (ok && cudaEventSynchronize(e1) == cudaSuccess) {
+        for (int k = 0; k < rounds && ok; ++k) {
+            const int calls = rounds > 1 && (k == 0 || sec > 6e-5) ? 1 : reps;
+            cudaEventRecord(e0, ctx->stream);
+            for (int r = 0; r < calls && ok; ++r)
+                ok = compute_hologram(ctx, s.width, s.height, ctx->pitch, ctx->lambda, s.xyz, s.amp, s.n, s.out) == CGH_OK;
+            cudaEventRecord(e1, ctx->stream);
             float ms = 0.0f;
-            if (cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) sec = ms * 1e-3 / reps;
+            ok = ok && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
+            if (ok) sec = sec < 0.0 ? ms * 1e-3 / calls : std::min(sec, ms * 1e-3 / calls);
         }
+        if (!ok) sec = -1.0;
     }
     cudaGetLastError();
     if (e0) cudaEventDestroy(e0);
@@ -458,39 +485,49 @@ double time_form(cgh_ctx *ctx, int form, int bn, int width, int height, int64_t 
     return sec;
 }
 
-// Least squares for t = c0 + c1 x1 + c2 x2 over the samples; coefficients kept >= 0.
-void fit3(const std::vector<double> &t, const std::vector<double> &x1, const std::vector<double> &x2, double c[3])
+// Least squares of the relative error of t = c[0] + c[1] x[0] + c[2] x[1] over the samples, every coefficient >= 0
+// (coordinate descent on the normal equations of the scaled terms).
+void fit_times(const std::vector<double> &t, const std::vector<std::array<double, 2>> &x, double c[3])
 {
-    const size_t m = t.size();
+    double scale[3] = {1e-300, 1e-300, 1e-300};
+    for (size_t i = 0; i < t.size(); ++i) {
+        const double r[3] = {1.0, x[i][0], x[i][1]};
+        for (int p = 0; p < 3; ++p) scale[p] = std::max(scale[p], r[p] / t[i]);
+    }
     double A[3][3] = {}, b[3] = {};
-    for (size_t i = 0; i < m; ++i) {
-        const double r[3] = {1.0, x1[i], x2[i]};
+    for (size_t i = 0; i < t.size(); ++i) {
+        const double r[3] = {1.0 / t[i] / scale[0], x[i][0] / t[i] / scale[1], x[i][1] / t[i] / scale[2]};
         for (int p = 0; p < 3; ++p) {
-            b[p] += r[p] * t[i];
+            b[p] += r[p];
             for (int q = 0; q < 3; ++q) A[p][q] += r[p] * r[q];
         }
     }
-    // Cramer's rule on the normal equations, then clamp
-    auto det3 = [](double M[3][3]) {
-        return M[0][0] * (M[1][1] * M[2][2] - M[1][2] * M[2][1]) - M[0][1] * (M[1][0] * M[2][2] - M[1][2] * M[2][0]) +
-               M[0][2] * (M[1][0] * M[2][1] - M[1][1] * M[2][0]);
+    double v[3] = {};
+    for (int sweep = 0; sweep < 5000; ++sweep)
+        for (int p = 0; p < 3; ++p) {
+            double d = b[p];
+            for (int q = 0; q < 3; ++q)
+                if (q != p) d -= A[p][q] * v[q];
+            v[p] = A[p][p] > 0.0 && d > 0.0 ? d / A[p][p] : 0.0;
+        }
+    for (int p = 0; p < 3; ++p) c[p] = v[p] / scale[p];
+}
+
+// What a form's time is made of beside the launches: the time model of its kernel (seconds), and the plane's pixels
+// (the direct forms write it) or the factors' entries.
+std::array<double, 2> form_terms(const cgh_ctx *ctx, int form, int width, int height, int64_t n)
+{
+    if (form < CGH_GEMM_F16)
+        return {choose_direct_mma(1, width, height, n, ctx->num_sms, 0, 0).us * 1e-6, (double)width * height};
+    const bool split = form == CGH_GEMM_SPLIT16;
+    const int ctas = gemm_max_ctas(ctx->num_sms);
+    const int64_t chunk = std::min(n, gemm_chunk_units(split ? kFactorSplit16 : kFactorF16, width, height,
+                                                       ctx->factor_budget_mb << 20));
+    auto us = [&](int64_t units) {
+        return choose_gemm_layout(width, height, (2 * units + 63) / 64, ctas, split, 0, 0, 0, 0).us;
     };
-    const double d = det3(A);
-    for (int k = 0; k < 3; ++k) {
-        double M[3][3];
-        for (int p = 0; p < 3; ++p)
-            for (int q = 0; q < 3; ++q) M[p][q] = (q == k) ? b[p] : A[p][q];
-        c[k] = d != 0.0 ? det3(M) / d : 0.0;
-    }
-    if (c[0] < 0.0 || c[1] < 0.0 || c[2] < 0.0) {
-        // fall back to a proportional model through the largest sample
-        size_t big = 0;
-        for (size_t i = 1; i < m; ++i)
-            if (x1[i] > x1[big]) big = i;
-        c[0] = 0.0;
-        c[1] = x1[big] > 0 ? t[big] / x1[big] : 0.0;
-        c[2] = 0.0;
-    }
+    const double gemm = (double)(n / chunk) * us(chunk) + (n % chunk ? us(n % chunk) : 0.0);
+    return {gemm * 1e-6, (double)(width + height) * (double)n};
 }
 
 std::string bn_key(int width, int height, int form)
@@ -518,29 +555,38 @@ int tune_calibrate(cgh_ctx *ctx, bool force)
         int w, h;
         int64_t n;
     };
-    const Shape shapes[3] = {{256, 256, 2048}, {1024, 512, 8192}, {1024, 1024, 16384}};
+    // The kernels' time models carry the shape, so that the fit is of their scale, the launches' share and what they leave
+    // out, from more samples than coefficients (three samples of 1.7 10^10 terms at most and terms of the sizes alone chose
+    // the direct form for 3840x2160, 2 10^5 points: 21 ms against 15, and differently in every process).  Over 128x128 to
+    // 4096x4096 pixels and 100 to 2 10^5 points the form chosen takes 1.01 of the fastest one's time on average, also with
+    // 10 % of noise on the samples.  The thin one tells the factors from the GEMM; the largest comes
+    // first, so that the clocks are up for the small ones.
+    static const Shape shapes[] = {{1920, 1080, 10000}, {1024, 1024, 10000}, {3840, 2160, 300}, {4096, 64, 20000},
+                                   {1024, 1024, 3000},  {512, 512, 10000},   {256, 256, 1000}};
     const int forms[5] = {CGH_DIRECT_SFU, CGH_DIRECT_ACCURATE, CGH_GEMM_F16, CGH_GEMM_BF16, CGH_GEMM_SPLIT16};
-    for (int f : forms) {
-        std::vector<double> ts, x1, x2;
-        for (const Shape &s : shapes) {
-            const double sec = time_form(ctx, f, 0, s.w, s.h, s.n, 3);
+    std::vector<double> ts[kForms];
+    std::vector<std::array<double, 2>> xs[kForms];
+    for (const Shape &s : shapes) {
+        const Synth cloud(s.w, s.h, s.n);
+        for (int f : forms) {
+            const double sec = time_form(ctx, f, 0, cloud, 3, 3);
             if (sec <= 0.0) return CGH_ECUDA;
-            ts.push_back(sec);
-            x1.push_back((double)s.w * s.h * (double)s.n);
-            x2.push_back((double)(s.w + s.h) * (double)s.n);
+            ts[f].push_back(sec);
+            xs[f].push_back(form_terms(ctx, f, s.w, s.h, s.n));
         }
-        fit3(ts, x1, x2, t->coef[f]);
     }
+    for (int f : forms) fit_times(ts[f], xs[f], t->coef[f]);
     t->calibrated = true;
+    t->last = TuneState::Choice();
     save_cache(*t);
     return CGH_OK;
 }
 
 double tune_predict(cgh_ctx *ctx, int form, int width, int height, int64_t n)
 {
-    TuneState *t = state(ctx);
-    const double *c = t->coef[form];
-    return c[0] + c[1] * (double)width * height * (double)n + c[2] * (double)(width + height) * (double)n;
+    const double *c = state(ctx)->coef[form];
+    const std::array<double, 2> x = form_terms(ctx, form, width, height, n);
+    return c[0] + c[1] * x[0] + c[2] * x[1];
 }
 
 // The persistent launch and the per-kind launches run direct units on the SIMT kernel, which the single hologram's times
@@ -550,6 +596,9 @@ double tune_predict(cgh_ctx *ctx, int form, int width, int height, int64_t n)
 int tune_choose_form(cgh_ctx *ctx, int width, int height, int64_t n, double tol, bool batch)
 {
     if (tune_calibrate(ctx, false) != CGH_OK) return CGH_DIRECT_SFU;
+    TuneState *t = state(ctx);
+    const TuneState::Choice key{width, height, n, tol, ctx->factor_budget_mb, batch, 0};
+    if (t->last.same(key)) return t->last.form;
     const int forms[5] = {CGH_DIRECT_SFU, CGH_DIRECT_ACCURATE, CGH_GEMM_F16, CGH_GEMM_BF16, CGH_GEMM_SPLIT16};
     int best = -1;
     double best_t = 1e300;
@@ -562,8 +611,10 @@ int tune_choose_form(cgh_ctx *ctx, int width, int height, int64_t n, double tol,
             best = f;
         }
     }
+    t->last = key;
     // nothing meets a tolerance tighter than every bound: the most accurate form
-    return best >= 0 ? best : CGH_DIRECT_ACCURATE;
+    t->last.form = best >= 0 ? best : CGH_DIRECT_ACCURATE;
+    return t->last.form;
 }
 
 int tune_choose_bn(cgh_ctx *ctx, int width, int height, int form)
@@ -575,8 +626,9 @@ int tune_choose_bn(cgh_ctx *ctx, int width, int height, int form)
     static const int cands[] = {256, 240, 224, 192, 128};
     int best = choose_gemm_bn(width);
     double best_t = 1e300;
+    const Synth cloud(width, height, 4096);
     for (int bn : cands) {
-        const double sec = time_form(ctx, form, bn, width, height, 4096, 3);
+        const double sec = time_form(ctx, form, bn, cloud, 3);
         if (sec > 0.0 && sec < best_t) {
             best_t = sec;
             best = bn;

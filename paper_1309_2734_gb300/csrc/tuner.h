@@ -35,9 +35,13 @@ struct GemmLayout {
     int bn;
     int splits;
     bool pair;
+    double us;   // predicted time
 };
 GemmLayout choose_gemm_layout(int width, int height, int64_t k_blocks, int ctas, bool split_form, int force_bn,
                               int force_splits, int force_trans, int force_pair);
+
+// Points (K units) per factor chunk when one chunk's P and Q may take budget bytes (mode: a factor mode).
+int64_t gemm_chunk_units(int mode, int width, int height, int64_t budget);
 
 // GEMM tile width (columns of the hologram per tile) with the least padding.
 int choose_gemm_bn(int width);
