@@ -70,9 +70,11 @@ enum {
 /* How the hologram is computed. */
 enum {
     CGH_FORM_AUTO = 0,          /* autotuner's choice for the accuracy class */
-    CGH_DIRECT_SFU = 1,         /* direct sum */
-    CGH_DIRECT_ACCURATE = 2,    /* direct sum; the same, but for CGH_OPT_DIRECT_SHAPE and cgh_batch, whose SIMT kernels
-                                   take the hardware (MUFU) cosine for CGH_DIRECT_SFU and a polynomial here */
+    CGH_DIRECT_SFU = 1,         /* direct sum (NRMS 3.5e-7 at display size; on the SIMT kernels of
+                                   CGH_OPT_DIRECT_SHAPE and cgh_batch the hardware (MUFU) sine and cosine) */
+    CGH_DIRECT_ACCURATE = 2,    /* direct sum, finer sines and cosines and accumulation chains half as long (NRMS
+                                   1.5e-7 on small clouds, 2e-7 at display size, a fifth slower; on the SIMT kernels
+                                   a polynomial) */
     CGH_GEMM_F16 = 3,           /* I = P Q^T, FP16 factors, FP32 accumulate */
     CGH_GEMM_BF16 = 4,          /* I = P Q^T, BF16 factors, FP32 accumulate */
     CGH_GEMM_SPLIT16 = 5        /* I = Ph Qh^T + Ph Ql^T + Pl Qh^T, hi+lo FP16 */

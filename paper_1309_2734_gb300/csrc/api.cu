@@ -22,7 +22,8 @@ namespace cgh {
 
 // The direct form on the tensor cores (planes = 2: the complex wave): prep, then one launch.
 int run_direct_mma(cgh_ctx *ctx, const DirectMmaLayout &lay, int planes, const char *name, int width, int height,
-                   double pitch, double lambda, const float *d_xyz, const float *d_amp, int64_t n, float *d_out)
+                   double pitch, double lambda, const float *d_xyz, const float *d_amp, int64_t n, float *d_out,
+                   bool accurate = false)
 {
     const int64_t n_pad = padded_points(n);
     const size_t geo_bytes = align_up((size_t)n_pad * sizeof(int4), 256);
@@ -51,7 +52,7 @@ int run_direct_mma(cgh_ctx *ctx, const DirectMmaLayout &lay, int planes, const c
     float *slots = reinterpret_cast<float *>(reinterpret_cast<char *>(counters) + cnt_bytes);
     return cuda_status(launch_direct_mma(lay, planes, geo, aux, amax, amp_parts, (int)n, width, height, d_out, slots,
                                          counters, ctx->d_status, (uint64_t)ctx->timeout_ms * 1000000ull, ctx->stream, ctx->drop_tile,
-                                         phase_ref(ctx)));
+                                         phase_ref(ctx), nullptr, 0.0f, 0.0f, accurate));
 }
 
 constexpr int kStreamMinPoints = 64;      // fewest points of one CTA's share in the balanced layout
@@ -68,7 +69,7 @@ int run_direct(cgh_ctx *ctx, bool sfu, int width, int height, double pitch, doub
     if (ctx->direct_shape == 0)
         return run_direct_mma(
             ctx, choose_direct_mma(1, width, height, n, ctx->num_sms, ctx->point_split, ctx->direct_ctas), 1, name,
-            width, height, pitch, lambda, d_xyz, d_amp, n, d_out);
+            width, height, pitch, lambda, d_xyz, d_amp, n, d_out, !sfu);
     const int64_t n_pad = padded_points(n);
     const size_t geo_bytes = align_up((size_t)n_pad * sizeof(int4), 256);
     const size_t aux_bytes = align_up((size_t)n_pad * sizeof(uint2), 256);

@@ -14,6 +14,13 @@
 //   1920x1080, 10^4 points 3.5e-7 (6.0e-7);  1283x717, 3001 points, piston and reference 3.2e-7 (4.1e-7);
 //   640x64, 3000 points 1.1e-7 (3.1e-7);  256x256, 1024 points 2.8e-7 (6.7e-7);  wave 3.5e-7 (5.9e-7).
 // (Without the half turn 640x64 gave 7.2e-7; chains of 1 / 4 / 8 groups at 1920x1080 3.1 / 8.6 / 17.6e-7.)
+// The accurate form takes its entries to 2.8e-8 (quarter_turn2) and chains of one group: with the above it would be coarser
+// on small clouds than the SIMT kernel's polynomial.  NRMS of the SIMT kernel / as above / with both:
+//   256x256, 20 points 1.6 / 2.5 / 1.5e-7, 300 points 2.2 / 3.0 / 1.5e-7, 2048 points 2.0 / 2.5 / 1.6e-7;
+//   640x64, 1024 points 1.27 / 1.50 / 0.95e-7;  1283x717, 3001 points 4.1 / 3.2 / 1.8e-7;  1920x1080, 2 10^5 points
+//   5.2 / - / 4.3e-7.  (From some 6 10^4 points on holograms of 256x256 or less the SIMT kernel's shorter partial sums are
+//   better, 1.5 against 1.8e-7.)
+// Time: 1920x1080, 10^4 points 0.370 ms (SIMT 1.89, as above 0.305), 1283x717, 3001 points 88 us (394, 79).
 //
 // The kernel starts while the points are being prepared (dependent launch) and reduces max |A| itself, so nothing is
 // cleared before: 256x256, 10^3 points with the quantiser 25.7 us (35.4 with plain launches, clears and prep blocks of
@@ -67,6 +74,7 @@ namespace {
 
 using dev::f2;
 using dev::half_turn2;
+using dev::quarter_turn2;
 
 constexpr int kWorkers = 512;
 constexpr int kMmaThreads = kWorkers + 64;   // the workers, the MMA warp, the loader warp
@@ -75,12 +83,16 @@ constexpr int kGroup = kDirectMmaGroup;      // points of a stage: 64 K elements
 constexpr int kPtSlots = 4;
 constexpr int kPtBytes = kGroup * (int)(sizeof(int4) + sizeof(uint2));
 constexpr int kChain = 2;                    // stages of an accumulation chain
+constexpr int kAccChain = 1;                 // the accurate form's
 constexpr int kSphChain = 4;                 // spherical: stages of half as many points
 constexpr float kEntryScale = 4096.0f;       // 2^12, the A side (amplitudes)
 // 2^-12, times 1 + 2.4e-7: the accumulation truncates, and a chain of two groups loses 2.9e-7 of its value on average
 // (measured on random clouds; 2.6e-7 on coherent ones); a spherical chain, with twice the MMAs, 4.6e-7
 constexpr float kUnscale = 2.44140625e-04f * (1.0f + 2.384185791015625e-07f);
 constexpr float kSphUnscale = 2.44140625e-04f * (1.0f + 4.76837158203125e-07f);
+// The accurate form's chains of one group lose 5e-8 (one point) to 1.1e-7 of their value in a random cloud, nothing where
+// many points add up in phase; the sum gets 4e-8 of it back (by one FMA: a unit in the last place from 1.5 on).
+constexpr float kAccUnscale = 2.44140625e-04f, kAccLoss = 4e-8f;
 
 template <int BN>
 struct MmaCfg {
@@ -186,7 +198,7 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&r)[8])
 // apart.  A side: 2^12 A (-cos a, sin a).  B side: its turns
 // walked backwards (b -> -b), (-cos b, -sin b); PLANES = 2: and the rows of the imaginary part, (-sin b, cos b), im_off
 // further on.
-template <int STEPS, bool B, int PLANES>
+template <int STEPS, bool B, int PLANES, bool ACC>
 __device__ __forceinline__ void side_entries(const int4 *geo, const uint2 *aux, bool swap, int row, uint32_t add,
                                              uint32_t step, uint32_t piston, float a_scale, uint32_t hi,
                                              uint32_t lo_off, uint32_t im_off)
@@ -210,8 +222,9 @@ __device__ __forceinline__ void side_entries(const int4 *geo, const uint2 *aux, 
         }
     }
     const float2 na = make_float2(-a.x, -a.y);
-    // U steps side by side: their chains of dependent operations overlap (one plane: 1.5 % over two; two planes: as two)
-    constexpr int kUnroll = PLANES == 1 ? 4 : 2;
+    // U steps side by side: their chains of dependent operations overlap (one plane: 1.5 % over two; two planes: as two;
+    // accurate: two are 2.5 % faster than four)
+    constexpr int kUnroll = PLANES == 1 && !ACC ? 4 : 2;
     auto steps = [&](auto uc, int k0) {
         constexpr int U = decltype(uc)::value;
         float2 s[U], c[U], x[U], y[U];
@@ -224,9 +237,18 @@ __device__ __forceinline__ void side_entries(const int4 *geo, const uint2 *aux, 
                 w[p].D += S[p];
             }
         }
-        half_turn2<U>(x, s, c);
+        if constexpr (ACC) {
+            quarter_turn2<U>(x, s, c);
 #pragma unroll
-        for (int j = 0; j < U; ++j) {
+            for (int j = 0; j < U; ++j) {
+                x[j] = B ? s[j] : __fmul2_rn(a, s[j]);
+                y[j] = B ? c[j] : __fmul2_rn(a, c[j]);
+            }
+        } else {
+            half_turn2<U>(x, s, c);
+        }
+#pragma unroll
+        for (int j = 0; j < U && !ACC; ++j) {
             if (B) {
                 x[j] = __ffma2_rn(s[j], s[j], f2(-1.0f));
                 y[j] = __fmul2_rn(s[j], c[j]);
@@ -376,12 +398,13 @@ struct MmaBars {
 // PLANES = 1: the amplitude hologram, tiles of 128 x BN pixels.  PLANES = 2: the complex wave, tiles of 128 x BN / 2
 // pixels, the B rows (and accumulator columns) of the imaginary part after those of the real part.
 // SPH: the amplitude hologram of the spherical model, 16 points a stage (three products each).
-template <int BN, int PLANES, bool SPH>
+// ACC: the accurate form (PLANES = 1), entries by quarter_turn2 and chains of one group.
+template <int BN, int PLANES, bool SPH, bool ACC>
 __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid_constant__ MmaArgs g)
 {
     using C = MmaCfg<BN>;
     constexpr int GROUP = SPH ? kSphMmaGroup : kGroup;
-    constexpr int CHAIN = SPH ? kSphChain : kChain;
+    constexpr int CHAIN = SPH ? kSphChain : ACC ? kAccChain : kChain;
     static_assert(!SPH || (PLANES == 1 && BN % 64 == 0), "row pairs of the amplitude hologram");
     if (SPH) grid_wait();
     if (SPH && !(g.amp_max[1] > g.phase_lo && g.amp_max[1] <= g.phase_hi)) return;   // another kernel's cloud
@@ -636,7 +659,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
                     }
                 }
 #pragma unroll
-                for (int k = 0; k < 8; ++k) v[k] = v[k] * (SPH ? kSphUnscale : kUnscale) * us;
+                for (int k = 0; k < 8; ++k)
+                    v[k] = (ACC ? fmaf(v[k], kAccLoss, v[k]) : v[k]) * (SPH ? kSphUnscale : ACC ? kAccUnscale : kUnscale) * us;
                 if (!g.a_rows) {   // lanes are columns: each store writes 32 consecutive pixels of a row
                     if (a < g.width)
 #pragma unroll
@@ -693,9 +717,9 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
                     sph_entries<TB / 32, true>(P, q, db, ob, pair & 1, add_b, ref_step(32 * kb), 0.0f,
                                                base + 2 * C::kA, C::kB);
                 } else {
-                    side_entries<kRowsA / 32, false, PLANES>(geo, aux, swap, ra, add_a, ref_step(32 * ka),
+                    side_entries<kRowsA / 32, false, PLANES, ACC>(geo, aux, swap, ra, add_a, ref_step(32 * ka),
                                                              g.ref.piston ? ~0u : 0u, a_scale, base, C::kA, 0);
-                    side_entries<TB / 32, true, PLANES>(geo, aux, swap, rb, add_b, ref_step(32 * kb), 0u, 0.0f,
+                    side_entries<TB / 32, true, PLANES, ACC>(geo, aux, swap, rb, add_b, ref_step(32 * kb), 0u, 0.0f,
                                                         base + 2 * C::kA, C::kB, TB * 128);
                 }
                 fence_proxy_async();
@@ -742,29 +766,29 @@ __global__ void __launch_bounds__(kMmaThreads, 1) direct_mma_kernel(const __grid
     }
 }
 
-template <int BN, int PLANES, bool SPH>
+template <int BN, int PLANES, bool SPH, bool ACC>
 cudaError_t launch_as(const MmaArgs &g, int ctas, cudaStream_t s)
 {
     static PerDeviceOnce configured;
     const cudaError_t e = configured.run([] {
-        return cudaFuncSetAttribute(direct_mma_kernel<BN, PLANES, SPH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        return cudaFuncSetAttribute(direct_mma_kernel<BN, PLANES, SPH, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     MmaCfg<BN>::kSmem);
     });
     if (e != cudaSuccess) return e;
-    return launch_dependent(direct_mma_kernel<BN, PLANES, SPH>, dim3(ctas), dim3(kMmaThreads), MmaCfg<BN>::kSmem, s, true, g);
+    return launch_dependent(direct_mma_kernel<BN, PLANES, SPH, ACC>, dim3(ctas), dim3(kMmaThreads), MmaCfg<BN>::kSmem, s, true, g);
 }
 
-template <int PLANES, bool SPH>
+template <int PLANES, bool SPH, bool ACC>
 cudaError_t launch_bn(int bn, const MmaArgs &g, int ctas, cudaStream_t s)
 {
     switch (bn) {
-    case 64: return launch_as<64, PLANES, SPH>(g, ctas, s);
-    case 128: return launch_as<128, PLANES, SPH>(g, ctas, s);
-    case 192: return launch_as<192, PLANES, SPH>(g, ctas, s);
+    case 64: return launch_as<64, PLANES, SPH, ACC>(g, ctas, s);
+    case 128: return launch_as<128, PLANES, SPH, ACC>(g, ctas, s);
+    case 192: return launch_as<192, PLANES, SPH, ACC>(g, ctas, s);
     case 224:
-        if constexpr (PLANES == 1 && !SPH) return launch_as<224, PLANES, SPH>(g, ctas, s);
+        if constexpr (PLANES == 1 && !SPH) return launch_as<224, PLANES, SPH, ACC>(g, ctas, s);
         else return cudaErrorInvalidValue;
-    case 256: return launch_as<256, PLANES, SPH>(g, ctas, s);
+    case 256: return launch_as<256, PLANES, SPH, ACC>(g, ctas, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -785,7 +809,7 @@ int direct_mma_launches(const DirectMmaLayout &lay, int group, int64_t n_points)
 cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4 *geo, const uint2 *aux,
                               const float *amp_max, int amp_parts, int n_points, int width, int height, float *out,
                               float *slots, int *counters, int *status, uint64_t timeout_ns, cudaStream_t s, int drop,
-                              const PhaseRef &ref, const float4 *ext, float phase_lo, float phase_hi)
+                              const PhaseRef &ref, const float4 *ext, float phase_lo, float phase_hi, bool accurate)
 {
     const int group = ext != nullptr ? kSphMmaGroup : kGroup;
     if (n_points < 1 || lay.ctas < 1 || (planes != 1 && planes != 2) || (uintptr_t)slots % 16 != 0)
@@ -825,9 +849,10 @@ cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4
         g.counters = counters != nullptr ? counters + k * tiles : nullptr;
         g.drop = k == 0 ? drop : -1;
         g.add = k > 0;
-        const cudaError_t e = ext != nullptr ? launch_bn<1, true>(lay.bn, g, lay.ctas, s)
-                              : planes == 2  ? launch_bn<2, false>(lay.bn, g, lay.ctas, s)
-                                             : launch_bn<1, false>(lay.bn, g, lay.ctas, s);
+        const cudaError_t e = ext != nullptr ? launch_bn<1, true, false>(lay.bn, g, lay.ctas, s)
+                              : planes == 2  ? launch_bn<2, false, false>(lay.bn, g, lay.ctas, s)
+                              : accurate     ? launch_bn<1, false, true>(lay.bn, g, lay.ctas, s)
+                                             : launch_bn<1, false, false>(lay.bn, g, lay.ctas, s);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

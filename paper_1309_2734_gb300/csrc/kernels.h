@@ -115,7 +115,7 @@ cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4
                               const float *amp_max, int amp_parts, int n_points, int width, int height, float *out,
                               float *slots, int *counters, int *status, uint64_t timeout_ns, cudaStream_t s, int drop = -1,
                               const PhaseRef &ref = PhaseRef(), const float4 *ext = nullptr, float phase_lo = 0.0f,
-                              float phase_hi = 0.0f);
+                              float phase_hi = 0.0f, bool accurate = false);
 
 // f2: the exact spherical wave of Eq. 1 (spherical.cu), direct SFU form.
 // Points prepared with the piston and ext.  planes = 1: the amplitude

@@ -82,6 +82,34 @@ def test_zero_amplitudes():
     assert not _field(c).any()
 
 
+@pytest.mark.parametrize("extra", [False, True])
+@pytest.mark.parametrize("w,h,n", [(256, 256, 9), (256, 256, 20), (256, 256, 32), (256, 256, 300), (256, 256, 2048), (640, 64, 1024),
+                                   (128, 128, 1000), (1283, 717, 33)])
+def test_accurate_form_is_no_coarser_than_the_simt_kernel(w, h, n, extra):
+    # the same cloud by the SIMT kernel with the cosine polynomial (a pinned thread block): its error is the bound, and
+    # 5 % for the draw of clouds and pixels
+    mma = simt = 0.0
+    for seed in range(3):
+        c = workloads.random_cloud(9700 + 10 * n + seed, w, h, n)
+        rng = np.random.default_rng(seed)
+        cols, rows = rng.integers(0, w, 20000), rng.integers(0, h, 20000)
+        tilt = (0.011, -0.007, 0.6) if extra else (0.0, 0.0, 0.0)
+        ref = oracle.model_wave_at(1 if extra else 0, c.pitch_m, c.lambda_m, c.xyz, c.amp, cols, rows, reference=tilt).real
+        xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
+        err = []
+        for shape in (0, 5):
+            with Hologram(w, h, c.pitch_m, c.lambda_m, form="direct_accurate") as hg:
+                hg.set_option(_lib.CGH_OPT_DIRECT_SHAPE, shape)
+                if extra:
+                    hg.set_phase_model("fresnel_piston")
+                    hg.set_reference(*tilt)
+                f = hg.point_cloud(xyz, amp)
+                hg.sync()
+                err.append(oracle.nrms(f.cpu().numpy()[rows, cols], ref))
+        mma, simt = mma + err[0] ** 2, simt + err[1] ** 2
+    assert mma <= simt * 1.05 ** 2, (mma ** 0.5, simt ** 0.5)
+
+
 MMA, SIMT = 1.5e-6, 1e-5   # the SIMT kernel's tolerance is that of its own tests
 
 
