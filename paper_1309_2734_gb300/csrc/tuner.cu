@@ -130,7 +130,8 @@ DirectMmaLayout choose_direct_mma(int planes, int width, int height, int64_t n_p
                 best.us = t;
             };
             if (split > 0) {
-                const int64_t s = std::min<int64_t>(split, groups), n = tiles * s;
+                // chunks of kPointTile points at least: each takes a slot of a whole tile
+                const int64_t s = std::min<int64_t>(split, (n_points + kPointTile - 1) / kPointTile), n = tiles * s;
                 consider(n, (n + num_sms - 1) / num_sms * ((groups + s - 1) / s), s);
                 continue;
             }

@@ -168,6 +168,22 @@ def test_points_beyond_one_launch(w, h, n):
         assert oracle.nrms((f[0] if wave else f)[rows, cols], ref) <= TOL
 
 
+def test_point_split_beyond_the_point_tiles():
+    # chunks of 256 points at least, however many are asked for: 30 tiles x 391 slots of 2 x 131,072 bytes (3.1 GB), a
+    # quarter more reserved, and not 3125 for each of them
+    c = workloads.random_cloud(9110, 1280, 720, 100000)
+    cols, rows, ref = _sampled(c, 100)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
+    with Hologram(c.width, c.height, c.pitch_m, c.lambda_m, form="direct_sfu") as h:
+        h.set_option(_lib.CGH_OPT_POINT_SPLIT, 4096)
+        f = h.point_cloud(xyz, amp)
+        h.sync()
+        assert free - torch.cuda.mem_get_info()[0] < 6 << 30
+    assert oracle.nrms(f.cpu().numpy()[rows, cols], ref) <= TOL
+
+
 def test_launches_share_the_points_evenly():
     # 12 tiles of 480,943 groups on 13 CTAs: 694 launches, none with fewer groups than the CTAs need.  To the tolerance
     # above come the launches' additions to the output, sqrt(694 / 2) 2^-25 = 5.6e-7
