@@ -233,17 +233,22 @@ def test_auto_single_hologram_meets_tolerance():
     assert oracle.nrms(f.cpu().numpy(), ref) <= 1e-5
 
 
-@pytest.mark.parametrize("tol_e9", [10000, 2_000_000])
-def test_video_batch_64_frames_sampled(tol_e9):
+@pytest.mark.parametrize("tol_e9,persistent", [(10000, False), (2_000_000, False), (10000, True), (2_000_000, True)])
+def test_video_batch_64_frames_sampled(tol_e9, persistent):
     """64 frames of uneven size (1024^2 / 1920x1080 / 3840x2160, 10^3..2x10^5 points), one
-    batch call at NRMS 1e-5 and at 2e-3 (autotuned forms), sampled pixels of every frame vs the oracle."""
+    batch call at NRMS 1e-5 and at 2e-3 (autotuned forms), sampled pixels of every frame vs the oracle: on the two streams
+    (the default at this size), and as one persistent launch (a pinned K chunk)."""
     frames = workloads.video_batch()
     dev = _dev(frames)
     outs = [torch.empty((c.height, c.width), device="cuda") for c in frames]
     with Hologram(8, 8, 8e-6, 532e-9, form="auto", timeout_ms=20000) as h:
         h.set_option(_lib.CGH_OPT_TOLERANCE_E9, tol_e9)
+        if persistent:
+            h.set_option(_lib.CGH_OPT_BATCH_CHUNK_MB, 128)
+        h.profile()
         batch(h, dev, outs)
         h.sync()
+        assert ("batch_persist" if persistent else "batch_lanes") in h.profile_read()
     rng = np.random.default_rng(64)
     for c, o in zip(frames, outs):
         cols = rng.integers(0, c.width, 24)

@@ -116,7 +116,7 @@ MMA, SIMT = 1.5e-6, 1e-5   # the SIMT kernel's tolerance is that of its own test
 @pytest.mark.parametrize("w,h,n,z,tol", [
     (129, 257, 15, (0.3, 0.5), MMA), (300, 200, 17, (0.2, 0.3), MMA), (1920, 224, 130, (0.4, 1.0), MMA), (130, 2000, 33, (0.5, 0.9), MMA),
     (1920, 1080, 65, (0.3, 1.0), MMA),      # the widest tile
-    (1920, 1080, 65, (0.2, 0.25), MMA),     # the narrowest tile
+    (1920, 1080, 65, (0.2, 0.25), MMA),     # corner points beyond the tiles' range of the remainder: the SIMT kernel
     (1920, 1080, 65, (0.05, 0.1), SIMT),     # beyond its bound: the SIMT kernel
     (1920, 1080, 65, (0.005, 1.0), SIMT),    # a close point among far ones: the SIMT kernel
     (1000, 600, 2050, (0.25, 0.6), MMA),
@@ -138,6 +138,44 @@ def test_spherical(w, h, n, z, tol, ref):
         hg.sync()
         got = f.cpu().numpy()
     assert oracle.nrms(got[rows, cols], want) <= tol
+
+
+def _sph_bound(c):
+    # the point preparation's bounds: the largest cross phase over tiles of 128 x 256 pixels (rad; a tile of 128 x bn takes
+    # up to 0.05 x 256 / bn) and the range of the remainder along a side (turns; up to 0.45)
+    x, y, z = c.xyz.astype(np.float64).T
+    q, Z = (c.pitch_m / z) ** 2, z / c.lambda_m
+    cx = np.maximum(abs(x), abs(c.width - 1 - x)) + 128
+    cy = np.maximum(abs(y), abs(c.height - 1 - y)) + 128
+    x64, x128, y64, y128 = (q * (2 * s * v + s * s) for v in (cx, cy) for s in (64, 128))
+    w = np.maximum(x128, y128)
+    return ((np.pi / 2 * Z * np.maximum(x64 * y128, x128 * y64)).max(),
+            (0.25 * Z * ((cx ** 2 + cy ** 2) * q + w) * w).max())
+
+
+@pytest.mark.parametrize("w,h,n,z,lo,hi", [
+    (1920, 1080, 600, (0.28, 0.281), 0.045, 0.05),   # the widest tile at nearly the largest cross phase it takes
+    (1920, 1080, 600, (0.25, 0.251), 0.05, 0.1),     # the narrowest, after the widest has declined
+    (1000, 600, 2050, (0.145, 0.146), 0.1, 0.2),     # only the narrowest takes it
+    (640, 360, 700, (0.0985, 0.099), 0.16, 0.2),     # nearly its largest cross phase
+    (300, 260, 65, (0.08, 0.081), 0.16, 0.2),
+])
+def test_spherical_tiles_near_their_bounds(w, h, n, z, lo, hi):
+    # Tolerance: the SIMT kernel's measured 9.5e-7 at most on such clouds, and the draw of pixels; the third order left out
+    # is 4e-7 of a term at the largest cross phase
+    c = workloads.random_cloud(9450 + w, w, h, n, z)
+    c.xyz[0] = (0.0, 0.0, z[0])
+    phase, spread = _sph_bound(c)
+    assert lo < phase <= hi and spread <= 0.45
+    rng = np.random.default_rng(4)
+    cols, rows = rng.integers(0, w, 3000), rng.integers(0, h, 3000)
+    want = oracle.model_wave_at(2, c.pitch_m, c.lambda_m, c.xyz, c.amp, cols, rows).real
+    xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
+    with Hologram(w, h, c.pitch_m, c.lambda_m, form="direct_sfu") as hg:
+        hg.set_phase_model("spherical")
+        f = hg.point_cloud(xyz, amp)
+        hg.sync()
+    assert oracle.nrms(f.cpu().numpy()[rows, cols], want) <= 1e-6
 
 
 @pytest.mark.parametrize("n", [1, 63, 64, 65, 256, 257, 1500])
