@@ -127,6 +127,20 @@ int factor_mode(int form)
 // into P and Q with leading dimension ld, on stream s.
 using FactorLaunch = std::function<cudaError_t(int64_t u0, int64_t nu, void *P, void *Q, int64_t ld, cudaStream_t s)>;
 
+// Largest W x H x points that prep, factors, GEMM and reduction are dependent launches for (about 0.2 ms).  Time with them
+// over without, FP16 / split FP16 / FP16 wave: 1920x1080, 6 10^9 terms 0.84 / 0.92 / 0.83, 2 10^10 0.92 / 0.98 / 0.93,
+// 3 10^10 0.97 / 1.01 / 0.98, 4 10^10 0.99 / 1.03 / 1.01, 6 10^10 1.02 / 1.04 / 0.99, 10^11 1.03 / 1.04 / 1.01; 1024x1024
+// and 2048x2048 up to 6 10^10 0.89 to 1.02.
+constexpr int64_t kDependentTerms = 30000000000ll;
+
+int64_t gemm_chunk_units(int mode, int width, int height, int64_t budget)
+{
+    const int planes = mode == kFactorSplit16 ? 2 : 1;
+    const int64_t bytes_per_unit = (int64_t)planes * (width + height) * 2 * 2;
+    const int64_t chunk = budget / bytes_per_unit / 32 * 32;
+    return chunk < 32 ? 32 : chunk;
+}
+
 // The GEMM over K units: per chunk of units the factors P and Q and the
 // tcgen05 GEMM over K splits, later chunks adding to the planes of the first;
 // then the fixed-order split reduction when there is more than one split.
@@ -138,17 +152,6 @@ using FactorLaunch = std::function<cudaError_t(int64_t u0, int64_t nu, void *P, 
 // 5x10^4 points: 0.428 ms without, 0.428-0.46 ms with 2-4 stages, so it is
 // off by default.)  The epilogue multiplies by *scale, the factor of Q (or
 // P) that keeps the FP16 operands within range.
-// Largest W x H x points that prep, factors, GEMM and reduction are dependent launches for (about 0.2 ms; 1920x1080,
-// 5 10^4 points, FP16: 2 % slower with them, 377 -> 383 us).
-constexpr int64_t kDependentTerms = 30000000000ll;
-int64_t gemm_chunk_units(int mode, int width, int height, int64_t budget)
-{
-    const int planes = mode == kFactorSplit16 ? 2 : 1;
-    const int64_t bytes_per_unit = (int64_t)planes * (width + height) * 2 * 2;
-    const int64_t chunk = budget / bytes_per_unit / 32 * 32;
-    return chunk < 32 ? 32 : chunk;
-}
-
 int gemm_units(cgh_ctx *ctx, int mode, int width, int height, int64_t n, const char *factor_name,
                const FactorLaunch &factors, const float *scale, float *d_out)
 {

@@ -28,7 +28,7 @@
 //
 // Time, prep included (before): 1920x1080, 10^4 points 0.305 ms (1.77; 68 G terms/ms); its complex wave 0.480 ms
 // (3.30); 1024x1024, 10^3 points 0.042 ms (0.117); 256x256, 10^3 points 0.021 ms (0.046); the spherical hologram,
-// 1920x1080, 10^4 points at 0.3-1 m 0.643 ms (7.36; with the narrowest tile, for points at 0.2 m, 1.53).
+// 1920x1080, 10^4 points at 0.3-1 m 0.644 ms (7.36; at 0.25 m, where only the narrowest tile's bound holds, 1.50).
 // What bounds it: the making of entries (0.26 of 0.31 ms with the MMAs left out), 30 instructions for two entries, 15
 // of them packed FMAs of two to three cycles, so the FMA pipe is about 80 % busy while entries are made (53 % over the
 // kernel); the tensor cores are active 36 % of the time.  128 x BN tiles: larger tiles share an entry among more pixels (BN = 64 / 128 /

@@ -2,7 +2,7 @@
 // middle line of Eq. 5), direct form, hardware sine: the SIMT kernel, which the
 // complex wave takes, and amplitude holograms whose points are too close to a
 // wide hologram for the tensor-core form (direct_mma.cu; 1920x1080, 10^4 points
-// at 0.3-1 m: 7.34 ms here, 0.66 ms there; 4.7e-7 against 8.9e-7 NRMS).
+// at 0.3-1 m: 7.36 ms here, 0.645 ms there; 4.7e-7 against 8.9e-7 NRMS).
 //
 // The phase of point j at pixel (m, n) in turns is t = sqrt(r^2 + z^2) / lambda
 // (r in metres).  With Z = z / lambda and u = r^2 / z^2,

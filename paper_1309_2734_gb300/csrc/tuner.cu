@@ -88,9 +88,11 @@ DirectLayout choose_layout(const DirectShape *shapes, int n_shapes, int width, i
 
 // Microseconds of one stage (32 points of a 128 x bn / planes tile; spherical: 16) of a CTA of the tensor-core direct
 // form, for the amplitude hologram, the complex wave and the spherical hologram, and per B row for each part of a tile
-// that its last CTA adds.  Measured on GB300 at 1920x1080 with 10^4 points (stages) and at 256x256 with 10^3 (parts); over 128x32 to 2048x2048 pixels
-// and 100 to 10^4 points the choice is within 8 % of the fastest tile and CTA count but for the smallest holograms
-// (under 30 us), where the spread of one of them is as large.
+// that its last CTA adds.  Measured on GB300 at 1920x1080 with 10^4 points (stages) and at 256x256 with 10^3 (parts).
+// Against every tile and orientation over 128x32 to 2048x2048 pixels, 100 to 3 10^4 points and the three forms, the choice
+// takes 1.02 of the fastest one's time on average; the worst are 1920x1080, 100 points (22.9 us, 16.8 with 128 rows),
+// 1283x717 with 1000 and 3000 points (47.9 and 78.6, 39.3 and 69.0 with 192 and 256) and the wave of 130x2000 with 1000
+// points (43.5, 37.3).
 struct MmaCost {
     int bn;
     double stage[3];
@@ -248,8 +250,8 @@ int choose_gemm_splits(int64_t tiles, int64_t k_blocks, int ctas)
 }
 
 // Stated NRMS bound of each form against the FP64 oracle (measured values are
-// below these: direct SFU ~4e-7, direct accurate ~1e-7, split FP16 ~3e-6,
-// FP16 ~3e-4, BF16 ~2e-3 on the display-size clouds).
+// below these: direct SFU 3.5e-7 and accurate 2e-7, on the batch's SIMT units 6e-7
+// and 4e-7, split FP16 2e-6, FP16 ~3e-4, BF16 ~2e-3 on the display-size clouds).
 double form_nrms_bound(int form)
 {
     switch (form) {

@@ -28,10 +28,10 @@
 //
 // 2048x2048, 10^5 points 2-10 mm behind the plane (before: a hardware sine and
 // cosine per pixel and point, lists counted, scanned by one thread and filled):
-// record 0.39 -> RECORD_MS ms, lists 0.105 -> LISTS_MS ms, preparation PREP_MS.  Bound by
-// instruction issue and the reads of the entries: about 50 instructions a warp
-// for a point and block, 55 % of whose pixels are inside the window (32 % with
-// rows of 32 pixels for a warp, 0.32 ms).
+// record 0.39 -> 0.25 ms, lists 0.105 -> 0.014 ms, preparation 0.015.  Bound by
+// instruction issue (62 % of the slots) and the reads of the entries: about 50
+// instructions a warp for a point and block, 56 % of whose pixels are inside the
+// window (rows of 32 pixels for a warp: 0.32 ms).
 #include <cmath>
 
 #include "device_util.cuh"
