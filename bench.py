@@ -41,18 +41,23 @@ FMA_PER_SM_PER_CLK = 128        # FP32 FMA-pipe operations per SM per clock
 DIRECT_FLOPS = 12               # direct forms, per evaluation: K = 2 (cosine, sine), three products of split FP16
 
 
+def simt_tile(width, height):
+    """The SIMT direct kernel's tile and its CGH_OPT_DIRECT_SHAPE: 128 x 64 pixels, or 256 x 32 where that pads a fifth
+    fewer pixels."""
+    def padded(tw, th):
+        return -(-width // tw) * tw * (-(-height // th) * th)
+    return (256, 32, 6) if padded(256, 32) * 6 < padded(128, 64) * 5 else (128, 64, 5)
+
+
 def direct_ops(form, width, height, n_points):
-    """The SIMT direct kernel's work per launch in FMA-pipe operations (the direct forms with a pinned thread block,
-    CGH_OPT_DIRECT_SHAPE; by default they run on the tensor cores, DIRECT_FLOPS), as the kernel does it: a CTA covers a 128 x 64
-    tile (256 x 32 where that pads a fifth fewer pixels); per point it takes the sine and cosine of the tile's
+    """The SIMT direct kernel's work per launch in FMA-pipe operations (--simt; by default the direct forms run on the
+    tensor cores, DIRECT_FLOPS), as the kernel does it: per point a CTA takes the sine and cosine of its tile's
     columns and rows once (the SFU form: one FFMA and the sine's range multiply per entry, and the amplitude's two
     multiplies per row entry; the accurate form: two polynomials of 8 FMA-pipe operations per entry), then every
     pixel costs two FMAs (one packed two-lane FMA per pair of columns).  Returns (operations, pipe, peak operations per SM per clock, operations per
     evaluation); the MUFU operations of the SFU form (two per entry, 0.05 per evaluation) bound nothing."""
-    def padded(tw, th):
-        return -(-width // tw) * tw * (-(-height // th) * th)
-    tw, th = (256, 32) if padded(256, 32) * 6 < padded(128, 64) * 5 else (128, 64)
-    tiles = padded(tw, th) // (tw * th)
+    tw, th, _ = simt_tile(width, height)
+    tiles = -(-width // tw) * -(-height // th)
     per_col, per_row = (2, 4) if form == "direct_sfu" else (16, 18)
     per_point_tile = 2 * tw * th + tw * per_col + th * per_row
     ops = n_points * tiles * per_point_tile
@@ -63,11 +68,11 @@ def direct_ops(form, width, height, n_points):
 # dram__bytes_write.sum), keyed by the SHA-1 of the kernel's sources they were
 # taken on; a changed source reports null until it is profiled again.
 NCU_TRAFFIC = [
-    # profiles/direct_mma-1920x1080-n10000.md: 0.340 MB read + 0.007 MB written (tuner.cu picks the tile and CTAs)
+    # 0.340 MB read + 0.077 MB written (tuner.cu picks the tile and CTAs)
     {"kernel": "direct_sfu", "form": "direct_sfu", "workload": "direct-1920x1080-n10000",
-     "src": ["direct_mma.cu", "half_turn.cuh", "sincospoly.h", "device_util.cuh", "tcgen05.cuh", "tuner.cu"],
-     "sha1": "3dcbd9d362a6953c3166959594f5a5d04ab321bc", "bytes_per_launch": 347392},
-    # profiles/gemm_f16-1920x1080-n50000.md: 600.757 MB read + 3.468 MB written per launch
+     "src": ["direct_mma.cu", "half_turn.cuh", "sincospoly.h", "sinpoly.h", "device_util.cuh", "tcgen05.cuh", "tuner.cu"],
+     "sha1": "e0203237e34af9acdc953f4ef84f1dce51e35903", "bytes_per_launch": 417536},
+    # 600.757 MB read + 3.468 MB written per launch
     {"kernel": "gemm_tcgen05", "form": "gemm_f16", "workload": "gemm-1920x1080-n50000",
      "src": ["gemm.cu", "gemm_dev.cuh", "tcgen05.cuh", "device_util.cuh"],
      "sha1": "43ea28564d17d32a63c9bd0dc4d6cbbcad3f1cca", "bytes_per_launch": 604224768},
@@ -331,6 +336,10 @@ def run_ours(args):
     q = torch.empty((H, W), dtype=torch.uint8, device="cuda")
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
     h = Hologram(W, H, cloud.pitch_m, cloud.lambda_m, form=args.form, stream=stream)
+    simt = args.simt and args.form.startswith("direct")
+    if simt:
+        from paper_1309_2734_gb300 import _lib
+        h.set_option(_lib.CGH_OPT_DIRECT_SHAPE, simt_tile(W, H)[2])
 
     def step():
         h.point_cloud(xyz, amp, out)
@@ -582,9 +591,9 @@ def run_ours(args):
                                   "speedup_vs_k20": t_k20 * 1e3 / ms, "kernel_ms": {k: v[1] for k, v in kp.items()},
                                   "step": "WRP record + Fresnel diffraction (2 FFTs, cached chirp spectrum) + kinoform8"}
 
-    # the batched workload: 64 frames of uneven size and point count in one cgh_batch call (persistent
-    # launches per form kind, captured in a CUDA graph and replayed), forms and tiles per frame from the
-    # autotuner at each accuracy class; NRMS on sampled pixels of every frame (CPU leg)
+    # the batched workload: 64 frames of uneven size and point count in one cgh_batch call (hologram by hologram on
+    # two streams at this size), the form per frame from the autotuner at each accuracy class; NRMS on sampled pixels
+    # of every frame (CPU leg)
     vbatch = {}
     if not args.no_batch:
         from paper_1309_2734_gb300 import _lib, batch as run_batch
@@ -691,6 +700,16 @@ def run_ours(args):
         achieved = (4.0 * W * H * k_units * passes * args.steps / (dom_ms * 1e-3) / 1e12) if dom_ms > 0 else None
         roof = {"bound": "tensor", "unit": "TFLOP/s", "gemm_k": 2 * k_units,
                 "peak_basis": "measured dense bf16 burst (fp16 nominal rate is the same)"}
+    elif simt:
+        dom = args.form
+        dom_launches, dom_ms = prof.get(dom, (0, 0.0))
+        ops, pipe, per_clk, per_eval = direct_ops(args.form, W, H, N)
+        peak = per_clk * torch.cuda.get_device_properties(local).multi_processor_count * \
+            (_peaks().get("sm_max_mhz") or 2070.0) * 1e-3
+        achieved = ops * args.steps / (dom_ms * 1e-3) / 1e9 if dom_ms > 0 else None
+        roof = {"bound": "alu", "unit": f"G {pipe} op/s",
+                "peak_basis": f"{per_clk} {pipe} op/clk/SM at the highest clock; {per_eval:.4f} op per evaluation (two FMAs "
+                              "a pixel and point, and the sines and cosines of the tile's columns and rows)"}
     else:
         # the tensor cores' part; what bounds the kernel is the making of the operands on the FMA pipe
         dom = args.form
@@ -699,7 +718,7 @@ def run_ours(args):
         roof = {"bound": "tensor", "unit": "TFLOP/s",
                 "peak_basis": f"measured dense bf16 burst (fp16 nominal rate is the same); {DIRECT_FLOPS} flop per "
                               "evaluation (K = 2, three products of split FP16)"}
-    traffic = ncu_traffic(dom, args.form, cloud.name)
+    traffic = None if simt else ncu_traffic(dom, args.form, cloud.name)
 
     cpu, nrms = (None, None)
     if not args.no_cpu_baseline:
@@ -718,11 +737,14 @@ def run_ours(args):
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None,
-        "dtype": {"gemm_f16": "f16", "gemm_bf16": "bf16", "gemm_split16": "f16x2 (hi+lo)"}.get(args.form, "f32"),
+        # the tensor-core direct forms make their operands in f32 and multiply them as hi+lo f16 pairs (22 bits)
+        "dtype": {"gemm_f16": "f16", "gemm_bf16": "bf16", "gemm_split16": "f16x2 (hi+lo)"}.get(
+            args.form, "f32" if simt else "f32 (products as f16x2 hi+lo, f32 sums)"),
         "data": "synthetic",
         "config": {"workload": cloud.name, "width": W, "height": H, "n_points": N, "form": args.form,
                    "step": ("prep + factors + tcgen05 GEMM (+ split reduction) + quantize8"
                             if args.form.startswith("gemm") else
+                            "prep + SIMT direct kernel (a pinned thread block) + quantize8" if simt else
                             "prep + direct kernel on the tensor cores (equal shares of the (tile, point) pairs, each "
                             "tile's parts summed in the kernel) + quantize8"),
                    "l2": "flushed between timed steps (256 MiB write, untimed)",
@@ -838,6 +860,8 @@ def main():
                     help="skip the Fresnel diffraction and wavefront-recording workloads of Tables 5-6")
     ap.add_argument("--no-large", action="store_true",
                     help="skip the 4096x4096, 10^6-point depth-layered case")
+    ap.add_argument("--simt", action="store_true",
+                    help="the headline's direct form on the SIMT kernel (a pinned thread block)")
     ap.add_argument("--no-small", action="store_true", help="skip the 256x256, 1,024-point cloud")
     ap.add_argument("--no-paper-workload", action="store_true",
                     help="skip the phase-only 1920x1080 workload of the paper's Tables 3-4")

@@ -73,7 +73,7 @@ enum {
     CGH_DIRECT_SFU = 1,         /* direct sum (NRMS 3.5e-7 at display size; on the SIMT kernels of
                                    CGH_OPT_DIRECT_SHAPE and cgh_batch the hardware (MUFU) sine and cosine) */
     CGH_DIRECT_ACCURATE = 2,    /* direct sum, finer sines and cosines and accumulation chains half as long (NRMS
-                                   1.5e-7 on small clouds, 2e-7 at display size, a fifth slower; on the SIMT kernels
+                                   1.5e-7 on small clouds, 2.6e-7 at display size, a fifth slower; on the SIMT kernels
                                    a polynomial) */
     CGH_GEMM_F16 = 3,           /* I = P Q^T, FP16 factors, FP32 accumulate */
     CGH_GEMM_BF16 = 4,          /* I = P Q^T, BF16 factors, FP32 accumulate */

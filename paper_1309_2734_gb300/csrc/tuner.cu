@@ -250,7 +250,7 @@ int choose_gemm_splits(int64_t tiles, int64_t k_blocks, int ctas)
 }
 
 // Stated NRMS bound of each form against the FP64 oracle (measured values are
-// below these: direct SFU 3.5e-7 and accurate 2e-7, on the batch's SIMT units 6e-7
+// below these: direct SFU 3.5e-7 and accurate 2.6e-7, on the batch's SIMT units 6e-7
 // and 4e-7, split FP16 2e-6, FP16 ~3e-4, BF16 ~2e-3 on the display-size clouds).
 double form_nrms_bound(int form)
 {

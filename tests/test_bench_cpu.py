@@ -1,5 +1,5 @@
-"""bench.py's host-side bookkeeping, without a GPU: the operation counts behind the direct kernel's roofline and
-the traffic records."""
+"""bench.py's host-side bookkeeping, without a GPU: the operation counts behind the SIMT direct kernel's roofline
+(--simt) and the traffic records."""
 import os
 import sys
 
