@@ -129,7 +129,8 @@ enum {
                                    the (pixel tile, point) pairs; 0 = automatic (up to one per SM; the hardware
                                    schedules those beyond the resident ones as others finish) */
     CGH_OPT_BATCH_MODE = 15,    /* cgh_batch: 0 = default: a batch of 10^11 terms (width x height x points) or more
-                                   hologram by hologram on two streams of the context's own (not under stream
+                                   whose holograms are large enough for launches of their own, hologram by
+                                   hologram on two streams of the context's own (not under stream
                                    capture, nor with another batch option, GEMM_BN, GEMM_CHUNK or
                                    GEMM_TRANSPOSE set); else one
                                    persistent launch for the whole batch (GEMM units on the tensor cores beside

@@ -112,11 +112,11 @@ constexpr int kSplit16ChunkKbBatch = 16;   // divides a factor group's 32 k-bloc
 
 // Form (and, for the GEMM forms, tile width) of every instance: the context's form, or the autotuner's choice.
 // forced > 0: that form for every instance; single: for the single-hologram forms of the lanes.
-void choose_forms(cgh_ctx *ctx, const cgh_instance *inst, int n, BatchPlan *plan, std::vector<int> &bn,
+void choose_forms(cgh_ctx *ctx, const cgh_instance *inst, int n, std::vector<int> &forms, std::vector<int> &bn,
                   int forced = 0, bool single = false)
 {
     const double tol = (double)ctx->tol_e9 * 1e-9;
-    plan->forms.assign(n, CGH_DIRECT_SFU);
+    forms.assign(n, CGH_DIRECT_SFU);
     bn.assign(n, 256);
     for (int i = 0; i < n; ++i) {
         if (inst[i].n_points == 0) continue;
@@ -124,7 +124,7 @@ void choose_forms(cgh_ctx *ctx, const cgh_instance *inst, int n, BatchPlan *plan
                       : ctx->form != CGH_FORM_AUTO
                           ? ctx->form
                           : tune_choose_form(ctx, inst[i].width, inst[i].height, inst[i].n_points, tol, !single);
-        plan->forms[i] = f;
+        forms[i] = f;
         if (f >= CGH_GEMM_F16 && !single)   // the single-hologram forms choose their own tiles
             bn[i] = ctx->gemm_bn > 0 ? ctx->gemm_bn
                                      : (ctx->form == CGH_FORM_AUTO ? tune_choose_bn(ctx, inst[i].width, inst[i].height, f)
@@ -251,7 +251,7 @@ constexpr int kDirectMaxChunks = 64;
 int build_plan_persist(cgh_ctx *ctx, const cgh_instance *inst, int n, BatchPlan *plan, int forced_form = 0)
 {
     std::vector<int> bn;
-    choose_forms(ctx, inst, n, plan, bn, forced_form);
+    choose_forms(ctx, inst, n, plan->forms, bn, forced_form);
     const int rows_f = persist_factor_rows(), pts_f = persist_factor_points();
     const int dtw = persist_direct_tile_w(), dth = persist_direct_tile_h();
     constexpr int kQ4NT = 8 * 256;   // float4s of one direct tile's totals
@@ -508,7 +508,7 @@ int build_plan_persist(cgh_ctx *ctx, const cgh_instance *inst, int n, BatchPlan 
 int build_plan_kinds(cgh_ctx *ctx, const cgh_instance *inst, int n, BatchPlan *plan)
 {
     std::vector<int> bn;
-    choose_forms(ctx, inst, n, plan, bn);
+    choose_forms(ctx, inst, n, plan->forms, bn);
     // arena layout
     Layout L;
     struct Off {
@@ -762,14 +762,9 @@ void destroy_batch_lanes(BatchLanes *L)
     delete L;
 }
 
-// Whether the batch's holograms go one by one through the single-hologram forms on two streams: their GEMMs take the
-// two-SM tiles and layouts of the time model, run at 0.8 of the tensor peak against the persistent launch's 0.6, and
-// one hologram's preparation and factors fill the other's tails.  From kLanesEvals terms in all; below it the
-// launches of many small holograms cost more than that gains.  12 frames of 10^3 to 10^5 points, split FP16: 9.9 ms
-// against 10.7 (FP16 3.5 against 3.8; one stream 9.7 but 3.65, three 9.9); 6 frames of 3 10^3 to 3 10^4 points (1.7
-// 10^11 terms) 1.48 against 1.68 (FP16 0.56 against 0.64); 4 small ones (4 10^10 terms) 0.41 against 0.44 (FP16 0.181
-// against 0.171).  Not under capture (the forms grow their workspaces), nor with options of the other
-// modes, a pinned tile width, chain or orientation among them.
+// Whether the batch's holograms may go one by one through the single-hologram forms on two streams: from kLanesEvals terms
+// in all, not under capture (the forms grow their workspaces), nor with options of the other modes, a pinned tile width,
+// chain or orientation among them.
 constexpr double kLanesEvals = 1e11;
 
 static bool lanes_serve(const cgh_ctx *ctx, const cgh_instance *inst, int n)
@@ -786,6 +781,40 @@ static bool lanes_serve(const cgh_ctx *ctx, const cgh_instance *inst, int n)
         return false;
     }
     return cs == cudaStreamCaptureStatusNone;
+}
+
+// And whether that pays: their GEMMs take the two-SM tiles and layouts of the time model, run at 0.8 of the tensor peak
+// against the persistent launch's 0.6, and one hologram's preparation and factors fill the other's tails, but every
+// hologram has its own launches.  What a term saves, more on holograms whose few 224-wide tiles the persistent launch fills
+// badly, against the launches of each hologram and the one tail of the persistent launch (fitted to the times below).  Two
+// streams over the persistent launch, FP16 / split FP16, 40 holograms:
+//   512x512      3 10^9 terms each 1.22 / 1.28, 10^10 0.80 / 0.70, 4 10^10 0.72 / 0.57;
+//   1024x1024    3 10^9 2.07 / 1.56, 10^10 1.09 / 0.73, 2 10^10 0.76 / 0.82;
+//   1920x1080    10^10 1.38 / 1.15, 2 10^10 1.15 / 0.98, 4 10^10 1.06 / 0.91, 10^11 (12) 0.88 / 0.94;
+//   3840x2160    10^10 1.36 / 1.17, 2 10^10 1.13 / 1.00, 4 10^10 0.98 / 0.94, 10^11 (12) 0.89 / 0.85;
+// two to four of 2 10^10 or more 0.4 to 1.0; one stream 9.7 ms against 9.9 on 12 mixed ones in split FP16, 3.65 against 3.5
+// in FP16, three streams 9.9.  The context's direct form runs on the tensor cores here and on the SIMT units there: 64
+// holograms of 1.6 10^7 terms 2.1, 3.3 10^7 0.97, 10^8 0.3 to 0.4.
+constexpr double kLanesPixels[2] = {1.5e6, 4e5};
+constexpr double kLanesSaveF16[3] = {0.3e-9, 1.6e-9, 2.5e-9};   // us a term: larger than the first, the second, the rest
+constexpr double kLanesSaveSplit[3] = {0.75e-9, 3.5e-9, 5e-9};
+constexpr double kLanesLaunchUs = 16.0, kLanesTailUs = 40.0;
+constexpr double kLanesDirect = 5e7;   // terms of a hologram, on average
+
+static bool lanes_pay(const cgh_ctx *ctx, const cgh_instance *inst, int n, const std::vector<int> &forms)
+{
+    const bool direct = ctx->form == CGH_DIRECT_SFU || ctx->form == CGH_DIRECT_ACCURATE;
+    double saved = kLanesTailUs, evals = 0.0;
+    int count = 0;
+    for (int i = 0; i < n; ++i) {
+        if (inst[i].n_points == 0) continue;
+        const double px = (double)inst[i].width * inst[i].height, terms = px * (double)inst[i].n_points;
+        const double *save = forms[i] == CGH_GEMM_F16 || forms[i] == CGH_GEMM_BF16 ? kLanesSaveF16 : kLanesSaveSplit;
+        ++count;
+        evals += terms;
+        saved += terms * save[px > kLanesPixels[0] ? 0 : px > kLanesPixels[1] ? 1 : 2] - kLanesLaunchUs;
+    }
+    return direct ? evals >= kLanesDirect * count : saved >= 0.0;
 }
 
 // The largest first, alternately on the lanes.
@@ -836,11 +865,14 @@ int run_batch(cgh_ctx *ctx, const cgh_instance *inst, int n)
     if (!ctx->batch) ctx->batch = new BatchPlan();
     BatchPlan *plan = ctx->batch;
     if (lanes_serve(ctx, inst, n)) {
-        std::vector<int> bn;
-        choose_forms(ctx, inst, n, plan, bn, 0, true);
-        plan->key.clear();   // the forms are this batch's now
-        ProfileScope ps(ctx, "batch_lanes", 1);
-        return run_batch_lanes(ctx, inst, n, plan->forms);
+        std::vector<int> forms, bn;
+        choose_forms(ctx, inst, n, forms, bn, 0, true);
+        if (lanes_pay(ctx, inst, n, forms)) {
+            plan->forms = forms;
+            plan->key.clear();   // the forms are this batch's now
+            ProfileScope ps(ctx, "batch_lanes", 1);
+            return run_batch_lanes(ctx, inst, n, forms);
+        }
     }
     const std::vector<uint64_t> key = plan_key(ctx, inst, n);
     if (!(plan->exec && plan->key == key)) {

@@ -368,3 +368,40 @@ def test_auto_is_near_the_fastest_form(w, h, n):
             hg.set_option(_lib.CGH_OPT_GEMM_GROUP, 1)
             auto = _best_us(lambda: hg.point_cloud(xyz, amp, out))
         assert auto <= 1.3 * min(us.values()), (auto, us)
+
+
+@pytest.mark.parametrize("form,frames,size,n,route", [
+    ("gemm_f16", 40, (1024, 1024), 3000, "batch_persist"),     # 3.1 10^9 terms each: half the time of launches of their own
+    ("gemm_split16", 40, (1024, 1024), 3000, "batch_persist"),
+    ("gemm_f16", 12, (1024, 1024), 19000, "batch_lanes"),
+    ("gemm_f16", 20, (512, 512), 30000, "batch_lanes"),
+    ("gemm_f16", 80, (512, 512), 6000, "batch_persist"),
+    ("gemm_split16", 11, (1920, 1080), 5000, "batch_persist"), # 10^10 terms each
+    ("gemm_split16", 7, (1920, 1080), 12000, "batch_lanes"),
+    ("gemm_f16", 7, (1920, 1080), 9000, "batch_persist"),
+    ("gemm_f16", 3, (1920, 1080), 17000, "batch_lanes"),       # few: 3.5 10^10 each
+    ("gemm_f16", 7, (1920, 1080), 27000, "batch_lanes"),
+    ("auto", 40, (1024, 1024), 3000, "batch_persist"),
+    ("direct_sfu", 40, (1024, 1024), 3000, "batch_lanes"),
+    ("direct_sfu", 2500, (128, 128), 2600, "batch_persist"),   # 4.3 10^7 terms each
+])
+def test_many_small_holograms_stay_in_one_launch(form, frames, size, n, route):
+    # 10^11 terms or more in all; the streams serve only holograms that are worth launches of their own
+    w, h = size
+    clouds = [workloads.random_cloud(970 + i, w, h, n) for i in range(2)]
+    two = _dev(clouds)
+    dev = [two[i % 2] for i in range(frames)]
+    outs = [torch.empty((h, w), device="cuda") for _ in range(frames)]
+    with Hologram(8, 8, 8e-6, 532e-9, form=form) as hg:
+        hg.profile()
+        batch(hg, dev, outs)
+        hg.sync()
+        assert set(hg.profile_read()) == {route}
+        if form == "auto":
+            assert set(_lib.cgh_batch_forms(hg.ctx)) == {_lib.CGH_GEMM_SPLIT16}
+    rng = np.random.default_rng(97)
+    cols, rows = rng.integers(0, w, 64), rng.integers(0, h, 64)
+    for i in (0, 1, frames - 2, frames - 1):
+        c = clouds[i % 2]
+        ref = oracle.field_at(c.pitch_m, c.lambda_m, c.xyz, c.amp, cols, rows)
+        assert oracle.nrms(outs[i].cpu().numpy()[rows, cols], ref) <= (1e-5 if form == "auto" else NRMS[form])
