@@ -111,8 +111,23 @@ int run_direct(cgh_ctx *ctx, bool sfu, int width, int height, double pitch, doub
 // k-blocks per TMEM accumulation chain of the split-FP16 form (3 passes each).  Between chains the MMAs wait for the
 // fold, so longer chains are faster, and the truncation of the accumulation grows with them: with the small products
 // first (gemm_mma) 8 / 16 / 24 / 32 k-blocks give 0.90 / 1.42 / 1.99 / 2.54e-6 NRMS and 248 / 237 / 232 / 233 us at
-// 1024x1024, 20,011 points (8 with the large products first: 2.8e-6, 245 us)
-constexpr int kSplit16ChunkKb = 24;
+// 1024x1024, 20,011 points (8 with the large products first: 2.8e-6, 245 us).  Each pass reads the chain's operands again,
+// so those of all units in flight have to stay in L2: where they would take more than kSplit16ChainBytes (thin holograms,
+// whose tiles share nothing: 16384x64, 8192x128, 2048x64 hold 120 MB), chains of 8: 16384x64, 3 10^4 points 1.49 -> 1.32 ms,
+// 4096x128 0.42 -> 0.385; at 64 MB (4096x256, 1024x1024) both lengths take the same.
+constexpr int kSplit16ChunkKb = 24, kSplit16ChunkKbThin = 8;
+constexpr double kSplit16ChainBytes = 100e6;
+
+static int split16_chunk_kb(const GemmPlan &plan, int width, int height)
+{
+    const int64_t a_rows = plan.trans ? width : height, b_rows = plan.trans ? height : width;
+    const int64_t tile_m = plan.pair ? 256 : 128, slots = plan.pair ? plan.ctas / 2 : plan.ctas;
+    const int64_t tiles = ((a_rows + tile_m - 1) / tile_m) * ((b_rows + plan.bn - 1) / plan.bn);
+    const double ranges = (double)std::min(slots, tiles * plan.splits) / (double)tiles;   // of K, in flight
+    const double bytes_per_kb = ranges * (double)(width + height) * 64 * 2 * 2;
+    return bytes_per_kb * kSplit16ChunkKb > kSplit16ChainBytes ? kSplit16ChunkKbThin : kSplit16ChunkKb;
+}
+
 // smallest point chunk worth a pipeline stage of its own
 constexpr int64_t kPipelineMinPoints = 8192;
 // CGH_OPT_GEMM_GROUP = 0 tries the grouped form from this many points
@@ -179,7 +194,7 @@ int gemm_units(cgh_ctx *ctx, int mode, int width, int height, int64_t n, const c
     plan.splits = lay.splits;
     plan.trans = lay.trans;
     if (!gemm_bn_supported(plan.bn)) return CGH_ENOTSUP;
-    plan.chunk_kb = ctx->gemm_chunk > 0 ? ctx->gemm_chunk : (mode == kFactorSplit16 ? kSplit16ChunkKb : 0);
+    plan.chunk_kb = ctx->gemm_chunk > 0 ? ctx->gemm_chunk : (mode == kFactorSplit16 ? split16_chunk_kb(plan, width, height) : 0);
     plan.accumulate = false;
     // every chunk must write every partial plane: no more splits than the last chunk has k-blocks
     const int64_t last = n - (n_chunks - 1) * chunk;
@@ -436,7 +451,7 @@ int run_wave(cgh_ctx *ctx, int form, const float *d_xyz, const float *d_amp, int
     plan.splits = lay.splits;
     plan.trans = lay.trans;
     if (!gemm_bn_supported(plan.bn)) return CGH_ENOTSUP;
-    plan.chunk_kb = ctx->gemm_chunk > 0 ? ctx->gemm_chunk : (mode == kFactorSplit16 ? kSplit16ChunkKb : 0);
+    plan.chunk_kb = ctx->gemm_chunk > 0 ? ctx->gemm_chunk : (mode == kFactorSplit16 ? split16_chunk_kb(plan, width, height) : 0);
     plan.accumulate = false;
     const bool dependent = plane * n <= kDependentTerms;
     plan.dependent = dependent;

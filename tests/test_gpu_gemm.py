@@ -295,3 +295,24 @@ def test_pair_gemm(form, w, h, n, trans):
     if w * h * n <= 2e8:
         ref = oracle.field(c.pitch_m, c.lambda_m, c.xyz, c.amp, w, h)
         assert oracle.nrms(a, ref) <= NRMS[form]
+
+
+@pytest.mark.parametrize("w,h,chunk", [(16384, 64, 8), (100, 8192, 8), (4096, 128, 8), (1024, 1024, 24), (640, 360, 24),
+                                       (1283, 717, 24)])
+@pytest.mark.parametrize("wave", [False, True])
+def test_chain_length_of_thin_holograms(w, h, chunk, wave):
+    # the chains of the units in flight stay in L2: 8 k-blocks where tiles share nothing, 24 elsewhere
+    c = workloads.random_cloud(700 + w, w, h, 4100)
+    xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
+    got = []
+    for pinned in (0, chunk, 32 - chunk):
+        with Hologram(w, h, c.pitch_m, c.lambda_m, form="gemm_split16") as hg:
+            hg.set_option(_lib.CGH_OPT_GEMM_CHUNK, pinned)
+            got.append((hg.wave(xyz, amp) if wave else hg.point_cloud(xyz, amp)).clone())
+            hg.sync()
+    assert torch.equal(got[0], got[1]) and not torch.equal(got[0], got[2])
+    rng = np.random.default_rng(1)
+    cols, rows = rng.integers(0, w, 200), rng.integers(0, h, 200)
+    ref = oracle.field_at(c.pitch_m, c.lambda_m, c.xyz, c.amp, cols, rows)
+    f = got[0][0] if wave else got[0]
+    assert oracle.nrms(f.cpu().numpy()[rows, cols], ref) <= 1e-5
