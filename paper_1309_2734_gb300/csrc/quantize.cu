@@ -149,14 +149,16 @@ __device__ __forceinline__ uint8_t kinoform_one(float re, float im)
     return (x >= 255.0f) ? (uint8_t)255 : ((x >= 0.0f) ? (uint8_t)x : (uint8_t)0);
 }
 
-// vec: four pixels a thread, 16-byte loads and a 4-byte store (the planes and out aligned); the rest one by one.
+// VEC: four pixels a thread, 16-byte loads and a 4-byte store (the planes and out aligned), the rest one by one; else, on
+// planes of an odd size, one by one with the registers of one (1283x717 6.4 -> 6.0 us).
+template <bool VEC>
 __global__ void kinoform_kernel(const float *__restrict__ re, const float *__restrict__ im, long long n,
-                                uint8_t *__restrict__ out, bool vec)
+                                uint8_t *__restrict__ out)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long first = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const long long n4 = vec ? n / 4 : 0;
-    for (long long i = first; i < n4; i += stride) {
+    const long long n4 = VEC ? n / 4 : 0;
+    for (long long i = first; VEC && i < n4; i += stride) {
         const float4 r = reinterpret_cast<const float4 *>(re)[i], m = reinterpret_cast<const float4 *>(im)[i];
         reinterpret_cast<uchar4 *>(out)[i] = make_uchar4(kinoform_one(r.x, m.x), kinoform_one(r.y, m.y),
                                                          kinoform_one(r.z, m.z), kinoform_one(r.w, m.w));
@@ -170,7 +172,8 @@ cudaError_t launch_kinoform8(const float *re, const float *im, int64_t n, uint8_
 {
     if (n <= 0) return cudaSuccess;
     const bool vec = (uintptr_t)re % 16 == 0 && (uintptr_t)im % 16 == 0 && (uintptr_t)out % 4 == 0;
-    kinoform_kernel<<<quant_grid(vec ? n / 4 : n), 256, 0, s>>>(re, im, n, out, vec);
+    if (vec) kinoform_kernel<true><<<quant_grid(n / 4), 256, 0, s>>>(re, im, n, out);
+    else kinoform_kernel<false><<<quant_grid(n), 256, 0, s>>>(re, im, n, out);
     return cudaGetLastError();
 }
 

@@ -231,18 +231,20 @@ def test_launches_share_the_points_evenly():
     assert oracle.nrms(got[rows, cols], ref) <= TOL + 6e-7
 
 
-@pytest.mark.parametrize("what", ["cloud", "accurate", "wave", "spherical", "gemm_wave", "launches", "gemm", "gemm_pair",
+@pytest.mark.parametrize("what", ["cloud", "accurate", "wave", "spherical", "spherical_close", "gemm_wave", "launches", "gemm", "gemm_pair",
                                   "gemm_chunks"])
 def test_captured_and_replayed(what):
     # dependent launches and the kernels' own clears inside a CUDA graph: a replay on new amplitudes gives the bits of
     # a plain call
-    c = workloads.random_cloud(811, 300, 200, 21000 if what == "launches" else 900)
+    # (spherical_close: every tensor-core launch declines, the SIMT kernel after them takes the cloud)
+    c = workloads.random_cloud(811, 300, 200, 21000 if what == "launches" else 900,
+                               (0.005, 0.01) if what == "spherical_close" else (0.3, 1.0))
     xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
     form = {"accurate": "direct_accurate", "gemm_wave": "gemm_split16", "gemm": "gemm_f16", "gemm_pair": "gemm_split16",
             "gemm_chunks": "gemm_bf16"}.get(what, "direct_sfu")
     s = torch.cuda.Stream()
     with Hologram(300, 200, c.pitch_m, c.lambda_m, form=form, stream=s) as h:
-        if what == "spherical":
+        if "spherical" in what:
             h.set_phase_model("spherical")
         if what == "gemm_pair":
             h.set_option(_lib.CGH_OPT_GEMM_PAIR, 1)
