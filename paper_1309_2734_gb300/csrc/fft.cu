@@ -556,21 +556,20 @@ __global__ void __launch_bounds__(1024) fft_rows_kernel(const float *__restrict_
     cp_async_wait_all();
     __syncthreads();
     rows_fft<MODE == kRowCrop>(sm, Lx, nseq, twx);
-    for (int q = 0; q < nseq; ++q) {
-        const int y = y0 + q;
-        if (y >= rows) break;
-        if (MODE == kRowCrop) {
+    const int live_rows = min(nseq, rows - y0);
+    if (MODE == kRowCrop) {
+        for (int q = 0; q < live_rows; ++q)
             for (int x = threadIdx.x; x < W; x += T) {
                 const float2 v = sm[saddr<kLayoutRows>(x, q, Lx, 0)];
-                out[(long long)y * W + x] = v.x;
-                out[plane + (long long)y * W + x] = v.y;
+                out[(long long)(y0 + q) * W + x] = v.x;
+                out[plane + (long long)(y0 + q) * W + x] = v.y;
             }
-        } else {
-            for (int x = threadIdx.x; x < Lx; x += T) {
-                const float2 v = sm[saddr<kLayoutRows>(x, q, Lx, 0)];
-                pad[(long long)y * Lx + x] = cmul(v, sx[x]);
-            }
-        }
+        return;
+    }
+    for (int x = threadIdx.x; x < Lx; x += T) {   // a column's factor once for the CTA's rows
+        const float2 f = sx[x];
+        for (int q = 0; q < live_rows; ++q)
+            pad[(long long)(y0 + q) * Lx + x] = cmul(sm[saddr<kLayoutRows>(x, q, Lx, 0)], f);
     }
 }
 
