@@ -797,8 +797,9 @@ cudaError_t launch_bn(int bn, const MmaArgs &g, int ctas, cudaStream_t s)
 
 // The totals take one FP32 addition per chain of 64 points, whose rounding grows with the square root of their number:
 // a launch adds at most kMmaLaunchPoints points of a tile in one CTA, and the next launch adds to its output
-// (2048x2048, 5 10^5 points: NRMS 4.3e-7; the SIMT kernel's 8.9e-7, one launch about 1.6e-6).  The groups are cut into
-// equal shares, so that with L > 1 launches each has at least groups / L > 320 ctas / tiles of them: every CTA has work.
+// (2048x2048, 5 10^5 points: NRMS 4.3e-7; the SIMT kernel's 8.9e-7, one launch about 1.6e-6).  Where the last launch
+// would be left with fewer groups than the CTAs need, the groups are cut into equal shares: with L > 1 launches each then
+// has at least groups / L > 320 ctas / tiles of them.
 int direct_mma_launches(const DirectMmaLayout &lay, int group, int64_t n_points)
 {
     const int64_t groups = (n_points + group - 1) / group;
@@ -816,7 +817,7 @@ cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4
         return cudaErrorInvalidValue;
     MmaArgs g{};
     const int launches = direct_mma_launches(lay, group, n_points);
-    const long long all_groups = (n_points + group - 1) / group;
+    const long long all_groups = (n_points + group - 1) / group, per = (all_groups + launches - 1) / launches;
     const int side_a = lay.a_rows ? height : width, side_b = lay.a_rows ? width : height;
     const int tb = lay.bn / planes;
     g.tiles_a = (side_a + kRowsA - 1) / kRowsA;
@@ -838,9 +839,11 @@ cudaError_t launch_direct_mma(const DirectMmaLayout &lay, int planes, const int4
     g.vec = width % 4 == 0 && (uintptr_t)out % 16 == 0 && ((long long)width * height) % 4 == 0;
     g.ref = ref;
     if (ext != nullptr && planes != 1) return cudaErrorInvalidValue;
-    for (long long k = 0; k < launches; ++k) {
-        const long long first = all_groups * k / launches;
-        g.groups = all_groups * (k + 1) / launches - first;
+    const bool even = tiles * ((all_groups - 1) % per + 1) < lay.ctas;
+    auto begin = [&](long long k) { return even ? all_groups * k / launches : std::min(all_groups, per * k); };
+    for (long long k = 0; begin(k) < all_groups; ++k) {
+        const long long first = begin(k);
+        g.groups = begin(k + 1) - first;
         g.units = tiles * g.groups;
         if (lay.ctas > g.units || g.units / lay.ctas >= 0x7ffffff0ll) return cudaErrorInvalidValue;
         g.geo = geo + first * group;

@@ -223,7 +223,7 @@ def test_point_split_beyond_the_point_tiles():
 
 
 def test_launches_share_the_points_evenly():
-    # 12 tiles of 480,943 groups on 13 CTAs: 694 launches, none with fewer groups than the CTAs need.  To the tolerance
+    # 12 tiles of 480,943 groups on 13 CTAs: 694 launches of 693 groups would leave the last one a single group.  To the tolerance
     # above come the launches' additions to the output, sqrt(694 / 2) 2^-25 = 5.6e-7
     c = workloads.random_cloud(611, 384, 896, 15390145)
     cols, rows, ref = _sampled(c, 24)
