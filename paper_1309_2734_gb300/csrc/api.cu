@@ -133,6 +133,13 @@ constexpr int64_t kPipelineMinPoints = 8192;
 // CGH_OPT_GEMM_GROUP = 0 tries the grouped form from this many points
 constexpr int64_t kGroupMinPoints = 65536;
 
+// Whether the GEMM forms look for points of one plane and column to group (with the piston, points of equal C may still
+// differ in depth).
+static bool may_group(const cgh_ctx *ctx, int64_t n)
+{
+    return !piston_on(ctx) && (ctx->gemm_group == 2 || (ctx->gemm_group == 0 && n >= kGroupMinPoints));
+}
+
 int factor_mode(int form)
 {
     return form == CGH_GEMM_BF16 ? kFactorBF16 : (form == CGH_GEMM_SPLIT16 ? kFactorSplit16 : kFactorF16);
@@ -319,8 +326,7 @@ int run_gemm(cgh_ctx *ctx, int form, int width, int height, double pitch, double
 {
     const int mode = factor_mode(form);
     const int64_t n_pad = padded_points(n);
-    // with the piston, points of equal C may still differ in depth: no grouping
-    bool try_group = !piston_on(ctx) && (ctx->gemm_group == 2 || (ctx->gemm_group == 0 && n >= kGroupMinPoints));
+    bool try_group = may_group(ctx, n);
     const PhaseRef ref = phase_ref(ctx);
     if (try_group) {   // the grouped form reads counts back: not while a graph is being captured
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -733,19 +739,20 @@ int wrp_record(cgh_ctx *ctx, const float *d_xyz, const float *d_amp, int64_t n, 
                                          planes, ctx->stream));
 }
 
-int resolve_form(cgh_ctx *ctx, int width, int height, int64_t n)
+// group: whether the call's GEMM forms may group points.
+int resolve_form(cgh_ctx *ctx, int width, int height, int64_t n, bool group)
 {
     if (ctx->phase_model == CGH_PHASE_SPHERICAL)   // one form computes Eq. 1
         return (ctx->form == CGH_FORM_AUTO || ctx->form == CGH_DIRECT_SFU) ? CGH_DIRECT_SFU : -1;
     if (ctx->form != CGH_FORM_AUTO) return ctx->form;
-    return tune_choose_form(ctx, width, height, n, (double)ctx->tol_e9 * 1e-9);
+    return tune_choose_form(ctx, width, height, n, (double)ctx->tol_e9 * 1e-9, group);
 }
 
 int compute_hologram(cgh_ctx *ctx, int width, int height, double pitch, double lambda, const float *d_xyz,
                      const float *d_amp, int64_t n, float *d_out)
 {
     if (n == 0) return cuda_status(cudaMemsetAsync(d_out, 0, (size_t)width * height * sizeof(float), ctx->stream));
-    const int form = resolve_form(ctx, width, height, n);
+    const int form = resolve_form(ctx, width, height, n, may_group(ctx, n));
     if (ctx->phase_model == CGH_PHASE_SPHERICAL)
         return form == CGH_DIRECT_SFU ? run_spherical(ctx, width, height, pitch, lambda, d_xyz, d_amp, n, 1, d_out)
                                       : CGH_ENOTSUP;
@@ -1087,7 +1094,7 @@ int cgh_wave(cgh_ctx *ctx, const float *d_xyz, const float *d_amp, int64_t n_poi
     DeviceGuard g(ctx->device);
     const int64_t plane = (int64_t)ctx->width * ctx->height;
     if (n_points == 0) return cuda_status(cudaMemsetAsync(d_out, 0, (size_t)2 * plane * sizeof(float), ctx->stream));
-    int form = resolve_form(ctx, ctx->width, ctx->height, n_points);
+    int form = resolve_form(ctx, ctx->width, ctx->height, n_points, false);
     if (ctx->phase_model == CGH_PHASE_SPHERICAL)
         return form == CGH_DIRECT_SFU ? run_spherical(ctx, ctx->width, ctx->height, ctx->pitch, ctx->lambda, d_xyz,
                                                       d_amp, n_points, 2, d_out)

@@ -273,7 +273,7 @@ int run_gemm(cgh_ctx *ctx, int form, int width, int height, double pitch, double
 int compute_hologram(cgh_ctx *ctx, int width, int height, double pitch, double lambda, const float *d_xyz,
                      const float *d_amp, int64_t n, float *d_out);
 int factor_mode(int form);
-int resolve_form(cgh_ctx *ctx, int width, int height, int64_t n);
+int resolve_form(cgh_ctx *ctx, int width, int height, int64_t n, bool group);
 int run_batch(cgh_ctx *ctx, const cgh_instance *inst, int n_inst);
 int batch_forms(const cgh_ctx *ctx, int *forms, int max_entries);
 int run_single_persistent(cgh_ctx *ctx, int form, const cgh_instance &inst);

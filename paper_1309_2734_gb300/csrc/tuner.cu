@@ -272,12 +272,12 @@ struct TuneState {
         int64_t n = 0;
         double tol = 0.0;
         int64_t budget_mb = 0;
-        bool batch = false;
+        bool gemm_only = false;
         int form = 0;
         bool same(const Choice &o) const
         {
             return width == o.width && height == o.height && n == o.n && tol == o.tol && budget_mb == o.budget_mb &&
-                   batch == o.batch;
+                   gemm_only == o.gemm_only;
         }
     } last;   // the choice of the call before: a program's holograms are mostly of one size
     std::map<std::string, int> bn;
@@ -595,19 +595,20 @@ double tune_predict(cgh_ctx *ctx, int form, int width, int height, int64_t n)
 // The persistent launch and the per-kind launches run direct units on the SIMT kernel, which the single hologram's times
 // say nothing about: there a GEMM form is taken wherever one is admissible.  Persistent launch, direct / split FP16:
 // 64 x 512x512, 2000 points 7386 / 539 us; 8 x 1920x1080, 100 points 424 / 90; 16 x 64x64, 100 points 42 / 33; the
-// direct form was ahead by 3 % at most (256 x 64x64, 100 points 287 / 295).
-int tune_choose_form(cgh_ctx *ctx, int width, int height, int64_t n, double tol, bool batch)
+// direct form was ahead by 3 % at most (256 x 64x64, 100 points 287 / 295).  And what grouping the points of a layered cloud
+// saves is not known beforehand: 512x512, 2 10^5 points on 16 planes 690 us direct, 690 split FP16, 270 grouped.
+int tune_choose_form(cgh_ctx *ctx, int width, int height, int64_t n, double tol, bool gemm_only)
 {
     if (tune_calibrate(ctx, false) != CGH_OK) return CGH_DIRECT_SFU;
     TuneState *t = state(ctx);
-    const TuneState::Choice key{width, height, n, tol, ctx->factor_budget_mb, batch, 0};
+    const TuneState::Choice key{width, height, n, tol, ctx->factor_budget_mb, gemm_only, 0};
     if (t->last.same(key)) return t->last.form;
     const int forms[5] = {CGH_DIRECT_SFU, CGH_DIRECT_ACCURATE, CGH_GEMM_F16, CGH_GEMM_BF16, CGH_GEMM_SPLIT16};
     int best = -1;
     double best_t = 1e300;
     for (int f : forms) {
         if (form_nrms_bound(f) > tol) continue;
-        if (batch && f < CGH_GEMM_F16 && tol >= form_nrms_bound(CGH_GEMM_SPLIT16)) continue;
+        if (gemm_only && f < CGH_GEMM_F16 && tol >= form_nrms_bound(CGH_GEMM_SPLIT16)) continue;
         const double tp = tune_predict(ctx, f, width, height, n);
         if (tp < best_t) {
             best_t = tp;

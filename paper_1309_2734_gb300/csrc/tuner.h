@@ -60,9 +60,9 @@ int choose_form(int width, int height, int64_t n_points, double tol, int num_sms
 int tune_calibrate(cgh_ctx *ctx, bool force);
 // Predicted seconds per hologram of a form.
 double tune_predict(cgh_ctx *ctx, int form, int width, int height, int64_t n);
-// Fastest admissible form by the calibrated model.  batch: for the batch's own launches, whose direct units are the
-// SIMT kernel's.
-int tune_choose_form(cgh_ctx *ctx, int width, int height, int64_t n, double tol, bool batch = false);
+// Fastest admissible form by the calibrated model.  gemm_only: a GEMM form where one is admissible -- the batch's own
+// launches, whose direct units are the SIMT kernel's, and clouds whose points the GEMM forms may group.
+int tune_choose_form(cgh_ctx *ctx, int width, int height, int64_t n, double tol, bool gemm_only);
 // Fastest GEMM tile width for a shape and form, timed on that shape.
 int tune_choose_bn(cgh_ctx *ctx, int width, int height, int form);
 

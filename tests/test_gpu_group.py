@@ -164,3 +164,20 @@ def test_layered_million_points_grouped_sampled(form):
         got = f[torch.from_numpy(rows).cuda(), torch.from_numpy(cols).cuda()].cpu().numpy()
     assert "group_factors" in names
     assert oracle.nrms(got, ref) <= NRMS[form]
+
+
+@pytest.mark.parametrize("w,h,n", [(512, 512, 100000), (640, 64, 200000), (512, 512, 65536)])
+def test_auto_leaves_layered_clouds_to_the_grouped_form(w, h, n):
+    # what grouping saves is not known when the form is chosen: from 65536 points on a GEMM form looks for it
+    c = workloads.layered_cloud(930 + w, w, h, n, 16)
+    xyz, amp = torch.from_numpy(c.xyz).cuda(), torch.from_numpy(c.amp).cuda()
+    with Hologram(w, h, c.pitch_m, c.lambda_m, form="auto") as hg:
+        _lib.check(_lib.cgh_autotune(hg.ctx, 0), "cgh_autotune")
+        hg.profile()
+        f = hg.point_cloud(xyz, amp)
+        hg.sync()
+        assert "group_factors" in hg.profile_read()
+    rng = np.random.default_rng(2)
+    cols, rows = rng.integers(0, w, 100), rng.integers(0, h, 100)
+    ref = oracle.field_at(c.pitch_m, c.lambda_m, c.xyz, c.amp, cols, rows)
+    assert oracle.nrms(f.cpu().numpy()[rows, cols], ref) <= 1e-5
