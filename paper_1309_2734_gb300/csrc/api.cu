@@ -213,6 +213,7 @@ int gemm_units(cgh_ctx *ctx, int mode, int width, int height, int64_t n, const c
     const size_t q_bytes = align_up((size_t)planes * width * ld_max * 2, 256);
     const size_t part_bytes = plan.splits > 1 ? (size_t)plan.splits * plane * sizeof(float) : 0;
     int rc = ensure(ctx, &ctx->ws, &ctx->ws_bytes, nbuf * (p_bytes + q_bytes) + part_bytes);
+    if (!rc && nbuf == 2) rc = ensure_side_stream(ctx);
     if (rc || ctx->reserve_only) return rc;
     char *fac = static_cast<char *>(ctx->ws);
     float *parts = reinterpret_cast<float *>(fac + nbuf * (p_bytes + q_bytes));
@@ -221,8 +222,6 @@ int gemm_units(cgh_ctx *ctx, int mode, int width, int height, int64_t n, const c
     // factors on the side stream when pipelining, else on the main stream
     cudaStream_t fs = ctx->stream;
     if (nbuf == 2) {
-        rc = ensure_side_stream(ctx);
-        if (rc) return rc;
         fs = ctx->side_stream;
         e = cudaEventRecord(ctx->ev_ready, ctx->stream);       // prep (and earlier work) done
         if (e == cudaSuccess) e = cudaStreamWaitEvent(fs, ctx->ev_ready, 0);
